@@ -137,8 +137,9 @@ int tpflbm_init(tpflbm_t h, const float *phi, const float *ux, const float *uy, 
 int tpflbm_init_forced(tpflbm_t h, const float *phi, const float *ux, const float *uy, const float *p,
                        const float *T, int which);
 
-/* Advance nsteps >= 0 time steps (one fused step-kernel launch each), enqueued
- * on the handle's stream; returns after enqueueing. */
+/* Advance nsteps >= 0 time steps, enqueued on the handle's stream; returns after
+ * enqueueing.  Each step is one fused kernel launch, except that a lattice of up to 304
+ * tiles of 32 x 8 nodes advances up to 1,024 steps per (cooperative) launch. */
 int tpflbm_step(tpflbm_t h, long long nsteps);
 
 /* Wait for the steps enqueued so far and report whether they completed: TPF_OK, or

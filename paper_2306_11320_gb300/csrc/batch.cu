@@ -87,8 +87,10 @@ k_step_batch(const InstDesc* __restrict__ inst, const int2* __restrict__ work, i
         const InstDesc& d = dsc[b];
         const typename S::elem* A = (const typename S::elem*)d.pop[parity];
         typename S::elem* B = (typename S::elem*)d.pop[parity ^ 1];
-        step_tile_general<BX, BY, S>(d.P, A, B, d.phiu, d.ref[parity], d.ref[parity ^ 1], sm, item.y & 0xffff,
-                                     item.y >> 16);
+        int x0, y0, tw, th;
+        tile_whole(d.P.nx, BX, item.y & 0xffff, x0, tw);
+        tile_whole(d.P.ny, BY, item.y >> 16, y0, th);
+        step_tile_general<BX, BY, S>(d.P, A, B, d.phiu, d.ref[parity], d.ref[parity ^ 1], sm, x0, y0, tw, th);
         // step_tile_general ends with a barrier: buffer b ^ 1 is free (its tile ended a
         // barrier ago), and after this one the next descriptor is visible
         if (wn < nwork && threadIdx.x < 32) store(b ^ 1);
@@ -241,9 +243,12 @@ k_step_batch_tma(const BatchTmaInst* __restrict__ inst, const int4* __restrict__
         if (tid == 0) gdesc = inst[item.x].d;
         __syncthreads();
         const DevParams& P = gdesc.P;
+        int x0, y0, tw, th;
+        tile_whole(P.nx, BX, item.y & 0xffff, x0, tw);
+        tile_whole(P.ny, BY, item.y >> 16, y0, th);
         step_tile_general<BX, BY, S>(P, (const E*)gdesc.pop[parity], (E*)gdesc.pop[parity ^ 1], gdesc.phiu,
                                      gdesc.ref[parity], gdesc.ref[parity ^ 1],
-                                     *reinterpret_cast<RingSmem<BX, BY>*>(dsm), item.y & 0xffff, item.y >> 16);
+                                     *reinterpret_cast<RingSmem<BX, BY>*>(dsm), x0, y0, tw, th);
         // step_tile_general ends with a barrier: gdesc is free again
     }
 }
@@ -431,7 +436,7 @@ int tpflbm_batch_create(int n, const int* nx, const int* ny, const tpflbm_params
     std::vector<InstDesc> desc(n);
     for (int k = 0; k < n; ++k) {
         tpflbm_t h = nullptr;
-        int rc = tpflbm_create(nx[k], ny[k], &params[k], &h);
+        int rc = tpf_create_member(nx[k], ny[k], &params[k], &h);
         if (rc != TPF_OK) {
             std::string why = std::string("lattice ") + std::to_string(k) + ": " + tpflbm_last_error(nullptr);
             tpflbm_batch_destroy(b);

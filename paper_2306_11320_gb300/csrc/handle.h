@@ -44,6 +44,12 @@ struct tpflbm {
     tpf::TmaMaps maps[2]{};             // maps[c]: reading pop[c]
     int bx0 = 0, by0 = 0, ntbx = 0, ntby = 0, grid_tma = 0;
     int2* tiles = nullptr;              // (x0, y0) of the TMA tiles in the order the kernel walks them
+    // many-step kernel (many_fn is null where the lattice does not take it): its tiles, the
+    // steps each has done, and the words they exchange
+    const void* many_fn = nullptr;
+    int many_tx = 0, many_ty = 0;
+    uint32_t* count = nullptr;
+    uint4* words = nullptr;
     // CUDA graphs of kGraphSteps steps starting from pop[0] / pop[1] (captured on first use)
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     // marks the steps enqueued so far for tpflbm_status_async's copy stream (created on first use)
@@ -51,3 +57,7 @@ struct tpflbm {
     long long t = 0;
     std::string err_msg;
 };
+
+// tpflbm_create for a member of an ensemble (without the many-step kernel's memory)
+extern "C" __attribute__((visibility("hidden"))) int tpf_create_member(int nx, int ny, const tpflbm_params* p,
+                                                                       tpflbm_t* out);

@@ -55,8 +55,15 @@ __device__ __forceinline__ float u_inlet(const DevParams& P, float y)
 
 // ---------------------------------------------------------------- storage
 
+// ld reads a population from global memory, lds from a staged copy in shared memory, st
+// stores it (st_dev: given its deviation from the reference too); through gives the value a
+// stored population decodes to.  Once: for a buffer that the same kernel writes later on.
+struct StoreF32Once;
+struct StoreF16Once;
 struct StoreF32 {
+    using Once = StoreF32Once;
     using elem = float;
+    static constexpr bool kRecords = false;
     // global memory (read-only path)
     template <class I>
     static __device__ __forceinline__ float ld(const float* __restrict__ p, I k, float, float) { return __ldg(p + k); }
@@ -65,9 +72,18 @@ struct StoreF32 {
     static __device__ __forceinline__ float lds(const float* p, I k, float, float) { return p[k]; }
     template <class I>
     static __device__ __forceinline__ void st(float* __restrict__ p, I k, float v, float, float) { p[k] = v; }
+    template <class I>
+    static __device__ __forceinline__ void st_dev(float* __restrict__ p, I k, float v, float, float) { p[k] = v; }
+    static __device__ __forceinline__ float through(float v, float, float, float, float) { return v; }
+};
+struct StoreF32Once : StoreF32 {
+    template <class I>
+    static __device__ __forceinline__ float ld(const float* p, I k, float, float) { return __ldcg(p + k); }
 };
 struct StoreF16 {
+    using Once = StoreF16Once;
     using elem = __half;
+    static constexpr bool kRecords = true;
     template <class I>
     static __device__ __forceinline__ float ld(const __half* __restrict__ p, I k, float inv_s, float ref)
     {
@@ -82,6 +98,23 @@ struct StoreF16 {
     static __device__ __forceinline__ void st(__half* __restrict__ p, I k, float v, float s, float ref)
     {
         p[k] = __float2half_rn((v - ref) * s);
+    }
+    template <class I>
+    static __device__ __forceinline__ void st_dev(__half* __restrict__ p, I k, float, float dev, float s)
+    {
+        p[k] = __float2half_rn(dev * s);
+    }
+    static __device__ __forceinline__ float through(float, float dev, float s, float inv_s, float ref)
+    {
+        return fmaf(__half2float(__float2half_rn(dev * s)), inv_s, ref);
+    }
+};
+
+struct StoreF16Once : StoreF16 {
+    template <class I>
+    static __device__ __forceinline__ float ld(const __half* p, I k, float inv_s, float ref)
+    {
+        return fmaf(__half2float(__ldcg(p + k)), inv_s, ref);
     }
 };
 

@@ -7,8 +7,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <type_traits>
-
 #include "lattice.cuh"
 
 namespace tpf {
@@ -30,7 +28,7 @@ namespace tpf {
 // halves; the writer encodes against the rounded record, so encoder and decoder see
 // the same reference bit for bit.
 template <class S>
-constexpr bool kRef = std::is_same<S, StoreF16>::value;
+constexpr bool kRef = S::kRecords;
 
 using RefT = uint2;  // one reference record: float32 zeroth moment, half2 first moment / cs2
 constexpr int kRecF = 0, kRecG = 1, kRecH = 2;  // record planes
@@ -71,6 +69,17 @@ __device__ __forceinline__ float ref_pop(int i, const RefVals& r)
 __device__ __forceinline__ float ref_g(int i, const RefVals& r)
 {
     return i == 0 ? wg(0) * r.m0 : fmaf(wg(i), r.m0, wq(i) * cdot(i, r.jx, r.jy));
+}
+
+// deviations v - ref_pop and v - ref_g with the reference's product in the same rounding
+// (the encoder's side)
+__device__ __forceinline__ float dev_pop(int i, const RefVals& r, float v)
+{
+    return i == 0 ? fmaf(-wq(0), r.m0, v) : fmaf(-wq(i), r.m0 + cdot(i, r.jx, r.jy), v);
+}
+__device__ __forceinline__ float dev_g(int i, const RefVals& r, float v)
+{
+    return i == 0 ? fmaf(-wg(0), r.m0, v) : v - ref_g(i, r);
 }
 
 // node that wrote population i at (x, y), whose record is its FP16 reference (for the
@@ -137,6 +146,77 @@ struct RingSmem {
     float h[9][SN];
 };
 
+// What lies one c_i away from node (x, y): the wall, the inlet, the outflow or node d.
+enum Link { kNode, kWall, kInlet, kOutflow };
+__device__ __forceinline__ Link link_of(const DevParams& P, int x, int y, int i, int& d)
+{
+    int dx = x + cx(i), dy = y + cy(i);
+    if (P.bc_x == 0) dx = wrap(dx, P.nx);
+    if (P.bc_y == 1) dy = wrap(dy, P.ny);
+    d = dy * P.nx + dx;
+    if (dy < 0 || dy >= P.ny) return kWall;
+    return dx < 0 ? kInlet : (dx >= P.nx ? kOutflow : kNode);
+}
+// temperature of the wall, and speed of the inlet, where link i of node (x, y) crosses it
+__device__ __forceinline__ float link_T_wall(const DevParams& P, int x, int i)
+{
+    const float xc = (float)x + 0.5f * cx(i);
+    return (cy(i) < 0) ? T_wall_bottom(P, xc) : T_wall_top(P, xc);
+}
+__device__ __forceinline__ float link_u_inlet(const DevParams& P, int y, int i)
+{
+    return u_inlet(P, (float)y + 0.5f + 0.5f * cy(i));
+}
+// the outflow's ghost column feeds node (x, y + c_iy) of the last column
+__device__ __forceinline__ bool link_copies(const DevParams& P, int x, int y, int i)
+{
+    return P.bc_x == 1 && x == P.nx - 1 && cx(i) < 0 && y + cy(i) >= 0 && y + cy(i) < P.ny;
+}
+// What the boundary sends back along link i as population o = opp(i): f and g, and h before
+// its Eq. 28 update.
+//   wall: halfway bounce-back of f and g; anti-bounce-back of h with the wall temperature
+__device__ __forceinline__ void wall_rule(int i, float Tw, float h, float& hin)
+{
+    hin = -h + 2.f * wq(opp(i)) * Tw;
+}
+//   velocity inlet: bounce-back carrying the inlet momentum and phi_in
+__device__ __forceinline__ void inlet_rule(const DevParams& P, int i, float u_in, float rho, float& f, float& g, float h,
+                                           float& hin)
+{
+    const int o = opp(i);
+    const float cu = cx(o) * u_in;
+    hin = -h + 2.f * wq(o) * P.T_in;
+    f = f + 2.f * wq(o) * P.phi_in * cu * kInvCs2;
+    g = g + 2.f * wq(o) * rho * cu * kInvCs2;
+}
+//   outflow: pressure anti-bounce-back of g (f and h arrive by the copy)
+__device__ __forceinline__ float outflow_rule(const DevParams& P, int i, const Macro& m, float g)
+{
+    const int o = opp(i);
+    const float cu = cx(o) * m.ux + cy(o) * m.uy;
+    const float sym = P.p_out * kInvCs2 +
+                      m.rho * (0.5f * cu * cu * kInvCs2 * kInvCs2 - 0.5f * (m.ux * m.ux + m.uy * m.uy) * kInvCs2);
+    return -g + 2.f * wq(o) * sym;
+}
+
+// The first-moment records of what a node emits (post-collision f, g, h; FP16), as the
+// decoder sees them; out(k, record) takes each.
+struct NodeRecords {
+    RefVals f{0.f, 0.f, 0.f}, g{0.f, 0.f, 0.f}, h{0.f, 0.f, 0.f};
+};
+template <class OUT>
+__device__ __forceinline__ void node_records(const Macro& m, const float* f, const float* g, const float* h,
+                                             NodeRecords& r, OUT out)
+{
+    float jfx, jfy, jgx, jgy, jhx, jhy;
+    dq9_moment1(f, jfx, jfy);
+    dq9_moment1(g, jgx, jgy);
+    dq9_moment1(h, jhx, jhy);
+    out(kRecF, ref_pack(m.phi, jfx * kInvCs2, jfy * kInvCs2, r.f));
+    out(kRecG, ref_pack(m.p * kInvCs2, jgx * kInvCs2, jgy * kInvCs2, r.g));
+    out(kRecH, ref_pack(m.T, jhx * kInvCs2, jhy * kInvCs2, r.h));
+}
+
 // Collide the node's populations and push them to their destinations, with every
 // boundary rule; for FP16 also leave the node's reference records in refB (every
 // population this node writes is encoded against them).  hold(i, k) and irc(k) give
@@ -149,26 +229,20 @@ __device__ __forceinline__ void collide_push(const DevParams& P, typename S::ele
     const long long pl = P.plane;
     const int n = y * P.nx + x;
     node_collide(P, m, f, g, h);
-    // FP16 reference records of what this node emits (as the decoder sees them)
-    RefVals rf{0.f, 0.f, 0.f}, rgv{0.f, 0.f, 0.f}, rh{0.f, 0.f, 0.f};
-    if constexpr (kRef<S>) {
-        float jfx, jfy, jgx, jgy, jhx, jhy;
-        dq9_moment1(f, jfx, jfy);
-        dq9_moment1(g, jgx, jgy);
-        dq9_moment1(h, jhx, jhy);
-        refB[kRecF * pl + n] = ref_pack(m.phi, jfx * kInvCs2, jfy * kInvCs2, rf);
-        refB[kRecG * pl + n] = ref_pack(m.p * kInvCs2, jgx * kInvCs2, jgy * kInvCs2, rgv);
-        refB[kRecH * pl + n] = ref_pack(m.T, jhx * kInvCs2, jhy * kInvCs2, rh);
-    }
+    NodeRecords r;
+    if constexpr (kRef<S>) node_records(m, f, g, h, r, [&](int k, RefT q) { refB[k * pl + n] = q; });
+    auto put_f = [&](int i, int d, float v) { S::st_dev(B + i * pl, d, v, dev_pop(i, r.f, v), P.s_f); };
+    auto put_g = [&](int i, int d, float v) { S::st_dev(B + (9 + i) * pl, d, v, dev_g(i, r.g, v), P.s_g); };
+    auto put_h = [&](int i, int d, float v) { S::st_dev(B + (18 + i) * pl, d, v, dev_pop(i, r.h, v), P.s_h); };
     if (interior) {
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
             const int d = n + cy(i) * P.nx + cx(i);
             const int kd = kown + cy(i) * SX + cx(i);
-            S::st(B + i * pl, d, f[i], P.s_f, ref_pop(i, rf));
-            S::st(B + (9 + i) * pl, d, g[i], P.s_g, ref_g(i, rgv));
+            put_f(i, d, f[i]);
+            put_g(i, d, g[i]);
             const float ho = hold(i, kd);
-            S::st(B + (18 + i) * pl, d, fmaf(h[i] - ho, irc(kd), ho), P.s_h, ref_pop(i, rh));
+            put_h(i, d, fmaf(h[i] - ho, irc(kd), ho));
         }
         return;
     }
@@ -176,96 +250,73 @@ __device__ __forceinline__ void collide_push(const DevParams& P, typename S::ele
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         const int o = opp(i);
-        int dx = x + cx(i), dy = y + cy(i);
-        if (P.bc_x == 0) dx = wrap(dx, P.nx);
-        if (P.bc_y == 1) dy = wrap(dy, P.ny);
-        const bool out_y = dy < 0 || dy >= P.ny;
-        const bool out_x = dx < 0 || dx >= P.nx;
-        if (out_y) {
-            // halfway bounce-back of f and g; anti-bounce-back of h with the wall
-            // temperature at the link's crossing point
-            const float xc = (float)x + 0.5f * cx(i);
-            const float Tw = (cy(i) < 0) ? T_wall_bottom(P, xc) : T_wall_top(P, xc);
-            S::st(B + o * pl, n, f[i], P.s_f, ref_pop(o, rf));
-            S::st(B + (9 + o) * pl, n, g[i], P.s_g, ref_g(o, rgv));
+        int d;
+        const Link link = link_of(P, x, y, i, d);
+        if (link == kWall || link == kInlet) {
+            float fo = f[i], go = g[i], hin;
+            if (link == kWall) wall_rule(i, link_T_wall(P, x, i), h[i], hin);
+            else inlet_rule(P, i, link_u_inlet(P, y, i), m.rho, fo, go, h[i], hin);
+            put_f(o, n, fo);
+            put_g(o, n, go);
             const float ho = hold(o, kown);
-            const float hin = -h[i] + 2.f * wq(o) * Tw;
-            S::st(B + (18 + o) * pl, n, fmaf(hin - ho, irc_own, ho), P.s_h, ref_pop(o, rh));
-        } else if (out_x && dx < 0) {
-            // velocity inlet: bounce-back carrying the inlet momentum and phi_in
-            const float ycr = (float)y + 0.5f + 0.5f * cy(i);
-            const float cu = cx(o) * u_inlet(P, ycr);
-            S::st(B + o * pl, n, f[i] + 2.f * wq(o) * P.phi_in * cu * kInvCs2, P.s_f, ref_pop(o, rf));
-            S::st(B + (9 + o) * pl, n, g[i] + 2.f * wq(o) * m.rho * cu * kInvCs2, P.s_g, ref_g(o, rgv));
-            const float ho = hold(o, kown);
-            const float hin = -h[i] + 2.f * wq(o) * P.T_in;
-            S::st(B + (18 + o) * pl, n, fmaf(hin - ho, irc_own, ho), P.s_h, ref_pop(o, rh));
-        } else if (out_x) {
-            // outflow: pressure anti-bounce-back of g (f and h arrive by the copy below)
-            const float cu = cx(o) * m.ux + cy(o) * m.uy;
-            const float sym = P.p_out * kInvCs2 +
-                              m.rho * (0.5f * cu * cu * kInvCs2 * kInvCs2 - 0.5f * (m.ux * m.ux + m.uy * m.uy) * kInvCs2);
-            S::st(B + (9 + o) * pl, n, -g[i] + 2.f * wq(o) * sym, P.s_g, ref_g(o, rgv));
+            put_h(o, n, fmaf(hin - ho, irc_own, ho));
+        } else if (link == kOutflow) {
+            put_g(o, n, outflow_rule(P, i, m, g[i]));
         } else {
-            const int d = dy * P.nx + dx;
             const int kd = kown + cy(i) * SX + cx(i);
-            S::st(B + i * pl, d, f[i], P.s_f, ref_pop(i, rf));
-            S::st(B + (9 + i) * pl, d, g[i], P.s_g, ref_g(i, rgv));
+            put_f(i, d, f[i]);
+            put_g(i, d, g[i]);
             const float ho = hold(i, kd);
-            S::st(B + (18 + i) * pl, d, fmaf(h[i] - ho, irc(kd), ho), P.s_h, ref_pop(i, rh));
+            put_h(i, d, fmaf(h[i] - ho, irc(kd), ho));
         }
         // zero-gradient outflow of f and h: the ghost column beyond x = nx-1 carries the
         // post-collision populations of the last column (this node wrote them, so they
         // are encoded against its own records).
-        if (P.bc_x == 1 && x == P.nx - 1 && cx(i) < 0) {
-            const int ey = y + cy(i);
-            if (ey >= 0 && ey < P.ny) {
-                const int d = ey * P.nx + x;
-                const int kd = kown + cy(i) * SX;
-                S::st(B + i * pl, d, f[i], P.s_f, ref_pop(i, rf));
-                const float ho = hold(i, kd);
-                S::st(B + (18 + i) * pl, d, fmaf(h[i] - ho, irc(kd), ho), P.s_h, ref_pop(i, rh));
-            }
+        if (link_copies(P, x, y, i)) {
+            const int dc = n + cy(i) * P.nx;
+            const int kd = kown + cy(i) * SX;
+            put_f(i, dc, f[i]);
+            const float ho = hold(i, kd);
+            put_h(i, dc, fmaf(h[i] - ho, irc(kd), ho));
         }
     }
 }
 
 // One tile through the general path: thread loads, ghost values and every boundary
 // rule.  Used for lattices whose rows do not meet TMA alignment, by the batched
-// ensemble, and in the TMA kernel for the tiles next to a periodic seam and the ragged
-// tiles.  (bx, by): tile coordinates.
+// ensemble, in the TMA kernel for the tiles next to a periodic seam and the ragged
+// tiles, and by the many-step kernel.  The tile covers nodes [x0, x0 + w) x [y0, y0 + h),
+// 1 <= w <= BX, 1 <= h <= BY.
+//
+// One thread per ring node issues that node's loads together with its own node's, so the
+// tile waits on one round trip to memory whatever its extent; ghost ring nodes take
+// their mirror's values from shared memory once those are in.
 template <int BX, int BY, class S>
 __device__ __forceinline__ void step_tile_general(const DevParams& P, const typename S::elem* __restrict__ A,
                                                   typename S::elem* __restrict__ B, float* __restrict__ phiu,
                                                   const RefT* __restrict__ refA, RefT* __restrict__ refB,
-                                                  RingSmem<BX, BY>& sm, int bx, int by)
+                                                  RingSmem<BX, BY>& sm, int x0, int y0, int w, int h_)
 {
-    constexpr int SX = RingSmem<BX, BY>::SX, SN = RingSmem<BX, BY>::SN;
+    constexpr int SX = RingSmem<BX, BY>::SX;
     const int tx = threadIdx.x % BX, ty = threadIdx.x / BX;
-    const int x0 = bx * BX, y0 = by * BY;
     const int x = x0 + tx, y = y0 + ty;
-    const bool active = x < P.nx && y < P.ny;
+    const bool active = tx < w && ty < h_;
     const long long pl = P.plane;
     const int n = y * P.nx + x;
     const int kown = (ty + 1) * SX + tx + 1;
-    const bool interior = x0 >= 1 && x0 + BX <= P.nx - 1 && y0 >= 1 && y0 + BY <= P.ny - 1;
+    const bool interior = x0 >= 1 && x0 + w <= P.nx - 1 && y0 >= 1 && y0 + h_ <= P.ny - 1;
 
-    // Whole tiles: one thread per ring node issues that node's loads together with the
-    // own node's, so the tile waits on one round trip to memory, and ghost ring nodes
-    // take their mirror's values from shared memory once those are in.  Ragged tiles
-    // walk every slot outside the lattice part of the tile.
     constexpr int kRing = 2 * (BX + BY) + 4;
     static_assert(kRing <= BX * BY, "one thread per ring node");
-    const bool whole = x0 + BX <= P.nx && y0 + BY <= P.ny;
     int rx = 0, ry = 0, wx = 0, wy = 0;
     bool rload = false, rghost = false;
     float ra[9], rc[9];
-    if (whole && (int)threadIdx.x < kRing) {
-        const int r = threadIdx.x;
-        if (r < SX) { rx = r; ry = 0; }
-        else if (r < 2 * SX) { rx = r - SX; ry = BY + 1; }
-        else if (r < 2 * SX + BY) { rx = 0; ry = r - 2 * SX + 1; }
-        else { rx = BX + 1; ry = r - 2 * SX - BY + 1; }
+    if ((int)threadIdx.x < 2 * (w + h_) + 4) {
+        const int r = threadIdx.x, sx = w + 2;
+        if (r < sx) { rx = r; ry = 0; }
+        else if (r < 2 * sx) { rx = r - sx; ry = h_ + 1; }
+        else if (r < 2 * sx + h_) { rx = 0; ry = r - 2 * sx + 1; }
+        else { rx = w + 1; ry = r - 2 * sx - h_ + 1; }
         wx = x0 + rx - 1;
         wy = y0 + ry - 1;
         if (P.bc_x == 0) wx = wrap(wx, P.nx);
@@ -290,84 +341,32 @@ __device__ __forceinline__ void step_tile_general(const DevParams& P, const type
 #pragma unroll
         for (int i = 0; i < 9; ++i) sm.h[i][kown] = h[i];
     }
-    if (whole) {
-        if (rload) {
-            const int k = ry * SX + rx;
-            float sf = 0.f, sh = 0.f;
+    if (rload) {
+        const int k = ry * SX + rx;
+        float sf = 0.f, sh = 0.f;
 #pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                sf += ra[i];
-                sh += rc[i];
-                sm.h[i][k] = rc[i];
-            }
-            sm.phi[k] = sf;
-            sm.T[k] = sh;
-            sm.irc[k] = __frcp_rn(fmaf(P.rcp_b, clamp1(sf), P.rcp_a));
+        for (int i = 0; i < 9; ++i) {
+            sf += ra[i];
+            sh += rc[i];
+            sm.h[i][k] = rc[i];
         }
-        // ghost ring nodes beyond walls, inlet and outflow (as phiT_at): phi mirrored,
-        // T by the boundary's rule; the mirror is the adjacent slot inside the lattice
-        if (__syncthreads_or(rghost) && rghost) {
-            const int gx = x0 + rx - 1, gy = y0 + ry - 1;
-            const int mx = min(max(wx, 0), P.nx - 1), my = min(max(wy, 0), P.ny - 1);
-            const int km = (ry + my - wy) * SX + rx + mx - wx;
-            const float tm = sm.T[km];
-            const float tx = (wx < 0) ? 2.f * P.T_in - tm : tm;
-            const bool oy = wy < 0 || wy >= P.ny;
-            const int k = ry * SX + rx;
-            sm.phi[k] = sm.phi[km];
-            sm.T[k] = oy ? 2.f * (wy < 0 ? T_wall_bottom(P, (float)gx) : T_wall_top(P, (float)gx)) - tx : tx;
-            sm.irc[k] = 0.f;
-            (void)gy;
-        }
-    } else {
-        auto get = [&](int gx, int gy, float& ph, float& tt) {
-            float a[9], c[9];
-            load_node<S, false>(P, A, refA, gx, gy, a, nullptr, c);
-            float sf = 0.f, sh = 0.f;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                sf += a[i];
-                sh += c[i];
-            }
-            ph = sf;
-            tt = sh;
-        };
-        for (int k = threadIdx.x; k < SN; k += BX * BY) {
-            const int lx = k % SX, ly = k / SX;
-            const bool own = lx >= 1 && lx <= BX && ly >= 1 && ly <= BY && (x0 + lx - 1) < P.nx && (y0 + ly - 1) < P.ny;
-            if (own) continue;
-            const int gx = x0 + lx - 1, gy = y0 + ly - 1;
-            int qx = gx, qy = gy;
-            if (P.bc_x == 0) qx = wrap(qx, P.nx);
-            if (P.bc_y == 1) qy = wrap(qy, P.ny);
-            const bool far = gx < -1 || gx > P.nx || gy < -1 || gy > P.ny;
-            if (far) {
-                sm.phi[k] = 0.f;
-                sm.T[k] = 0.f;
-                sm.irc[k] = 0.f;
-                continue;
-            }
-            if (qx >= 0 && qx < P.nx && qy >= 0 && qy < P.ny) {
-                float a[9], c[9];
-                load_node<S, false>(P, A, refA, qx, qy, a, nullptr, c);
-                float sf = 0.f, sh = 0.f;
-#pragma unroll
-                for (int i = 0; i < 9; ++i) {
-                    sf += a[i];
-                    sh += c[i];
-                    sm.h[i][k] = c[i];
-                }
-                sm.phi[k] = sf;
-                sm.T[k] = sh;
-                sm.irc[k] = __frcp_rn(fmaf(P.rcp_b, clamp1(sf), P.rcp_a));
-            } else {
-                float ph, tt;
-                phiT_at(P, gx, gy, get, ph, tt);
-                sm.phi[k] = ph;
-                sm.T[k] = tt;
-                sm.irc[k] = 0.f;
-            }
-        }
+        sm.phi[k] = sf;
+        sm.T[k] = sh;
+        sm.irc[k] = __frcp_rn(fmaf(P.rcp_b, clamp1(sf), P.rcp_a));
+    }
+    // ghost ring nodes beyond walls, inlet and outflow (as phiT_at): phi mirrored,
+    // T by the boundary's rule; the mirror is the adjacent slot inside the lattice
+    if (__syncthreads_or(rghost) && rghost) {
+        const int gx = x0 + rx - 1;
+        const int mx = min(max(wx, 0), P.nx - 1), my = min(max(wy, 0), P.ny - 1);
+        const int km = (ry + my - wy) * SX + rx + mx - wx;
+        const float tm = sm.T[km];
+        const float tg = (wx < 0) ? 2.f * P.T_in - tm : tm;
+        const bool oy = wy < 0 || wy >= P.ny;
+        const int k = ry * SX + rx;
+        sm.phi[k] = sm.phi[km];
+        sm.T[k] = oy ? 2.f * (wy < 0 ? T_wall_bottom(P, (float)gx) : T_wall_top(P, (float)gx)) - tg : tg;
+        sm.irc[k] = 0.f;
     }
     __syncthreads();
     if (active) {
@@ -387,6 +386,19 @@ __device__ __forceinline__ void step_tile_general(const DevParams& P, const type
     }
     __syncthreads();  // the caller may reuse sm for the next tile
 }
+// Tile b of an axis of n nodes: start and extent.  Whole tiles of B nodes first, the
+// ragged one last (tile_whole), or nt = ceil(n / B) tiles of nearly equal extent
+// (tile_even; at least B / 2 nodes each once nt > 1).
+__device__ __forceinline__ void tile_whole(int n, int B, int b, int& x0, int& w)
+{
+    x0 = b * B;
+    w = min(B, n - x0);
+}
+__device__ __forceinline__ void tile_even(int n, int nt, int b, int& x0, int& w)
+{
+    x0 = (int)((long long)b * n / nt);
+    w = (int)((long long)(b + 1) * n / nt) - x0;
+}
 
 template <int BX, int BY, class S>
 __global__ void __launch_bounds__(BX * BY, 3)
@@ -394,7 +406,422 @@ k_step_general(const DevParams P, const typename S::elem* __restrict__ A, typena
                float* __restrict__ phiu, const RefT* __restrict__ refA, RefT* __restrict__ refB)
 {
     __shared__ RingSmem<BX, BY> sm;
-    step_tile_general<BX, BY, S>(P, A, B, phiu, refA, refB, sm, blockIdx.x, blockIdx.y);
+    int x0, y0, w, h;
+    tile_even(P.nx, gridDim.x, blockIdx.x, x0, w);
+    tile_even(P.ny, gridDim.y, blockIdx.y, y0, h);
+    step_tile_general<BX, BY, S>(P, A, B, phiu, refA, refB, sm, x0, y0, w, h);
+}
+
+// ------------------------------------------------------- many steps per launch
+//
+// Lattices small enough that every tile has a CTA of its own on the GPU at once advance
+// many steps in one cooperative launch.  A step of such a lattice is latency: one launch
+// per step pays the kernel boundary and the kernel's start on top of the memory round trip
+// and the arithmetic.  Here each CTA keeps its tile's populations in shared memory from
+// the first step, which reads the population buffer A, to the last, which writes B; (phi u)
+// stays in registers.  B is the other buffer after an odd number of steps, and A itself
+// after an even one, as one launch per step would leave them: whoever reads a slot in the
+// first step has done so before the slot's writer gets through its second.
+//
+// What the tiles exchange goes through L2 as self-validating words: the populations i of
+// the three LBEs that arrive at a node (f_i, g_i, h_i) and the number of the step that
+// they begin, 16 bytes read and written as one.  A reader polls the word itself until the
+// number is right, so a step has no fence, no flag and no second round trip.  Words exist
+// for the nodes on the rim of each tile (slots of two sets of 9 planes, used in turn):
+// whoever pushes to such a node writes the word, its tile reads the ones that came from
+// outside, and the tiles that have the node in their ring read all nine, for its phi, T
+// and h_i.  A slot is written again two steps later by a tile that has by then received
+// a push of the step between from every tile that reads the slot (they lie within two
+// nodes of the writer), so it has been read.
+//
+// FP16 storage: a population is rounded through its code as it is emitted and travels
+// decoded (the writer knows the reference), so that a step gives the very values that the
+// one-step kernels store, without records in between.
+//
+// What a step costs (512 x 128, in cycles of a CTA): the words' way through L2 and the
+// slowest neighbour 3,700, the moments 900, the macroscopic state 1,000, collisions and
+// pushes 2,200; it is bound by this chain, not by bandwidth (about 5 MB of words per step).
+// Measured against one launch per step (us/step, same process): 128 x 32 5.4 -> 2.8, 512 x
+// 128 6.7 -> 3.7, 160 x 320 6.4 -> 3.6, 331 x 117 5.5 -> 3.5; FP16 7.8 -> 3.3, 10.3 -> 4.3,
+// 10.6 -> 4.3, 12.7 -> 4.4.  Tried: step counters per tile with release/acquire and the
+// populations in L2 (4.3 and 5.3 at 128 x 32 and 512 x 128); 32 x 4 tiles (3.8, 5.6: each
+// thread then reads twice the words); testing the kind of each link in turn instead of
+// masks (3.4, 4.1).
+//
+// The waits are bounded: a CTA that gives up raises err and returns, and so do the
+// others, which look at err now and then; with err up no later launch starts.
+
+__device__ __forceinline__ uint4 ld_word(const uint4* p)
+{
+    unsigned long long lo, hi;
+    asm volatile("{\n .reg .b128 t;\n ld.relaxed.gpu.global.b128 t, [%2];\n mov.b128 {%0, %1}, t;\n}\n"
+                 : "=l"(lo), "=l"(hi)
+                 : "l"(p));
+    return make_uint4((uint32_t)lo, (uint32_t)(lo >> 32), (uint32_t)hi, (uint32_t)(hi >> 32));
+}
+__device__ __forceinline__ void st_word(uint4* p, float f, float g, float h, uint32_t tag)
+{
+    const unsigned long long lo = ((unsigned long long)__float_as_uint(g) << 32) | __float_as_uint(f);
+    const unsigned long long hi = ((unsigned long long)tag << 32) | __float_as_uint(h);
+    asm volatile("{\n .reg .b128 t;\n mov.b128 t, {%1, %2};\n st.relaxed.gpu.global.b128 [%0], t;\n}\n" ::"l"(p),
+                 "l"(lo), "l"(hi));
+}
+
+constexpr uint32_t kWordWaitLimit = 1u << 22;  // polls, about half a microsecond each
+
+// Shared memory of one tile: the populations of its nodes and its ring (of the ring
+// nodes f and h), their phi, T and 1/(rho c_p), the list of words it reads, and per node
+// what its links need: the slots of the words it writes, wall temperatures (by c_ix) and
+// inlet velocities (by c_iy) at the crossing points.
+template <int BX, int BY>
+struct ManySmem {
+    static constexpr int SX = BX + 2, SN = (BX + 2) * (BY + 2), NT = BX * BY;
+    static constexpr int kRing = 2 * (BX + BY) + 4;
+    static constexpr int kWords = 9 * kRing + 6 * (BX + BY);
+    float f[9][SN], g[9][SN], h[9][SN];
+    float phi[SN], T[SN], irc[SN];
+    uint2 word[kWords];  // x: slot in a word set; y: i * SN + ring slot, bit 31: g_i is used too
+    uint32_t slot[9][NT];
+    float Tw[3][NT], uin[3][NT];
+    int nwords;
+};
+
+// A node's links, worked out once per launch: bit i of each mask.
+struct TileMasks {
+    uint32_t wall, inlet, outflow, copies;
+    uint32_t inside;  // what lies one c_i away is a node of the tile
+    uint32_t rim;     // it is a node on the rim of its tile
+};
+
+// Collide a node and push its populations: into the tile's shared memory, and as words of
+// step `tag` into set `out` for nodes on a rim.  The slot of population i at a node is read
+// (as h_i before the step) and written by the one node that pushes to it.
+template <class S, class SM>
+__device__ __forceinline__ void tile_push(const DevParams& P, const TileMasks& M, SM& sm, uint4* out, uint32_t tag,
+                                          int kown, const Macro& m, float* f, float* g, float* h)
+{
+    const int tid = threadIdx.x;
+    node_collide(P, m, f, g, h);
+    NodeRecords r;
+    if constexpr (kRef<S>) node_records(m, f, g, h, r, [](int, RefT) {});
+    auto thru_f = [&](int i, float v) { return S::through(v, dev_pop(i, r.f, v), P.s_f, P.is_f, ref_pop(i, r.f)); };
+    auto thru_g = [&](int i, float v) { return S::through(v, dev_g(i, r.g, v), P.s_g, P.is_g, ref_g(i, r.g)); };
+    auto thru_h = [&](int i, float v) { return S::through(v, dev_pop(i, r.h, v), P.s_h, P.is_h, ref_pop(i, r.h)); };
+    auto word = [&](int i, int j, float vf, float vg, float vh) {
+        st_word(out + (uint32_t)(i * (int)P.plane) + sm.slot[j][tid], vf, vg, vh, tag);
+    };
+    if (M.wall | M.inlet | M.outflow) {
+#pragma unroll
+        for (int i = 1; i < 9; ++i) {
+            const int o = opp(i);
+            if ((M.wall | M.inlet) >> i & 1) {
+                float vf = f[i], vg = g[i], hin;
+                if (M.wall >> i & 1) wall_rule(i, sm.Tw[cx(i) + 1][tid], h[i], hin);
+                else inlet_rule(P, i, sm.uin[cy(i) + 1][tid], m.rho, vf, vg, h[i], hin);
+                const float hold = sm.h[o][kown];
+                vf = thru_f(o, vf);
+                vg = thru_g(o, vg);
+                const float vh = thru_h(o, fmaf(hin - hold, sm.irc[kown], hold));
+                sm.f[o][kown] = vf;
+                sm.g[o][kown] = vg;
+                sm.h[o][kown] = vh;
+                if (M.rim & 1) word(o, 0, vf, vg, vh);
+            } else if (M.outflow >> i & 1) {
+                sm.g[o][kown] = thru_g(o, outflow_rule(P, i, m, g[i]));
+            }
+            if (cx(i) < 0 && M.copies >> i & 1) {
+                const int j = cy(i) == 0 ? 0 : (cy(i) > 0 ? 2 : 4);  // the copy's destination: a node of the column
+                const int kd = kown + cy(i) * SM::SX;
+                const float hold = sm.h[i][kd];
+                const float vf = thru_f(i, f[i]), vh = thru_h(i, fmaf(h[i] - hold, sm.irc[kd], hold));
+                if (M.inside >> j & 1) {
+                    sm.f[i][kd] = vf;
+                    sm.h[i][kd] = vh;
+                }
+                if (M.rim >> j & 1) word(i, j, vf, 0.f, vh);
+            }
+        }
+    }
+    // links to nodes: everything is read before anything is written (the compiler cannot
+    // tell the slots apart), and the words, which other tiles wait for, go first
+    float ho[9], ic[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const int kd = kown + cy(i) * SM::SX + cx(i);
+        ho[i] = sm.h[i][kd];
+        ic[i] = sm.irc[kd];
+    }
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        f[i] = thru_f(i, f[i]);
+        g[i] = thru_g(i, g[i]);
+        h[i] = thru_h(i, fmaf(h[i] - ho[i], ic[i], ho[i]));
+    }
+    if (M.rim) {
+        uint32_t slot[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) slot[i] = sm.slot[i][tid];
+#pragma unroll
+        for (int i = 0; i < 9; ++i)
+            if (M.rim >> i & 1) st_word(out + (uint32_t)(i * (int)P.plane) + slot[i], f[i], g[i], h[i], tag);
+    }
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const int kd = kown + cy(i) * SM::SX + cx(i);
+        if (M.inside >> i & 1) {
+            sm.f[i][kd] = f[i];
+            sm.g[i][kd] = g[i];
+            sm.h[i][kd] = h[i];
+        }
+    }
+}
+
+template <int BX, int BY, class S>
+__global__ void __launch_bounds__(BX * BY, 512 / (BX * BY))
+k_step_many(const DevParams P, const typename S::elem* A, typename S::elem* B, float* phiu, const RefT* refA, RefT* refB,
+            uint4* words, uint32_t* count, int ntx, int nty, int nsteps, int* err)
+{
+    using SM = ManySmem<BX, BY>;
+    constexpr int SX = SM::SX, SN = SM::SN, NT = BX * BY;
+    constexpr int kPerThread = (SM::kWords + NT - 1) / NT;
+    static_assert(2 * SM::kRing <= NT, "one thread per ring moment");
+    extern __shared__ __align__(128) unsigned char dsm[];
+    SM& sm = *reinterpret_cast<SM*>(dsm);
+    const int tid = threadIdx.x;
+    int x0, y0, w, h_;
+    tile_even(P.nx, ntx, blockIdx.x % ntx, x0, w);
+    tile_even(P.ny, nty, blockIdx.x / ntx, y0, h_);
+    const long long pl = P.plane;
+    // steps this tile has done, ever (the same for all tiles between launches): the
+    // numbers of this launch's words start after it
+    const uint32_t base = count[blockIdx.x];
+    const int e0 = *(volatile int*)err;
+    if (tid == 0) sm.nwords = 0;
+    if (__syncthreads_or(e0)) return;
+
+    const int tx = tid % BX, ty = tid / BX;
+    const int x = x0 + tx, y = y0 + ty;
+    const bool active = tx < w && ty < h_;
+    const int n = y * P.nx + x;
+    const int kown = (ty + 1) * SX + tx + 1;
+    const bool interior = x0 >= 1 && x0 + w <= P.nx - 1 && y0 >= 1 && y0 + h_ <= P.ny - 1;
+    const int nring = 2 * (w + h_) + 4;
+    // slot (rx, ry) of ring node r; true when it lies inside the lattice, at (wx, wy)
+    auto ring_node = [&](int r, int& rx, int& ry, int& wx, int& wy) {
+        const int sx = w + 2;
+        if (r < sx) { rx = r; ry = 0; }
+        else if (r < 2 * sx) { rx = r - sx; ry = h_ + 1; }
+        else if (r < 2 * sx + h_) { rx = 0; ry = r - 2 * sx + 1; }
+        else { rx = w + 1; ry = r - 2 * sx - h_ + 1; }
+        wx = x0 + rx - 1;
+        wy = y0 + ry - 1;
+        if (P.bc_x == 0) wx = wrap(wx, P.nx);
+        if (P.bc_y == 1) wy = wrap(wy, P.ny);
+        return wx >= 0 && wx < P.nx && wy >= 0 && wy < P.ny;
+    };
+    // this thread's moment of the ring: thread r takes phi (and 1/(rho c_p)), thread
+    // kRing + r takes T, of ring slot kr.  Ghost nodes beyond walls, inlet and outflow sum
+    // their mirror's populations (the adjacent slot inside the lattice, km) and follow
+    // phiT_at: phi is mirrored; T is 2 T_wall - T at a wall, 2 T_in - T at the inlet.
+    const bool ring_h = tid >= SM::kRing;
+    const int ring = ring_h ? tid - SM::kRing : tid;
+    int kr = -1, km = 0;
+    bool ghost = false, g_in = false, g_wall = false;
+    float gT2 = 0.f;  // twice the wall's temperature
+    if (ring < nring) {
+        int rx, ry, wx, wy;
+        ghost = !ring_node(ring, rx, ry, wx, wy);
+        kr = km = ry * SX + rx;
+        if (ghost) {
+            const int mx = min(max(wx, 0), P.nx - 1), my = min(max(wy, 0), P.ny - 1);
+            km = (ry + my - wy) * SX + rx + mx - wx;
+            g_in = wx < 0;
+            g_wall = wy < 0 || wy >= P.ny;
+            const int gx = x0 + rx - 1;
+            if (g_wall) gT2 = 2.f * (wy < 0 ? T_wall_bottom(P, (float)gx) : T_wall_top(P, (float)gx));
+        }
+    }
+
+    // the words this tile reads: all nine of each ring node, and of its own nodes those
+    // that arrive from outside the tile (at the outflow, f and h of the last column come
+    // from the column's other nodes)
+    {
+        auto append = [&](bool take, uint2 v) {
+            const unsigned m = __ballot_sync(0xffffffffu, take);
+            int at = 0;
+            if ((tid & 31) == 0 && m) at = atomicAdd(&sm.nwords, __popc(m));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (take) sm.word[at + __popc(m & ((1u << (tid & 31)) - 1u))] = v;
+        };
+        const int rr = (9 * nring + NT - 1) / NT;
+        for (int j = 0; j < rr; ++j) {
+            const int idx = tid + j * NT, i = idx / nring;
+            int rx = 0, ry = 0, wx = 0, wy = 0;
+            bool take = i < 9 && ring_node(idx - i * nring, rx, ry, wx, wy);
+            append(take, make_uint2((uint32_t)(i * pl + (long long)wy * P.nx + wx), (uint32_t)(i * SN + ry * SX + rx)));
+        }
+        for (int i = 1; i < 9; ++i) {
+            const int lx = tx - cx(i), ly = ty - cy(i);  // the source, in the tile's coordinates
+            int sx = x - cx(i), sy = y - cy(i);
+            if (P.bc_x == 0) sx = wrap(sx, P.nx);
+            if (P.bc_y == 1) sy = wrap(sy, P.ny);
+            const bool in_y = sy >= 0 && sy < P.ny;
+            const bool out_tile = lx < 0 || lx >= w || ly < 0 || ly >= h_;
+            const bool copied = sx >= P.nx;  // outflow: written by (nx - 1, sy)
+            const bool take = active && in_y && sx >= 0 && (copied ? (ly < 0 || ly >= h_) : out_tile);
+            append(take, make_uint2((uint32_t)(i * pl + n), (uint32_t)(i * SN + kown) | (copied ? 0u : 1u << 31)));
+        }
+    }
+    TileMasks M{0, 0, 0, 0, 0, 0};
+    if (active) {
+#pragma unroll
+        for (int j = 0; j < 9; ++j) {
+            const int lx = tx + cx(j), ly = ty + cy(j);
+            const bool in = lx >= 0 && lx < w && ly >= 0 && ly < h_;
+            int d;
+            const Link link = link_of(P, x, y, j, d);
+            M.wall |= (uint32_t)(link == kWall) << j;
+            M.inlet |= (uint32_t)(link == kInlet) << j;
+            M.outflow |= (uint32_t)(link == kOutflow) << j;
+            M.copies |= (uint32_t)link_copies(P, x, y, j) << j;
+            M.inside |= (uint32_t)(link == kNode && in) << j;
+            M.rim |= (uint32_t)(link == kNode && (!in || lx == 0 || lx == w - 1 || ly == 0 || ly == h_ - 1)) << j;
+            sm.slot[j][tid] = (uint32_t)d;
+            if (link == kWall) sm.Tw[cx(j) + 1][tid] = link_T_wall(P, x, j);
+            if (link == kInlet) sm.uin[cy(j) + 1][tid] = link_u_inlet(P, y, j);
+        }
+    }
+
+    float pu_x = 0.f, pu_y = 0.f;
+    if (active) {
+        pu_x = phiu[n];
+        pu_y = phiu[pl + n];
+    }
+    // first step: the populations from the buffer
+    int rx, ry, wx, wy;
+    if (tid < nring && ring_node(tid, rx, ry, wx, wy)) {
+        float ra[9], rc[9];
+        load_node<typename S::Once, false>(P, A, refA, wx, wy, ra, nullptr, rc);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            sm.f[i][kr] = ra[i];
+            sm.h[i][kr] = rc[i];
+        }
+    }
+    if (active) {
+        float f[9], g[9], h[9];
+        load_node<typename S::Once>(P, A, refA, x, y, f, g, h);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            sm.f[i][kown] = f[i];
+            sm.g[i][kown] = g[i];
+            sm.h[i][kown] = h[i];
+        }
+    }
+    __syncthreads();
+    const int nwords = sm.nwords;
+    uint2 rd[kPerThread];  // the words this thread reads
+#pragma unroll
+    for (int j = 0; j < kPerThread; ++j)
+        rd[j] = tid + j * NT < nwords ? sm.word[tid + j * NT] : make_uint2(0, 0);
+
+    for (int s = 0; s < nsteps; ++s) {
+        if (s > 0) {
+            bool ok = true;
+            // the words of this step, written by the tiles around during the last one
+            const uint32_t tag = base + (uint32_t)s;
+            const uint4* in = words + (size_t)(tag & 1) * 9 * pl;
+            uint4 v[kPerThread];
+            bool all = true;
+#pragma unroll
+            for (int j = 0; j < kPerThread; ++j) v[j].w = tag - 1;
+            for (uint32_t it = 1;; ++it) {
+#pragma unroll
+                for (int j = 0; j < kPerThread; ++j)
+                    if (tid + j * NT < nwords && v[j].w != tag) v[j] = ld_word(in + rd[j].x);
+                all = true;
+#pragma unroll
+                for (int j = 0; j < kPerThread; ++j) all = all && (tid + j * NT >= nwords || v[j].w == tag);
+                if (all) break;
+                if (it >= kWordWaitLimit || ((it & 1023) == 0 && *(volatile int*)err)) {
+                    ok = false;
+                    break;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < kPerThread; ++j) {
+                if (tid + j * NT >= nwords) continue;
+                const uint32_t at = rd[j].y & 0x7fffffffu;
+                (&sm.f[0][0])[at] = __uint_as_float(v[j].x);
+                if (rd[j].y >> 31) (&sm.g[0][0])[at] = __uint_as_float(v[j].y);
+                (&sm.h[0][0])[at] = __uint_as_float(v[j].z);
+            }
+            if (__syncthreads_or(!ok)) {
+                if (tid == 0) atomicExch(err, 1);
+                return;
+            }
+        }
+        float f[9], g[9], h[9], sf = 0.f, sh = 0.f, sr = 0.f;
+        {
+            const float(*rq)[SN] = ring_h ? sm.h : sm.f;
+            float q[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                f[i] = sm.f[i][kown];
+                g[i] = sm.g[i][kown];
+                h[i] = sm.h[i][kown];
+                q[i] = kr >= 0 ? rq[i][km] : 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                sf += f[i];
+                sh += h[i];
+                sr += q[i];
+            }
+        }
+        if (active) {
+            sm.phi[kown] = sf;
+            sm.T[kown] = sh;
+            sm.irc[kown] = __frcp_rn(fmaf(P.rcp_b, clamp1(sf), P.rcp_a));
+        }
+        if (kr >= 0) {
+            if (!ring_h) {
+                sm.phi[kr] = sr;
+                sm.irc[kr] = ghost ? 0.f : __frcp_rn(fmaf(P.rcp_b, clamp1(sr), P.rcp_a));
+            } else {
+                if (g_in) sr = 2.f * P.T_in - sr;
+                if (g_wall) sr = gT2 - sr;
+                sm.T[kr] = sr;
+            }
+        }
+        __syncthreads();
+        if (active) {
+            float phin[9], Tn[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const int k = kown + cy(i) * SX + cx(i);
+                phin[i] = sm.phi[k];
+                Tn[i] = sm.T[k];
+            }
+            const Macro m = node_macro(P, f, g, h, phin, Tn, pu_x, pu_y);
+            pu_x = m.phi * m.ux;
+            pu_y = m.phi * m.uy;
+            if (s + 1 < nsteps) {
+                const uint32_t tag = base + (uint32_t)s + 1;
+                tile_push<S>(P, M, sm, words + (size_t)(tag & 1) * 9 * pl, tag, kown, m, f, g, h);
+            } else {
+                collide_push<S, SX>(
+                    P, B, refB, x, y, kown, interior, m, f, g, h, [&](int i, int k) { return sm.h[i][k]; },
+                    [&](int k) { return sm.irc[k]; });
+            }
+        }
+        __syncthreads();
+    }
+    if (active) {
+        phiu[n] = pu_x;
+        phiu[pl + n] = pu_y;
+    }
+    if (tid == 0) count[blockIdx.x] = base + (uint32_t)nsteps;
 }
 
 // ------------------------------------------------------------ TMA kernel
@@ -861,7 +1288,11 @@ k_step_tma(const DevParams P, const __grid_constant__ TmaMaps maps, const typena
             const bool inner = by >= by0 && by < by0 + ntby;
             bx = (inner && idx >= bx0) ? idx + ntbx : idx;
         }
-        step_tile_general<BX, BY, S>(P, A, B, phiu, refA, refB, *reinterpret_cast<RingSmem<BX, BY>*>(dsm), bx, by);
+        int x0, y0, w, h;
+        tile_whole(P.nx, BX, bx, x0, w);
+        tile_whole(P.ny, BY, by, y0, h);
+        step_tile_general<BX, BY, S>(P, A, B, phiu, refA, refB, *reinterpret_cast<RingSmem<BX, BY>*>(dsm), x0, y0, w,
+                                     h);
     }
 }
 

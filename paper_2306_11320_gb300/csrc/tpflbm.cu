@@ -477,16 +477,31 @@ namespace {
 thread_local std::string g_create_error;
 
 constexpr int kStagePlanes = 9;
+// Many-step kernel: lattices of at most kManyMaxTiles tiles of kManyBX x kManyBY nodes, two
+// CTAs on each of 152 SMs (its registers allow no more: the line lies where the tiles stop
+// having a CTA each; setup_many checks it against the device).  kManySteps steps per launch,
+// so that no launch holds the GPU for more than a few milliseconds.
+constexpr int kManyBX = 32, kManyBY = 8;
+constexpr int kManyMaxTiles = 2 * 152;
+constexpr long long kManySteps = 1024;
+bool many_tiles(int nx, int ny, int& tx, int& ty)
+{
+    tx = (nx + kManyBX - 1) / kManyBX;
+    ty = (ny + kManyBY - 1) / kManyBY;
+    return (long long)tx * ty <= kManyMaxTiles;
+}
 
 size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
 long long plane_of(int nx, int ny) { return (((long long)nx * ny + 63) / 64) * 64; }
 
 struct Layout {
-    size_t pop0, pop1, ref0, ref1, phiu, stage, red, err, snap, tiles, total;
+    size_t pop0, pop1, ref0, ref1, phiu, stage, red, err, snap, tiles, count, words, total;
 };
 
-Layout layout_of(int nx, int ny, int storage)
+// `many`: with the word sets of the many-step kernel, for lattices small enough for it (the
+// members of an ensemble, which is stepped as a whole, do without)
+Layout layout_of(int nx, int ny, int storage, bool many)
 {
     const long long pl = plane_of(nx, ny);
     const bool f16 = storage == TPF_STORAGE_FP16;
@@ -504,6 +519,11 @@ Layout layout_of(int nx, int ny, int storage)
     L.snap = off; off = align256(off + 3 * (size_t)pl * 4);
     // the TMA step kernel's tile list (x0, y0 per tile)
     L.tiles = off; off = align256(off + (size_t)((nx + kBX - 1) / kBX) * ((ny + kBY - 1) / kBY) * sizeof(int2));
+    // the many-step kernel's step counts per tile and its two word sets
+    int mtx = 0, mty = 0;
+    const bool words = many && many_tiles(nx, ny, mtx, mty);
+    L.count = off; off = align256(off + (words ? (size_t)mtx * mty * sizeof(uint32_t) : 0));
+    L.words = off; off = align256(off + (words ? 18 * (size_t)pl * sizeof(uint4) : 0));
     L.total = off;
     return L;
 }
@@ -717,13 +737,31 @@ void setup_tma(tpflbm_t h)
     h->tma = true;
 }
 
-int finish_create(tpflbm_t h, int nx, int ny, const tpflbm_params* p, void* ws, size_t bytes, bool owns)
+// The many-step kernel, for lattices whose tiles all have a CTA on the GPU at once.
+template <class S>
+void setup_many(tpflbm_t h)
+{
+    using SM = ManySmem<kManyBX, kManyBY>;
+    const auto fn = k_step_many<kManyBX, kManyBY, S>;
+    if (!many_tiles(h->nx, h->ny, h->many_tx, h->many_ty)) return;
+    int coop = 0, per_sm = 0;
+    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device) != cudaSuccess || !coop ||
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SM)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kManyBX * kManyBY, sizeof(SM)) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    if (h->many_tx * h->many_ty <= per_sm * h->num_sms) h->many_fn = (const void*)fn;
+}
+
+int finish_create(tpflbm_t h, int nx, int ny, const tpflbm_params* p, void* ws, size_t bytes, bool owns,
+                  bool many)
 {
     h->nx = nx; h->ny = ny; h->hp = *p;
     h->dp = make_dev_params(nx, ny, *p);
     cudaGetDevice(&h->device);
     cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
-    const Layout L = layout_of(nx, ny, p->storage);
+    const Layout L = layout_of(nx, ny, p->storage, many);
     h->ws = ws; h->ws_bytes = bytes; h->owns = owns;
     char* b = (char*)ws;
     h->pop[0] = b + L.pop0;
@@ -736,9 +774,19 @@ int finish_create(tpflbm_t h, int nx, int ny, const tpflbm_params* p, void* ws, 
     h->err = (int*)(b + L.err);
     h->snap = (float*)(b + L.snap);
     h->tiles = (int2*)(b + L.tiles);
+    h->count = (uint32_t*)(b + L.count);
+    h->words = (uint4*)(b + L.words);
     if (cudaMemset(h->err, 0, sizeof(int)) != cudaSuccess) return cuda_fail(h, cudaGetLastError(), "cudaMemset");
-    if (p->storage == TPF_STORAGE_FP16) setup_tma<StoreF16>(h);
+    const bool f16 = p->storage == TPF_STORAGE_FP16;
+    if (f16) setup_tma<StoreF16>(h);
     else setup_tma<StoreF32>(h);
+    if (many && L.total > L.count) {
+        // steps are numbered from 1: no word of a new lattice is valid
+        if (cudaMemset(h->count, 0, L.total - L.count) != cudaSuccess)
+            return cuda_fail(h, cudaGetLastError(), "cudaMemset");
+        if (f16) setup_many<StoreF16>(h);
+        else setup_many<StoreF32>(h);
+    }
     return TPF_OK;
 }
 
@@ -760,6 +808,21 @@ void launch_step(tpflbm_t h)
         k_step_general<kBX, kBY, S><<<grd, kBX * kBY, 0, h->stream>>>(P, A, B, h->phiu, h->ref[c], h->ref[c ^ 1]);
     }
     h->cur ^= 1;
+}
+
+// n steps of a lattice that takes the many-step kernel, in one launch
+cudaError_t launch_many(tpflbm_t h, int n)
+{
+    const int c = h->cur, d = c ^ (n & 1);
+    void *A = h->pop[c], *B = h->pop[d];
+    RefT *rA = h->ref[c], *rB = h->ref[d];
+    void* args[] = {&h->dp,   &A,        &B,          &h->phiu,    &rA, &rB,
+                    &h->words, &h->count, &h->many_tx, &h->many_ty, &n,  &h->err};
+    const cudaError_t e =
+        cudaLaunchCooperativeKernel(h->many_fn, dim3(h->many_tx * h->many_ty), dim3(kManyBX * kManyBY), args,
+                                    sizeof(ManySmem<kManyBX, kManyBY>), h->stream);
+    if (e == cudaSuccess) h->cur = d;
+    return e;
 }
 
 // error raised by a step kernel (bounded waits that ran out)
@@ -825,17 +888,17 @@ size_t tpflbm_workspace_bytes(int nx, int ny, const tpflbm_params* p)
 {
     std::string why;
     if (validate(nx, ny, p, why) != TPF_OK) return 0;
-    return layout_of(nx, ny, p->storage).total;
+    return layout_of(nx, ny, p->storage, true).total;
 }
 
-int tpflbm_create(int nx, int ny, const tpflbm_params* p, tpflbm_t* out)
+static int create_impl(int nx, int ny, const tpflbm_params* p, bool many, tpflbm_t* out)
 {
     if (!out) return fail(nullptr, TPF_ERR_INVALID_ARG, "out is NULL");
     *out = nullptr;
     std::string why;
     int rc = validate(nx, ny, p, why);
     if (rc != TPF_OK) return fail(nullptr, rc, why);
-    const size_t bytes = layout_of(nx, ny, p->storage).total;
+    const size_t bytes = layout_of(nx, ny, p->storage, many).total;
     void* ws = nullptr;
     cudaError_t e = cudaMalloc(&ws, bytes);
     if (e != cudaSuccess) {
@@ -848,7 +911,7 @@ int tpflbm_create(int nx, int ny, const tpflbm_params* p, tpflbm_t* out)
         cudaFree(ws);
         return fail(nullptr, TPF_ERR_OOM, "host allocation failed");
     }
-    rc = finish_create(h, nx, ny, p, ws, bytes, true);
+    rc = finish_create(h, nx, ny, p, ws, bytes, true, many);
     if (rc != TPF_OK) {
         g_create_error = h->err_msg;
         cudaFree(ws);
@@ -859,6 +922,13 @@ int tpflbm_create(int nx, int ny, const tpflbm_params* p, tpflbm_t* out)
     return TPF_OK;
 }
 
+int tpflbm_create(int nx, int ny, const tpflbm_params* p, tpflbm_t* out) { return create_impl(nx, ny, p, true, out); }
+
+int tpf_create_member(int nx, int ny, const tpflbm_params* p, tpflbm_t* out)
+{
+    return create_impl(nx, ny, p, false, out);
+}
+
 int tpflbm_create_in(int nx, int ny, const tpflbm_params* p, void* workspace, size_t bytes, tpflbm_t* out)
 {
     if (!out) return fail(nullptr, TPF_ERR_INVALID_ARG, "out is NULL");
@@ -867,10 +937,10 @@ int tpflbm_create_in(int nx, int ny, const tpflbm_params* p, void* workspace, si
     int rc = validate(nx, ny, p, why);
     if (rc != TPF_OK) return fail(nullptr, rc, why);
     if (!workspace || ((uintptr_t)workspace & 255)) return fail(nullptr, TPF_ERR_INVALID_ARG, "workspace must be 256-byte aligned device memory");
-    if (bytes < layout_of(nx, ny, p->storage).total) return fail(nullptr, TPF_ERR_INVALID_ARG, "workspace too small");
+    if (bytes < layout_of(nx, ny, p->storage, true).total) return fail(nullptr, TPF_ERR_INVALID_ARG, "workspace too small");
     tpflbm_t h = new (std::nothrow) tpflbm;
     if (!h) return fail(nullptr, TPF_ERR_OOM, "host allocation failed");
-    rc = finish_create(h, nx, ny, p, workspace, bytes, false);
+    rc = finish_create(h, nx, ny, p, workspace, bytes, false, true);
     if (rc != TPF_OK) {
         g_create_error = h->err_msg;
         delete h;
@@ -931,6 +1001,15 @@ int tpflbm_init_forced(tpflbm_t h, const float* phi, const float* ux, const floa
 int tpflbm_step(tpflbm_t h, long long nsteps)
 {
     if (!h || nsteps < 0) return TPF_ERR_INVALID_ARG;
+    if (h->many_fn) {
+        while (nsteps > 0) {
+            const int n = (int)(nsteps < kManySteps ? nsteps : kManySteps);
+            TPF_CUDA(h, launch_many(h, n));
+            nsteps -= n;
+            h->t += n;
+        }
+        return TPF_OK;
+    }
     // whole chunks from a CUDA graph when the stream can be captured (not the legacy
     // default stream); kGraphSteps is even, so a chunk leaves the parity unchanged
     while (h->stream && nsteps >= kGraphSteps) {
