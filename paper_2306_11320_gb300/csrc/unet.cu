@@ -412,7 +412,11 @@ k_conv3x3_wgrad(const bf16* __restrict__ x, const bf16* __restrict__ dz, int N, 
 // coordinates, never on the innermost (channel) one, so every copy starts on a
 // 16-byte boundary.  Same roles as the forward kernel: one thread copies, one thread
 // issues tcgen05.mma (FP32 accumulator in 64 TMEM columns), four warps read TMEM and
-// add into dW.
+// add into dW.  db[co] += sum_p dz[p][co] is summed by the two warps left over, from the
+// staged dz boxes, in the CTAs of the first tap group and input-channel tile (partial sums
+// per 64-pixel stage, so no longer chains of additions than 64 and the stages of a CTA).  As a
+// kernel of its own, one thread per channel and pixel range, it read dz again and took
+// 9.6 us beside the 25 us of the weight gradient at (4, 64, 256, 64, 64).
 constexpr int kWgStages = 4;
 constexpr int kWgPix = 64;   // pixels per K step (one row segment)
 // taps per CTA: one, or the three rows (dh) of one column offset (dw), which share their
@@ -431,7 +435,7 @@ __device__ __forceinline__ uint64_t mnmajor_desc(uint32_t addr, uint32_t lbo)
 template <int TAPS>
 __global__ void __launch_bounds__(128, 1)
 k_conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap mdz, const __grid_constant__ CUtensorMap mx, int N, int H,
-                   int W, int Cin, int Cout, int chunks_per_cta, float* __restrict__ dw)
+                   int W, int Cin, int Cout, int chunks_per_cta, float* __restrict__ dw, float* __restrict__ db)
 {
     static_assert(TAPS == 1 || TAPS == 3, "one tap, or the three rows of one column offset");
     constexpr int kBlk = kWgPix * 128;      // one 64-channel x 64-pixel box
@@ -454,11 +458,12 @@ k_conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap mdz, const __grid_constan
     const int c_begin = split * chunks_per_cta;
     const int c_end = min(c_begin + chunks_per_cta, nchunks);
     const int ksteps = c_end > c_begin ? c_end - c_begin : 0;
+    const bool bias = db && g == 0 && blockIdx.y == 0;
 
     if (tid == 0) {
         for (int s = 0; s < kWgStages; ++s) {
             mb_init(&full[s], 1);
-            mb_init(&empty[s], 1);
+            mb_init(&empty[s], bias ? 3 : 1);  // the MMAs and, with the bias, its two warps
         }
         mb_init(&done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -524,6 +529,35 @@ k_conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap mdz, const __grid_constan
         }
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(sa(&done))
                      : "memory");
+    } else if (warp >= 2 && bias) {
+        // warp 2 + q sums box q, lane l its channels 2 l and 2 l + 1: 16-byte piece l / 4 of
+        // the 128-byte rows, which the swizzle puts at piece (l / 4) ^ (pixel % 8)
+        const int q = warp - 2, cb = co0 + 64 * q + 2 * lane;
+        float b0 = 0.f, b1 = 0.f;
+        for (int k = 0; k < ksteps; ++k) {
+            const int s = k % kWgStages;
+            if (!mb_wait(&full[s], (k / kWgStages) & 1)) break;
+            if (co0 + 64 * q < Cout) {
+                const unsigned char* a = st0 + s * kStage + q * kBlk + 4 * (lane & 3);
+                float p0 = 0.f, p1 = 0.f;
+#pragma unroll 16
+                for (int p = 0; p < kWgPix; ++p) {
+                    const float2 v = __bfloat1622float2(
+                        *reinterpret_cast<const __nv_bfloat162*>(a + 128 * p + 16 * ((lane >> 2) ^ (p & 7))));
+                    p0 += v.x;
+                    p1 += v.y;
+                }
+                b0 += p0;
+                b1 += p1;
+            }
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sa(&empty[s])) : "memory");
+        }
+        if (cb < Cout) {  // (Cout is even)
+            atomicAdd(db + cb, b0);
+            atomicAdd(db + cb + 1, b1);
+        }
     }
     __syncwarp();
 
@@ -552,17 +586,6 @@ k_conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap mdz, const __grid_constan
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
 }
 
-// db[co] += sum_p dz[p][co]: one thread per channel per pixel range
-__global__ void k_bias_grad(const bf16* __restrict__ dz, long long P, int Cout, long long per, float* __restrict__ db)
-{
-    const int co = blockIdx.x * blockDim.x + threadIdx.x;
-    if (co >= Cout) return;
-    const long long p0 = (long long)blockIdx.y * per, p1 = p0 + per < P ? p0 + per : P;
-    float acc = 0.f;
-    for (long long p = p0; p < p1; ++p) acc += __bfloat162float(dz[p * Cout + co]);
-    atomicAdd(db + co, acc);
-}
-
 // flipped transpose for the data gradient: wd[tap][ci][co] = w[8 - tap][co][ci]
 __global__ void k_flip_weights(const bf16* __restrict__ w, int Cin, int Cout, bf16* __restrict__ wd)
 {
@@ -572,6 +595,137 @@ __global__ void k_flip_weights(const bf16* __restrict__ w, int Cin, int Cout, bf
         const long long r = k / Cout;
         const int ci = (int)(r % Cin), tap = (int)(r / Cin);
         wd[k] = w[((size_t)(8 - tap) * Cout + co) * Cin + ci];
+    }
+}
+
+// The element-wise kernels come in two forms: eight channels (one 16-byte piece) per thread
+// where every channel count and offset is a multiple of eight and every tensor 16-byte
+// aligned (all of the network's calls), and one element per thread for the rest.  They
+// move memory and nothing else; the scalar forms spent their time on 2-byte accesses and
+// 64-bit divisions per element (batch 4 at 512 x 128: upsampling the last level 98 us, now
+// see below).
+struct Piece {
+    float v[8];
+};
+__device__ __forceinline__ Piece ld8(const bf16* p)
+{
+    const uint4 q = *reinterpret_cast<const uint4*>(p);
+    const uint32_t u[4] = {q.x, q.y, q.z, q.w};
+    Piece r;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {  // bf16 is the upper half of float32
+        r.v[2 * j] = __uint_as_float(u[j] << 16);
+        r.v[2 * j + 1] = __uint_as_float(u[j] & 0xffff0000u);
+    }
+    return r;
+}
+__device__ __forceinline__ void st8(bf16* p, const Piece& r)
+{
+    uint32_t u[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const __nv_bfloat162 t = __floats2bfloat162_rn(r.v[2 * j], r.v[2 * j + 1]);
+        u[j] = *reinterpret_cast<const uint32_t*>(&t);
+    }
+    *reinterpret_cast<uint4*>(p) = make_uint4(u[0], u[1], u[2], u[3]);
+}
+// zero where the mask's element is not positive
+__device__ __forceinline__ void relu_back8(Piece& d, const Piece& y)
+{
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        if (!(y.v[j] > 0.f)) d.v[j] = 0.f;
+}
+
+__global__ void k_relu_mask8(bf16* __restrict__ d, const bf16* __restrict__ y, long long pieces)
+{
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < pieces; k += (long long)gridDim.x * blockDim.x) {
+        Piece v = ld8(d + 8 * k);
+        relu_back8(v, ld8(y + 8 * k));
+        st8(d + 8 * k, v);
+    }
+}
+// The image kernels below: blockIdx.y walks the rows (of all images), threads the pieces of
+// a row; C8 pieces per pixel.
+__global__ void k_pool8(const bf16* __restrict__ x, int rows, int W, int C8, bf16* __restrict__ y)
+{
+    const int Wo = W / 2, C = 8 * C8;
+    for (int r = blockIdx.y; r < rows; r += gridDim.y)  // output row: image rows 2 r, 2 r + 1
+        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < Wo * C8; k += gridDim.x * blockDim.x) {
+            const int w = k / C8, c = 8 * (k - w * C8);
+            const bf16* b = x + ((size_t)2 * r * W + 2 * w) * C + c;
+            const Piece p0 = ld8(b), p1 = ld8(b + C), p2 = ld8(b + (size_t)W * C), p3 = ld8(b + (size_t)W * C + C);
+            Piece o;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) o.v[j] = 0.25f * (p0.v[j] + p1.v[j] + p2.v[j] + p3.v[j]);
+            st8(y + ((size_t)r * Wo + w) * C + c, o);
+        }
+}
+// rows: coarse rows; one thread serves the 2 x 2 fine pixels of a coarse one
+__global__ void k_pool_back8(const bf16* __restrict__ dy, int rows, int W, int C8, bf16* __restrict__ dx, int accumulate)
+{
+    const int Wo = W / 2, C = 8 * C8;
+    for (int r = blockIdx.y; r < rows; r += gridDim.y)
+        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < Wo * C8; k += gridDim.x * blockDim.x) {
+            const int w = k / C8, c = 8 * (k - w * C8);
+            const Piece g = ld8(dy + ((size_t)r * Wo + w) * C + c);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                bf16* d = dx + ((size_t)(2 * r + q / 2) * W + 2 * w + q % 2) * C + c;
+                Piece v, old;
+                if (accumulate) old = ld8(d);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v.v[j] = accumulate ? 0.25f * g.v[j] + old.v[j] : 0.25f * g.v[j];
+                st8(d, v);
+            }
+        }
+}
+__global__ void k_up_into8(const bf16* __restrict__ x, int rows, int W, int C8, bf16* __restrict__ y, int Ctot, int cofs)
+{
+    const int Wo = W / 2, C = 8 * C8;
+    for (int r = blockIdx.y; r < rows; r += gridDim.y)
+        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < Wo * C8; k += gridDim.x * blockDim.x) {
+            const int w = k / C8, c = 8 * (k - w * C8);
+            const uint4 v = *reinterpret_cast<const uint4*>(x + ((size_t)r * Wo + w) * C + c);
+            bf16* d = y + ((size_t)2 * r * W + 2 * w) * Ctot + cofs + c;
+            *reinterpret_cast<uint4*>(d) = v;
+            *reinterpret_cast<uint4*>(d + Ctot) = v;
+            *reinterpret_cast<uint4*>(d + (size_t)W * Ctot) = v;
+            *reinterpret_cast<uint4*>(d + (size_t)W * Ctot + Ctot) = v;
+        }
+}
+__global__ void k_up_back8(const bf16* __restrict__ dy, int rows, int W, int Ctot, int cofs, int C8, bf16* __restrict__ dx)
+{
+    const int Wo = W / 2, C = 8 * C8;
+    for (int r = blockIdx.y; r < rows; r += gridDim.y)
+        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < Wo * C8; k += gridDim.x * blockDim.x) {
+            const int w = k / C8, c = 8 * (k - w * C8);
+            const bf16* b = dy + ((size_t)2 * r * W + 2 * w) * Ctot + cofs + c;
+            const Piece p0 = ld8(b), p1 = ld8(b + Ctot), p2 = ld8(b + (size_t)W * Ctot),
+                        p3 = ld8(b + (size_t)W * Ctot + Ctot);
+            Piece o;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) o.v[j] = p0.v[j] + p1.v[j] + p2.v[j] + p3.v[j];
+            st8(dx + ((size_t)r * Wo + w) * C + c, o);
+        }
+}
+__global__ void k_channels8(const bf16* __restrict__ src, int Sc, int sofs, long long pixels, int C8,
+                            bf16* __restrict__ dst, int Dc, int dofs, int accumulate)
+{
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < pixels * C8; k += (long long)gridDim.x * blockDim.x) {
+        const long long p = k / C8;
+        const int c = 8 * (int)(k - p * C8);
+        const bf16* a = src + p * Sc + sofs + c;
+        bf16* d = dst + p * Dc + dofs + c;
+        if (!accumulate) {
+            *reinterpret_cast<uint4*>(d) = *reinterpret_cast<const uint4*>(a);
+            continue;
+        }
+        Piece v = ld8(a);
+        const Piece old = ld8(d);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v.v[j] += old.v[j];
+        st8(d, v);
     }
 }
 
@@ -659,6 +813,110 @@ __global__ void k_channels(const bf16* __restrict__ src, int Sc, int sofs, long 
     }
 }
 
+// The head with one pixel per thread: its C channels in 16-byte pieces, the weights in
+// shared memory, the outputs of a block leaving through shared memory in one run.  C a
+// multiple of 8, at most 8 outputs, 16-byte aligned x.
+template <int CO>
+__global__ void __launch_bounds__(256)
+k_head8(const bf16* __restrict__ x, long long pixels, int C, const float* __restrict__ Wt, const float* __restrict__ b,
+        float* __restrict__ out)
+{
+    extern __shared__ float shw[];  // C x CO weights, then 256 x CO outputs
+    float* sho = shw + C * CO;
+    for (int k = threadIdx.x; k < C * CO; k += 256) shw[k] = Wt[k];
+    float bo[CO];
+#pragma unroll
+    for (int o = 0; o < CO; ++o) bo[o] = b[o];
+    __syncthreads();
+    for (long long p0 = blockIdx.x * 256LL; p0 < pixels; p0 += gridDim.x * 256LL) {
+        const long long p = p0 + threadIdx.x;
+        if (p < pixels) {
+            float s[CO];
+#pragma unroll
+            for (int o = 0; o < CO; ++o) s[o] = bo[o];
+            for (int c = 0; c < C; c += 8) {
+                const Piece v = ld8(x + p * C + c);
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+#pragma unroll
+                    for (int o = 0; o < CO; ++o) s[o] = fmaf(v.v[j], shw[(c + j) * CO + o], s[o]);
+            }
+#pragma unroll
+            for (int o = 0; o < CO; ++o) sho[threadIdx.x * CO + o] = s[o];
+        }
+        __syncthreads();
+        const int m = (int)(pixels - p0 < 256 ? pixels - p0 : 256) * CO;
+        for (int k = threadIdx.x; k < m; k += 256) out[p0 * CO + k] = sho[k];
+        __syncthreads();
+    }
+}
+// Head gradients, C = 8 G with G a power of two up to 32: lane l of a warp holds channels
+// 8 (l % G) .. + 7 of pixel l / G, their weights and the FP32 partial sums of dW and db in
+// registers over all its pixels; shuffles, shared memory and one atomic per block and
+// parameter add them up.  Bound by reading x and dout and writing dx.  (Adding every
+// pixel's products into shared memory with atomics serialised each warp on the same C x CO
+// words: 1,147 us at 262,144 pixels, C = 32, 5 outputs.)
+template <int CO>
+__global__ void __launch_bounds__(256)
+k_head_back8(const bf16* __restrict__ x, const float* __restrict__ dout, long long pixels, int C,
+             const float* __restrict__ Wt, bf16* __restrict__ dx, float* __restrict__ dW, float* __restrict__ db)
+{
+    extern __shared__ float sh[];  // C * CO + CO sums
+    const int G = C >> 3, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int cg = lane & (G - 1), ps = lane / G, PP = 32 / G;
+    float w[8][CO], acc[8][CO], accb[CO];
+#pragma unroll
+    for (int o = 0; o < CO; ++o) {
+        accb[o] = 0.f;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            w[j][o] = Wt[(8 * cg + j) * CO + o];
+            acc[j][o] = 0.f;
+        }
+    }
+    for (int k = threadIdx.x; k < (C + 1) * CO; k += 256) sh[k] = 0.f;
+    __syncthreads();
+    for (long long p = ((long long)blockIdx.x * 8 + warp) * PP + ps; p < pixels; p += (long long)gridDim.x * 8 * PP) {
+        float d[CO];
+#pragma unroll
+        for (int o = 0; o < CO; ++o) d[o] = dout[p * CO + o];
+        const Piece v = ld8(x + p * C + 8 * cg);
+        Piece r;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            float s = 0.f;
+#pragma unroll
+            for (int o = 0; o < CO; ++o) {
+                s = fmaf(d[o], w[j][o], s);
+                acc[j][o] = fmaf(v.v[j], d[o], acc[j][o]);
+            }
+            r.v[j] = s;
+        }
+        st8(dx + p * C + 8 * cg, r);
+#pragma unroll
+        for (int o = 0; o < CO; ++o) accb[o] += d[o];
+    }
+    for (int m = G; m < 32; m <<= 1) {
+#pragma unroll
+        for (int o = 0; o < CO; ++o) {
+            accb[o] += __shfl_xor_sync(0xffffffffu, accb[o], m);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[j][o] += __shfl_xor_sync(0xffffffffu, acc[j][o], m);
+        }
+    }
+    if (ps == 0) {
+#pragma unroll
+        for (int o = 0; o < CO; ++o) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) atomicAdd(&sh[(8 * cg + j) * CO + o], acc[j][o]);
+            if (cg == 0) atomicAdd(&sh[C * CO + o], accb[o]);
+        }
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < C * CO; k += 256) atomicAdd(&dW[k], sh[k]);
+    for (int k = threadIdx.x; k < CO; k += 256) atomicAdd(&db[k], sh[C * CO + k]);
+}
+
 // 1x1 head: out[p][o] = b[o] + sum_c x[p][c] W[c][o] (FP32 weights and output)
 __global__ void k_head(const bf16* __restrict__ x, long long pixels, int C, const float* __restrict__ Wt,
                        const float* __restrict__ b, int Cout, float* __restrict__ out)
@@ -698,7 +956,7 @@ __global__ void k_head_back(const bf16* __restrict__ x, const float* __restrict_
 }
 
 // mean squared error with channel weights; grad = d loss / d pred; loss accumulated in FP64
-__global__ void k_mse(const float* __restrict__ pred, const float* __restrict__ target, const float* __restrict__ wch,
+__global__ void __launch_bounds__(256) k_mse(const float* __restrict__ pred, const float* __restrict__ target, const float* __restrict__ wch,
                       long long count, int C, float* __restrict__ grad, double* __restrict__ loss)
 {
     double acc = 0.0;
@@ -710,7 +968,15 @@ __global__ void k_mse(const float* __restrict__ pred, const float* __restrict__ 
         if (grad) grad[k] = 2.f * d * wc * inv;
     }
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, acc / (double)count);
+    // one atomic per block: they queue up on the one word (one per warp of 1,024 blocks took
+    // 19 us at 1.3 M elements)
+    __shared__ double part[8];
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) acc += part[w];
+        atomicAdd(loss, acc / (double)count);
+    }
 }
 
 // Adam on FP32 master weights, refreshing the bf16 copy used by the convolutions
@@ -768,6 +1034,15 @@ int grid_of(long long count)
     long long b = (count + 255) / 256;
     return (int)(b < 152 * 32 ? (b < 1 ? 1 : b) : 152 * 32);
 }
+
+// whether tensors and channel counts allow 16-byte pieces
+template <class... P>
+bool pieces(int channels, P... p)
+{
+    return channels % 8 == 0 && ((... | (uintptr_t)p) & 15) == 0;
+}
+// grid of the row kernels: `per_row` pieces in each of `rows` rows
+dim3 grid_rows(int rows, int per_row) { return dim3((per_row + 255) / 256, rows < 65535 ? rows : 65535); }
 
 int status(cudaError_t e) { return e == cudaSuccess ? TPF_OK : TPF_ERR_CUDA; }
 
@@ -906,13 +1181,9 @@ bool wgrad_tc(const bf16* x, const bf16* dz, int N, int H, int W, int Cin, int C
     splits = (nchunks + per - 1) / per;
     dim3 grd(ctiles, itiles, (9 / taps) * (unsigned)splits);
     if (taps == 3)
-        k_conv3x3_wgrad_tc<3><<<grd, 128, smem, s>>>(mdz, mx, N, H, W, Cin, Cout, (int)per, dw);
+        k_conv3x3_wgrad_tc<3><<<grd, 128, smem, s>>>(mdz, mx, N, H, W, Cin, Cout, (int)per, dw, db);
     else
-        k_conv3x3_wgrad_tc<1><<<grd, 128, smem, s>>>(mdz, mx, N, H, W, Cin, Cout, (int)per, dw);
-    if (db) {
-        const long long ys = P < 256 ? P : 256, pper = (P + ys - 1) / ys;
-        k_bias_grad<<<dim3((Cout + 127) / 128, (unsigned)((P + pper - 1) / pper)), 128, 0, s>>>(dz, P, Cout, pper, db);
-    }
+        k_conv3x3_wgrad_tc<1><<<grd, 128, smem, s>>>(mdz, mx, N, H, W, Cin, Cout, (int)per, dw, db);
     return true;
 }
 
@@ -997,6 +1268,10 @@ int tpfnet_conv3x3_wgrad(const void* x, const void* dz, int N, int H, int W, int
 
 int tpfnet_relu_mask(void* d, const void* y, long long count, void* stream)
 {
+    if (pieces((int)(count % 8), d, y)) {
+        k_relu_mask8<<<grid_of(count / 8), 256, 0, (cudaStream_t)stream>>>((bf16*)d, (const bf16*)y, count / 8);
+        return status(cudaGetLastError());
+    }
     k_relu_mask<<<grid_of(count), 256, 0, (cudaStream_t)stream>>>((bf16*)d, (const bf16*)y, count);
     return status(cudaGetLastError());
 }
@@ -1004,12 +1279,22 @@ int tpfnet_relu_mask(void* d, const void* y, long long count, void* stream)
 int tpfnet_pool(const void* x, int N, int H, int W, int C, void* y, void* stream)
 {
     if (H % 2 || W % 2) return TPF_ERR_INVALID_ARG;
+    if (pieces(C, x, y)) {
+        k_pool8<<<grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, N * (H / 2), W,
+                                                                                         C / 8, (bf16*)y);
+        return status(cudaGetLastError());
+    }
     k_pool<<<grid_of((long long)N * H * W * C / 4), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, N, H, W, C, (bf16*)y);
     return status(cudaGetLastError());
 }
 
 int tpfnet_pool_back(const void* dy, int N, int H, int W, int C, void* dx, int accumulate, void* stream)
 {
+    if (H % 2 == 0 && W % 2 == 0 && pieces(C, dy, dx)) {
+        k_pool_back8<<<grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream>>>(
+            (const bf16*)dy, N * (H / 2), W, C / 8, (bf16*)dx, accumulate);
+        return status(cudaGetLastError());
+    }
     k_pool_back<<<grid_of((long long)N * H * W * C), 256, 0, (cudaStream_t)stream>>>((const bf16*)dy, N, H, W, C, (bf16*)dx,
                                                                                     accumulate);
     return status(cudaGetLastError());
@@ -1017,6 +1302,11 @@ int tpfnet_pool_back(const void* dy, int N, int H, int W, int C, void* dx, int a
 
 int tpfnet_up_into(const void* x, int N, int H, int W, int C, void* y, int Ctot, int cofs, void* stream)
 {
+    if (H % 2 == 0 && W % 2 == 0 && pieces(C | Ctot | cofs, x, y)) {
+        k_up_into8<<<grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream>>>(
+            (const bf16*)x, N * (H / 2), W, C / 8, (bf16*)y, Ctot, cofs);
+        return status(cudaGetLastError());
+    }
     k_up_into<<<grid_of((long long)N * H * W * C), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, N, H, W, C, (bf16*)y,
                                                                                   Ctot, cofs);
     return status(cudaGetLastError());
@@ -1024,6 +1314,11 @@ int tpfnet_up_into(const void* x, int N, int H, int W, int C, void* y, int Ctot,
 
 int tpfnet_up_back(const void* dy, int N, int H, int W, int Ctot, int cofs, int C, void* dx, void* stream)
 {
+    if (H % 2 == 0 && W % 2 == 0 && pieces(C | Ctot | cofs, dy, dx)) {
+        k_up_back8<<<grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream>>>(
+            (const bf16*)dy, N * (H / 2), W, Ctot, cofs, C / 8, (bf16*)dx);
+        return status(cudaGetLastError());
+    }
     k_up_back<<<grid_of((long long)N * H * W * C / 4), 256, 0, (cudaStream_t)stream>>>((const bf16*)dy, N, H, W, Ctot, cofs,
                                                                                        C, (bf16*)dx);
     return status(cudaGetLastError());
@@ -1032,6 +1327,11 @@ int tpfnet_up_back(const void* dy, int N, int H, int W, int Ctot, int cofs, int 
 int tpfnet_channels(const void* src, int Sc, int sofs, long long pixels, int C, void* dst, int Dc, int dofs,
                     int accumulate, void* stream)
 {
+    if (pieces(C | Sc | sofs | Dc | dofs, src, dst)) {
+        k_channels8<<<grid_of(pixels * (C / 8)), 256, 0, (cudaStream_t)stream>>>((const bf16*)src, Sc, sofs, pixels, C / 8,
+                                                                               (bf16*)dst, Dc, dofs, accumulate);
+        return status(cudaGetLastError());
+    }
     k_channels<<<grid_of(pixels * C), 256, 0, (cudaStream_t)stream>>>((const bf16*)src, Sc, sofs, pixels, C, (bf16*)dst, Dc,
                                                                      dofs, accumulate);
     return status(cudaGetLastError());
@@ -1040,6 +1340,23 @@ int tpfnet_channels(const void* src, int Sc, int sofs, long long pixels, int C, 
 int tpfnet_head(const void* x, long long pixels, int C, const float* Wt, const float* b, int Cout, float* out,
                 void* stream)
 {
+    const int blocks = (int)((pixels + 255) / 256 < 152 * 8 ? (pixels + 255) / 256 : 152 * 8);
+    const int smem = (C + 256) * Cout * (int)sizeof(float);
+    if (pixels > 0 && Cout >= 1 && Cout <= 8 && smem <= 48 * 1024 && pieces(C, x)) {
+        cudaStream_t s = (cudaStream_t)stream;
+        auto run = [&](auto kern) { kern<<<blocks, 256, smem, s>>>((const bf16*)x, pixels, C, Wt, b, out); };
+        switch (Cout) {
+        case 1: run(k_head8<1>); break;
+        case 2: run(k_head8<2>); break;
+        case 3: run(k_head8<3>); break;
+        case 4: run(k_head8<4>); break;
+        case 5: run(k_head8<5>); break;
+        case 6: run(k_head8<6>); break;
+        case 7: run(k_head8<7>); break;
+        default: run(k_head8<8>); break;
+        }
+        return status(cudaGetLastError());
+    }
     k_head<<<grid_of(pixels * Cout), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, pixels, C, Wt, b, Cout, out);
     return status(cudaGetLastError());
 }
@@ -1049,6 +1366,26 @@ int tpfnet_head_back(const void* x, const float* dout, long long pixels, int C, 
 {
     const int smem = (C * Cout + Cout) * (int)sizeof(float);
     if (smem > 48 * 1024) return TPF_ERR_INVALID_ARG;
+    const int G = C / 8;
+    if (pixels > 0 && Cout >= 1 && Cout <= 8 && G >= 1 && G <= 32 && (G & (G - 1)) == 0 && pieces(C, x, dx)) {
+        const long long per = 8 * (32 / G);  // pixels per block and turn
+        const int blocks = (int)((pixels + per - 1) / per < 152 * 2 ? (pixels + per - 1) / per : 152 * 2);
+        cudaStream_t s = (cudaStream_t)stream;
+        auto run = [&](auto kern) {
+            kern<<<blocks, 256, smem, s>>>((const bf16*)x, dout, pixels, C, Wt, (bf16*)dx, dW, db);
+        };
+        switch (Cout) {
+        case 1: run(k_head_back8<1>); break;
+        case 2: run(k_head_back8<2>); break;
+        case 3: run(k_head_back8<3>); break;
+        case 4: run(k_head_back8<4>); break;
+        case 5: run(k_head_back8<5>); break;
+        case 6: run(k_head_back8<6>); break;
+        case 7: run(k_head_back8<7>); break;
+        default: run(k_head_back8<8>); break;
+        }
+        return status(cudaGetLastError());
+    }
     k_head_back<<<grid_of(pixels) < 304 ? grid_of(pixels) : 304, 256, smem, (cudaStream_t)stream>>>(
         (const bf16*)x, dout, pixels, C, Wt, Cout, (bf16*)dx, dW, db);
     return status(cudaGetLastError());
@@ -1057,7 +1394,7 @@ int tpfnet_head_back(const void* x, const float* dout, long long pixels, int C, 
 int tpfnet_mse(const float* pred, const float* target, const float* wch, long long count, int C, float* grad,
                double* loss, void* stream)
 {
-    k_mse<<<grid_of(count) < 1024 ? grid_of(count) : 1024, 256, 0, (cudaStream_t)stream>>>(pred, target, wch, count, C, grad,
+    k_mse<<<grid_of(count) < 304 ? grid_of(count) : 304, 256, 0, (cudaStream_t)stream>>>(pred, target, wch, count, C, grad,
                                                                                           loss);
     return status(cudaGetLastError());
 }
