@@ -51,6 +51,35 @@ int tpfnet_status(void);
 int tpfnet_conv3x3_dgrad(const void *dz, int N, int H, int W, int Cout, const void *wt, int Cin, void *wflip,
                          void *dx, void *stream);
 
+/* The same pieces in the forms that a whole network's passes join, so that no concatenation,
+ * split or ReLU mask is a pass of its own:
+ *   conv3x3_into: the output goes to Cout channels of a tensor with ldy channels per pixel
+ *     (y points at the first of them; ldy even);
+ *   flip_weights: the flipped, transposed weights of up to 16 layers (host arrays of device
+ *     pointers and sizes) in one launch;
+ *   dgrad_masked: the data gradient from weights flipped before, zero where mask (laid out as
+ *     dx; the layer's input, a ReLU output) is not positive; mask may be NULL;
+ *   pool_from: pooling of C channels of a tensor with ldx channels per pixel;
+ *   pool_back_skip: dx = dy / 4 + skip (lds channels per pixel), zero where mask (ldm) is not
+ *     positive;
+ *   up_back_masked, head_back_masked: the adjoints, dx zero where the mask (laid out as dx; for
+ *     the head its input x) is not positive.
+ * Pooling and upsampling in these forms take channel counts and offsets that are multiples of 8
+ * and 16-byte aligned tensors. */
+int tpfnet_conv3x3_into(const void *x, int N, int H, int W, int Cin, const void *wt, const float *bias, int Cout,
+                        int relu, void *y, int ldy, void *stream);
+int tpfnet_flip_weights(int layers, const void *const *wt, const int *cin, const int *cout, void *const *wflip,
+                        void *stream);
+int tpfnet_conv3x3_dgrad_masked(const void *dz, int N, int H, int W, int Cout, const void *wflip, int Cin,
+                                const void *mask, void *dx, void *stream);
+int tpfnet_pool_from(const void *x, int N, int H, int W, int C, int ldx, void *y, void *stream);
+int tpfnet_pool_back_skip(const void *dy, int N, int H, int W, int C, const void *skip, int lds, const void *mask,
+                          int ldm, void *dx, void *stream);
+int tpfnet_up_back_masked(const void *dy, int N, int H, int W, int Ctot, int cofs, int C, const void *mask, void *dx,
+                          void *stream);
+int tpfnet_head_back_masked(const void *x, const float *dout, long long pixels, int C, const float *Wt, int Cout,
+                            void *dx, float *dW, float *db, void *stream);
+
 /* Weight and bias gradients of conv3x3, ADDED to dw ([9][Cout][Cin] float32) and db
  * (Cout float32, or NULL).  Cin % 32 == 0, Cout % 32 == 0. */
 int tpfnet_conv3x3_wgrad(const void *x, const void *dz, int N, int H, int W, int Cin, int Cout, float *dw,

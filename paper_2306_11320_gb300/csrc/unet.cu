@@ -37,7 +37,8 @@ __device__ __forceinline__ void mma_bf16(float* d, const uint32_t* a, const uint
 template <int BN>
 __global__ void __launch_bounds__(128)
 k_conv3x3(const bf16* __restrict__ x, int N, int H, int W, int Cin, const bf16* __restrict__ wt,
-          const float* __restrict__ bias, int Cout, int relu, bf16* __restrict__ y)
+          const float* __restrict__ bias, int Cout, int relu, bf16* __restrict__ y, int ldy,
+          const bf16* __restrict__ mask)
 {
     __shared__ __align__(16) bf16 As[kBM][kKC + kPad];
     __shared__ __align__(16) bf16 Bs[BN][kKC + kPad];
@@ -106,10 +107,15 @@ k_conv3x3(const bf16* __restrict__ x, int N, int H, int W, int Cin, const bf16* 
                 v0 = fmaxf(v0, 0.f);
                 v1 = fmaxf(v1, 0.f);
             }
+            const size_t px = ((size_t)n * H + h) * W + ww;
+            if (mask) {
+                if (!(__bfloat162float(mask[px * Cout + co]) > 0.f)) v0 = 0.f;
+                if (!(__bfloat162float(mask[px * Cout + co + 1]) > 0.f)) v1 = 0.f;
+            }
             __nv_bfloat162 o;
             o.x = __float2bfloat16_rn(v0);
             o.y = __float2bfloat16_rn(v1);
-            *reinterpret_cast<__nv_bfloat162*>(y + (((size_t)n * H + h) * W + ww) * Cout + co) = o;
+            *reinterpret_cast<__nv_bfloat162*>(y + px * ldy + co) = o;
         }
     }
 }
@@ -193,7 +199,8 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 template <int BN, int KC>
 __global__ void __launch_bounds__(128, 1)
 k_conv3x3_tc(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUtensorMap mw, int H, int W, int Cin,
-             int Cout, int BW, int BH, const float* __restrict__ bias, int relu, bf16* __restrict__ y)
+             int Cout, int BW, int BH, const float* __restrict__ bias, int relu, bf16* __restrict__ y, int ldy,
+             const bf16* __restrict__ mask)
 {
     static_assert(BN == 32 || BN == 64 || BN == 128 || BN == 256, "TMEM columns: a power of two from 32");
     constexpr int kABytes = 128 * KC * 2, kBBytes = BN * KC * 2;
@@ -279,7 +286,9 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUt
     tc_fence_after();
     const int m = warp * 32 + lane;
     const int hh = h0 + m / BW, ww = w0 + m % BW;
-    bf16* out = y + (((size_t)n * H + hh) * W + ww) * Cout + co0;
+    const size_t px = ((size_t)n * H + hh) * W + ww;
+    bf16* out = y + px * ldy + co0;
+    const bf16* mrow = mask ? mask + px * Cout + co0 : nullptr;
 #pragma unroll 1
     for (int c = 0; c < BN; c += 8) {
         uint32_t r[8];
@@ -288,6 +297,9 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUt
                      : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c));
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         uint32_t o[4];
+        uint4 mk = make_uint4(0, 0, 0, 0);
+        if (mrow) mk = *reinterpret_cast<const uint4*>(mrow + c);
+        const uint32_t mu[4] = {mk.x, mk.y, mk.z, mk.w};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             float v0 = __uint_as_float(r[2 * j]) + (bias ? bias[co0 + c + 2 * j] : 0.f);
@@ -295,6 +307,10 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUt
             if (relu) {
                 v0 = fmaxf(v0, 0.f);
                 v1 = fmaxf(v1, 0.f);
+            }
+            if (mrow) {  // bf16 is the upper half of float32
+                if (!(__uint_as_float(mu[j] << 16) > 0.f)) v0 = 0.f;
+                if (!(__uint_as_float(mu[j] & 0xffff0000u) > 0.f)) v1 = 0.f;
             }
             __nv_bfloat162 t;
             t.x = __float2bfloat16_rn(v0);
@@ -586,15 +602,31 @@ k_conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap mdz, const __grid_constan
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
 }
 
-// flipped transpose for the data gradient: wd[tap][ci][co] = w[8 - tap][co][ci]
-__global__ void k_flip_weights(const bf16* __restrict__ w, int Cin, int Cout, bf16* __restrict__ wd)
+// flipped transposes for the data gradients: wd[tap][ci][co] = w[8 - tap][co][ci], of up to
+// kMaxFlips layers in one launch (blockIdx.y; 3 us each on its own)
+constexpr int kMaxFlips = 16;
+struct FlipList {
+    const bf16* w[kMaxFlips];
+    bf16* wd[kMaxFlips];
+    int cin[kMaxFlips], cout[kMaxFlips];
+};
+__global__ void __launch_bounds__(256) k_flip_weights(const FlipList L)
 {
-    const long long total = 9LL * Cin * Cout;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < total; k += (long long)gridDim.x * blockDim.x) {
-        const int co = (int)(k % Cout);
-        const long long r = k / Cout;
-        const int ci = (int)(r % Cin), tap = (int)(r / Cin);
-        wd[k] = w[((size_t)(8 - tap) * Cout + co) * Cin + ci];
+    // 32 x 32 (co, ci) tiles of one tap through shared memory, so that both sides are read
+    // and written in whole rows
+    __shared__ bf16 t[32][33];
+    const int l = blockIdx.y, cin = L.cin[l], cout = L.cout[l];
+    const int ti = cin / 32, to = cout / 32;
+    const bf16* w = L.w[l];
+    bf16* wd = L.wd[l];
+    for (int k = blockIdx.x; k < 9 * ti * to; k += gridDim.x) {
+        const int tap = k / (ti * to), ci0 = 32 * ((k / to) % ti), co0 = 32 * (k % to);
+        for (int r = threadIdx.x >> 5; r < 32; r += 8)
+            t[r][threadIdx.x & 31] = w[((size_t)(8 - tap) * cout + co0 + r) * cin + ci0 + (threadIdx.x & 31)];
+        __syncthreads();
+        for (int r = threadIdx.x >> 5; r < 32; r += 8)
+            wd[((size_t)tap * cin + ci0 + r) * cout + co0 + (threadIdx.x & 31)] = t[threadIdx.x & 31][r];
+        __syncthreads();
     }
 }
 
@@ -647,36 +679,48 @@ __global__ void k_relu_mask8(bf16* __restrict__ d, const bf16* __restrict__ y, l
 }
 // The image kernels below: blockIdx.y walks the rows (of all images), threads the pieces of
 // a row; C8 pieces per pixel.
-__global__ void k_pool8(const bf16* __restrict__ x, int rows, int W, int C8, bf16* __restrict__ y)
+// x: ldx channels per pixel
+__global__ void k_pool8(const bf16* __restrict__ x, int rows, int W, int C8, int ldx, bf16* __restrict__ y)
 {
     const int Wo = W / 2, C = 8 * C8;
     for (int r = blockIdx.y; r < rows; r += gridDim.y)  // output row: image rows 2 r, 2 r + 1
         for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < Wo * C8; k += gridDim.x * blockDim.x) {
             const int w = k / C8, c = 8 * (k - w * C8);
-            const bf16* b = x + ((size_t)2 * r * W + 2 * w) * C + c;
-            const Piece p0 = ld8(b), p1 = ld8(b + C), p2 = ld8(b + (size_t)W * C), p3 = ld8(b + (size_t)W * C + C);
+            const bf16* b = x + ((size_t)2 * r * W + 2 * w) * ldx + c;
+            const Piece p0 = ld8(b), p1 = ld8(b + ldx), p2 = ld8(b + (size_t)W * ldx),
+                        p3 = ld8(b + (size_t)W * ldx + ldx);
             Piece o;
 #pragma unroll
             for (int j = 0; j < 8; ++j) o.v[j] = 0.25f * (p0.v[j] + p1.v[j] + p2.v[j] + p3.v[j]);
             st8(y + ((size_t)r * Wo + w) * C + c, o);
         }
 }
-// rows: coarse rows; one thread serves the 2 x 2 fine pixels of a coarse one
-__global__ void k_pool_back8(const bf16* __restrict__ dy, int rows, int W, int C8, bf16* __restrict__ dx, int accumulate)
+// rows: coarse rows; one thread serves the 2 x 2 fine pixels of a coarse one.  dx = dy / 4,
+// plus `add` (lda channels per pixel; may be dx itself) when given, zero where `mask` (ldm
+// channels per pixel) is not positive when given.
+__global__ void k_pool_back8(const bf16* __restrict__ dy, int rows, int W, int C8, const bf16* add, int lda,
+                             const bf16* __restrict__ mask, int ldm, bf16* dx)
 {
     const int Wo = W / 2, C = 8 * C8;
     for (int r = blockIdx.y; r < rows; r += gridDim.y)
         for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < Wo * C8; k += gridDim.x * blockDim.x) {
             const int w = k / C8, c = 8 * (k - w * C8);
             const Piece g = ld8(dy + ((size_t)r * Wo + w) * C + c);
+            Piece old[4], mk[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                bf16* d = dx + ((size_t)(2 * r + q / 2) * W + 2 * w + q % 2) * C + c;
-                Piece v, old;
-                if (accumulate) old = ld8(d);
+                const size_t px = (size_t)(2 * r + q / 2) * W + 2 * w + q % 2;
+                if (add) old[q] = ld8(add + px * lda + c);
+                if (mask) mk[q] = ld8(mask + px * ldm + c);
+            }
 #pragma unroll
-                for (int j = 0; j < 8; ++j) v.v[j] = accumulate ? 0.25f * g.v[j] + old.v[j] : 0.25f * g.v[j];
-                st8(d, v);
+            for (int q = 0; q < 4; ++q) {
+                const size_t px = (size_t)(2 * r + q / 2) * W + 2 * w + q % 2;
+                Piece v;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v.v[j] = add ? 0.25f * g.v[j] + old[q].v[j] : 0.25f * g.v[j];
+                if (mask) relu_back8(v, mk[q]);
+                st8(dx + px * C + c, v);
             }
         }
 }
@@ -694,7 +738,9 @@ __global__ void k_up_into8(const bf16* __restrict__ x, int rows, int W, int C8, 
             *reinterpret_cast<uint4*>(d + (size_t)W * Ctot + Ctot) = v;
         }
 }
-__global__ void k_up_back8(const bf16* __restrict__ dy, int rows, int W, int Ctot, int cofs, int C8, bf16* __restrict__ dx)
+// zero where `mask` (laid out as dx) is not positive, when given
+__global__ void k_up_back8(const bf16* __restrict__ dy, int rows, int W, int Ctot, int cofs, int C8,
+                           const bf16* __restrict__ mask, bf16* __restrict__ dx)
 {
     const int Wo = W / 2, C = 8 * C8;
     for (int r = blockIdx.y; r < rows; r += gridDim.y)
@@ -706,7 +752,9 @@ __global__ void k_up_back8(const bf16* __restrict__ dy, int rows, int W, int Cto
             Piece o;
 #pragma unroll
             for (int j = 0; j < 8; ++j) o.v[j] = p0.v[j] + p1.v[j] + p2.v[j] + p3.v[j];
-            st8(dx + ((size_t)r * Wo + w) * C + c, o);
+            const size_t at = ((size_t)r * Wo + w) * C + c;
+            if (mask) relu_back8(o, ld8(mask + at));
+            st8(dx + at, o);
         }
 }
 __global__ void k_channels8(const bf16* __restrict__ src, int Sc, int sofs, long long pixels, int C8,
@@ -859,7 +907,8 @@ k_head8(const bf16* __restrict__ x, long long pixels, int C, const float* __rest
 template <int CO>
 __global__ void __launch_bounds__(256)
 k_head_back8(const bf16* __restrict__ x, const float* __restrict__ dout, long long pixels, int C,
-             const float* __restrict__ Wt, bf16* __restrict__ dx, float* __restrict__ dW, float* __restrict__ db)
+             const float* __restrict__ Wt, bf16* __restrict__ dx, float* __restrict__ dW, float* __restrict__ db,
+             int relu)
 {
     extern __shared__ float sh[];  // C * CO + CO sums
     const int G = C >> 3, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -892,6 +941,7 @@ k_head_back8(const bf16* __restrict__ x, const float* __restrict__ dout, long lo
             }
             r.v[j] = s;
         }
+        if (relu) relu_back8(r, v);
         st8(dx + p * C + 8 * cg, r);
 #pragma unroll
         for (int o = 0; o < CO; ++o) accb[o] += d[o];
@@ -1084,7 +1134,7 @@ int tc_bn(int N, int H, int W, int Cout, int& BW, int& BH)
 // false (nothing launched) otherwise.
 template <int BN, int KC>
 bool launch_tc(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, const float* bias, int Cout, int relu,
-               bf16* y, cudaStream_t s, int BW, int BH)
+               bf16* y, int ldy, const bf16* mask, cudaStream_t s, int BW, int BH)
 {
     auto fn = encode_fn();
     if (!fn) return false;
@@ -1116,29 +1166,29 @@ bool launch_tc(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, cons
         return false;
     }
     dim3 grd(N * (H / BH) * (W / BW), Cout / BN);
-    k_conv3x3_tc<BN, KC><<<grd, 128, smem, s>>>(mx, mw, H, W, Cin, Cout, BW, BH, bias, relu, y);
+    k_conv3x3_tc<BN, KC><<<grd, 128, smem, s>>>(mx, mw, H, W, Cin, Cout, BW, BH, bias, relu, y, ldy, mask);
     return true;
 }
 
 bool conv_tc(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, const float* bias, int Cout, int relu,
-             bf16* y, cudaStream_t s)
+             bf16* y, int ldy, const bf16* mask, cudaStream_t s)
 {
     int BW = 0, BH = 0;
     const int bn = tc_bn(N, H, W, Cout, BW, BH);
-    if (!bn || (((uintptr_t)x | (uintptr_t)wt | (uintptr_t)y) & 15)) return false;
+    if (!bn || (((uintptr_t)x | (uintptr_t)wt | (uintptr_t)y | (uintptr_t)mask) & 15) || ldy % 8) return false;
     if (Cin % 64 == 0) {
         switch (bn) {
-        case 256: return launch_tc<256, 64>(x, N, H, W, Cin, wt, bias, Cout, relu, y, s, BW, BH);
-        case 128: return launch_tc<128, 64>(x, N, H, W, Cin, wt, bias, Cout, relu, y, s, BW, BH);
-        case 64: return launch_tc<64, 64>(x, N, H, W, Cin, wt, bias, Cout, relu, y, s, BW, BH);
-        default: return launch_tc<32, 64>(x, N, H, W, Cin, wt, bias, Cout, relu, y, s, BW, BH);
+        case 256: return launch_tc<256, 64>(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, BW, BH);
+        case 128: return launch_tc<128, 64>(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, BW, BH);
+        case 64: return launch_tc<64, 64>(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, BW, BH);
+        default: return launch_tc<32, 64>(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, BW, BH);
         }
     }
     switch (bn) {
-    case 256: return launch_tc<256, 32>(x, N, H, W, Cin, wt, bias, Cout, relu, y, s, BW, BH);
-    case 128: return launch_tc<128, 32>(x, N, H, W, Cin, wt, bias, Cout, relu, y, s, BW, BH);
-    case 64: return launch_tc<64, 32>(x, N, H, W, Cin, wt, bias, Cout, relu, y, s, BW, BH);
-    default: return launch_tc<32, 32>(x, N, H, W, Cin, wt, bias, Cout, relu, y, s, BW, BH);
+    case 256: return launch_tc<256, 32>(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, BW, BH);
+    case 128: return launch_tc<128, 32>(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, BW, BH);
+    case 64: return launch_tc<64, 32>(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, BW, BH);
+    default: return launch_tc<32, 32>(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, BW, BH);
     }
 }
 
@@ -1191,21 +1241,61 @@ bool wgrad_tc(const bf16* x, const bf16* dz, int N, int H, int W, int Cin, int C
 
 extern "C" {
 
-int tpfnet_conv3x3(const void* x, int N, int H, int W, int Cin, const void* wt, const float* bias, int Cout, int relu,
-                   void* y, void* stream)
+static int conv_any(const void* x, int N, int H, int W, int Cin, const void* wt, const float* bias, int Cout, int relu,
+                    void* y, int ldy, const void* mask, void* stream)
 {
     if (!x || !wt || !y || N < 1 || H < 1 || W < 1 || Cin % kKC || Cout % 32) return TPF_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    if (conv_tc((const bf16*)x, N, H, W, Cin, (const bf16*)wt, bias, Cout, relu, (bf16*)y, s))
+    if (conv_tc((const bf16*)x, N, H, W, Cin, (const bf16*)wt, bias, Cout, relu, (bf16*)y, ldy, (const bf16*)mask, s))
         return status(cudaGetLastError());
     const int wblocks = (W + kBM - 1) / kBM;
     if (Cout % 64 == 0) {
         dim3 grd(wblocks * N * H, Cout / 64);
-        k_conv3x3<64><<<grd, 128, 0, s>>>((const bf16*)x, N, H, W, Cin, (const bf16*)wt, bias, Cout, relu, (bf16*)y);
+        k_conv3x3<64><<<grd, 128, 0, s>>>((const bf16*)x, N, H, W, Cin, (const bf16*)wt, bias, Cout, relu, (bf16*)y,
+                                      ldy, (const bf16*)mask);
     } else {
         dim3 grd(wblocks * N * H, Cout / 32);
-        k_conv3x3<32><<<grd, 128, 0, s>>>((const bf16*)x, N, H, W, Cin, (const bf16*)wt, bias, Cout, relu, (bf16*)y);
+        k_conv3x3<32><<<grd, 128, 0, s>>>((const bf16*)x, N, H, W, Cin, (const bf16*)wt, bias, Cout, relu, (bf16*)y,
+                                      ldy, (const bf16*)mask);
     }
+    return status(cudaGetLastError());
+}
+
+int tpfnet_conv3x3(const void* x, int N, int H, int W, int Cin, const void* wt, const float* bias, int Cout, int relu,
+                   void* y, void* stream)
+{
+    return conv_any(x, N, H, W, Cin, wt, bias, Cout, relu, y, Cout, nullptr, stream);
+}
+
+int tpfnet_conv3x3_into(const void* x, int N, int H, int W, int Cin, const void* wt, const float* bias, int Cout,
+                        int relu, void* y, int ldy, void* stream)
+{
+    if (ldy < Cout || ldy % 2) return TPF_ERR_INVALID_ARG;
+    return conv_any(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, nullptr, stream);
+}
+
+int tpfnet_conv3x3_dgrad_masked(const void* dz, int N, int H, int W, int Cout, const void* wflip, int Cin,
+                                const void* mask, void* dx, void* stream)
+{
+    return conv_any(dz, N, H, W, Cout, wflip, nullptr, Cin, 0, dx, Cin, mask, stream);
+}
+
+int tpfnet_flip_weights(int layers, const void* const* wt, const int* cin, const int* cout, void* const* wflip,
+                        void* stream)
+{
+    if (layers < 1 || layers > kMaxFlips || !wt || !cin || !cout || !wflip) return TPF_ERR_INVALID_ARG;
+    FlipList L{};
+    int most = 0;
+    for (int l = 0; l < layers; ++l) {
+        if (!wt[l] || !wflip[l] || cin[l] < 32 || cout[l] < 32 || cin[l] % 32 || cout[l] % 32) return TPF_ERR_INVALID_ARG;
+        L.w[l] = (const bf16*)wt[l];
+        L.wd[l] = (bf16*)wflip[l];
+        L.cin[l] = cin[l];
+        L.cout[l] = cout[l];
+        const int tiles = 9 * (cin[l] / 32) * (cout[l] / 32);
+        if (tiles > most) most = tiles;
+    }
+    k_flip_weights<<<dim3(most < 304 ? most : 304, layers), 256, 0, (cudaStream_t)stream>>>(L);
     return status(cudaGetLastError());
 }
 
@@ -1232,9 +1322,7 @@ int tpfnet_conv3x3_dgrad(const void* dz, int N, int H, int W, int Cout, const vo
                          void* stream)
 {
     if (!dz || !wt || !wflip || !dx || Cin % 32 || Cout % kKC) return TPF_ERR_INVALID_ARG;
-    cudaStream_t s = (cudaStream_t)stream;
-    k_flip_weights<<<grid_of(9LL * Cin * Cout), 256, 0, s>>>((const bf16*)wt, Cin, Cout, (bf16*)wflip);
-    int rc = status(cudaGetLastError());
+    int rc = tpfnet_flip_weights(1, &wt, &Cin, &Cout, &wflip, stream);
     if (rc) return rc;
     return tpfnet_conv3x3(dz, N, H, W, Cout, wflip, nullptr, Cin, 0, dx, stream);
 }
@@ -1281,7 +1369,7 @@ int tpfnet_pool(const void* x, int N, int H, int W, int C, void* y, void* stream
     if (H % 2 || W % 2) return TPF_ERR_INVALID_ARG;
     if (pieces(C, x, y)) {
         k_pool8<<<grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, N * (H / 2), W,
-                                                                                         C / 8, (bf16*)y);
+                                                                                         C / 8, C, (bf16*)y);
         return status(cudaGetLastError());
     }
     k_pool<<<grid_of((long long)N * H * W * C / 4), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, N, H, W, C, (bf16*)y);
@@ -1292,7 +1380,7 @@ int tpfnet_pool_back(const void* dy, int N, int H, int W, int C, void* dx, int a
 {
     if (H % 2 == 0 && W % 2 == 0 && pieces(C, dy, dx)) {
         k_pool_back8<<<grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream>>>(
-            (const bf16*)dy, N * (H / 2), W, C / 8, (bf16*)dx, accumulate);
+            (const bf16*)dy, N * (H / 2), W, C / 8, accumulate ? (const bf16*)dx : nullptr, C, nullptr, 0, (bf16*)dx);
         return status(cudaGetLastError());
     }
     k_pool_back<<<grid_of((long long)N * H * W * C), 256, 0, (cudaStream_t)stream>>>((const bf16*)dy, N, H, W, C, (bf16*)dx,
@@ -1316,11 +1404,42 @@ int tpfnet_up_back(const void* dy, int N, int H, int W, int Ctot, int cofs, int 
 {
     if (H % 2 == 0 && W % 2 == 0 && pieces(C | Ctot | cofs, dy, dx)) {
         k_up_back8<<<grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream>>>(
-            (const bf16*)dy, N * (H / 2), W, Ctot, cofs, C / 8, (bf16*)dx);
+            (const bf16*)dy, N * (H / 2), W, Ctot, cofs, C / 8, nullptr, (bf16*)dx);
         return status(cudaGetLastError());
     }
     k_up_back<<<grid_of((long long)N * H * W * C / 4), 256, 0, (cudaStream_t)stream>>>((const bf16*)dy, N, H, W, Ctot, cofs,
                                                                                        C, (bf16*)dx);
+    return status(cudaGetLastError());
+}
+
+int tpfnet_pool_from(const void* x, int N, int H, int W, int C, int ldx, void* y, void* stream)
+{
+    if (!x || !y || N < 1 || H < 2 || W < 2 || H % 2 || W % 2 || C < 8 || ldx < C || !pieces(C | ldx, x, y))
+        return TPF_ERR_INVALID_ARG;
+    k_pool8<<<grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, N * (H / 2), W, C / 8,
+                                                                                     ldx, (bf16*)y);
+    return status(cudaGetLastError());
+}
+
+int tpfnet_pool_back_skip(const void* dy, int N, int H, int W, int C, const void* skip, int lds, const void* mask,
+                          int ldm, void* dx, void* stream)
+{
+    if (!dy || !skip || !mask || !dx || N < 1 || H < 2 || W < 2 || H % 2 || W % 2 || C < 8 || lds < C || ldm < C ||
+        !pieces(C | lds | ldm, dy, skip, mask, dx))
+        return TPF_ERR_INVALID_ARG;
+    k_pool_back8<<<grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream>>>(
+        (const bf16*)dy, N * (H / 2), W, C / 8, (const bf16*)skip, lds, (const bf16*)mask, ldm, (bf16*)dx);
+    return status(cudaGetLastError());
+}
+
+int tpfnet_up_back_masked(const void* dy, int N, int H, int W, int Ctot, int cofs, int C, const void* mask, void* dx,
+                          void* stream)
+{
+    if (!dy || !mask || !dx || N < 1 || H < 2 || W < 2 || H % 2 || W % 2 || C < 8 || cofs < 0 || cofs + C > Ctot ||
+        !pieces(C | Ctot | cofs, dy, mask, dx))
+        return TPF_ERR_INVALID_ARG;
+    k_up_back8<<<grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream>>>(
+        (const bf16*)dy, N * (H / 2), W, Ctot, cofs, C / 8, (const bf16*)mask, (bf16*)dx);
     return status(cudaGetLastError());
 }
 
@@ -1361,8 +1480,8 @@ int tpfnet_head(const void* x, long long pixels, int C, const float* Wt, const f
     return status(cudaGetLastError());
 }
 
-int tpfnet_head_back(const void* x, const float* dout, long long pixels, int C, const float* Wt, int Cout, void* dx,
-                     float* dW, float* db, void* stream)
+static int head_back_any(const void* x, const float* dout, long long pixels, int C, const float* Wt, int Cout, void* dx,
+                         float* dW, float* db, int relu, void* stream)
 {
     const int smem = (C * Cout + Cout) * (int)sizeof(float);
     if (smem > 48 * 1024) return TPF_ERR_INVALID_ARG;
@@ -1372,7 +1491,7 @@ int tpfnet_head_back(const void* x, const float* dout, long long pixels, int C, 
         const int blocks = (int)((pixels + per - 1) / per < 152 * 2 ? (pixels + per - 1) / per : 152 * 2);
         cudaStream_t s = (cudaStream_t)stream;
         auto run = [&](auto kern) {
-            kern<<<blocks, 256, smem, s>>>((const bf16*)x, dout, pixels, C, Wt, (bf16*)dx, dW, db);
+            kern<<<blocks, 256, smem, s>>>((const bf16*)x, dout, pixels, C, Wt, (bf16*)dx, dW, db, relu);
         };
         switch (Cout) {
         case 1: run(k_head_back8<1>); break;
@@ -1388,7 +1507,20 @@ int tpfnet_head_back(const void* x, const float* dout, long long pixels, int C, 
     }
     k_head_back<<<grid_of(pixels) < 304 ? grid_of(pixels) : 304, 256, smem, (cudaStream_t)stream>>>(
         (const bf16*)x, dout, pixels, C, Wt, Cout, (bf16*)dx, dW, db);
-    return status(cudaGetLastError());
+    const int rc = status(cudaGetLastError());
+    return rc || !relu ? rc : tpfnet_relu_mask(dx, x, pixels * C, stream);
+}
+
+int tpfnet_head_back(const void* x, const float* dout, long long pixels, int C, const float* Wt, int Cout, void* dx,
+                     float* dW, float* db, void* stream)
+{
+    return head_back_any(x, dout, pixels, C, Wt, Cout, dx, dW, db, 0, stream);
+}
+
+int tpfnet_head_back_masked(const void* x, const float* dout, long long pixels, int C, const float* Wt, int Cout,
+                            void* dx, float* dW, float* db, void* stream)
+{
+    return head_back_any(x, dout, pixels, C, Wt, Cout, dx, dW, db, 1, stream);
 }
 
 int tpfnet_mse(const float* pred, const float* target, const float* wch, long long count, int C, float* grad,

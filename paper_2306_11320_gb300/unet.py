@@ -22,6 +22,13 @@ _fp, _dp = C.POINTER(C.c_float), C.POINTER(C.c_double)
 
 SIGNATURES = {
     "tpfnet_conv3x3": [_vp, _ip, _ip, _ip, _ip, _vp, _vp, _ip, _ip, _vp, _vp],
+    "tpfnet_conv3x3_into": [_vp, _ip, _ip, _ip, _ip, _vp, _vp, _ip, _ip, _vp, _ip, _vp],
+    "tpfnet_conv3x3_dgrad_masked": [_vp, _ip, _ip, _ip, _ip, _vp, _ip, _vp, _vp, _vp],
+    "tpfnet_flip_weights": [_ip, _vp, _vp, _vp, _vp, _vp],
+    "tpfnet_pool_from": [_vp, _ip, _ip, _ip, _ip, _ip, _vp, _vp],
+    "tpfnet_pool_back_skip": [_vp, _ip, _ip, _ip, _ip, _vp, _ip, _vp, _ip, _vp, _vp],
+    "tpfnet_up_back_masked": [_vp, _ip, _ip, _ip, _ip, _ip, _ip, _vp, _vp, _vp],
+    "tpfnet_head_back_masked": [_vp, _vp, _ll, _ip, _vp, _ip, _vp, _vp, _vp, _vp],
     "tpfnet_conv3x3_tcgen05": [_ip, _ip, _ip, _ip, _ip],
     "tpfnet_conv3x3_wgrad_tcgen05": [_ip, _ip, _ip, _ip, _ip],
     "tpfnet_status": [],
@@ -85,6 +92,12 @@ class UNet:
         self.stream = stream if stream is not None else torch.cuda.current_stream()
         rng = np.random.default_rng(seed)
         self.P, self.Pb, self.G, self.M, self.V = {}, {}, {}, {}, {}
+        # every parameter is a view into one flat tensor per kind (each starting on a 256-byte
+        # boundary), so that Adam and clearing the gradients are one launch each
+        total = sum(-(-taps * a * b // 128) * 128 + -(-b // 128) * 128 for _, a, b, taps in self.specs)
+        self._flat = {k: torch.zeros(total, dtype=torch.bfloat16 if k == "Pb" else torch.float32, device="cuda")
+                      for k in ("P", "G", "M", "V", "Pb")}
+        self._used = 0
         for name, a, b, taps in self.specs:
             fan_in = taps * (self.cin if name == "e0a" else a)
             w = rng.standard_normal((taps, b, a) if taps == 9 else (a, b)) * np.sqrt(2.0 / fan_in)
@@ -97,11 +110,27 @@ class UNet:
 
     def _add(self, key, arr, bf16):
         t = self.torch
-        self.P[key] = t.from_numpy(np.ascontiguousarray(arr)).cuda()
-        self.G[key] = t.zeros_like(self.P[key])
-        self.M[key] = t.zeros_like(self.P[key])
-        self.V[key] = t.zeros_like(self.P[key])
-        self.Pb[key] = self.P[key].to(t.bfloat16) if bf16 else None
+        n, o = arr.size, self._used
+        self._used += -(-n // 128) * 128
+        for kind in ("P", "G", "M", "V", "Pb"):
+            getattr(self, kind)[key] = self._flat[kind][o:o + n].view(arr.shape)
+        self.P[key].copy_(t.from_numpy(np.ascontiguousarray(arr)))
+        self.Pb[key].copy_(self.P[key])
+        if not bf16:
+            self.Pb[key] = None
+
+    def _is_flat(self, kinds):
+        """Whether every tensor of these kinds is still the view into its flat tensor that
+        _add made (a caller may have put tensors of its own in their place)."""
+        o = 0
+        for name, a, b, taps in self.specs:
+            for key, n in ((name + ".W", taps * a * b), (name + ".b", b)):
+                for kind in kinds:
+                    v, f = getattr(self, kind)[key], self._flat[kind]
+                    if v is not None and (v.numel() != n or v.data_ptr() != f.data_ptr() + o * f.element_size()):
+                        return False
+                o += -(-n // 128) * 128
+        return True
 
     # ------------------------------------------------------- parameter I/O
     def set_reference_params(self, params):
@@ -153,22 +182,27 @@ class UNet:
         for lvl, (h, w, c) in enumerate(dims):
             nm = ["e0", "e1", "e2", "b"][lvl]
             self.B[nm + "a"] = t.empty((N, h, w, c), **bf)
-            self.B[nm] = t.empty((N, h, w, c), **bf)
+            if lvl == 3:
+                self.B[nm] = t.empty((N, h, w, c), **bf)
             if lvl > 0:
                 cin = dims[lvl - 1][2]
                 self.B["pool%d" % lvl] = t.empty((N, h, w, cin), **bf)
         for lvl, (h, w, c) in ((2, dims[2]), (1, dims[1]), (0, dims[0])):
             cup = dims[lvl + 1][2] if lvl == 2 else self.ch[lvl + 1]
             self.B["cat%d" % lvl] = t.empty((N, h, w, cup + c), **bf)
+            # the encoder's output is the concatenation's second part (written there)
+            self.B["e%d" % lvl] = self.B["cat%d" % lvl][..., cup:]
             self.B["d%da" % lvl] = t.empty((N, h, w, c), **bf)
             self.B["d%d" % lvl] = t.empty((N, h, w, c), **bf)
         self.out = t.empty((N, H, W, self.cout), dtype=t.float32, device="cuda")
         # gradient buffers (one per activation shape)
-        self.D = {k: t.empty_like(v) for k, v in self.B.items()}
+        self.D = {k: t.empty(v.shape, **bf) for k, v in self.B.items()}
+        for (h, w, c) in dims:
+            self.D["_tmp_%d_%d" % (h, c)] = t.empty((N, h, w, c), **bf)
         self.D["x"] = t.empty((N, H, W, self.cinp), **bf)
         self.D["out"] = t.empty_like(self.out)
-        maxw = max(9 * a * b for _, a, b, taps in self.specs if taps == 9)
-        self.wflip = t.empty(maxw, **bf)
+        # flipped weights of every layer whose data gradient is wanted (all but the first)
+        self.wflip = {n: t.empty(9 * a * b, **bf) for n, a, b, taps in self.specs if taps == 9 and n != "e0a"}
         self.loss = t.zeros(1, dtype=t.float64, device="cuda")
         self._shape = (N, H, W)
 
@@ -177,8 +211,9 @@ class UNet:
             raise RuntimeError("tpfnet kernel %s failed (%d)" % (what, rc))
 
     def _conv(self, name, x, N, H, W, cin, cout, y, relu=1):
-        self._chk(self.lib.tpfnet_conv3x3(_p(x), N, H, W, cin, _p(self.Pb[name + ".W"]), _p(self.P[name + ".b"]),
-                                          cout, relu, _p(y), self._s()), name)
+        """y: (N, H, W, cout), possibly a channel range of a wider tensor."""
+        self._chk(self.lib.tpfnet_conv3x3_into(_p(x), N, H, W, cin, _p(self.Pb[name + ".W"]), _p(self.P[name + ".b"]),
+                                               cout, relu, _p(y), y.stride(2), self._s()), name)
 
     def _s(self):
         return C.c_void_p(self.stream.cuda_stream)
@@ -199,20 +234,17 @@ class UNet:
         prev, pc = B["e0"], c0
         for lvl, (nm, c) in enumerate((("e1", c1), ("e2", c2), ("b", c3)), start=1):
             h, w = dims[lvl]
-            self._chk(L.tpfnet_pool(_p(prev), N, 2 * h, 2 * w, pc, _p(B["pool%d" % lvl]), s), "pool")
+            self._chk(L.tpfnet_pool_from(_p(prev), N, 2 * h, 2 * w, pc, prev.stride(2), _p(B["pool%d" % lvl]), s), "pool")
             ka, kb = ("b_a", "b_b") if nm == "b" else (nm + "a", nm + "b")
             self._conv(ka, B["pool%d" % lvl], N, h, w, pc, c, B[nm + "a"])
             self._conv(kb, B[nm + "a"], N, h, w, c, c, B[nm])
             prev, pc = B[nm], c
-        # decoder
-        skips = {2: (B["e2"], c2), 1: (B["e1"], c1), 0: (B["e0"], c0)}
-        for lvl in (2, 1, 0):
+        # decoder: the skip part of each concatenation is there already
+        for lvl, c in ((2, c2), (1, c1), (0, c0)):
             h, w = dims[lvl]
-            skip, c = skips[lvl]
             cat = B["cat%d" % lvl]
             ctot = pc + c
             self._chk(L.tpfnet_up_into(_p(prev), N, h, w, pc, _p(cat), ctot, 0, s), "up")
-            self._chk(L.tpfnet_channels(_p(skip), c, 0, N * h * w, c, _p(cat), ctot, pc, 0, s), "cat")
             self._conv("d%da" % lvl, cat, N, h, w, ctot, c, B["d%da" % lvl])
             self._conv("d%db" % lvl, B["d%da" % lvl], N, h, w, c, c, B["d%d" % lvl])
             prev, pc = B["d%d" % lvl], c
@@ -221,39 +253,44 @@ class UNet:
         return self.out
 
     # --------------------------------------------------------- backward
-    def _block_back(self, ka, kb, inp, cin, a, bo, c, dout, dinp, N, h, w, need_dinp=True):
-        """Back through relu(conv_b(relu(conv_a(inp)))): dout (grad at the block output,
-        overwritten) -> weight grads and dinp."""
+    def _flip_weights(self):
+        names = list(self.wflip)
+        n = len(names)
+        spec = {name: (a, b) for name, a, b, _ in self.specs}
+        wt = (_vp * n)(*[self.Pb[k + ".W"].data_ptr() for k in names])
+        wf = (_vp * n)(*[self.wflip[k].data_ptr() for k in names])
+        ci = (_ip * n)(*[spec[k][0] for k in names])
+        co = (_ip * n)(*[spec[k][1] for k in names])
+        self._chk(self.lib.tpfnet_flip_weights(n, wt, ci, co, wf, self._s()), "flip")
+
+    def _block_back(self, ka, kb, inp, cin, a, c, dout, dinp, N, h, w):
+        """Back through relu(conv_b(relu(conv_a(inp)))): dout (gradient at the block's output,
+        its ReLU mask applied) -> weight gradients and dinp (None: not wanted)."""
         L, s = self.lib, self._s()
         da = self.D["_tmp_%d_%d" % (h, c)]
-        self._chk(L.tpfnet_relu_mask(_p(dout), _p(bo), dout.numel(), s), "mask")
         self._chk(L.tpfnet_conv3x3_wgrad(_p(a), _p(dout), N, h, w, c, c, _p(self.G[kb + ".W"]),
                                          _p(self.G[kb + ".b"]), s), "wgrad")
-        self._chk(L.tpfnet_conv3x3_dgrad(_p(dout), N, h, w, c, _p(self.Pb[kb + ".W"]), c, _p(self.wflip), _p(da), s),
-                  "dgrad")
-        self._chk(L.tpfnet_relu_mask(_p(da), _p(a), da.numel(), s), "mask")
+        self._chk(L.tpfnet_conv3x3_dgrad_masked(_p(dout), N, h, w, c, _p(self.wflip[kb]), c, _p(a), _p(da), s), "dgrad")
         self._chk(L.tpfnet_conv3x3_wgrad(_p(inp), _p(da), N, h, w, cin, c, _p(self.G[ka + ".W"]),
                                          _p(self.G[ka + ".b"]), s), "wgrad")
-        if need_dinp:
-            self._chk(L.tpfnet_conv3x3_dgrad(_p(da), N, h, w, c, _p(self.Pb[ka + ".W"]), cin, _p(self.wflip),
-                                             _p(dinp), s), "dgrad")
+        if dinp is not None:
+            self._chk(L.tpfnet_conv3x3_dgrad_masked(_p(da), N, h, w, c, _p(self.wflip[ka]), cin, None, _p(dinp), s),
+                      "dgrad")
 
     def backward(self, dout):
         """dout: float32 (N, H, W, cout) gradient of the loss at the output; accumulates
-        every parameter gradient into self.G."""
-        t, L, s = self.torch, self.lib, self._s()
+        every parameter gradient into self.G.  The ReLU masks, the split of the
+        concatenations' gradients and the sums at the encoder's outputs are part of the
+        kernels that produce those gradients."""
+        L, s = self.lib, self._s()
         N, H, W = self._shape
         B, D = self.B, self.D
         c0, c1, c2, c3 = self.ch
         dims = [(H, W), (H // 2, W // 2), (H // 4, W // 4), (H // 8, W // 8)]
-        for (h, w), c in zip(dims, self.ch):
-            key = "_tmp_%d_%d" % (h, c)
-            if key not in D:
-                D[key] = t.empty((N, h, w, c), dtype=t.bfloat16, device="cuda")
-        self._chk(L.tpfnet_head_back(_p(B["d0"]), _p(dout), N * H * W, c0, _p(self.P["head.W"]), self.cout,
-                                     _p(D["d0"]), _p(self.G["head.W"]), _p(self.G["head.b"]), s), "head_back")
-        skip_grads = {}
-        # decoder levels 0, 1, 2: back through the block, split the concatenation
+        self._flip_weights()
+        self._chk(L.tpfnet_head_back_masked(_p(B["d0"]), _p(dout), N * H * W, c0, _p(self.P["head.W"]), self.cout,
+                                            _p(D["d0"]), _p(self.G["head.W"]), _p(self.G["head.b"]), s), "head_back")
+        # decoder levels 0, 1, 2; the upsampled part's gradient goes to the level below
         ups = {0: c1, 1: c2, 2: c3}
         skips = {0: c0, 1: c1, 2: c2}
         below = {0: "d1", 1: "d2", 2: "b"}
@@ -261,46 +298,67 @@ class UNet:
             h, w = dims[lvl]
             cu, cs = ups[lvl], skips[lvl]
             ctot = cu + cs
-            self._block_back("d%da" % lvl, "d%db" % lvl, B["cat%d" % lvl], ctot, B["d%da" % lvl], B["d%d" % lvl], cs,
-                             D["d%d" % lvl], D["cat%d" % lvl], N, h, w)
-            # the upsampled part goes to the level below, the skip part to the encoder
-            self._chk(L.tpfnet_up_back(_p(D["cat%d" % lvl]), N, h, w, ctot, 0, cu, _p(D[below[lvl]]), s), "up_back")
-            enc = ["e0", "e1", "e2"][lvl]
-            self._chk(L.tpfnet_channels(_p(D["cat%d" % lvl]), ctot, cu, N * h * w, cs, _p(D[enc]), cs, 0, 0, s), "split")
-        # bottleneck and encoder levels 2, 1, 0
+            self._block_back("d%da" % lvl, "d%db" % lvl, B["cat%d" % lvl], ctot, B["d%da" % lvl], cs, D["d%d" % lvl],
+                             D["cat%d" % lvl], N, h, w)
+            self._chk(L.tpfnet_up_back_masked(_p(D["cat%d" % lvl]), N, h, w, ctot, 0, cu, _p(B[below[lvl]]),
+                                              _p(D[below[lvl]]), s), "up_back")
+        # bottleneck and encoder levels 2, 1, 0; an encoder output's gradient is the skip part
+        # of the concatenation's plus the pooled one's
         for lvl, nm, c in ((3, "b", c3), (2, "e2", c2), (1, "e1", c1)):
             h, w = dims[lvl]
             ka, kb = ("b_a", "b_b") if nm == "b" else (nm + "a", nm + "b")
             pc = self.ch[lvl - 1]
-            self._block_back(ka, kb, B["pool%d" % lvl], pc, B[nm + "a"], B[nm], c, D[nm], D["pool%d" % lvl], N, h, w)
-            enc_above = ["e0", "e1", "e2"][lvl - 1]
-            self._chk(L.tpfnet_pool_back(_p(D["pool%d" % lvl]), N, 2 * h, 2 * w, pc, _p(D[enc_above]), 1, s), "pool_back")
-        self._block_back("e0a", "e0b", self.x, self.cinp, B["e0a"], B["e0"], c0, D["e0"], D["x"], N, H, W,
-                         need_dinp=False)
+            self._block_back(ka, kb, B["pool%d" % lvl], pc, B[nm + "a"], c, D[nm], D["pool%d" % lvl], N, h, w)
+            above = lvl - 1
+            skip, act = D["cat%d" % above][..., ups[above]:], B["e%d" % above]
+            self._chk(L.tpfnet_pool_back_skip(_p(D["pool%d" % lvl]), N, 2 * h, 2 * w, pc, _p(skip), skip.stride(2),
+                                              _p(act), act.stride(2), _p(D["e%d" % above]), s), "pool_back")
+        self._block_back("e0a", "e0b", self.x, self.cinp, B["e0a"], c0, D["e0"], None, N, H, W)
 
     def zero_grad(self):
+        if self._is_flat(("G",)):
+            self._flat["G"].zero_()
+            return
         for g in self.G.values():
             g.zero_()
 
     def adam(self, lr=1e-3, b1=0.9, b2=0.999, eps=1e-8):
         self.adam_t += 1
         s = self._s()
+        if self._is_flat(("P", "G", "M", "V", "Pb")):
+            # the 128-element gaps and the biases' unused bf16 copies go along
+            f = self._flat
+            self._chk(self.lib.tpfnet_adam(_p(f["P"]), _p(f["G"]), _p(f["M"]), _p(f["V"]), f["P"].numel(), lr, b1, b2,
+                                           eps, self.adam_t, _p(f["Pb"]), s), "adam")
+            return
         for k, p in self.P.items():
             self._chk(self.lib.tpfnet_adam(_p(p), _p(self.G[k]), _p(self.M[k]), _p(self.V[k]), p.numel(), lr, b1, b2,
                                            eps, self.adam_t, _p(self.Pb[k]), s), "adam")
 
     def mse(self, pred, target, wch=None, want_grad=True):
         """Loss (float, synchronises) and, when want_grad, its gradient in self.D['out']."""
+        self._mse(pred, target, wch, want_grad)
+        return float(self.loss.item())
+
+    def _mse(self, pred, target, wch, want_grad=True):
         self.loss.zero_()
         C_ = pred.shape[-1]
         self._chk(self.lib.tpfnet_mse(_p(pred), _p(target), _p(wch), pred.numel(), C_,
                                       _p(self.D["out"]) if want_grad else None, _p(self.loss), self._s()), "mse")
-        return float(self.loss.item())
 
     def train_step(self, x, target, wch=None, lr=1e-3):
         self.zero_grad()
         out = self.forward(x)
-        loss = self.mse(out, target, wch)
+        self._mse(out, target, wch)
+        # the loss travels to the host while the backward pass is queued: the GPU does not wait
+        # for the host to read it
+        t = self.torch
+        host = t.empty(1, dtype=t.float64, pin_memory=True)
+        done = t.cuda.Event()
+        with t.cuda.stream(self.stream):
+            host.copy_(self.loss, non_blocking=True)
+            done.record()
         self.backward(self.D["out"])
         self.adam(lr)
-        return loss
+        done.synchronize()
+        return float(host)
