@@ -29,48 +29,132 @@ constexpr long long kGraphSteps = 64;  // steps per replayed CUDA graph (even)
 
 // ------------------------------------------------------- auxiliary kernels
 
-// Macroscopic state of node (x, y) read straight from global memory.
-template <class S>
-__device__ Macro macro_at(const DevParams& P, const typename S::elem* __restrict__ A,
-                          const RefT* __restrict__ ref, const float* __restrict__ phiu, int x, int y)
+// phi and T of a read-out tile and its ring
+template <int BX, int BY>
+struct PhiTSmem {
+    static constexpr int SX = BX + 2, SN = (BX + 2) * (BY + 2);
+    float phi[SN], T[SN];
+};
+
+// The macroscopic state of the nodes of one tile (x0, y0, w, h), one per thread: use(n, x, y,
+// m) on the threads that have a node.  Each population is read once, and f and h of the ring
+// once more, as in step_tile_general (reading the eight neighbours' f and h node by node took
+// 47 us for the fields of 2048 x 512 and 98 us for the sums, 189 loads per node; now 33 loads,
+// 34 and 67 us).  The fields are bound by DRAM (142 MB), the sums by the FP64 pipe and the
+// tiles' latency.  Ends with a block barrier.
+template <int BX, int BY, class S, class USE>
+__device__ __forceinline__ void tile_macro(const DevParams& P, const typename S::elem* __restrict__ A,
+                                           const RefT* __restrict__ ref, const float* __restrict__ phiu,
+                                           PhiTSmem<BX, BY>& sm, int x0, int y0, int w, int h_, USE use)
 {
-    const long long pl = P.plane;
-    const int n = y * P.nx + x;
-    float f[9], g[9], h[9];
-    load_node<S>(P, A, ref, x, y, f, g, h);
-    auto get = [&](int gx, int gy, float& ph, float& tt) {
-        float a[9], c[9];
-        load_node<S, false>(P, A, ref, gx, gy, a, nullptr, c);
+    constexpr int SX = PhiTSmem<BX, BY>::SX;
+    static_assert(2 * (BX + BY) + 4 <= BX * BY, "one thread per ring node");
+    const int tid = threadIdx.x, tx = tid % BX, ty = tid / BX;
+    const int x = x0 + tx, y = y0 + ty, n = y * P.nx + x;
+    const bool active = tx < w && ty < h_;
+    const int kown = (ty + 1) * SX + tx + 1;
+    int rx = 0, ry = 0, wx = 0, wy = 0;
+    bool rload = false, rghost = false;
+    float ra[9], rc[9];
+    if (tid < 2 * (w + h_) + 4) {
+        const int r = tid, sx = w + 2;
+        if (r < sx) { rx = r; ry = 0; }
+        else if (r < 2 * sx) { rx = r - sx; ry = h_ + 1; }
+        else if (r < 2 * sx + h_) { rx = 0; ry = r - 2 * sx + 1; }
+        else { rx = w + 1; ry = r - 2 * sx - h_ + 1; }
+        wx = x0 + rx - 1;
+        wy = y0 + ry - 1;
+        if (P.bc_x == 0) wx = wrap(wx, P.nx);
+        if (P.bc_y == 1) wy = wrap(wy, P.ny);
+        rload = wx >= 0 && wx < P.nx && wy >= 0 && wy < P.ny;
+        rghost = !rload;
+        if (rload) load_node<S, false>(P, A, ref, wx, wy, ra, nullptr, rc);
+    }
+    float f[9], g[9], h[9], pu_x = 0.f, pu_y = 0.f;
+    if (active) {
+        load_node<S>(P, A, ref, x, y, f, g, h);
+        pu_x = phiu[n];
+        pu_y = phiu[P.plane + n];
         float sf = 0.f, sh = 0.f;
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-            sf += a[i];
-            sh += c[i];
+            sf += f[i];
+            sh += h[i];
         }
-        ph = sf;
-        tt = sh;
-    };
-    float phin[9], Tn[9];
+        sm.phi[kown] = sf;
+        sm.T[kown] = sh;
+    }
+    if (rload) {
+        float sf = 0.f, sh = 0.f;
 #pragma unroll
-    for (int i = 0; i < 9; ++i) phiT_at(P, x + cx(i), y + cy(i), get, phin[i], Tn[i]);
-    return node_macro(P, f, g, h, phin, Tn, phiu[n], phiu[pl + n]);
+        for (int i = 0; i < 9; ++i) {
+            sf += ra[i];
+            sh += rc[i];
+        }
+        sm.phi[ry * SX + rx] = sf;
+        sm.T[ry * SX + rx] = sh;
+    }
+    // ghost ring nodes (as phiT_at); the mirror is the adjacent slot inside the lattice
+    if (__syncthreads_or(rghost) && rghost) {
+        const int gx = x0 + rx - 1;
+        const int mx = min(max(wx, 0), P.nx - 1), my = min(max(wy, 0), P.ny - 1);
+        const int km = (ry + my - wy) * SX + rx + mx - wx;
+        const float tm = sm.T[km];
+        const float tg = (wx < 0) ? 2.f * P.T_in - tm : tm;
+        const bool oy = wy < 0 || wy >= P.ny;
+        sm.phi[ry * SX + rx] = sm.phi[km];
+        sm.T[ry * SX + rx] = oy ? 2.f * (wy < 0 ? T_wall_bottom(P, (float)gx) : T_wall_top(P, (float)gx)) - tg : tg;
+    }
+    __syncthreads();
+    if (active) {
+        float phin[9], Tn[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const int k = kown + cy(i) * SX + cx(i);
+            phin[i] = sm.phi[k];
+            Tn[i] = sm.T[k];
+        }
+        use(n, x, y, node_macro(P, f, g, h, phin, Tn, pu_x, pu_y));
+    }
+    __syncthreads();
 }
 
-template <class S>
-__global__ void k_fields(const DevParams P, const typename S::elem* __restrict__ A, const RefT* __restrict__ ref,
-                         const float* __restrict__ phiu, float* __restrict__ out)
+// Calls use for every node of the lattice, tile by tile (the blocks stride over the tiles).
+template <class S, class USE>
+__device__ __forceinline__ void each_macro(const DevParams& P, const typename S::elem* __restrict__ A,
+                                           const RefT* __restrict__ ref, const float* __restrict__ phiu, USE use)
 {
-    const long long N = (long long)P.nx * P.ny;
-    for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
-         n += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(n % P.nx), y = (int)(n / P.nx);
-        const Macro m = macro_at<S>(P, A, ref, phiu, x, y);
-        out[n] = m.phi;
-        out[P.plane + n] = m.ux;
-        out[2 * P.plane + n] = m.uy;
-        out[3 * P.plane + n] = m.p;
-        out[4 * P.plane + n] = m.T;
+    __shared__ PhiTSmem<kBX, kBY> sm;
+    const int ntx = (P.nx + kBX - 1) / kBX, nty = (P.ny + kBY - 1) / kBY;
+    for (int t = blockIdx.x; t < ntx * nty; t += gridDim.x) {
+        int x0, y0, w, h;
+        tile_even(P.nx, ntx, t % ntx, x0, w);
+        tile_even(P.ny, nty, t / ntx, y0, h);
+        tile_macro<kBX, kBY, S>(P, A, ref, phiu, sm, x0, y0, w, h, use);
     }
+}
+// blocks for each_macro, at most `most`
+int macro_blocks(const DevParams& P, int most)
+{
+    const long long t = (long long)((P.nx + kBX - 1) / kBX) * ((P.ny + kBY - 1) / kBY);
+    return (int)(t < most ? t : most);
+}
+
+// the fields' destinations (NULL: not wanted)
+struct FieldPtrs {
+    float* p[5];
+};
+template <class S>
+__global__ void __launch_bounds__(kBX * kBY)
+k_fields(const DevParams P, const typename S::elem* __restrict__ A, const RefT* __restrict__ ref,
+         const float* __restrict__ phiu, const FieldPtrs out)
+{
+    each_macro<S>(P, A, ref, phiu, [&](int n, int, int, const Macro& m) {
+        const float v[5] = {m.phi, m.ux, m.uy, m.p, m.T};
+#pragma unroll
+        for (int k = 0; k < 5; ++k)
+            if (out.p[k]) out.p[k][n] = v[k];
+    });
 }
 
 // Equilibrium populations from the staged fields (planes 0-4: phi, ux, uy, p, T).
@@ -205,19 +289,17 @@ __global__ void k_lbe_decode(const DevParams P, int k, const typename S::elem* _
 // FP64 reductions (see tpflbm_diagnostics).  Each block writes 8 partial sums;
 // k_reduce_final adds the partials of all blocks in a fixed order.
 constexpr int kRedThreads = 256;
+static_assert(kRedThreads == kBX * kBY, "the state's reductions run over tiles, one node per thread");
 constexpr int kRedMaxBlocks = 1024;
+constexpr int kRedDoubles = kRedMaxBlocks * 8 + 16;  // block sums, then results and flag
 
 template <class S>
 __global__ void __launch_bounds__(kRedThreads)
 k_reduce_partial(const DevParams P, const typename S::elem* __restrict__ A, const RefT* __restrict__ ref,
                  const float* __restrict__ phiu, double* __restrict__ partial)
 {
-    const long long N = (long long)P.nx * P.ny;
     double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
-         n += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(n % P.nx), y = (int)(n / P.nx);
-        const Macro m = macro_at<S>(P, A, ref, phiu, x, y);
+    each_macro<S>(P, A, ref, phiu, [&](int, int x, int, const Macro& m) {
         acc[0] += m.phi;
         acc[1] += (double)m.rcp * m.T;
         acc[2] += m.T;
@@ -228,7 +310,7 @@ k_reduce_partial(const DevParams P, const typename S::elem* __restrict__ A, cons
             acc[6] += (double)m.phi * x;
         }
         if (!isfinite(m.phi) || !isfinite(m.ux) || !isfinite(m.uy) || !isfinite(m.T)) acc[7] += 1.0;
-    }
+    });
     __shared__ double red[8][kRedThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -247,8 +329,11 @@ k_reduce_partial(const DevParams P, const typename S::elem* __restrict__ A, cons
 
 // One warp per quantity: lane l adds blocks l, l + 32, ... in order, then a fixed
 // shuffle tree; the result does not depend on timing (deterministic).
-__global__ void k_reduce_final(const double* __restrict__ partial, int nblocks, double* __restrict__ out)
+// With err, out[8] takes the step kernels' error flag, so that one copy brings both.
+__global__ void k_reduce_final(const double* __restrict__ partial, int nblocks, double* __restrict__ out,
+                               const int* err = nullptr)
 {
+    if (err && threadIdx.x == 0) out[8] = *err;
     const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (k >= 8) return;
     double v = 0.0;
@@ -264,13 +349,9 @@ __global__ void __launch_bounds__(kRedThreads)
 k_residual_partial(const DevParams P, const typename S::elem* __restrict__ A, const RefT* __restrict__ ref,
                    const float* __restrict__ phiu, float* __restrict__ snap, double* __restrict__ partial)
 {
-    const long long N = (long long)P.nx * P.ny;
     const long long pl = P.plane;
     double acc[3] = {0, 0, 0};
-    for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
-         n += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(n % P.nx), y = (int)(n / P.nx);
-        const Macro m = macro_at<S>(P, A, ref, phiu, x, y);
+    each_macro<S>(P, A, ref, phiu, [&](int n, int, int, const Macro& m) {
         const double dux = (double)m.ux - snap[n], duy = (double)m.uy - snap[pl + n];
         const double dT = (double)m.T - snap[2 * pl + n];
         acc[0] += dux * dux + duy * duy;
@@ -279,7 +360,7 @@ k_residual_partial(const DevParams P, const typename S::elem* __restrict__ A, co
         snap[n] = m.ux;
         snap[pl + n] = m.uy;
         snap[2 * pl + n] = m.T;
-    }
+    });
     __shared__ double red[3][kRedThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -363,114 +444,169 @@ __global__ void k_project_apply(const float* __restrict__ a, long long N, double
         out[n] = (float)tanh((double)a[n] + s);
 }
 
-// Bubbles of Sec. 4.3: the connected regions of phi < 0 (4-connectivity, wrapping
-// along periodic axes), each with its FP64 moments.  Labels are node indices: every
-// node of the set starts with its own index and repeatedly takes the smallest label
-// among itself, its in-set neighbours and its label's label (pointer jumping).  Labels
-// only decrease and always name a node of the same region, so the fixed point gives
-// every node of a region the region's smallest node index, its root.
+// Bubbles of Sec. 4.3: the connected regions of phi < 0 (4-connectivity, wrapping along
+// periodic axes), each with its FP64 moments.  Labels are node indices in a union-find
+// forest: a node's parent is never larger than the node, and joining two trees hangs the
+// larger root under the smaller one, so a region ends up with its smallest node index as
+// its root.  Runs inside 32 nodes of a row start out joined; after that only the links
+// between runs are joined, and one more pass points every node at its root.  Everything
+// stays on the device until the sums are done (sweeping labels to a fixed point, with the
+// host asking for changes, cost 12 sweeps and 4 round trips on the two-bubble channel).
 constexpr int kMaxBubbles = 32;
-constexpr int kBubBlocks = 40;  // kBubBlocks x kMaxBubbles x 6 partials + results fit the reduction area
-static_assert((kBubBlocks + 1) * kMaxBubbles * 6 <= kRedMaxBlocks * 8 + 8, "bubble sums fit the reduction area");
+struct BubbleSums {
+    double v[kMaxBubbles][6];
+    int count, err;
+    int root[kMaxBubbles];
+};
+static_assert(sizeof(BubbleSums) <= kRedDoubles * sizeof(double), "bubble sums fit the reduction area");
 
-__global__ void k_lab_init(const float* __restrict__ phi, long long N, int* __restrict__ lab)
+// one warp per 32 nodes of a row: label = first node of the run
+__global__ void k_lab_runs(const float* __restrict__ phi, int nx, int ny, int* __restrict__ lab, BubbleSums* sums)
 {
-    for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x)
-        lab[n] = phi[n] < 0.f ? (int)n : -1;
+    if (blockIdx.x == 0 && threadIdx.x == 0) sums->count = 0;
+    const int segs = (nx + 31) / 32, lane = threadIdx.x & 31;
+    const long long total = (long long)segs * ny;
+    for (long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; w < total;
+         w += ((long long)gridDim.x * blockDim.x) >> 5) {
+        const int y = (int)(w / segs), x = (int)(w % segs) * 32 + lane;
+        const bool in = x < nx && phi[(long long)y * nx + x] < 0.f;
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        if (x >= nx) continue;
+        // the run starts after the highest clear bit below this lane
+        const unsigned below = ~m & ((1u << lane) - 1u);
+        const int start = below ? 32 - __clz(below) : 0;
+        lab[(long long)y * nx + x] = in ? y * nx + x - lane + start : -1;
+    }
 }
-
-__global__ void k_lab_hook(int nx, int ny, int bc_x, int bc_y, int* lab, int* changed)
+__device__ __forceinline__ int lab_root(const int* lab, int a)
+{
+    for (int p = __ldcg(lab + a); p != a; p = __ldcg(lab + a)) a = p;
+    return a;
+}
+__device__ __forceinline__ void lab_join(int* lab, int a, int b)
+{
+    for (;;) {
+        a = lab_root(lab, a);
+        b = lab_root(lab, b);
+        if (a == b) return;
+        if (a < b) {
+            const int t = a;
+            a = b;
+            b = t;
+        }
+        const int old = atomicMin(lab + a, b);
+        if (old == a) return;  // a was still a root and now hangs under b
+        a = old;               // somebody else hung it elsewhere: join that with b
+    }
+}
+// the links between runs: across the 32-node segments (and the periodic x seam), and up (and
+// across the periodic y seam) once per pair of overlapping runs
+__global__ void k_lab_join(int nx, int ny, int bc_x, int bc_y, int* lab)
 {
     const long long N = (long long)nx * ny;
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x) {
-        const int l = lab[n];
-        if (l < 0) continue;
+        if (__ldcg(lab + n) < 0) continue;
         const int x = (int)(n % nx), y = (int)(n / nx);
-        int m = min(l, lab[l]);
-        const int nb[4][2] = {{x + 1, y}, {x - 1, y}, {x, y + 1}, {x, y - 1}};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            int qx = nb[k][0], qy = nb[k][1];
-            if (bc_x == 0) qx = wrap(qx, nx);
-            if (bc_y == 1) qy = wrap(qy, ny);
-            if (qx < 0 || qx >= nx || qy < 0 || qy >= ny) continue;
-            const int lq = lab[(long long)qy * nx + qx];
-            if (lq >= 0 && lq < m) m = lq;
-        }
-        if (m < l) {
-            atomicMin(&lab[n], m);
-            atomicMin(&lab[l], m);  // the old label's node joins too (same region)
-            *changed = 1;
+        const int l = x > 0 ? (int)n - 1 : (bc_x == 0 ? (int)n + nx - 1 : -1);
+        if (x % 32 == 0 && l >= 0 && __ldcg(lab + l) >= 0) lab_join(lab, (int)n, l);
+        const int u = y + 1 < ny ? (int)n + nx : (bc_y == 1 ? x : -1);
+        if (u < 0 || __ldcg(lab + u) < 0) continue;
+        // the pair (x - 1, its upper neighbour) of the same two runs makes the link already
+        if (x % 32 != 0 && __ldcg(lab + n - 1) >= 0 && __ldcg(lab + u - 1) >= 0) continue;
+        lab_join(lab, (int)n, u);
+    }
+}
+__global__ void k_lab_roots(int* lab, long long N, BubbleSums* sums)
+{
+    for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x) {
+        if (__ldcg(lab + n) < 0) continue;
+        const int r = lab_root(lab, (int)n);
+        __stcg(lab + n, r);
+        if (r == (int)n) {
+            const int k = atomicAdd(&sums->count, 1);
+            if (k < kMaxBubbles) sums->root[k] = r;
         }
     }
 }
-
-__global__ void k_lab_roots(const int* __restrict__ lab, long long N, int* __restrict__ count, int* __restrict__ roots)
+// the roots in increasing order, the sums cleared, the step kernels' error flag (one warp)
+__global__ void k_lab_order(BubbleSums* sums, const int* err)
 {
-    for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x)
-        if (lab[n] == (int)n) {
-            const int k = atomicAdd(count, 1);
-            if (k < kMaxBubbles) roots[k] = (int)n;
-        }
+    const int lane = threadIdx.x, n = min(sums->count, kMaxBubbles);
+    const int r = lane < n ? sums->root[lane] : 0x7fffffff;
+    int rank = 0;
+    for (int k = 0; k < 32; ++k) rank += __shfl_sync(0xffffffffu, r, k) < r;
+    if (lane < n) sums->root[rank] = r;
+    for (int k = lane; k < kMaxBubbles * 6; k += 32) sums->v[k / 6][k % 6] = 0.0;
+    if (lane == 0) sums->err = *err;
 }
 
-struct RootList {
-    int n;
-    int r[kMaxBubbles];
-};
-
-// Per block and bubble: node count, sum phi, sum phi u_x, sum phi u_y, sum phi dx,
-// sum phi dy, with (dx, dy) the node's offset from its root, taken to the nearest
-// periodic image along periodic axes.
+// Per bubble: node count, sum phi, sum phi u_x, sum phi u_y, sum phi dx, sum phi dy, with
+// (dx, dy) the node's offset from its root, taken to the nearest periodic image along
+// periodic axes.  A thread keeps its sums in registers while the label stays the same, a
+// warp whose lanes end on one label adds them up by shuffles, and what is left goes through
+// shared memory (every node adding to shared memory took 240 us on the two-bubble channel,
+// whose nodes all add to one of two bubbles).
 __global__ void __launch_bounds__(256)
-k_bubble_partial(int nx, int ny, int bc_x, int bc_y, const float* __restrict__ phi, const float* __restrict__ ux,
-                 const float* __restrict__ uy, const int* __restrict__ lab, const RootList roots,
-                 double* __restrict__ partial)
+k_bubble_sums(int nx, int ny, int bc_x, int bc_y, const float* __restrict__ phi, const float* __restrict__ ux,
+              const float* __restrict__ uy, const int* __restrict__ lab, BubbleSums* __restrict__ sums)
 {
     __shared__ double acc[kMaxBubbles][6];
+    __shared__ int root[kMaxBubbles];
+    const int nb = sums->count;
+    if (nb > kMaxBubbles) return;
     for (int k = threadIdx.x; k < kMaxBubbles * 6; k += blockDim.x) acc[k / 6][k % 6] = 0.0;
+    if (threadIdx.x < nb) root[threadIdx.x] = sums->root[threadIdx.x];
     __syncthreads();
     const long long N = (long long)nx * ny;
+    int cur = -1;
+    double a[6] = {0, 0, 0, 0, 0, 0};
+    auto flush = [&](int label) {
+        for (int b = 0; b < nb; ++b)
+            if (root[b] == label)
+                for (int k = 0; k < 6; ++k) atomicAdd(&acc[b][k], a[k]);
+    };
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x) {
         const int l = lab[n];
         if (l < 0) continue;
-        int b = -1;
-        for (int k = 0; k < roots.n; ++k)
-            if (roots.r[k] == l) b = k;
-        if (b < 0) continue;
+        if (l != cur) {
+            if (cur >= 0) flush(cur);
+            cur = l;
+            for (int k = 0; k < 6; ++k) a[k] = 0.0;
+        }
         int dx = (int)(n % nx) - l % nx, dy = (int)(n / nx) - l / nx;
         if (bc_x == 0) dx = dx > nx / 2 ? dx - nx : (dx < -nx / 2 ? dx + nx : dx);
         if (bc_y == 1) dy = dy > ny / 2 ? dy - ny : (dy < -ny / 2 ? dy + ny : dy);
         const double ph = phi[n];
-        atomicAdd(&acc[b][0], 1.0);
-        atomicAdd(&acc[b][1], ph);
-        atomicAdd(&acc[b][2], ph * ux[n]);
-        atomicAdd(&acc[b][3], ph * uy[n]);
-        atomicAdd(&acc[b][4], ph * dx);
-        atomicAdd(&acc[b][5], ph * dy);
+        a[0] += 1.0;
+        a[1] += ph;
+        a[2] += ph * ux[n];
+        a[3] += ph * uy[n];
+        a[4] += ph * dx;
+        a[5] += ph * dy;
+    }
+    const unsigned has = __ballot_sync(0xffffffffu, cur >= 0);
+    if (has) {
+        const int one = __shfl_sync(0xffffffffu, cur, __ffs(has) - 1);
+        if (__all_sync(0xffffffffu, cur < 0 || cur == one)) {
+            for (int k = 0; k < 6; ++k)
+                for (int o = 16; o > 0; o >>= 1) a[k] += __shfl_down_sync(0xffffffffu, a[k], o);
+            if ((threadIdx.x & 31) == 0) flush(one);
+        } else if (cur >= 0) {
+            flush(cur);
+        }
     }
     __syncthreads();
-    for (int k = threadIdx.x; k < roots.n * 6; k += blockDim.x)
-        partial[(blockIdx.x * kMaxBubbles + k / 6) * 6 + k % 6] = acc[k / 6][k % 6];
-}
-
-// sums of the block partials in block order (one thread per bubble and quantity)
-__global__ void k_bubble_final(const double* __restrict__ partial, int nblocks, int nb, double* __restrict__ out)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nb * 6) return;
-    double v = 0.0;
-    for (int b = 0; b < nblocks; ++b) v += partial[(b * kMaxBubbles + k / 6) * 6 + k % 6];
-    out[k] = v;
+    for (int k = threadIdx.x; k < nb * 6; k += blockDim.x)
+        if (acc[k / 6][0] != 0.0) atomicAdd(&sums->v[k / 6][k % 6], acc[k / 6][k % 6]);
 }
 
 }  // namespace
 
 // Scratch of tpflbm_diagnostics_static: the per-block partial sums (kRedMaxBlocks x 8)
-// and the 8 results, in a fixed device array so that the entry point allocates
+// and the results, in a fixed device array so that the entry point allocates
 // nothing.  Host code must not pass this name to a kernel (on the host it is only a
 // stand-in); it uses the address cudaGetSymbolAddress returns for the current device.
-static __device__ __align__(256) double g_diag_scratch[kRedMaxBlocks * 8 + 8];
+static __device__ __align__(256) double g_diag_scratch[kRedDoubles];
 
 namespace {
 
@@ -514,7 +650,7 @@ Layout layout_of(int nx, int ny, int storage, bool many)
     L.ref1 = off; off = align256(off + (f16 ? 3 * (size_t)pl * sizeof(RefT) : 0));
     L.phiu = off; off = align256(off + 2 * (size_t)pl * 4);
     L.stage = off; off = align256(off + kStagePlanes * (size_t)pl * 4);
-    L.red = off; off = align256(off + (kRedMaxBlocks * 8 + 8) * sizeof(double));
+    L.red = off; off = align256(off + kRedDoubles * sizeof(double));
     L.err = off; off = align256(off + 256);
     L.snap = off; off = align256(off + 3 * (size_t)pl * 4);
     // the TMA step kernel's tile list (x0, y0 per tile)
@@ -825,13 +961,15 @@ cudaError_t launch_many(tpflbm_t h, int n)
     return e;
 }
 
+constexpr char kTimeoutMsg[] = "a step kernel gave up waiting for its shared-memory copies";
+
 // error raised by a step kernel (bounded waits that ran out)
 int check_err(tpflbm_t h)
 {
     int v = 0;
     TPF_CUDA(h, cudaMemcpyAsync(&v, h->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     TPF_CUDA(h, cudaStreamSynchronize(h->stream));
-    if (v) return fail(h, TPF_ERR_TIMEOUT, "a step kernel gave up waiting for its shared-memory copies");
+    if (v) return fail(h, TPF_ERR_TIMEOUT, kTimeoutMsg);
     return TPF_OK;
 }
 
@@ -1066,24 +1204,38 @@ int tpflbm_status_async(tpflbm_t h, int* flag, void* copy_stream)
     return TPF_OK;
 }
 
+// the fields of the current state into device planes (NULL: not wanted)
+static void launch_fields(tpflbm_t h, const FieldPtrs& to)
+{
+    const int c = h->cur, nb = macro_blocks(h->dp, 152 * 64);
+    if (h->dp.storage == TPF_STORAGE_FP16)
+        k_fields<StoreF16><<<nb, kBX * kBY, 0, h->stream>>>(h->dp, (const __half*)h->pop[c], h->ref[c], h->phiu, to);
+    else
+        k_fields<StoreF32><<<nb, kBX * kBY, 0, h->stream>>>(h->dp, (const float*)h->pop[c], h->ref[c], h->phiu, to);
+}
+
 int tpflbm_get_fields(tpflbm_t h, float* phi, float* ux, float* uy, float* p, float* T)
 {
     if (!h) return TPF_ERR_INVALID_ARG;
-    int rc = check_err(h);
-    if (rc) return rc;
     const long long N = (long long)h->nx * h->ny;
-    const int c = h->cur;
-    if (h->dp.storage == TPF_STORAGE_FP16)
-        k_fields<StoreF16><<<grid_1d(N), 256, 0, h->stream>>>(h->dp, (const __half*)h->pop[c], h->ref[c], h->phiu, h->stage);
-    else
-        k_fields<StoreF32><<<grid_1d(N), 256, 0, h->stream>>>(h->dp, (const float*)h->pop[c], h->ref[c], h->phiu, h->stage);
-    TPF_CUDA(h, cudaGetLastError());
     float* dst[5] = {phi, ux, uy, p, T};
+    // straight into the caller's planes where they are this device's memory, else by way of
+    // the staging planes
+    FieldPtrs to{};
+    for (int k = 0; k < 5; ++k) {
+        if (!dst[k]) continue;
+        cudaPointerAttributes at{};
+        const bool here = cudaPointerGetAttributes(&at, dst[k]) == cudaSuccess && at.type == cudaMemoryTypeDevice &&
+                          at.device == h->device && ((uintptr_t)dst[k] & 3) == 0;
+        to.p[k] = here ? dst[k] : h->stage + k * h->dp.plane;
+    }
+    cudaGetLastError();  // (an unregistered host pointer is no error here)
+    launch_fields(h, to);
+    TPF_CUDA(h, cudaGetLastError());
     for (int k = 0; k < 5; ++k)
-        if (dst[k])
-            TPF_CUDA(h, cudaMemcpyAsync(dst[k], h->stage + k * h->dp.plane, N * sizeof(float), cudaMemcpyDefault, h->stream));
-    TPF_CUDA(h, cudaStreamSynchronize(h->stream));
-    return TPF_OK;
+        if (dst[k] && to.p[k] != dst[k])
+            TPF_CUDA(h, cudaMemcpyAsync(dst[k], to.p[k], N * sizeof(float), cudaMemcpyDefault, h->stream));
+    return check_err(h);  // waits for the stream
 }
 
 int tpflbm_get_state(tpflbm_t h, float* f, float* g, float* hh, float* phiu)
@@ -1138,26 +1290,42 @@ int tpflbm_set_state(tpflbm_t h, const float* f, const float* g, const float* hh
     return TPF_OK;
 }
 
+// blocks of the state's reductions: four per SM that strides over its tiles
+static int red_blocks(const DevParams& P) { return macro_blocks(P, 152 * 4); }
+
+// results and error flag of a reduction, in one copy; waits for the stream
+static int red_results(tpflbm_t h, int nb, double v[9])
+{
+    double* res = h->red + kRedMaxBlocks * 8;
+    k_reduce_final<<<1, 256, 0, h->stream>>>(h->red, nb, res, h->err);
+    TPF_CUDA(h, cudaGetLastError());
+    TPF_CUDA(h, cudaMemcpyAsync(v, res, 9 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    TPF_CUDA(h, cudaStreamSynchronize(h->stream));
+    return v[8] != 0.0 ? fail(h, TPF_ERR_TIMEOUT, kTimeoutMsg) : TPF_OK;
+}
+
 int tpflbm_diagnostics(tpflbm_t h, double out[8])
 {
     if (!h || !out) return TPF_ERR_INVALID_ARG;
-    int rc = check_err(h);
-    if (rc) return rc;
-    const long long N = (long long)h->nx * h->ny;
-    long long b = (N + kRedThreads - 1) / kRedThreads;
-    const int nb = (int)(b < kRedMaxBlocks ? b : kRedMaxBlocks);
-    const int c = h->cur;
+    const int nb = red_blocks(h->dp), c = h->cur;
     if (h->dp.storage == TPF_STORAGE_FP16)
         k_reduce_partial<StoreF16><<<nb, kRedThreads, 0, h->stream>>>(h->dp, (const __half*)h->pop[c], h->ref[c], h->phiu, h->red);
     else
         k_reduce_partial<StoreF32><<<nb, kRedThreads, 0, h->stream>>>(h->dp, (const float*)h->pop[c], h->ref[c], h->phiu, h->red);
     TPF_CUDA(h, cudaGetLastError());
-    double* res = h->red + kRedMaxBlocks * 8;
-    k_reduce_final<<<1, 256, 0, h->stream>>>(h->red, nb, res);
-    TPF_CUDA(h, cudaGetLastError());
-    TPF_CUDA(h, cudaMemcpyAsync(out, res, 8 * sizeof(double), cudaMemcpyDefault, h->stream));
-    TPF_CUDA(h, cudaStreamSynchronize(h->stream));
-    if (out[7] > 0) return fail(h, TPF_ERR_NONFINITE, "non-finite values in the state");
+    double v[9];
+    const int rc = red_results(h, nb, v);
+    if (rc) return rc;
+    // (out may be device memory)
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, out) == cudaSuccess && at.type == cudaMemoryTypeDevice) {
+        TPF_CUDA(h, cudaMemcpyAsync(out, v, 8 * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+        TPF_CUDA(h, cudaStreamSynchronize(h->stream));
+    } else {
+        cudaGetLastError();
+        std::memcpy(out, v, 8 * sizeof(double));
+    }
+    if (v[7] > 0) return fail(h, TPF_ERR_NONFINITE, "non-finite values in the state");
     return TPF_OK;
 }
 
@@ -1181,9 +1349,7 @@ int tpflbm_diagnostics_static(int nx, int ny, const tpflbm_params* p, const void
 
     DevParams P = make_dev_params(nx, ny, *p);
     P.plane = plane;
-    const long long N = (long long)nx * ny;
-    const long long b = (N + kRedThreads - 1) / kRedThreads;
-    const int nb = (int)(b < kRedMaxBlocks ? b : kRedMaxBlocks);
+    const int nb = red_blocks(P);
     cudaStream_t s = (cudaStream_t)stream;
     if (f16)
         k_reduce_partial<StoreF16><<<nb, kRedThreads, 0, s>>>(P, (const __half*)pop, (const RefT*)ref, phiu, scratch);
@@ -1226,23 +1392,16 @@ int tpflbm_state_buffers(tpflbm_t h, void** pop, void** ref, void** phiu, long l
 int tpflbm_residual(tpflbm_t h, double dT, double out[3])
 {
     if (!h || !out || !(dT > 0)) return fail(h, TPF_ERR_INVALID_ARG, "tpflbm_residual needs out and dT > 0");
-    int rc = check_err(h);
-    if (rc) return rc;
     const long long N = (long long)h->nx * h->ny;
-    long long b = (N + kRedThreads - 1) / kRedThreads;
-    const int nb = (int)(b < kRedMaxBlocks ? b : kRedMaxBlocks);
-    const int c = h->cur;
+    const int nb = red_blocks(h->dp), c = h->cur;
     if (h->dp.storage == TPF_STORAGE_FP16)
         k_residual_partial<StoreF16><<<nb, kRedThreads, 0, h->stream>>>(h->dp, (const __half*)h->pop[c], h->ref[c], h->phiu, h->snap, h->red);
     else
         k_residual_partial<StoreF32><<<nb, kRedThreads, 0, h->stream>>>(h->dp, (const float*)h->pop[c], h->ref[c], h->phiu, h->snap, h->red);
     TPF_CUDA(h, cudaGetLastError());
-    double* res = h->red + kRedMaxBlocks * 8;
-    k_reduce_final<<<1, 256, 0, h->stream>>>(h->red, nb, res);
-    TPF_CUDA(h, cudaGetLastError());
-    double sums[8];
-    TPF_CUDA(h, cudaMemcpyAsync(sums, res, 8 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    TPF_CUDA(h, cudaStreamSynchronize(h->stream));
+    double sums[9];
+    const int rc = red_results(h, nb, sums);
+    if (rc) return rc;
     const long long K = h->t - h->snap_t;
     const bool first = h->snap_t < 0;
     h->snap_t = h->t;
@@ -1309,67 +1468,37 @@ int tpflbm_bubbles(tpflbm_t h, int max_bubbles, double* out, int* count)
 {
     if (!h || max_bubbles < 0 || (max_bubbles > 0 && !out) || !count)
         return fail(h, TPF_ERR_INVALID_ARG, "tpflbm_bubbles needs count, and out when max_bubbles > 0");
-    int rc = check_err(h);
-    if (rc) return rc;
     const long long N = (long long)h->nx * h->ny;
     const long long pl = h->dp.plane;
-    const int c = h->cur;
-    // phi, u_x, u_y of the current state into staging planes 0-2 (as tpflbm_get_fields)
-    if (h->dp.storage == TPF_STORAGE_FP16)
-        k_fields<StoreF16><<<grid_1d(N), 256, 0, h->stream>>>(h->dp, (const __half*)h->pop[c], h->ref[c], h->phiu, h->stage);
-    else
-        k_fields<StoreF32><<<grid_1d(N), 256, 0, h->stream>>>(h->dp, (const float*)h->pop[c], h->ref[c], h->phiu, h->stage);
+    // phi, u_x, u_y of the current state into staging planes 0-2
+    FieldPtrs to{};
+    for (int k = 0; k < 3; ++k) to.p[k] = h->stage + k * pl;
+    launch_fields(h, to);
     TPF_CUDA(h, cudaGetLastError());
     int* lab = (int*)(h->stage + 5 * pl);
-    int* roots = (int*)(h->stage + 6 * pl);  // kMaxBubbles entries
-    int* flags = h->err + 1;                   // [0] changed, [1] root count
-    k_lab_init<<<grid_1d(N), 256, 0, h->stream>>>(h->stage, N, lab);
+    BubbleSums* dev = (BubbleSums*)h->red;
+    const int nb = grid_1d(N);
+    k_lab_runs<<<nb, 256, 0, h->stream>>>(h->stage, h->nx, h->ny, lab, dev);
+    k_lab_join<<<nb, 256, 0, h->stream>>>(h->nx, h->ny, h->dp.bc_x, h->dp.bc_y, lab);
+    k_lab_roots<<<nb, 256, 0, h->stream>>>(lab, N, dev);
+    k_lab_order<<<1, 32, 0, h->stream>>>(dev, h->err);
+    k_bubble_sums<<<nb < 152 * 4 ? nb : 152 * 4, 256, 0, h->stream>>>(h->nx, h->ny, h->dp.bc_x, h->dp.bc_y, h->stage,
+                                                                      h->stage + pl, h->stage + 2 * pl, lab, dev);
     TPF_CUDA(h, cudaGetLastError());
-    // propagate to the fixed point, checking for changes every 4 sweeps; a region of
-    // n nodes settles within n sweeps (pointer jumping makes it far fewer)
-    const long long max_sweeps = N + 8;
-    long long sweeps = 0;
-    for (;;) {
-        int changed = 0;
-        TPF_CUDA(h, cudaMemsetAsync(flags, 0, sizeof(int), h->stream));
-        for (int k = 0; k < 4; ++k)
-            k_lab_hook<<<grid_1d(N), 256, 0, h->stream>>>(h->nx, h->ny, h->dp.bc_x, h->dp.bc_y, lab, flags);
-        TPF_CUDA(h, cudaGetLastError());
-        TPF_CUDA(h, cudaMemcpyAsync(&changed, flags, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-        TPF_CUDA(h, cudaStreamSynchronize(h->stream));
-        sweeps += 4;
-        if (!changed) break;
-        if (sweeps > max_sweeps) return fail(h, TPF_ERR_UNSUPPORTED, "tpflbm_bubbles: labelling did not settle");
-    }
-    TPF_CUDA(h, cudaMemsetAsync(flags + 1, 0, sizeof(int), h->stream));
-    k_lab_roots<<<grid_1d(N), 256, 0, h->stream>>>(lab, N, flags + 1, roots);
-    TPF_CUDA(h, cudaGetLastError());
-    RootList rl{};
-    int nroots = 0;
-    TPF_CUDA(h, cudaMemcpyAsync(&nroots, flags + 1, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    TPF_CUDA(h, cudaMemcpyAsync(rl.r, roots, sizeof(rl.r), cudaMemcpyDeviceToHost, h->stream));
+    BubbleSums got;
+    TPF_CUDA(h, cudaMemcpyAsync(&got, dev, sizeof(got), cudaMemcpyDeviceToHost, h->stream));
     TPF_CUDA(h, cudaStreamSynchronize(h->stream));
+    if (got.err) return fail(h, TPF_ERR_TIMEOUT, kTimeoutMsg);
+    const int nroots = got.count;
     if (nroots > kMaxBubbles)
         return fail(h, TPF_ERR_UNSUPPORTED, "tpflbm_bubbles: more than 32 separate regions of phi < 0");
-    rl.n = nroots;
-    std::sort(rl.r, rl.r + nroots);
     *count = nroots;
     if (nroots == 0 || max_bubbles == 0) return TPF_OK;
-    double* part = h->red;
-    double* res = h->red + kBubBlocks * kMaxBubbles * 6;
-    k_bubble_partial<<<kBubBlocks, 256, 0, h->stream>>>(h->nx, h->ny, h->dp.bc_x, h->dp.bc_y, h->stage, h->stage + pl,
-                                                        h->stage + 2 * pl, lab, rl, part);
-    TPF_CUDA(h, cudaGetLastError());
-    k_bubble_final<<<1, kMaxBubbles * 6, 0, h->stream>>>(part, kBubBlocks, nroots, res);
-    TPF_CUDA(h, cudaGetLastError());
-    double sums[kMaxBubbles * 6];
-    TPF_CUDA(h, cudaMemcpyAsync(sums, res, nroots * 6 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    TPF_CUDA(h, cudaStreamSynchronize(h->stream));
     // per bubble: nodes, sum phi, u_b, v_b, x_b, y_b; ordered by x_b, then y_b
     double rows[kMaxBubbles][6];
     for (int k = 0; k < nroots; ++k) {
-        const double* v = sums + 6 * k;
-        const int xr = rl.r[k] % h->nx, yr = rl.r[k] / h->nx;
+        const double* v = got.v[k];
+        const int xr = got.root[k] % h->nx, yr = got.root[k] / h->nx;
         double xb = xr + v[4] / v[1], yb = yr + v[5] / v[1];
         if (h->dp.bc_x == 0) xb = std::fmod(xb + h->nx, (double)h->nx);
         if (h->dp.bc_y == 1) yb = std::fmod(yb + h->ny, (double)h->ny);
