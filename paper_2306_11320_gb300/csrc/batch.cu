@@ -38,10 +38,11 @@ constexpr int kVarBY[kNumVariants] = {4, 8, 16, 4, kStepBY};
 // Persistent CTAs walk the work list of (instance, tile) pairs; each tile goes
 // through the general tile routine with its instance's parameters and buffers.
 // resident threads per SM the batch kernel is built for: the general tile path is
-// latency-bound, and FP32 at 2 CTAs of 256 threads per SM (107 registers) ran 20% slower
-// than at 3; FP16 keeps 2 (at 80 registers it spills)
+// latency-bound.  FP32 32 x 4 tiles on the 256-lattice ensemble: 0.427 ms per step at 768 (80
+// registers, with spills), 0.403 at 640 (five CTAs, 102 registers), 0.417 at 896, 0.444 at
+// 1,024; FP16 is fastest at 512 (128 registers)
 template <class S>
-constexpr int kBatchThreadsPerSM = kRef<S> ? 512 : 768;
+constexpr int kBatchThreadsPerSM = kRef<S> ? 512 : 640;
 // The instance descriptor of a work item is copied word by word by warp 0 (32-bit words;
 // InstDesc is plain data).  The next item's copy is loaded into registers while the
 // current tile runs and stored into the other shared buffer after it, so no tile waits
@@ -130,11 +131,14 @@ static_assert(alignof(BatchTmaInst) % 64 == 0 && sizeof(BatchTmaInst) % 64 == 0,
 // lattice's TMA rectangle is laid out
 constexpr int kTBX = kStepBX, kTBY = kStepBY;
 
+// Three descriptors beside the two stages: the descriptor of the tile after next lands while
+// the current tile still reads its own.
 template <class S>
 struct BatchLayout {
     using L = TmaLayout<kTBX, kTBY, S>;
-    static constexpr int OFF_D = L::STAGE;
-    static constexpr int STAGE = L::STAGE + L::rnd((int)sizeof(BatchTileDesc));
+    static constexpr int DESC = L::rnd((int)sizeof(BatchTileDesc));
+    static constexpr int OFF_D = 2 * L::STAGE;
+    static constexpr int BYTES = OFF_D + 3 * DESC;
 };
 
 __device__ __forceinline__ void mbar_expect_tx_only(uint64_t* bar, uint32_t bytes)
@@ -159,12 +163,10 @@ k_step_batch_tma(const BatchTmaInst* __restrict__ inst, const int4* __restrict__
     using L = TmaLayout<BX, BY, S>;
     using BL = BatchLayout<S>;
     using E = typename S::elem;
-    static_assert(sizeof(RingSmem<BX, BY>) <= 2 * BL::STAGE, "general-path tiles reuse the stages");
+    static_assert(sizeof(RingSmem<BX, BY>) <= 2 * L::STAGE, "general-path tiles reuse the stages");
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ __align__(8) uint64_t bar[2];
-    // issue placement and staging as in k_step_tma
-    constexpr bool kLate = kRef<S>;
-    __shared__ PhiSmem<BX, BY> smb[kLate ? 2 : 1];
+    __shared__ PhiSmem<BX, BY> smb[2];
     __shared__ BatchTileDesc gdesc;  // general-path tiles
     const int tid = threadIdx.x;
 
@@ -175,63 +177,70 @@ k_step_batch_tma(const BatchTmaInst* __restrict__ inst, const int4* __restrict__
     }
     __syncthreads();
 
-    auto issue = [&](int t, int s) {
-        // item: lattice, tile (bx | by << 16), seam side, boundary tile
+    // the copies of this CTA's k-th tile, work item t, into stage k % 2 and descriptor k % 3
+    auto issue = [&](int t, int k) {
+        // item: lattice, tile (bx | by << 16), seam side, extent and boundary flag
         const int4 item = titem[t];
         const BatchTmaInst& I = inst[item.x];
         const TmaMaps& M = I.maps[parity];
-        const int x0 = (item.y & 0xffff) * BX, y0 = (item.y >> 16) * BY;
-        unsigned char* st = dsm + s * BL::STAGE;
+        const int x0 = (item.y & 0xffff) * BX, y0 = (item.y >> 16) * BY, s = k & 1;
         // the descriptor's bytes join the tile's on the same mbarrier (expected without an
         // arrival; the tile's copies bring the one arrival)
         fence_proxy_async();
         mbar_expect_tx_only(&bar[s], (uint32_t)sizeof(BatchTileDesc));
-        bulk_load(st + BL::OFF_D, &I.d, (uint32_t)sizeof(BatchTileDesc), &bar[s]);
-        tma_issue_tile<BX, BY, S>(M, st, &bar[s], x0, y0);
+        bulk_load(dsm + BL::OFF_D + k % 3 * BL::DESC, &I.d, (uint32_t)sizeof(BatchTileDesc), &bar[s]);
+        tma_issue_tile<BX, BY, S>(M, dsm + s * L::STAGE, &bar[s], x0, y0);
     };
 
+    // Where the copies are issued: as in k_step_tma, the tile after next goes into the current
+    // tile's stage once that has been read (right after the ring barrier for tiles without
+    // boundary nodes).  Its descriptor slot was last read by the tile before this one, which
+    // every warp has left by then.
     int it = 0;
     int t = blockIdx.x;
     int4 cur = t < nt ? titem[t] : make_int4(0, 0, 0, 0);
-    if (t < nt && tid == 0) issue(t, 0);
+    if (tid == 0) {
+        if (t < nt) issue(t, 0);
+        if (t + (int)gridDim.x < nt) issue(t + gridDim.x, 1);
+    }
     for (; t < nt; t += gridDim.x, ++it) {
         const int s = it & 1;
-        const int tn = t + gridDim.x;
+        const int tn = t + gridDim.x, t2 = t + 2 * gridDim.x;
         const int4 nxt = tn < nt ? titem[tn] : make_int4(0, 0, 0, 0);
-        if constexpr (!kLate) {
-            if (tn < nt && tid == 0) issue(tn, s ^ 1);
-        }
-        PhiSmem<BX, BY>& sm = smb[kLate ? s : 0];
+        PhiSmem<BX, BY>& sm = smb[s];
         const bool ok = mbar_wait_bounded(&bar[s], (it >> 1) & 1);
-        unsigned char* st = dsm + s * BL::STAGE;
+        unsigned char* st = dsm + s * L::STAGE;
         // the lattice's parameters and buffers, landed with the populations (read before
         // the block's vote only for shared-memory indices the tile body keeps in range)
-        const BatchTileDesc& D = *reinterpret_cast<const BatchTileDesc*>(st + BL::OFF_D);
+        const BatchTileDesc& D = *reinterpret_cast<const BatchTileDesc*>(dsm + BL::OFF_D + it % 3 * BL::DESC);
         const DevParams& P = D.P;
         const int x0 = (cur.y & 0xffff) * BX, y0 = (cur.y >> 16) * BY;
         auto on_abort = [&]() {
             if (tid == 0) {
                 atomicExch(inst[cur.x].d.err, 1);
                 mbar_wait_bounded(&bar[s], (it >> 1) & 1);
-                if (!kLate && tn < nt) mbar_wait_bounded(&bar[s ^ 1], ((it + 1) >> 1) & 1);
+                if (tn < nt) mbar_wait_bounded(&bar[s ^ 1], ((it + 1) >> 1) & 1);
             }
         };
-        auto after_ring = [&]() {
-            if constexpr (kLate) {
-                if (tn < nt && tid == 0) issue(tn, s ^ 1);
-            }
+        auto refill = [&]() {
+            if (t2 < nt && tid == 0) issue(t2, it + 2);
         };
-        // the buffers are read only after the block's vote; which body runs and whether the
-        // seam patch does come from the work item, the same on every thread
+        auto no_refill = [&]() {};
+        // the buffers are read only after the block's vote; which body runs, its extent and
+        // whether the seam patch runs come from the work item, the same on every thread
         const E* A = (const E*)D.pop[parity];
         E* B = (E*)D.pop[parity ^ 1];
         RefT* refB = D.ref[parity ^ 1];
-        if (cur.w ? tma_tile<BX, BY, S, true, false>(P, A, B, D.phiu, refB, st, sm, x0, y0, cur.z, ok, on_abort,
-                                                     after_ring)
-                  : tma_tile<BX, BY, S, false, false>(P, A, B, D.phiu, refB, st, sm, x0, y0, 0, ok, on_abort,
-                                                      after_ring))
+        if (cur.w & 1) {
+            if (tma_tile<BX, BY, S, true, false>(P, A, B, D.phiu, refB, st, sm, x0, y0, cur.w >> 8 & 0xff, cur.w >> 16,
+                                                 cur.z, ok, on_abort, no_refill))
+                return;
+            __syncthreads();  // every warp is done with stage s
+            refill();
+        } else if (tma_tile<BX, BY, S, false, true>(P, A, B, D.phiu, refB, st, sm, x0, y0, BX, BY, 0, ok, on_abort,
+                                                    refill)) {
             return;
-        if constexpr (!kLate) __syncthreads();  // stage s and sm are free for the next copies
+        }
         cur = nxt;
     }
 
@@ -257,13 +266,13 @@ template <class S>
 void launch_tma(const BatchTmaInst* inst, const int4* titem, int nt, const int2* gitem, int ng, int parity, int grid,
                 cudaStream_t s)
 {
-    k_step_batch_tma<S><<<grid, kTBX * kTBY, 2 * BatchLayout<S>::STAGE, s>>>(inst, titem, nt, gitem, ng, parity);
+    k_step_batch_tma<S><<<grid, kTBX * kTBY, BatchLayout<S>::BYTES, s>>>(inst, titem, nt, gitem, ng, parity);
 }
 
 template <class S>
 int occupancy_tma()
 {
-    const int smem = 2 * BatchLayout<S>::STAGE;
+    const int smem = BatchLayout<S>::BYTES;
     if (cudaFuncSetAttribute(k_step_batch_tma<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -517,14 +526,15 @@ int tpflbm_batch_create(int n, const int* nx, const int* ny, const tpflbm_params
                 for (auto& l : lists) work.insert(work.end(), l.begin(), l.end());
             };
             concat(tma);
-            // TMA items also carry the tile's seam side (as seam_side) and whether it
-            // touches the lattice boundary (as the single-lattice kernel decides it)
+            // TMA items also carry the tile's seam side (as seam_side), its extent, and
+            // whether it touches the lattice boundary (as the single-lattice kernel decides it)
             std::vector<int4> titem(work.size());
             for (size_t i = 0; i < work.size(); ++i) {
                 const int k = work[i].x, x0 = (work[i].y & 0xffff) * BX, y0 = (work[i].y >> 16) * BY;
-                const int seam = b->inst[k]->hp.bc_x != 0 ? 0 : (x0 == 0 ? -1 : (x0 + BX == nx[k] ? 1 : 0));
+                const int seam = b->inst[k]->hp.bc_x != 0 ? 0 : (x0 == 0 ? -1 : (x0 + BX >= nx[k] ? 1 : 0));
                 const bool eg = x0 <= 1 || x0 + BX >= nx[k] - 1 || y0 <= 1 || y0 + BY >= ny[k] - 1;
-                titem[i] = make_int4(k, work[i].y, seam, eg ? 1 : 0);
+                titem[i] = make_int4(k, work[i].y, seam,
+                                     (eg ? 1 : 0) | std::min(BX, nx[k] - x0) << 8 | std::min(BY, ny[k] - y0) << 16);
             }
             b->ntma = (int)titem.size();
             work.clear();

@@ -308,17 +308,23 @@ __device__ __forceinline__ void step_tile_general(const DevParams& P, const type
 
     constexpr int kRing = 2 * (BX + BY) + 4;
     static_assert(kRing <= BX * BY, "one thread per ring node");
-    int rx = 0, ry = 0, wx = 0, wy = 0;
-    bool rload = false, rghost = false;
-    float ra[9], rc[9];
-    if ((int)threadIdx.x < 2 * (w + h_) + 4) {
+    // slot (rx, ry) of this thread's ring node (worked out again where it is needed: nothing
+    // of it stays in registers while the loads are out)
+    auto ring_slot = [&](int& rx, int& ry) {
         const int r = threadIdx.x, sx = w + 2;
         if (r < sx) { rx = r; ry = 0; }
         else if (r < 2 * sx) { rx = r - sx; ry = h_ + 1; }
         else if (r < 2 * sx + h_) { rx = 0; ry = r - 2 * sx + 1; }
         else { rx = w + 1; ry = r - 2 * sx - h_ + 1; }
-        wx = x0 + rx - 1;
-        wy = y0 + ry - 1;
+    };
+    int kr = 0;
+    bool rload = false, rghost = false;
+    float ra[9], rc[9];
+    if ((int)threadIdx.x < 2 * (w + h_) + 4) {
+        int rx, ry;
+        ring_slot(rx, ry);
+        kr = ry * SX + rx;
+        int wx = x0 + rx - 1, wy = y0 + ry - 1;
         if (P.bc_x == 0) wx = wrap(wx, P.nx);
         if (P.bc_y == 1) wy = wrap(wy, P.ny);
         rload = wx >= 0 && wx < P.nx && wy >= 0 && wy < P.ny;
@@ -342,31 +348,32 @@ __device__ __forceinline__ void step_tile_general(const DevParams& P, const type
         for (int i = 0; i < 9; ++i) sm.h[i][kown] = h[i];
     }
     if (rload) {
-        const int k = ry * SX + rx;
         float sf = 0.f, sh = 0.f;
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
             sf += ra[i];
             sh += rc[i];
-            sm.h[i][k] = rc[i];
+            sm.h[i][kr] = rc[i];
         }
-        sm.phi[k] = sf;
-        sm.T[k] = sh;
-        sm.irc[k] = __frcp_rn(fmaf(P.rcp_b, clamp1(sf), P.rcp_a));
+        sm.phi[kr] = sf;
+        sm.T[kr] = sh;
+        sm.irc[kr] = __frcp_rn(fmaf(P.rcp_b, clamp1(sf), P.rcp_a));
     }
     // ghost ring nodes beyond walls, inlet and outflow (as phiT_at): phi mirrored,
     // T by the boundary's rule; the mirror is the adjacent slot inside the lattice
     if (__syncthreads_or(rghost) && rghost) {
-        const int gx = x0 + rx - 1;
+        int rx, ry;
+        ring_slot(rx, ry);
+        const int gx = x0 + rx - 1, gy = y0 + ry - 1;
+        const int wx = P.bc_x == 0 ? wrap(gx, P.nx) : gx, wy = P.bc_y == 1 ? wrap(gy, P.ny) : gy;
         const int mx = min(max(wx, 0), P.nx - 1), my = min(max(wy, 0), P.ny - 1);
-        const int km = (ry + my - wy) * SX + rx + mx - wx;
+        const int km = kr + (my - wy) * SX + mx - wx;
         const float tm = sm.T[km];
         const float tg = (wx < 0) ? 2.f * P.T_in - tm : tm;
         const bool oy = wy < 0 || wy >= P.ny;
-        const int k = ry * SX + rx;
-        sm.phi[k] = sm.phi[km];
-        sm.T[k] = oy ? 2.f * (wy < 0 ? T_wall_bottom(P, (float)gx) : T_wall_top(P, (float)gx)) - tg : tg;
-        sm.irc[k] = 0.f;
+        sm.phi[kr] = sm.phi[km];
+        sm.T[kr] = oy ? 2.f * (wy < 0 ? T_wall_bottom(P, (float)gx) : T_wall_top(P, (float)gx)) - tg : tg;
+        sm.irc[kr] = 0.f;
     }
     __syncthreads();
     if (active) {
@@ -829,10 +836,11 @@ k_step_many(const DevParams P, const typename S::elem* A, typename S::elem* B, f
 // Persistent CTAs walk a tile list: first the TMA tiles, then the remaining tiles
 // through the general path.  TMA tiles are the whole tiles whose halo lies inside the
 // lattice along each periodic axis (x0 >= XP, x0 + BX + XP <= nx; y0 >= 2,
-// y0 + BY + 2 <= ny), which along a walled or inlet/outflow axis are all whole tiles:
-// there the box reaches past the lattice, the copy fills it with zeros, and the tile
-// takes its ghost ring nodes and its boundary nodes' FP16 records by the boundary
-// rules instead.  For a TMA tile one elected thread issues 3D bulk
+// y0 + BY + 2 <= ny), which along a walled or inlet/outflow axis are all tiles, the ragged
+// last one too: there the box reaches past the lattice, the copy fills it with zeros, and
+// the tile takes its ghost ring nodes and its boundary nodes' FP16 records by the boundary
+// rules instead (with FP32 storage, along a periodic x axis of two tiles and more, too: see
+// seam_side).  For a TMA tile one elected thread issues 3D bulk
 // tensor copies (cp.async.bulk.tensor) of the 9 f planes and the 9 h planes over the
 // tile plus a one-node ring (widened to XP columns each side for the 16-byte rule),
 // the 9 g planes and the 2 (phi u) planes over the tile, and for FP16 the 3 planes of
@@ -898,7 +906,7 @@ struct TmaLayout {
 
 // Which side of a periodic x seam a TMA tile sits on: -1 its left ring column wraps to
 // x = nx - 1, +1 its right one to x = 0, 0 neither.  Seam tiles are staged by TMA with
-// FP32 storage only, and only in lattices at least two tiles wide (so no tile has both
+// FP32 storage only, and only in lattices more than a tile wide (so no tile has both
 // sides); otherwise they take the general path and this is 0 for every TMA tile.  With
 // FP16 storage (records to patch as well) the seam code pushed the kernel to its
 // 128-register cap and slowed every tile (the 2048 x 512 channel, which has no seam,
@@ -907,7 +915,7 @@ template <int BX>
 __device__ __forceinline__ int seam_side(const DevParams& P, int x0)
 {
     if (P.bc_x != 0) return 0;
-    return x0 == 0 ? -1 : (x0 + BX == P.nx ? 1 : 0);
+    return x0 == 0 ? -1 : (x0 + BX >= P.nx ? 1 : 0);
 }
 
 struct TmaMaps {
@@ -947,14 +955,14 @@ struct PhiSmem {
 // block barrier.
 template <int BX, int BY, class S>
 __device__ __noinline__ void seam_patch(unsigned char* st, int seam, const typename S::elem* __restrict__ A, int nx,
-                                        int ny, long long pl, int y0)
+                                        int ny, long long pl, int y0, int w)
 {
     static_assert(!kRef<S>, "FP16 tiles are not staged across a seam");
     using L = TmaLayout<BX, BY, S>;
     using E = typename S::elem;
     E* bF = (E*)(st + L::OFF_F);
     E* bH = (E*)(st + L::OFF_H);
-    const int fc = seam < 0 ? L::XP - 1 : L::XP + BX, gx = seam < 0 ? nx - 1 : 0;
+    const int fc = seam < 0 ? L::XP - 1 : L::XP + w, gx = seam < 0 ? nx - 1 : 0;
     for (int k = threadIdx.x; k < 9 * L::FH; k += BX * BY) {
         const int i = k / L::FH, y = y0 - 1 + k % L::FH;
         if (y < 0 || y >= ny) continue;
@@ -971,17 +979,20 @@ __device__ __noinline__ void seam_patch(unsigned char* st, int seam, const typen
 // on_abort() runs on every thread and the tile returns true when any wait ran out),
 // after_ring() on every thread, then per node the macroscopic state, the collisions
 // and the push to B.  EDGE: the tile touches the lattice boundary (ghost ring nodes,
-// boundary records, boundary-aware push for every node); seam (seam_side): the wrapped
-// column of a periodic x seam comes from A first.  EDGE and seam must be the
+// boundary records, boundary-aware push for every node), and may be ragged: it covers w x h_
+// nodes (w and h_ are BX and BY otherwise); seam (seam_side): the wrapped
+// column of a periodic x seam comes from A first.  EDGE, seam, w and h_ must be the
 // same on every thread and must not come from a staged P (it is not to be trusted
 // before the vote).
 template <int BX, int BY, class S, bool EDGE, bool PRELOAD, class OnAbort, class AfterRing>
 __device__ __forceinline__ bool tma_tile(const DevParams& P, const typename S::elem* __restrict__ A,
                                          typename S::elem* __restrict__ B, float* __restrict__ phiu,
                                          RefT* __restrict__ refB,
-                                         unsigned char* st, PhiSmem<BX, BY>& sm, int x0, int y0, int seam, bool ok,
-                                         OnAbort on_abort, AfterRing after_ring)
+                                         unsigned char* st, PhiSmem<BX, BY>& sm, int x0, int y0, int w_, int h__,
+                                         int seam, bool ok, OnAbort on_abort, AfterRing after_ring)
 {
+    // (constants where the tile cannot be ragged)
+    const int w = EDGE ? w_ : BX, h_ = EDGE ? h__ : BY;
     using L = TmaLayout<BX, BY, S>;
     using E = typename S::elem;
     constexpr int SX = BX + 2;
@@ -1014,7 +1025,7 @@ __device__ __forceinline__ bool tma_tile(const DevParams& P, const typename S::e
                     on_abort();
                     return true;
                 }
-                seam_patch<BX, BY, S>(st, seam, A, P.nx, P.ny, P.plane, y0);
+                seam_patch<BX, BY, S>(st, seam, A, P.nx, P.ny, P.plane, y0, w);
             }
         }
     }
@@ -1035,6 +1046,7 @@ __device__ __forceinline__ bool tma_tile(const DevParams& P, const typename S::e
     const int lx = tx + 1, ly = ty + 1, kown = ly * SX + lx;
     const int x = x0 + tx, y = y0 + ty;
     const int n = y * P.nx + x;
+    const bool active = !edge || (tx < w && ty < h_);
     const bool bnode = edge && on_boundary(x, y);
     float f[9], g[9], h[9], phin[9], Tn[9];
     {
@@ -1058,9 +1070,11 @@ __device__ __forceinline__ bool tma_tile(const DevParams& P, const typename S::e
             sf += f[i];
             sh += h[i];
         }
-        sm.phi[kown] = sf;
-        sm.T[kown] = sh;
-        sm.irc[kown] = __frcp_rn(fmaf(P.rcp_b, clamp1(sf), P.rcp_a));
+        if (active) {
+            sm.phi[kown] = sf;
+            sm.T[kown] = sh;
+            sm.irc[kown] = __frcp_rn(fmaf(P.rcp_b, clamp1(sf), P.rcp_a));
+        }
     }
     // PRELOAD (tiles without boundary nodes): the rest of the tile's reads of the stage,
     // done before the ring barrier so that the stage is free after it: the destinations'
@@ -1082,14 +1096,19 @@ __device__ __forceinline__ bool tma_tile(const DevParams& P, const typename S::e
         pu_x = sU[ty * BX + tx];
         pu_y = sU[(BY + ty) * BX + tx];
     }
-    // ring: 2 (BX + BY) + 4 nodes, one zeroth moment (f or h) per thread
-    if (tid < 2 * kRing) {
-        const int r = tid < kRing ? tid : tid - kRing;
+    // ring: 2 (w + h_) + 4 nodes, one zeroth moment (f or h) per thread
+    auto ring_slot = [&](int r, int& rx, int& ry) {
+        const int sx = w + 2;
+        if (r < sx) { rx = r; ry = 0; }
+        else if (r < 2 * sx) { rx = r - sx; ry = h_ + 1; }
+        else if (r < 2 * sx + h_) { rx = 0; ry = r - 2 * sx + 1; }
+        else { rx = w + 1; ry = r - 2 * sx - h_ + 1; }
+    };
+    const int nring = 2 * (w + h_) + 4;  // <= kRing
+    if (tid < 2 * nring) {
+        const bool ring_f = tid < nring;
         int rx, ry;
-        if (r < SX) { rx = r; ry = 0; }
-        else if (r < 2 * SX) { rx = r - SX; ry = BY + 1; }
-        else if (r < 2 * SX + BY) { rx = 0; ry = r - 2 * SX + 1; }
-        else { rx = BX + 1; ry = r - 2 * SX - BY + 1; }
+        ring_slot(ring_f ? tid : tid - nring, rx, ry);
         const int k = ry * SX + rx;
         const int gx = x0 + rx - 1, gy = y0 + ry - 1;
         const bool ghost = edge && is_ghost(gx, gy);
@@ -1097,7 +1116,7 @@ __device__ __forceinline__ bool tma_tile(const DevParams& P, const typename S::e
         float s = 0.f;
         if (ghost) {
             // filled below from the node it mirrors
-        } else if (tid < kRing) {
+        } else if (ring_f) {
 #pragma unroll
             for (int i = 0; i < 9; ++i) s += decF(sF, P.is_f, kRecF, i, rx, ry, rb);
             sm.phi[k] = s;
@@ -1112,13 +1131,9 @@ __device__ __forceinline__ bool tma_tile(const DevParams& P, const typename S::e
         // ghost ring nodes beyond walls, inlet and outflow: phi mirrored, T by the
         // boundary's rule (as phiT_at does for the general path)
         __syncthreads();
-        if (tid < kRing) {
-            const int r = tid;
+        if (tid < nring) {
             int rx, ry;
-            if (r < SX) { rx = r; ry = 0; }
-            else if (r < 2 * SX) { rx = r - SX; ry = BY + 1; }
-            else if (r < 2 * SX + BY) { rx = 0; ry = r - 2 * SX + 1; }
-            else { rx = BX + 1; ry = r - 2 * SX - BY + 1; }
+            ring_slot(tid, rx, ry);
             const int gx = x0 + rx - 1, gy = y0 + ry - 1;
             const bool ox = (!kSeams || P.bc_x != 0) && (gx < 0 || gx >= P.nx), oy = gy < 0 || gy >= P.ny;
             if (ox || oy) {
@@ -1140,6 +1155,7 @@ __device__ __forceinline__ bool tma_tile(const DevParams& P, const typename S::e
         return true;
     }
     after_ring();
+    if (!active) return false;
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         const int k = kown + cy(i) * SX + cx(i);
@@ -1259,11 +1275,13 @@ k_step_tma(const DevParams P, const __grid_constant__ TmaMaps maps, const typena
         const bool edge_tile = x0 <= 1 || x0 + BX >= P.nx - 1 || y0 <= 1 || y0 + BY >= P.ny - 1;
         const int seam = seam_side<BX>(P, x0);
         if (edge_tile) {
-            if (tma_tile<BX, BY, S, true, false>(P, A, B, phiu, refB, st, sm, x0, y0, seam, ok, on_abort, no_refill))
+            if (tma_tile<BX, BY, S, true, false>(P, A, B, phiu, refB, st, sm, x0, y0, min(BX, P.nx - x0),
+                                                 min(BY, P.ny - y0), seam, ok, on_abort, no_refill))
                 return;
             __syncthreads();  // every warp is done with stage s
             refill();
-        } else if (tma_tile<BX, BY, S, false, true>(P, A, B, phiu, refB, st, sm, x0, y0, 0, ok, on_abort, refill)) {
+        } else if (tma_tile<BX, BY, S, false, true>(P, A, B, phiu, refB, st, sm, x0, y0, BX, BY, 0, ok, on_abort,
+                                                    refill)) {
             return;
         }
     }
