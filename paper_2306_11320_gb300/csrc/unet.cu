@@ -143,6 +143,17 @@ __device__ __forceinline__ void mb_init(uint64_t* b, uint32_t n)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sa(b)), "r"(n) : "memory");
 }
+// one lane of a converged warp.  The warps that issue copies and MMAs run their loops with
+// all lanes and pick the issuing one with this around each issue: tcgen05.mma and the bulk
+// copies take their operands from uniform registers, and in a branch that one lane took by
+// its number the compiler cannot know them to be uniform (an MMA of 128 x 32 x 16 then took
+// 210 cycles to issue).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}\n" : "=r"(p));
+    return p != 0;
+}
 __device__ __forceinline__ void mb_expect_tx(uint64_t* b, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(sa(b)), "r"(bytes) : "memory");
@@ -161,12 +172,12 @@ __device__ __forceinline__ bool mb_wait(uint64_t* b, uint32_t parity)
     atomicExch(&g_tc_err, 1);
     return false;
 }
-__device__ __forceinline__ void tma_2d(void* dst, const CUtensorMap* m, uint64_t* b, int c0, int c1)
+__device__ __forceinline__ void tma_3d(void* dst, const CUtensorMap* m, uint64_t* b, int c0, int c1, int c2)
 {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
             sa(dst)),
-        "l"((uint64_t)m), "r"(c0), "r"(c1), "r"(sa(b))
+        "l"((uint64_t)m), "r"(c0), "r"(c1), "r"(c2), "r"(sa(b))
         : "memory");
 }
 __device__ __forceinline__ void tma_4d(void* dst, const CUtensorMap* m, uint64_t* b, int c0, int c1, int c2, int c3)
@@ -193,6 +204,19 @@ __host__ __device__ constexpr uint32_t tc_idesc(int M, int N)
 {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
+// d (+)= A B; and an arrival on bar once every MMA issued so far has finished
+__device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, bool accumulate)
+{
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"((uint32_t)accumulate)
+        : "memory");
+}
+__device__ __forceinline__ void tc_commit(uint64_t* bar)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(sa(bar)) : "memory");
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
@@ -208,7 +232,7 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUt
     extern __shared__ __align__(1024) unsigned char tsm[];
     __shared__ __align__(8) uint64_t full[kTcStages], empty[kTcStages], done;
     __shared__ uint32_t tmem_base;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     // 1024-byte aligned stages (the swizzle pattern repeats every 512 bytes)
     unsigned char* st0 = tsm + ((1024 - (sa(tsm) & 1023)) & 1023);
     const int bpr = W / BW, bpi = bpr * (H / BH);  // pixel blocks per row of blocks, per image
@@ -236,7 +260,7 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUt
     tc_fence_after();
     const uint32_t tmem = tmem_base;
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
         // producer: stage k % S holds tap k / kc, channels (k % kc) * 32
         int issued = 0;
         for (int k = 0; k < ksteps; ++k) {
@@ -244,15 +268,18 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUt
             if (k >= kTcStages && !mb_wait(&empty[s], ((k / kTcStages) - 1) & 1)) break;
             unsigned char* a = st0 + s * kStage;
             const int tap = k / kc, c0 = (k % kc) * KC;
-            mb_expect_tx(&full[s], kStage);
-            tma_4d(a, &mx, &full[s], c0, w0 + tap % 3 - 1, h0 + tap / 3 - 1, n);
-            tma_2d(a + kABytes, &mw, &full[s], c0, tap * Cout + co0);
+            if (elect_one()) {
+                mb_expect_tx(&full[s], kStage);
+                tma_4d(a, &mx, &full[s], c0, w0 + tap % 3 - 1, h0 + tap / 3 - 1, n);
+                tma_3d(a + kABytes, &mw, &full[s], c0, co0, tap);
+            }
+            __syncwarp();
             issued = k + 1;
         }
         // copies still in flight (only after a wait ran out) land before the CTA ends
         for (int k = issued > kTcStages ? issued - kTcStages : 0; k < issued; ++k)
             mb_wait(&full[k % kTcStages], (k / kTcStages) & 1);
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         // MMA issuer
         constexpr uint32_t idesc = tc_idesc(128, BN);
         for (int k = 0; k < ksteps; ++k) {
@@ -260,24 +287,16 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUt
             if (!mb_wait(&full[s], (k / kTcStages) & 1)) break;
             tc_fence_after();
             const uint32_t a = sa(st0 + s * kStage), b = a + kABytes;
+            if (elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < KC / 16; ++kk) {
-                const uint64_t ad = kmajor_desc<KC>(a + 32 * kk), bd = kmajor_desc<KC>(b + 32 * kk);
-                const uint32_t acc = (k | kk) != 0;
-                asm volatile(
-                    "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                    " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-                    "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-                    : "memory");
+                for (int kk = 0; kk < KC / 16; ++kk)
+                    tc_mma(tmem, kmajor_desc<KC>(a + 32 * kk), kmajor_desc<KC>(b + 32 * kk), idesc, (k | kk) != 0);
+                tc_commit(&empty[s]);  // stage s is free once these MMAs have read it
             }
-            // stage s is free once these MMAs have read it
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             sa(&empty[s]))
-                         : "memory");
+            __syncwarp();
         }
         // the accumulator is complete once every MMA issued has finished
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(sa(&done))
-                     : "memory");
+        if (elect_one()) tc_commit(&done);
     }
     __syncwarp();
 
@@ -323,6 +342,214 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUt
     __syncthreads();
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN) : "memory");
+}
+
+// ------------------------------------------ tcgen05 convolution on halo tiles
+//
+// The same GEMMs with the activations staged once per CTA instead of once per tap.  A CTA
+// takes MT (1 or 2) blocks of 8 x 16 output pixels side by side (M = 128 each) and BN output
+// channels.  One TMA box per KC channels brings the block's pixels and their one-pixel
+// frame, (8 MT + 2) x 18 rows of KC channels, zero outside the image.  A tap's operand is
+// then a window into that box: 16 groups (image rows) of 8 rows (pixels), the groups one row
+// of the box apart, starting (dh + 1) box rows and dw + 1 pixels in.  The box starts on a
+// swizzle boundary and the swizzle follows the address bits, so a window may start at any of
+// its rows.  The weights of each (tap, channel chunk) come through a ring of stages; taps
+// outermost, as in k_conv3x3_tc, so that the FP32 sums are the same bit for bit.
+//
+// What this saves is the way from L2 to the SM, which bounded the per-tap form: 184 MB of
+// copies for (4, 128, 512, 32, 32) against 40 MB here, 113 MB against 30 MB for (4, 64, 256,
+// 64, 64).
+constexpr int kHaloChunks = 12;  // channel chunks of a box (Cin <= 768)
+constexpr int kHaloStages = 8;   // weight stages at most
+constexpr int kHaloRows = 18;    // box rows: 16 image rows and the frame
+
+// K-major descriptor with 8-row groups sbo bytes apart (kmajor_desc: 16 KC)
+template <int KC>
+__device__ __forceinline__ uint64_t kmajor_desc_sbo(uint32_t addr, uint32_t sbo)
+{
+    constexpr uint64_t mode = KC == 64 ? 2 : 4;
+    return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(sbo >> 4) << 32) |
+           ((uint64_t)1 << 46) | (mode << 61);
+}
+// bytes of one chunk's box, a multiple of the swizzle's 1024
+__host__ __device__ constexpr int halo_bytes(int MT, int KC)
+{
+    return ((8 * MT + 2) * kHaloRows * 2 * KC + 1023) / 1024 * 1024;
+}
+
+// The weights' way through shared memory: a stage holds T taps (1, 3 or 9) of CC channel chunks
+// of the BN output channels, S stages in use.
+struct HaloStages {
+    int T, CC, S;
+};
+
+template <int KC, int MT>
+__global__ void __launch_bounds__(128 * MT)
+k_conv3x3_halo(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUtensorMap mw, int H, int W, int Cin,
+               int Cout, int BN, const HaloStages st, const float* __restrict__ bias, int relu, bf16* __restrict__ y,
+               int ldy, const bf16* __restrict__ mask)
+{
+    constexpr int kPitch = 8 * MT + 2, kABytes = halo_bytes(MT, KC), kABox = kPitch * kHaloRows * 2 * KC;
+    extern __shared__ __align__(1024) unsigned char tsm[];
+    __shared__ __align__(8) uint64_t fullA[kHaloChunks], fullB[kHaloStages], emptyB[kHaloStages], done;
+    __shared__ uint32_t tmem_base;
+    __shared__ __align__(16) float sbias[256];
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    unsigned char* sA = tsm + ((1024 - (sa(tsm) & 1023)) & 1023);
+    const int kc = Cin / KC, kBBytes = BN * KC * 2, kStage = st.T * st.CC * kBBytes;
+    unsigned char* sB = sA + kc * kABytes;
+    const int bpr = W / (8 * MT), bpi = bpr * (H / 16);
+    const int n = blockIdx.x / bpi, rem = blockIdx.x % bpi;
+    const int h0 = (rem / bpr) * 16, w0 = (rem % bpr) * 8 * MT;
+    const int co0 = blockIdx.y * BN;
+    uint32_t cols = 32;
+    while ((int)cols < MT * BN) cols *= 2;
+
+    if (tid == 0) {
+        for (int c = 0; c < kc; ++c) mb_init(&fullA[c], 1);
+        for (int s = 0; s < st.S; ++s) {
+            mb_init(&fullB[s], 1);
+            mb_init(&emptyB[s], 1);
+        }
+        mb_init(&done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sa(&tmem_base)),
+                     "r"(cols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    for (int k = tid; k < BN; k += 128 * MT) sbias[k] = bias ? bias[co0 + k] : 0.f;
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_base;
+
+    // Stage k covers taps t .. t + T - 1 and chunks c .. c + CC - 1.  All counters advance by
+    // additions: divisions by the runtime counts cost more than a stage's MMAs.
+    if (warp == 0) {
+        // producer: a chunk's box ahead of the weights that need it first
+        int s = 0, t = 0, c = 0, issued = 0;
+        uint32_t round = 0;  // times the ring has gone round
+        for (; t < 9; ++issued) {
+            if (round && !mb_wait(&emptyB[s], (round - 1) & 1)) break;
+            if (elect_one()) {
+                if (t == 0)
+                    for (int j = c; j < c + st.CC; ++j) {
+                        mb_expect_tx(&fullA[j], kABox);
+                        tma_4d(sA + j * kABytes, &mx, &fullA[j], j * KC, w0 - 1, h0 - 1, n);
+                    }
+                mb_expect_tx(&fullB[s], kStage);
+                for (int j = 0; j < st.CC; ++j)
+                    tma_3d(sB + s * kStage + j * st.T * kBBytes, &mw, &fullB[s], (c + j) * KC, co0, t);
+            }
+            __syncwarp();
+            if (++s == st.S) { s = 0; ++round; }
+            c += st.CC;
+            if (c == kc) { c = 0; t += st.T; }
+        }
+        if (t < 9) {  // a wait ran out: the copies still in flight land before the CTA ends
+            for (int j = 0; j < kc && j < issued * st.CC; ++j) mb_wait(&fullA[j], 0);
+            for (int k = issued > st.S ? issued - st.S : 0; k < issued; ++k)
+                mb_wait(&fullB[k % st.S], (k / st.S) & 1);
+        }
+    } else if (warp == 1) {
+        const uint32_t idesc = tc_idesc(128, BN);
+        int s = 0, t = 0, c = 0;
+        uint32_t round = 0;
+        bool ok = true;
+        while (t < 9 && ok) {
+            if (t == 0)
+                for (int j = c; j < c + st.CC && ok; ++j) ok = mb_wait(&fullA[j], 0);
+            ok = ok && mb_wait(&fullB[s], round & 1);
+            if (!ok) break;
+            tc_fence_after();
+            if (elect_one()) {
+                // a tap's window starts t / 3 = dh + 1 box rows and t % 3 = dw + 1 pixels in
+                int row = t / 3 * kPitch + t % 3, tw = t % 3;
+                for (int u = 0; u < st.T; ++u) {
+                    uint32_t a0 = sa(sA) + (uint32_t)(c * kABytes + row * 2 * KC);
+                    uint32_t b0 = sa(sB) + (uint32_t)(s * kStage + u * kBBytes);
+                    for (int j = 0; j < st.CC; ++j) {
+                        const uint64_t ad = kmajor_desc_sbo<KC>(a0, kPitch * 2 * KC), bd = kmajor_desc<KC>(b0);
+                        const bool first = (t | u | c | j) == 0;
+                        // (the address is the descriptor's low field: no step leaves it)
+#pragma unroll
+                        for (int kk = 0; kk < KC / 16; ++kk)
+#pragma unroll
+                            for (int q = 0; q < MT; ++q)
+                                tc_mma(tmem + (uint32_t)(q * BN), ad + (16 * KC * q + 32 * kk) / 16, bd + 2 * kk, idesc,
+                                       !(first && kk == 0));
+                        a0 += kABytes;
+                        b0 += st.T * kBBytes;
+                    }
+                    ++row;
+                    if (++tw == 3) { tw = 0; row += kPitch - 3; }
+                }
+                tc_commit(&emptyB[s]);
+            }
+            __syncwarp();
+            if (++s == st.S) { s = 0; ++round; }
+            c += st.CC;
+            if (c == kc) { c = 0; t += st.T; }
+        }
+        if (elect_one()) tc_commit(&done);
+    }
+    __syncwarp();
+
+    // epilogue: warps 4 q .. 4 q + 3 hold block q; thread (warp w, lane l) its pixel m = 32 (w % 4)
+    // + l, at row m / 8 and column m % 8 of the block
+    const int q = warp >> 2, m = (warp & 3) * 32 + lane;
+    const size_t px = ((size_t)n * H + h0 + m / 8) * W + w0 + 8 * q + m % 8;
+    bf16* out = y + px * ldy + co0;
+    const bf16* mrow = mask ? mask + px * Cout + co0 : nullptr;
+    mb_wait(&done, 0);
+    tc_fence_after();
+#pragma unroll 1
+    for (int c = 0; c < BN; c += 32) {
+        uint32_t r[32];
+        const uint32_t at = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(q * BN + c);
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+            "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+              "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+              "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+              "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+            : "r"(at));
+        uint4 mk[4];
+        if (mrow) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) mk[j] = *reinterpret_cast<const uint4*>(mrow + c + 8 * j);
+        }
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            uint32_t o[4];
+            const uint32_t mu[4] = {mk[j].x, mk[j].y, mk[j].z, mk[j].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float2 bb = *reinterpret_cast<const float2*>(&sbias[c + 8 * j + 2 * e]);
+                float v0 = __uint_as_float(r[8 * j + 2 * e]) + bb.x, v1 = __uint_as_float(r[8 * j + 2 * e + 1]) + bb.y;
+                if (relu) {
+                    v0 = fmaxf(v0, 0.f);
+                    v1 = fmaxf(v1, 0.f);
+                }
+                if (mrow) {  // bf16 is the upper half of float32
+                    if (!(__uint_as_float(mu[e] << 16) > 0.f)) v0 = 0.f;
+                    if (!(__uint_as_float(mu[e] & 0xffff0000u) > 0.f)) v1 = 0.f;
+                }
+                const __nv_bfloat162 t2 = __floats2bfloat162_rn(v0, v1);
+                o[e] = *reinterpret_cast<const uint32_t*>(&t2);
+            }
+            *reinterpret_cast<uint4*>(out + c + 8 * j) = make_uint4(o[0], o[1], o[2], o[3]);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols) : "memory");
 }
 
 // dW[tap][co][ci] += sum_p dz[p][co] x[p + off(tap)][ci], db[co] += sum_p dz[p][co].
@@ -462,7 +689,7 @@ k_conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap mdz, const __grid_constan
     extern __shared__ __align__(1024) unsigned char tsm[];
     __shared__ __align__(8) uint64_t full[kWgStages], empty[kWgStages], done;
     __shared__ uint32_t tmem_base;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     unsigned char* st0 = tsm + ((1024 - (sa(tsm) & 1023)) & 1023);
     const int co0 = blockIdx.x * 128, ci0 = blockIdx.y * 64;
     // TAPS 1: tap = z % 9; TAPS 3: taps dwi, dwi + 3, dwi + 6 (dh = -1, 0, 1) with dwi = z % 3
@@ -495,7 +722,7 @@ k_conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap mdz, const __grid_constan
     tc_fence_after();
     const uint32_t tmem = tmem_base;
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
         int issued = 0;
         for (int k = 0; k < ksteps; ++k) {
             const int s = k % kWgStages;
@@ -506,45 +733,39 @@ k_conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap mdz, const __grid_constan
             // the second dz box only when it holds channels: otherwise TMEM lanes 64-127
             // accumulate whatever that smem holds and are never read
             const bool a2 = co0 + 64 < Cout;
-            mb_expect_tx(&full[s], a2 ? kStage : kStage - kBlk);
-            tma_4d(a, &mdz, &full[s], co0, w0, h, n);
-            if (a2) tma_4d(a + kBlk, &mdz, &full[s], co0 + 64, w0, h, n);
+            if (elect_one()) {
+                mb_expect_tx(&full[s], a2 ? kStage : kStage - kBlk);
+                tma_4d(a, &mdz, &full[s], co0, w0, h, n);
+                if (a2) tma_4d(a + kBlk, &mdz, &full[s], co0 + 64, w0, h, n);
 #pragma unroll
-            for (int t = 0; t < TAPS; ++t) {
-                const int dh = (tap0 + 3 * t) / 3 - 1;
-                tma_4d(a + (2 + t) * kBlk, &mx, &full[s], ci0, w0 + dwd, h + dh, n);
+                for (int t = 0; t < TAPS; ++t) {
+                    const int dh = (tap0 + 3 * t) / 3 - 1;
+                    tma_4d(a + (2 + t) * kBlk, &mx, &full[s], ci0, w0 + dwd, h + dh, n);
+                }
             }
+            __syncwarp();
             issued = k + 1;
         }
         for (int k = issued > kWgStages ? issued - kWgStages : 0; k < issued; ++k)
             mb_wait(&full[k % kWgStages], (k / kWgStages) & 1);
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         for (int k = 0; k < ksteps; ++k) {
             const int s = k % kWgStages;
             if (!mb_wait(&full[s], (k / kWgStages) & 1)) break;
             tc_fence_after();
             const uint32_t a = sa(st0 + s * kStage);
+            if (elect_one()) {
 #pragma unroll
-            for (int t = 0; t < TAPS; ++t) {
-                const uint32_t b = a + (2 + t) * kBlk;
+                for (int t = 0; t < TAPS; ++t)
 #pragma unroll
-                for (int kk = 0; kk < kWgPix / 16; ++kk) {
-                    // 16 K rows = two 8-row groups
-                    const uint64_t ad = mnmajor_desc(a + 2048 * kk, kBlk), bd = mnmajor_desc(b + 2048 * kk, kBlk);
-                    const uint32_t acc = (k | kk) != 0;
-                    asm volatile(
-                        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + 64 * t),
-                        "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-                        : "memory");
-                }
+                    for (int kk = 0; kk < kWgPix / 16; ++kk)  // 16 K rows = two 8-row groups
+                        tc_mma(tmem + 64 * t, mnmajor_desc(a + 2048 * kk, kBlk),
+                               mnmajor_desc(a + (2 + t) * kBlk + 2048 * kk, kBlk), idesc, (k | kk) != 0);
+                tc_commit(&empty[s]);
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             sa(&empty[s]))
-                         : "memory");
+            __syncwarp();
         }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(sa(&done))
-                     : "memory");
+        if (elect_one()) tc_commit(&done);
     } else if (warp >= 2 && bias) {
         // warp 2 + q sums box q, lane l its channels 2 l and 2 l + 1: 16-byte piece l / 4 of
         // the 128-byte rows, which the swizzle puts at piece (l / 4) ^ (pixel % 8)
@@ -1130,35 +1351,41 @@ int tc_bn(int N, int H, int W, int Cout, int& BW, int& BH)
     return 32;
 }
 
+// tensor maps of the convolutions: pixel boxes of an NHWC tensor
+bool pixel_map(CUtensorMap* m, const bf16* x, int N, int H, int W, int C, int KC, int bw, int bh)
+{
+    auto fn = encode_fn();
+    if (!fn) return false;
+    cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
+    cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
+    cuuint32_t box[4] = {(cuuint32_t)KC, (cuuint32_t)bw, (cuuint32_t)bh, 1};
+    cuuint32_t es[4] = {1, 1, 1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void*)x, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              KC == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+// and KC channels x BN output channels x T taps of the [9][Cout][Cin] weights
+bool weight_map(CUtensorMap* m, const bf16* wt, int Cin, int Cout, int KC, int BN, int T)
+{
+    auto fn = encode_fn();
+    if (!fn) return false;
+    cuuint64_t dims[3] = {(cuuint64_t)Cin, (cuuint64_t)Cout, 9};
+    cuuint64_t strides[2] = {(cuuint64_t)Cin * 2, (cuuint64_t)Cout * Cin * 2};
+    cuuint32_t box[3] = {(cuuint32_t)KC, (cuuint32_t)BN, (cuuint32_t)T};
+    cuuint32_t es[3] = {1, 1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, (void*)wt, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              KC == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // The tcgen05 convolution for 16-byte aligned tensors of a shape tc_bn takes; returns
 // false (nothing launched) otherwise.
 template <int BN, int KC>
 bool launch_tc(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, const float* bias, int Cout, int relu,
                bf16* y, int ldy, const bf16* mask, cudaStream_t s, int BW, int BH)
 {
-    auto fn = encode_fn();
-    if (!fn) return false;
     CUtensorMap mx, mw;
-    {
-        cuuint64_t dims[4] = {(cuuint64_t)Cin, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
-        cuuint64_t strides[3] = {(cuuint64_t)Cin * 2, (cuuint64_t)W * Cin * 2, (cuuint64_t)H * W * Cin * 2};
-        cuuint32_t box[4] = {(cuuint32_t)KC, (cuuint32_t)BW, (cuuint32_t)BH, 1};
-        cuuint32_t es[4] = {1, 1, 1, 1};
-        if (fn(&mx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void*)x, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               KC == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
-            CUDA_SUCCESS)
-            return false;
-    }
-    {
-        cuuint64_t dims[2] = {(cuuint64_t)Cin, (cuuint64_t)9 * Cout};
-        cuuint64_t strides[1] = {(cuuint64_t)Cin * 2};
-        cuuint32_t box[2] = {(cuuint32_t)KC, (cuuint32_t)BN};
-        cuuint32_t es[2] = {1, 1};
-        if (fn(&mw, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)wt, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               KC == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
-            CUDA_SUCCESS)
-            return false;
-    }
+    if (!pixel_map(&mx, x, N, H, W, Cin, KC, BW, BH) || !weight_map(&mw, wt, Cin, Cout, KC, BN, 1)) return false;
     const int smem = kTcStages * (128 + BN) * KC * 2 + 1024;
     // set on every call: the attribute belongs to the current device
     if (cudaFuncSetAttribute(k_conv3x3_tc<BN, KC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
@@ -1170,12 +1397,62 @@ bool launch_tc(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, cons
     return true;
 }
 
+// The halo form, for images that divide into blocks of 8 x 16 pixels and channel counts whose
+// boxes fit in shared memory; false (nothing launched) otherwise.
+template <int KC, int MT>
+bool launch_halo(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, const float* bias, int Cout, int relu,
+                 bf16* y, int ldy, const bf16* mask, cudaStream_t s, int BN)
+{
+    const int kc = Cin / KC, a = kc * halo_bytes(MT, KC) + 1024, b = BN * KC * 2;
+    if (kc > kHaloChunks) return false;
+    // The fewest and largest weight stages that fit: a wait and its loop cost about as much as
+    // eight MMAs.  With more CTAs than SMs, two to an SM: all nine taps at once, three at a
+    // time, or one, or a few channel chunks of one; where the boxes alone leave no room for a
+    // second CTA, the per-tap kernel is the better one ((4, 32, 128, 384, 128): 24.6 us against
+    // 31.1).  With at most one CTA per SM its whole shared memory.
+    const long long ctas = (long long)N * (H / 16) * (W / (8 * MT)) * (Cout / BN);
+    const int limit = ctas > 152 ? 112 * 1024 : 226 * 1024;
+    HaloStages st{0, 0, 0};
+    auto take = [&](int T, int CC, int S) {
+        if (st.S || CC < 1 || kc % CC || (long long)a + (long long)S * T * CC * b > limit) return;
+        st = {T, CC, S};
+    };
+    take(9, kc, 1);
+    take(3, kc, 3);
+    take(1, kc, 4);
+    take(1, kc, 3);
+    take(1, kc / 2, 4);
+    take(1, kc / 3, 4);
+    take(1, 1, 4);
+    take(1, 1, 3);
+    if (!st.S) return false;
+    const int smem = a + st.S * st.T * st.CC * b;
+    CUtensorMap mx, mw;
+    if (!pixel_map(&mx, x, N, H, W, Cin, KC, 8 * MT + 2, kHaloRows) || !weight_map(&mw, wt, Cin, Cout, KC, BN, st.T))
+        return false;
+    // set on every call: the attribute belongs to the current device
+    if (cudaFuncSetAttribute(k_conv3x3_halo<KC, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    dim3 grd(N * (H / 16) * (W / (8 * MT)), Cout / BN);
+    k_conv3x3_halo<KC, MT><<<grd, 128 * MT, smem, s>>>(mx, mw, H, W, Cin, Cout, BN, st, bias, relu, y, ldy, mask);
+    return true;
+}
+
 bool conv_tc(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, const float* bias, int Cout, int relu,
              bf16* y, int ldy, const bf16* mask, cudaStream_t s)
 {
     int BW = 0, BH = 0;
     const int bn = tc_bn(N, H, W, Cout, BW, BH);
     if (!bn || (((uintptr_t)x | (uintptr_t)wt | (uintptr_t)y | (uintptr_t)mask) & 15) || ldy % 8) return false;
+    if (H % 16 == 0 && W % 8 == 0) {
+        // two blocks per CTA where that still gives every SM a CTA (half the weight traffic)
+        const bool two = W % 16 == 0 && (long long)N * H * W / 256 * (Cout / bn) >= 152;
+        const auto f = Cin % 64 == 0 ? (two ? launch_halo<64, 2> : launch_halo<64, 1>)
+                                     : (two ? launch_halo<32, 2> : launch_halo<32, 1>);
+        if (f(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, bn)) return true;
+    }
     if (Cin % 64 == 0) {
         switch (bn) {
         case 256: return launch_tc<256, 64>(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, BW, BH);

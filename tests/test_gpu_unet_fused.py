@@ -131,6 +131,7 @@ def test_parameters_of_the_callers_own():
     x = torch.randn((1, 16, 64, 32), device="cuda", generator=g).to(torch.bfloat16)
     y = torch.randn((1, 16, 64, 5), device="cuda", generator=g)
     la, lb = a.train_step(x, y), b.train_step(x, y)
-    assert la == lb
+    # (the loss is an FP64 sum of one atomic per block, in any order: at most 304 roundings)
+    assert abs(la - lb) <= 304 * 2.0 ** -53 * la
     for k in a.G:  # the order of the weight gradients' atomic sums is the only difference
         assert float((a.G[k] - b.G[k]).norm()) <= 1e-5 * float(a.G[k].norm()), k
