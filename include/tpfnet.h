@@ -34,8 +34,8 @@ int tpfnet_conv3x3(const void *x, int N, int H, int W, int Cin, const void *wt, 
  * tensor memory. */
 int tpfnet_conv3x3_tcgen05(int N, int H, int W, int Cin, int Cout);
 
-/* 1 when tpfnet_conv3x3_wgrad runs the tcgen05 kernel for a shape (W a multiple of 64,
- * 16-byte aligned tensors), 0 for the mma.sync kernel.  The tcgen05 weight gradient
+/* 1 when tpfnet_conv3x3_wgrad runs a tcgen05 kernel for a shape (W a multiple of 64, or W of 8
+ * and H of 16; 16-byte aligned tensors), 0 for the mma.sync kernel.  The tcgen05 weight gradient
  * reduces over pixels with both operands staged MN-major by TMA (one pixel's channels
  * per 128-byte row) and adds each CTA's FP32 partial sums into dw with atomics. */
 int tpfnet_conv3x3_wgrad_tcgen05(int N, int H, int W, int Cin, int Cout);

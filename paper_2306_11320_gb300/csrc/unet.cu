@@ -890,6 +890,198 @@ __device__ __forceinline__ void relu_back8(Piece& d, const Piece& y)
         if (!(y.v[j] > 0.f)) d.v[j] = 0.f;
 }
 
+// ------------------------------------------ tcgen05 weight gradient on halo tiles
+//
+// The weight gradient with 8 x 16 pixel blocks as K steps of 128 and one column offset dw of
+// the taps per CTA: a stage holds the block of dz (64 output channels per box, two boxes when
+// there are more) and the block of x shifted by dw with a row above and below, 18 rows of 8
+// pixels by CK input channels.  Both are MN-major, one pixel's channels per row.  The three
+// taps of the column are one MMA: its N runs over three blocks of CK channels that lie one
+// image row (eight rows of shared memory) apart, so the operand's windows are the taps' shifts
+// and dz is read from shared memory once for the three.  M = 128 output channels (past the
+// boxes that exist, lanes hold sums that are not read), N = 3 CK, K = 16 pixels = two image
+// rows.  db is summed from the dz boxes by four more warps in the CTAs of dw = -1 and the
+// first input channels, each thread eight channels of every fourth pixel.  Partial sums of a
+// CTA go to dw in vector reductions.
+//
+// Weight and bias gradient, batch 4 (us, against one tap or column of taps per stage with its
+// own x box): 512 x 128 32 -> 32 62 -> 24, 96 -> 32 122 -> 44; 256 x 64 64 -> 64 29 -> 19, 192 ->
+// 64 62 -> 22; 64 x 16 256 -> 256 31 -> 13.  Bound by the MMAs (N = 192 takes the tensor pipe as
+// long as shared memory takes to deliver its operands) and, at 64 channels and fewer, by the
+// kernel's start and the reductions at its end.  The sums are more accurate than before
+// (fewer accumulations in a row): 2.5e-6 -> 1.1e-6 of dw at 512 x 128, 7.5e-7 -> 4.9e-7 at 256 x
+// 64 (relative L2 against float64).
+constexpr int kWhDz = 128 * 128;  // a dz box: 128 pixels of 64 channels
+constexpr int kWhStages = 4;
+
+// MN-major descriptor: rows of CK channels (64 or 128 bytes, swizzled over the row), groups of
+// eight rows sbo bytes apart along K, blocks of a row's channels lbo bytes apart along M or N
+template <int CK>
+__device__ __forceinline__ uint64_t mnmajor_desc2(uint32_t addr, uint32_t lbo, uint32_t sbo)
+{
+    constexpr uint64_t mode = CK == 64 ? 2 : 4;
+    return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(sbo >> 4) << 32) |
+           ((uint64_t)1 << 46) | (mode << 61);
+}
+__device__ __forceinline__ void red_add4(float* p, const uint32_t* r)
+{
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(__uint_as_float(r[0])),
+                 "f"(__uint_as_float(r[1])), "f"(__uint_as_float(r[2])), "f"(__uint_as_float(r[3]))
+                 : "memory");
+}
+
+template <int CK>
+__global__ void __launch_bounds__(256)
+k_conv3x3_wgrad_halo(const __grid_constant__ CUtensorMap mdz, const __grid_constant__ CUtensorMap mx, int N, int H,
+                     int W, int Cin, int Cout, int tiles_per_cta, float* __restrict__ dw, float* __restrict__ db)
+{
+    constexpr int kX = 18 * 8 * 2 * CK, kRow = 8 * 2 * CK;  // x box, one image row of it
+    constexpr uint32_t kCols = CK == 64 ? 256 : 128;        // TMEM columns: 3 CK in use
+    // MN-major A and B (transpose bits)
+    constexpr uint32_t idesc = tc_idesc(128, 3 * CK) | (1u << 15) | (1u << 16);
+    extern __shared__ __align__(1024) unsigned char tsm[];
+    __shared__ __align__(8) uint64_t full[kWhStages], empty[kWhStages], done;
+    __shared__ uint32_t tmem_base;
+    __shared__ float sdb[4][128];
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    unsigned char* st0 = tsm + ((1024 - (sa(tsm) & 1023)) & 1023);
+    const int co0 = blockIdx.x * 128, ci0 = blockIdx.y * CK;
+    const int g = blockIdx.z % 3, split = blockIdx.z / 3;
+    const int nb = co0 + 64 < Cout ? 2 : 1;  // dz boxes
+    const int boxes = Cout > 64 ? 2 : 1;     // room for them
+    const int kStage = boxes * kWhDz + kX;
+    const int bpr = W / 8, bpi = bpr * (H / 16), tiles = N * bpi;
+    const int begin = split * tiles_per_cta, end = min(begin + tiles_per_cta, tiles), steps = max(end - begin, 0);
+    const bool bias = db && g == 0 && blockIdx.y == 0;
+
+    if (tid == 0) {
+        for (int s = 0; s < kWhStages; ++s) {
+            mb_init(&full[s], 1);
+            mb_init(&empty[s], bias ? 5 : 1);  // the MMAs and, with the bias, its four warps
+        }
+        mb_init(&done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sa(&tmem_base)),
+                     "r"(kCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_base;
+
+    if (warp == 0) {
+        int n = begin / bpi, rem = begin - n * bpi, row = rem / bpr, col = rem - row * bpr, issued = 0;
+        for (; issued < steps; ++issued) {
+            const int s = issued % kWhStages;
+            if (issued >= kWhStages && !mb_wait(&empty[s], (issued / kWhStages - 1) & 1)) break;
+            if (elect_one()) {
+                unsigned char* a = st0 + s * kStage;
+                mb_expect_tx(&full[s], nb * kWhDz + kX);
+                tma_4d(a, &mdz, &full[s], co0, 8 * col, 16 * row, n);
+                if (nb == 2) tma_4d(a + kWhDz, &mdz, &full[s], co0 + 64, 8 * col, 16 * row, n);
+                tma_4d(a + boxes * kWhDz, &mx, &full[s], ci0, 8 * col + g - 1, 16 * row - 1, n);
+            }
+            __syncwarp();
+            if (++col == bpr) {
+                col = 0;
+                if (++row * bpr == bpi) { row = 0; ++n; }
+            }
+        }
+        if (issued < steps)  // a wait ran out: the copies still in flight land before the CTA ends
+            for (int k = max(issued - kWhStages, 0); k < issued; ++k) mb_wait(&full[k % kWhStages], (k / kWhStages) & 1);
+    } else if (warp == 1) {
+        for (int k = 0; k < steps; ++k) {
+            const int s = k % kWhStages;
+            if (!mb_wait(&full[s], (k / kWhStages) & 1)) break;
+            tc_fence_after();
+            if (elect_one()) {
+                const uint32_t a = sa(st0 + s * kStage), b = a + boxes * kWhDz;
+                // (with one dz box the second block of M is the first one's rows 8 and on)
+                const uint64_t ad = mnmajor_desc2<64>(a, nb == 2 ? kWhDz : 1024, 1024);
+                const uint64_t bd = mnmajor_desc2<CK>(b, kRow, kRow);
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk)  // two image rows each
+                    tc_mma(tmem, ad + 2048 / 16 * kk, bd + 2 * kRow / 16 * kk, idesc, (k | kk) != 0);
+                tc_commit(&empty[s]);
+            }
+            __syncwarp();
+        }
+        if (elect_one()) tc_commit(&done);
+    } else if (warp >= 4 && bias) {
+        // lane: 16-byte piece lane % 8 of a row, pixels 32 (warp - 4) + 4 j + lane / 8
+        const int piece = lane & 7, p0 = 32 * (warp - 4) + (lane >> 3);
+        float acc[2][8] = {};
+        for (int k = 0; k < steps; ++k) {
+            const int s = k % kWhStages;
+            if (!mb_wait(&full[s], (k / kWhStages) & 1)) break;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                if (q >= nb) break;
+                const unsigned char* a = st0 + s * kStage + q * kWhDz;
+                float part[8] = {};
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int p = p0 + 4 * j;
+                    const Piece v = ld8(reinterpret_cast<const bf16*>(a + 128 * p + 16 * (piece ^ (p & 7))));
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) part[e] += v.v[e];
+                }
+#pragma unroll
+                for (int e = 0; e < 8; ++e) acc[q][e] += part[e];
+            }
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sa(&empty[s])) : "memory");
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                float v = acc[q][e];
+                v += __shfl_xor_sync(0xffffffffu, v, 8);
+                v += __shfl_xor_sync(0xffffffffu, v, 16);
+                if (lane < 8) sdb[warp - 4][64 * q + 8 * piece + e] = v;
+            }
+        }
+    }
+    __syncwarp();
+
+    // thread (warp w, lane l) owns output channel co0 + 32 (w % 4) + l (its TMEM lane); warps 4-7
+    // take the second half of the columns
+    mb_wait(&done, 0);
+    tc_fence_after();
+    const int co = co0 + (warp & 3) * 32 + lane;
+    const bool mine = steps > 0 && co < Cout;
+    constexpr int kHalf = 3 * CK / 2;
+#pragma unroll 1
+    for (int c = (warp >> 2) * kHalf; c < ((warp >> 2) + 1) * kHalf; c += 16) {
+        uint32_t r[16];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+            "%15}, [%16];"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+              "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+            : "r"(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (mine) {
+            // columns c .. c + 15: tap 3 (c / CK) + g, input channels ci0 + c % CK and on
+            float* dst = dw + ((size_t)(3 * (c / CK) + g) * Cout + co) * Cin + ci0 + c % CK;
+#pragma unroll
+            for (int j = 0; j < 16; j += 4) red_add4(dst + j, r + j);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (bias && tid < 128 && co0 + tid < Cout)  // one atomic per CTA and channel
+        atomicAdd(db + co0 + tid, (sdb[0][tid] + sdb[1][tid]) + (sdb[2][tid] + sdb[3][tid]));
+    if (warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
+}
+
 __global__ void k_relu_mask8(bf16* __restrict__ d, const bf16* __restrict__ y, long long pieces)
 {
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < pieces; k += (long long)gridDim.x * blockDim.x) {
@@ -1407,9 +1599,9 @@ bool launch_halo(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, co
     if (kc > kHaloChunks) return false;
     // The fewest and largest weight stages that fit: a wait and its loop cost about as much as
     // eight MMAs.  With more CTAs than SMs, two to an SM: all nine taps at once, three at a
-    // time, or one, or a few channel chunks of one; where the boxes alone leave no room for a
-    // second CTA, the per-tap kernel is the better one ((4, 32, 128, 384, 128): 24.6 us against
-    // 31.1).  With at most one CTA per SM its whole shared memory.
+    // time, or one; where the boxes leave no room for that, the per-tap kernel is the better
+    // one ((4, 32, 128, 384, 128): 22.9 us against 31.1, (4, 16, 64, 256, 256): 16.8 against
+    // 17.7).  With at most one CTA per SM its whole shared memory, and parts of a tap if need be.
     const long long ctas = (long long)N * (H / 16) * (W / (8 * MT)) * (Cout / BN);
     const int limit = ctas > 152 ? 112 * 1024 : 226 * 1024;
     HaloStages st{0, 0, 0};
@@ -1421,10 +1613,11 @@ bool launch_halo(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, co
     take(3, kc, 3);
     take(1, kc, 4);
     take(1, kc, 3);
-    take(1, kc / 2, 4);
-    take(1, kc / 3, 4);
-    take(1, 1, 4);
-    take(1, 1, 3);
+    if (ctas <= 152) {
+        take(1, kc / 2, 4);
+        take(1, kc / 3, 4);
+        take(1, 1, 4);
+    }
     if (!st.S) return false;
     const int smem = a + st.S * st.T * st.CC * b;
     CUtensorMap mx, mw;
@@ -1469,12 +1662,44 @@ bool conv_tc(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, const 
     }
 }
 
+// The halo form of the weight gradient, for images that divide into blocks of 8 x 16 pixels;
+// false (nothing launched) otherwise.
+template <int CK>
+bool launch_wgrad_halo(const bf16* x, const bf16* dz, int N, int H, int W, int Cin, int Cout, float* dw, float* db,
+                       cudaStream_t s)
+{
+    CUtensorMap mdz, mx;
+    if (!pixel_map(&mdz, dz, N, H, W, Cout, 64, 8, 16) || !pixel_map(&mx, x, N, H, W, Cin, CK, 8, 18)) return false;
+    const int stage = (Cout > 64 ? 2 : 1) * kWhDz + 18 * 8 * 2 * CK, smem = kWhStages * stage + 1024;
+    if (cudaFuncSetAttribute(k_conv3x3_wgrad_halo<CK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    // split the blocks over about as many CTAs as run at once
+    const long long tiles = (long long)N * (H / 16) * (W / 8);
+    const int ctiles = (Cout + 127) / 128, itiles = Cin / CK;
+    const long long base = 3LL * ctiles * itiles, target = smem <= 112 * 1024 ? 304 : 152;
+    long long splits = target / base;
+    if (splits > tiles) splits = tiles;
+    if (splits < 1) splits = 1;
+    const long long per = (tiles + splits - 1) / splits;
+    splits = (tiles + per - 1) / per;
+    k_conv3x3_wgrad_halo<CK><<<dim3(ctiles, itiles, 3 * (unsigned)splits), 256, smem, s>>>(mdz, mx, N, H, W, Cin, Cout,
+                                                                                          (int)per, dw, db);
+    return true;
+}
+
 // The tcgen05 weight gradient for W a multiple of 64 and 16-byte aligned tensors;
 // false (nothing launched) otherwise.  Adds into dw (and db).
 bool wgrad_tc(const bf16* x, const bf16* dz, int N, int H, int W, int Cin, int Cout, float* dw, float* db,
               cudaStream_t s)
 {
-    if (W % kWgPix != 0 || (((uintptr_t)x | (uintptr_t)dz) & 15)) return false;
+    if (((uintptr_t)x | (uintptr_t)dz) & 15) return false;
+    if (H % 16 == 0 && W % 8 == 0 && (uintptr_t)dw % 16 == 0) {
+        const auto f = Cin % 64 == 0 ? launch_wgrad_halo<64> : launch_wgrad_halo<32>;
+        if (f(x, dz, N, H, W, Cin, Cout, dw, db, s)) return true;
+    }
+    if (W % kWgPix != 0) return false;
     auto fn = encode_fn();
     if (!fn) return false;
     CUtensorMap mdz, mx;
@@ -1585,7 +1810,8 @@ int tpfnet_conv3x3_tcgen05(int N, int H, int W, int Cin, int Cout)
 
 int tpfnet_conv3x3_wgrad_tcgen05(int N, int H, int W, int Cin, int Cout)
 {
-    return N >= 1 && H >= 1 && W >= 1 && Cin % 32 == 0 && Cout % 32 == 0 && W % kWgPix == 0 && encode_fn() ? 1 : 0;
+    const bool tiles = W % kWgPix == 0 || (H % 16 == 0 && W % 8 == 0);
+    return N >= 1 && H >= 1 && W >= 1 && Cin % 32 == 0 && Cout % 32 == 0 && tiles && encode_fn() ? 1 : 0;
 }
 
 int tpfnet_status(void)

@@ -135,3 +135,45 @@ def test_parameters_of_the_callers_own():
     assert abs(la - lb) <= 304 * 2.0 ** -53 * la
     for k in a.G:  # the order of the weight gradients' atomic sums is the only difference
         assert float((a.G[k] - b.G[k]).norm()) <= 1e-5 * float(a.G[k].norm()), k
+
+
+# images that divide into 8 x 16 blocks: one block, two side by side, rows of blocks; channel
+# counts of one chunk and several, whole and half boxes; (4, 16, 64, 256, 256) and (1, 16, 16,
+# 384, 64) have too many channels for the boxes of two CTAs on an SM
+@pytest.mark.parametrize("N,H,W,Cin,Cout", [(1, 16, 8, 32, 32), (1, 16, 16, 64, 64), (2, 32, 24, 96, 96),
+                                            (1, 48, 40, 64, 160), (3, 16, 32, 192, 64), (1, 16, 16, 384, 64),
+                                            (4, 16, 64, 256, 256), (2, 128, 256, 32, 128)])
+def test_block_convolutions(N, H, W, Cin, Cout):
+    """Forward, data and weight gradients against float64.  Bounds, element by element: a
+    float32 sum of n terms is within n 2^-24 sum |terms|, a stored bf16 within 2^-8 of its
+    value; weight gradients are added to what is there."""
+    lib = _lib()
+    x, wt, dz = _rnd(N, H, W, Cin).relu(), _rnd(9, Cout, Cin, seed=1), _rnd(N, H, W, Cout, seed=2)
+    g = torch.Generator(device="cuda").manual_seed(H + W)
+    b = torch.randn(Cout, device="cuda", generator=g)
+    dw0, db0 = torch.randn((9, Cout, Cin), device="cuda", generator=g), torch.randn(Cout, device="cuda", generator=g)
+    y, dx, wf, dw, db = torch.empty_like(dz), torch.empty_like(x), torch.empty_like(wt), dw0.clone(), db0.clone()
+    _ok(lib.tpfnet_conv3x3(_p(x), N, H, W, Cin, _p(wt), _p(b), Cout, 0, _p(y), None),
+        lib.tpfnet_conv3x3_dgrad(_p(dz), N, H, W, Cout, _p(wt), Cin, _p(wf), _p(dx), None),
+        lib.tpfnet_conv3x3_wgrad(_p(x), _p(dz), N, H, W, Cin, Cout, _p(dw), _p(db), None))
+    assert lib.tpfnet_status() == 0
+    F = torch.nn.functional
+    k = wt.double().view(3, 3, Cout, Cin).permute(2, 3, 0, 1).contiguous()
+    xd, dd = x.double().permute(0, 3, 1, 2).contiguous(), dz.double().permute(0, 3, 1, 2).contiguous()
+    u, nhwc = 2.0 ** -24, lambda t: t.permute(0, 2, 3, 1)
+
+    def near(got, ref, mag, n, store):
+        assert ((got.double() - ref).abs() <= n * u * mag + store * ref.abs()).all()
+
+    ref, mag = F.conv2d(xd, k, b.double(), padding=1), F.conv2d(xd.abs(), k.abs(), b.double().abs(), padding=1)
+    near(y, nhwc(ref), nhwc(mag), 9 * Cin + 1, 2.0 ** -8)
+    ref, mag = F.conv_transpose2d(dd, k, padding=1), F.conv_transpose2d(dd.abs(), k.abs(), padding=1)
+    near(dx, nhwc(ref), nhwc(mag), 9 * Cout, 2.0 ** -8)
+    px = N * H * W
+    pad = F.pad(xd, (1, 1, 1, 1))
+    for tap in range(9):
+        win = pad[:, :, tap // 3:tap // 3 + H, tap % 3:tap % 3 + W]
+        ref = torch.einsum("nohw,nihw->oi", dd, win) + dw0[tap].double()
+        mag = torch.einsum("nohw,nihw->oi", dd.abs(), win.abs()) + dw0[tap].double().abs()
+        near(dw[tap], ref, mag, px + 1, 0.0)
+    near(db, dd.sum((0, 2, 3)) + db0.double(), dd.abs().sum((0, 2, 3)) + db0.double().abs(), px + 1, 0.0)
