@@ -110,6 +110,23 @@ int tpfnet_head(const void *x, long long pixels, int C, const float *Wt, const f
 int tpfnet_head_back(const void *x, const float *dout, long long pixels, int C, const float *Wt, int Cout,
                      void *dx, float *dW, float *db, void *stream);
 
+/* The whole forward pass of the 4-level network: the calls above in order, queued by one call.
+ * weight and bias: the fourteen 3x3 layers in the order they run (encoder levels 0-3, decoder
+ * levels 2-0, two layers each); the activations' buffers are the caller's and keep what a
+ * backward pass needs (cat[l]: ch[l + 1] upsampled channels, then the encoder's ch[l]). */
+typedef struct tpfnet_unet {
+    int cin, cout, ch[4];      /* input channels (padded), outputs, channels per level */
+    const void *weight[14];
+    const float *bias[14];
+    const float *head_w, *head_b;
+    void *enc[4];              /* between the two layers of encoder level l */
+    void *pool[3];             /* pooled outputs of levels 0-2 */
+    void *cat[3];              /* concatenations of levels 0-2 */
+    void *deep;                /* output of level 3 */
+    void *dec_a[3], *dec[3];   /* between the two layers, and output, of decoder level l */
+} tpfnet_unet;
+int tpfnet_unet_forward(const tpfnet_unet *u, const void *x, int N, int H, int W, float *out, void *stream);
+
 /* loss += mean_k (pred[k] - target[k])^2 wch[k % C] (FP64, device); grad[k] = d loss /
  * d pred[k] (or NULL to skip); wch may be NULL (all ones). */
 int tpfnet_mse(const float *pred, const float *target, const float *wch, long long count, int C, float *grad,

@@ -394,8 +394,9 @@ __device__ __forceinline__ void step_tile_general(const DevParams& P, const type
     __syncthreads();  // the caller may reuse sm for the next tile
 }
 // Tile b of an axis of n nodes: start and extent.  Whole tiles of B nodes first, the
-// ragged one last (tile_whole), or nt = ceil(n / B) tiles of nearly equal extent
-// (tile_even; at least B / 2 nodes each once nt > 1).
+// ragged one last (tile_whole), or nt = ceil(n / B) tiles of nearly equal extent (tile_even:
+// the many-step kernel, whose step takes as long as its fullest tile; where tiles come in
+// waves, whole ones are 1% faster).
 __device__ __forceinline__ void tile_whole(int n, int B, int b, int& x0, int& w)
 {
     x0 = b * B;
@@ -414,8 +415,8 @@ k_step_general(const DevParams P, const typename S::elem* __restrict__ A, typena
 {
     __shared__ RingSmem<BX, BY> sm;
     int x0, y0, w, h;
-    tile_even(P.nx, gridDim.x, blockIdx.x, x0, w);
-    tile_even(P.ny, gridDim.y, blockIdx.y, y0, h);
+    tile_whole(P.nx, BX, blockIdx.x, x0, w);
+    tile_whole(P.ny, BY, blockIdx.y, y0, h);
     step_tile_general<BX, BY, S>(P, A, B, phiu, refA, refB, sm, x0, y0, w, h);
 }
 

@@ -128,8 +128,8 @@ __device__ __forceinline__ void each_macro(const DevParams& P, const typename S:
     const int ntx = (P.nx + kBX - 1) / kBX, nty = (P.ny + kBY - 1) / kBY;
     for (int t = blockIdx.x; t < ntx * nty; t += gridDim.x) {
         int x0, y0, w, h;
-        tile_even(P.nx, ntx, t % ntx, x0, w);
-        tile_even(P.ny, nty, t / ntx, y0, h);
+        tile_whole(P.nx, kBX, t % ntx, x0, w);
+        tile_whole(P.ny, kBY, t / ntx, y0, h);
         tile_macro<kBX, kBY, S>(P, A, ref, phiu, sm, x0, y0, w, h, use);
     }
 }

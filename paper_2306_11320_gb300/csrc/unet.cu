@@ -17,6 +17,36 @@ namespace {
 
 typedef __nv_bfloat16 bf16;
 
+// Programmatic dependent launch: every kernel here is launched so that its CTAs may start
+// while the kernel before it on the stream drains, and waits for that kernel's end (and its
+// memory) before it touches global memory.  What runs ahead is the launch itself and a tensor
+// core kernel's set-up (barriers, tensor memory, descriptors), about 2 us of each of the 20 to
+// 60 short kernels of a forward or training step.  pdl_next lets the next kernel start; the
+// tensor core kernels say so once they hold their tensor memory (a waiting successor must
+// not take it from a CTA that has yet to allocate).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_enter()
+{
+    pdl_wait();
+    pdl_next();
+}
+template <class... K, class... A>
+cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, K(args)...);
+}
+
 constexpr int kBM = 64;  // output pixels per CTA (one row segment)
 constexpr int kKC = 32;  // input channels per K chunk
 constexpr int kPad = 8;  // smem row padding (bf16) against bank conflicts
@@ -40,6 +70,7 @@ k_conv3x3(const bf16* __restrict__ x, int N, int H, int W, int Cin, const bf16* 
           const float* __restrict__ bias, int Cout, int relu, bf16* __restrict__ y, int ldy,
           const bf16* __restrict__ mask)
 {
+    pdl_enter();
     __shared__ __align__(16) bf16 As[kBM][kKC + kPad];
     __shared__ __align__(16) bf16 Bs[BN][kKC + kPad];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -255,9 +286,11 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUt
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    pdl_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_next();
     const uint32_t tmem = tmem_base;
 
     if (warp == 0) {
@@ -420,10 +453,12 @@ k_conv3x3_halo(const __grid_constant__ CUtensorMap mx, const __grid_constant__ C
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    pdl_wait();
     for (int k = tid; k < BN; k += 128 * MT) sbias[k] = bias ? bias[co0 + k] : 0.f;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_next();
     const uint32_t tmem = tmem_base;
 
     // Stage k covers taps t .. t + T - 1 and chunks c .. c + CC - 1.  All counters advance by
@@ -562,6 +597,7 @@ __global__ void __launch_bounds__(128)
 k_conv3x3_wgrad(const bf16* __restrict__ x, const bf16* __restrict__ dz, int N, int H, int W, int Cin, int Cout,
                 int pix_per_cta, float* __restrict__ dw, float* __restrict__ db)
 {
+    pdl_enter();
     constexpr int RB = WM / 16;        // row blocks
     constexpr int NG = 4 / RB;         // n-tile groups
     constexpr int NTW = 4 / NG;        // n-tiles (of 8 ci) per warp
@@ -717,9 +753,11 @@ k_conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap mdz, const __grid_constan
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    pdl_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_next();
     const uint32_t tmem = tmem_base;
 
     if (warp == 0) {
@@ -833,6 +871,7 @@ struct FlipList {
 };
 __global__ void __launch_bounds__(256) k_flip_weights(const FlipList L)
 {
+    pdl_enter();
     // 32 x 32 (co, ci) tiles of one tap through shared memory, so that both sides are read
     // and written in whole rows
     __shared__ bf16 t[32][33];
@@ -968,9 +1007,11 @@ k_conv3x3_wgrad_halo(const __grid_constant__ CUtensorMap mdz, const __grid_const
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    pdl_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_next();
     const uint32_t tmem = tmem_base;
 
     if (warp == 0) {
@@ -1084,6 +1125,7 @@ k_conv3x3_wgrad_halo(const __grid_constant__ CUtensorMap mdz, const __grid_const
 
 __global__ void k_relu_mask8(bf16* __restrict__ d, const bf16* __restrict__ y, long long pieces)
 {
+    pdl_enter();
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < pieces; k += (long long)gridDim.x * blockDim.x) {
         Piece v = ld8(d + 8 * k);
         relu_back8(v, ld8(y + 8 * k));
@@ -1095,6 +1137,7 @@ __global__ void k_relu_mask8(bf16* __restrict__ d, const bf16* __restrict__ y, l
 // x: ldx channels per pixel
 __global__ void k_pool8(const bf16* __restrict__ x, int rows, int W, int C8, int ldx, bf16* __restrict__ y)
 {
+    pdl_enter();
     const int Wo = W / 2, C = 8 * C8;
     for (int r = blockIdx.y; r < rows; r += gridDim.y)  // output row: image rows 2 r, 2 r + 1
         for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < Wo * C8; k += gridDim.x * blockDim.x) {
@@ -1114,6 +1157,7 @@ __global__ void k_pool8(const bf16* __restrict__ x, int rows, int W, int C8, int
 __global__ void k_pool_back8(const bf16* __restrict__ dy, int rows, int W, int C8, const bf16* add, int lda,
                              const bf16* __restrict__ mask, int ldm, bf16* dx)
 {
+    pdl_enter();
     const int Wo = W / 2, C = 8 * C8;
     for (int r = blockIdx.y; r < rows; r += gridDim.y)
         for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < Wo * C8; k += gridDim.x * blockDim.x) {
@@ -1139,6 +1183,7 @@ __global__ void k_pool_back8(const bf16* __restrict__ dy, int rows, int W, int C
 }
 __global__ void k_up_into8(const bf16* __restrict__ x, int rows, int W, int C8, bf16* __restrict__ y, int Ctot, int cofs)
 {
+    pdl_enter();
     const int Wo = W / 2, C = 8 * C8;
     for (int r = blockIdx.y; r < rows; r += gridDim.y)
         for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < Wo * C8; k += gridDim.x * blockDim.x) {
@@ -1155,6 +1200,7 @@ __global__ void k_up_into8(const bf16* __restrict__ x, int rows, int W, int C8, 
 __global__ void k_up_back8(const bf16* __restrict__ dy, int rows, int W, int Ctot, int cofs, int C8,
                            const bf16* __restrict__ mask, bf16* __restrict__ dx)
 {
+    pdl_enter();
     const int Wo = W / 2, C = 8 * C8;
     for (int r = blockIdx.y; r < rows; r += gridDim.y)
         for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < Wo * C8; k += gridDim.x * blockDim.x) {
@@ -1173,6 +1219,7 @@ __global__ void k_up_back8(const bf16* __restrict__ dy, int rows, int W, int Cto
 __global__ void k_channels8(const bf16* __restrict__ src, int Sc, int sofs, long long pixels, int C8,
                             bf16* __restrict__ dst, int Dc, int dofs, int accumulate)
 {
+    pdl_enter();
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < pixels * C8; k += (long long)gridDim.x * blockDim.x) {
         const long long p = k / C8;
         const int c = 8 * (int)(k - p * C8);
@@ -1192,6 +1239,7 @@ __global__ void k_channels8(const bf16* __restrict__ src, int Sc, int sofs, long
 
 __global__ void k_relu_mask(bf16* __restrict__ d, const bf16* __restrict__ y, long long count)
 {
+    pdl_enter();
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < count; k += (long long)gridDim.x * blockDim.x)
         if (!(__bfloat162float(y[k]) > 0.f)) d[k] = __float2bfloat16_rn(0.f);
 }
@@ -1199,6 +1247,7 @@ __global__ void k_relu_mask(bf16* __restrict__ d, const bf16* __restrict__ y, lo
 // 2x2 average pooling and its adjoint; nearest upsampling and its adjoint
 __global__ void k_pool(const bf16* __restrict__ x, int N, int H, int W, int C, bf16* __restrict__ y)
 {
+    pdl_enter();
     const int Ho = H / 2, Wo = W / 2;
     const long long total = (long long)N * Ho * Wo * C;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < total; k += (long long)gridDim.x * blockDim.x) {
@@ -1216,6 +1265,7 @@ __global__ void k_pool(const bf16* __restrict__ x, int N, int H, int W, int C, b
 // dx[fine] (+)= dy[coarse] / 4
 __global__ void k_pool_back(const bf16* __restrict__ dy, int N, int H, int W, int C, bf16* __restrict__ dx, int accumulate)
 {
+    pdl_enter();
     const long long total = (long long)N * H * W * C;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < total; k += (long long)gridDim.x * blockDim.x) {
         const int c = (int)(k % C);
@@ -1231,6 +1281,7 @@ __global__ void k_pool_back(const bf16* __restrict__ dy, int N, int H, int W, in
 // y[n, h, w, cofs + c] = x[n, h/2, w/2, c] : upsampled x into channels [cofs, cofs + C) of a Ctot tensor
 __global__ void k_up_into(const bf16* __restrict__ x, int N, int H, int W, int C, bf16* __restrict__ y, int Ctot, int cofs)
 {
+    pdl_enter();
     const long long total = (long long)N * H * W * C;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < total; k += (long long)gridDim.x * blockDim.x) {
         const int c = (int)(k % C);
@@ -1244,6 +1295,7 @@ __global__ void k_up_into(const bf16* __restrict__ x, int N, int H, int W, int C
 // dx[coarse] = sum of the 4 fine dy values in channels [cofs, cofs + C) of a Ctot tensor
 __global__ void k_up_back(const bf16* __restrict__ dy, int N, int H, int W, int Ctot, int cofs, int C, bf16* __restrict__ dx)
 {
+    pdl_enter();
     const int Ho = H / 2, Wo = W / 2;
     const long long total = (long long)N * Ho * Wo * C;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < total; k += (long long)gridDim.x * blockDim.x) {
@@ -1263,6 +1315,7 @@ __global__ void k_up_back(const bf16* __restrict__ dy, int N, int H, int W, int 
 __global__ void k_channels(const bf16* __restrict__ src, int Sc, int sofs, long long pixels, int C, bf16* __restrict__ dst,
                            int Dc, int dofs, int accumulate)
 {
+    pdl_enter();
     const long long total = pixels * C;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < total; k += (long long)gridDim.x * blockDim.x) {
         const int c = (int)(k % C);
@@ -1282,6 +1335,7 @@ __global__ void __launch_bounds__(256)
 k_head8(const bf16* __restrict__ x, long long pixels, int C, const float* __restrict__ Wt, const float* __restrict__ b,
         float* __restrict__ out)
 {
+    pdl_enter();
     extern __shared__ float shw[];  // C x CO weights, then 256 x CO outputs
     float* sho = shw + C * CO;
     for (int k = threadIdx.x; k < C * CO; k += 256) shw[k] = Wt[k];
@@ -1323,6 +1377,7 @@ k_head_back8(const bf16* __restrict__ x, const float* __restrict__ dout, long lo
              const float* __restrict__ Wt, bf16* __restrict__ dx, float* __restrict__ dW, float* __restrict__ db,
              int relu)
 {
+    pdl_enter();
     extern __shared__ float sh[];  // C * CO + CO sums
     const int G = C >> 3, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int cg = lane & (G - 1), ps = lane / G, PP = 32 / G;
@@ -1384,6 +1439,7 @@ k_head_back8(const bf16* __restrict__ x, const float* __restrict__ dout, long lo
 __global__ void k_head(const bf16* __restrict__ x, long long pixels, int C, const float* __restrict__ Wt,
                        const float* __restrict__ b, int Cout, float* __restrict__ out)
 {
+    pdl_enter();
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < pixels * Cout; k += (long long)gridDim.x * blockDim.x) {
         const int o = (int)(k % Cout);
         const long long p = k / Cout;
@@ -1397,6 +1453,7 @@ __global__ void k_head_back(const bf16* __restrict__ x, const float* __restrict_
                             const float* __restrict__ Wt, int Cout, bf16* __restrict__ dx, float* __restrict__ dW,
                             float* __restrict__ db)
 {
+    pdl_enter();
     extern __shared__ float sh[];  // C * Cout + Cout partial sums
     for (int k = threadIdx.x; k < C * Cout + Cout; k += blockDim.x) sh[k] = 0.f;
     __syncthreads();
@@ -1422,6 +1479,7 @@ __global__ void k_head_back(const bf16* __restrict__ x, const float* __restrict_
 __global__ void __launch_bounds__(256) k_mse(const float* __restrict__ pred, const float* __restrict__ target, const float* __restrict__ wch,
                       long long count, int C, float* __restrict__ grad, double* __restrict__ loss)
 {
+    pdl_enter();
     double acc = 0.0;
     const float inv = 1.f / (float)count;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < count; k += (long long)gridDim.x * blockDim.x) {
@@ -1447,6 +1505,7 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ gr, floa
                        long long count, float lr, float b1, float b2, float eps, float c1, float c2,
                        bf16* __restrict__ pb)
 {
+    pdl_enter();
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < count; k += (long long)gridDim.x * blockDim.x) {
         const float gk = gr[k];
         const float mk = b1 * m[k] + (1.f - b1) * gk;
@@ -1461,6 +1520,7 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ gr, floa
 
 __global__ void k_to_bf16(const float* __restrict__ x, long long count, bf16* __restrict__ y)
 {
+    pdl_enter();
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < count; k += (long long)gridDim.x * blockDim.x)
         y[k] = __float2bfloat16_rn(x[k]);
 }
@@ -1473,6 +1533,7 @@ struct Affine {
 __global__ void k_pack(const float* __restrict__ src, const float* __restrict__ base, long long plane, int C,
                        long long pixels, Affine a, void* __restrict__ dst, int Cd, int bf)
 {
+    pdl_enter();
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < pixels * C; k += (long long)gridDim.x * blockDim.x) {
         const int c = (int)(k % C);
         const long long p = k / C;
@@ -1485,6 +1546,7 @@ __global__ void k_pack(const float* __restrict__ src, const float* __restrict__ 
 __global__ void k_unpack(const float* __restrict__ src, long long pixels, int C, Affine a, const float* __restrict__ base,
                          float* __restrict__ dst, long long plane)
 {
+    pdl_enter();
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < pixels * C; k += (long long)gridDim.x * blockDim.x) {
         const int c = (int)(k % C);
         const long long p = k / C;
@@ -1585,7 +1647,7 @@ bool launch_tc(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, cons
         return false;
     }
     dim3 grd(N * (H / BH) * (W / BW), Cout / BN);
-    k_conv3x3_tc<BN, KC><<<grd, 128, smem, s>>>(mx, mw, H, W, Cin, Cout, BW, BH, bias, relu, y, ldy, mask);
+    launch_pdl(k_conv3x3_tc<BN, KC>, grd, 128, smem, s, mx, mw, H, W, Cin, Cout, BW, BH, bias, relu, y, ldy, mask);
     return true;
 }
 
@@ -1629,7 +1691,7 @@ bool launch_halo(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, co
         return false;
     }
     dim3 grd(N * (H / 16) * (W / (8 * MT)), Cout / BN);
-    k_conv3x3_halo<KC, MT><<<grd, 128 * MT, smem, s>>>(mx, mw, H, W, Cin, Cout, BN, st, bias, relu, y, ldy, mask);
+    launch_pdl(k_conv3x3_halo<KC, MT>, grd, 128 * MT, smem, s, mx, mw, H, W, Cin, Cout, BN, st, bias, relu, y, ldy, mask);
     return true;
 }
 
@@ -1684,7 +1746,7 @@ bool launch_wgrad_halo(const bf16* x, const bf16* dz, int N, int H, int W, int C
     if (splits < 1) splits = 1;
     const long long per = (tiles + splits - 1) / splits;
     splits = (tiles + per - 1) / per;
-    k_conv3x3_wgrad_halo<CK><<<dim3(ctiles, itiles, 3 * (unsigned)splits), 256, smem, s>>>(mdz, mx, N, H, W, Cin, Cout,
+    launch_pdl(k_conv3x3_wgrad_halo<CK>, dim3(ctiles, itiles, 3 * (unsigned)splits), 256, smem, s, mdz, mx, N, H, W, Cin, Cout,
                                                                                           (int)per, dw, db);
     return true;
 }
@@ -1733,9 +1795,9 @@ bool wgrad_tc(const bf16* x, const bf16* dz, int N, int H, int W, int Cin, int C
     splits = (nchunks + per - 1) / per;
     dim3 grd(ctiles, itiles, (9 / taps) * (unsigned)splits);
     if (taps == 3)
-        k_conv3x3_wgrad_tc<3><<<grd, 128, smem, s>>>(mdz, mx, N, H, W, Cin, Cout, (int)per, dw, db);
+        launch_pdl(k_conv3x3_wgrad_tc<3>, grd, 128, smem, s, mdz, mx, N, H, W, Cin, Cout, (int)per, dw, db);
     else
-        k_conv3x3_wgrad_tc<1><<<grd, 128, smem, s>>>(mdz, mx, N, H, W, Cin, Cout, (int)per, dw, db);
+        launch_pdl(k_conv3x3_wgrad_tc<1>, grd, 128, smem, s, mdz, mx, N, H, W, Cin, Cout, (int)per, dw, db);
     return true;
 }
 
@@ -1753,11 +1815,11 @@ static int conv_any(const void* x, int N, int H, int W, int Cin, const void* wt,
     const int wblocks = (W + kBM - 1) / kBM;
     if (Cout % 64 == 0) {
         dim3 grd(wblocks * N * H, Cout / 64);
-        k_conv3x3<64><<<grd, 128, 0, s>>>((const bf16*)x, N, H, W, Cin, (const bf16*)wt, bias, Cout, relu, (bf16*)y,
+        launch_pdl(k_conv3x3<64>, grd, 128, 0, s, (const bf16*)x, N, H, W, Cin, (const bf16*)wt, bias, Cout, relu, (bf16*)y,
                                       ldy, (const bf16*)mask);
     } else {
         dim3 grd(wblocks * N * H, Cout / 32);
-        k_conv3x3<32><<<grd, 128, 0, s>>>((const bf16*)x, N, H, W, Cin, (const bf16*)wt, bias, Cout, relu, (bf16*)y,
+        launch_pdl(k_conv3x3<32>, grd, 128, 0, s, (const bf16*)x, N, H, W, Cin, (const bf16*)wt, bias, Cout, relu, (bf16*)y,
                                       ldy, (const bf16*)mask);
     }
     return status(cudaGetLastError());
@@ -1797,7 +1859,7 @@ int tpfnet_flip_weights(int layers, const void* const* wt, const int* cin, const
         const int tiles = 9 * (cin[l] / 32) * (cout[l] / 32);
         if (tiles > most) most = tiles;
     }
-    k_flip_weights<<<dim3(most < 304 ? most : 304, layers), 256, 0, (cudaStream_t)stream>>>(L);
+    launch_pdl(k_flip_weights, dim3(most < 304 ? most : 304, layers), 256, 0, (cudaStream_t)stream, L);
     return status(cudaGetLastError());
 }
 
@@ -1849,10 +1911,10 @@ int tpfnet_conv3x3_wgrad(const void* x, const void* dz, int N, int H, int W, int
     splits = (P + per - 1) / per;
     dim3 grd(Cin / kWN, Cout / WM, 9 * (int)splits);
     if (WM == 64)
-        k_conv3x3_wgrad<64><<<grd, 128, 0, (cudaStream_t)stream>>>((const bf16*)x, (const bf16*)dz, N, H, W, Cin, Cout,
+        launch_pdl(k_conv3x3_wgrad<64>, grd, 128, 0, (cudaStream_t)stream, (const bf16*)x, (const bf16*)dz, N, H, W, Cin, Cout,
                                                                    (int)per, dw, db);
     else
-        k_conv3x3_wgrad<32><<<grd, 128, 0, (cudaStream_t)stream>>>((const bf16*)x, (const bf16*)dz, N, H, W, Cin, Cout,
+        launch_pdl(k_conv3x3_wgrad<32>, grd, 128, 0, (cudaStream_t)stream, (const bf16*)x, (const bf16*)dz, N, H, W, Cin, Cout,
                                                                    (int)per, dw, db);
     return status(cudaGetLastError());
 }
@@ -1860,10 +1922,10 @@ int tpfnet_conv3x3_wgrad(const void* x, const void* dz, int N, int H, int W, int
 int tpfnet_relu_mask(void* d, const void* y, long long count, void* stream)
 {
     if (pieces((int)(count % 8), d, y)) {
-        k_relu_mask8<<<grid_of(count / 8), 256, 0, (cudaStream_t)stream>>>((bf16*)d, (const bf16*)y, count / 8);
+        launch_pdl(k_relu_mask8, grid_of(count / 8), 256, 0, (cudaStream_t)stream, (bf16*)d, (const bf16*)y, count / 8);
         return status(cudaGetLastError());
     }
-    k_relu_mask<<<grid_of(count), 256, 0, (cudaStream_t)stream>>>((bf16*)d, (const bf16*)y, count);
+    launch_pdl(k_relu_mask, grid_of(count), 256, 0, (cudaStream_t)stream, (bf16*)d, (const bf16*)y, count);
     return status(cudaGetLastError());
 }
 
@@ -1871,22 +1933,22 @@ int tpfnet_pool(const void* x, int N, int H, int W, int C, void* y, void* stream
 {
     if (H % 2 || W % 2) return TPF_ERR_INVALID_ARG;
     if (pieces(C, x, y)) {
-        k_pool8<<<grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, N * (H / 2), W,
+        launch_pdl(k_pool8, grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream, (const bf16*)x, N * (H / 2), W,
                                                                                          C / 8, C, (bf16*)y);
         return status(cudaGetLastError());
     }
-    k_pool<<<grid_of((long long)N * H * W * C / 4), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, N, H, W, C, (bf16*)y);
+    launch_pdl(k_pool, grid_of((long long)N * H * W * C / 4), 256, 0, (cudaStream_t)stream, (const bf16*)x, N, H, W, C, (bf16*)y);
     return status(cudaGetLastError());
 }
 
 int tpfnet_pool_back(const void* dy, int N, int H, int W, int C, void* dx, int accumulate, void* stream)
 {
     if (H % 2 == 0 && W % 2 == 0 && pieces(C, dy, dx)) {
-        k_pool_back8<<<grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream>>>(
+        launch_pdl(k_pool_back8, grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream, 
             (const bf16*)dy, N * (H / 2), W, C / 8, accumulate ? (const bf16*)dx : nullptr, C, nullptr, 0, (bf16*)dx);
         return status(cudaGetLastError());
     }
-    k_pool_back<<<grid_of((long long)N * H * W * C), 256, 0, (cudaStream_t)stream>>>((const bf16*)dy, N, H, W, C, (bf16*)dx,
+    launch_pdl(k_pool_back, grid_of((long long)N * H * W * C), 256, 0, (cudaStream_t)stream, (const bf16*)dy, N, H, W, C, (bf16*)dx,
                                                                                     accumulate);
     return status(cudaGetLastError());
 }
@@ -1894,11 +1956,11 @@ int tpfnet_pool_back(const void* dy, int N, int H, int W, int C, void* dx, int a
 int tpfnet_up_into(const void* x, int N, int H, int W, int C, void* y, int Ctot, int cofs, void* stream)
 {
     if (H % 2 == 0 && W % 2 == 0 && pieces(C | Ctot | cofs, x, y)) {
-        k_up_into8<<<grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream>>>(
+        launch_pdl(k_up_into8, grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream, 
             (const bf16*)x, N * (H / 2), W, C / 8, (bf16*)y, Ctot, cofs);
         return status(cudaGetLastError());
     }
-    k_up_into<<<grid_of((long long)N * H * W * C), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, N, H, W, C, (bf16*)y,
+    launch_pdl(k_up_into, grid_of((long long)N * H * W * C), 256, 0, (cudaStream_t)stream, (const bf16*)x, N, H, W, C, (bf16*)y,
                                                                                   Ctot, cofs);
     return status(cudaGetLastError());
 }
@@ -1906,11 +1968,11 @@ int tpfnet_up_into(const void* x, int N, int H, int W, int C, void* y, int Ctot,
 int tpfnet_up_back(const void* dy, int N, int H, int W, int Ctot, int cofs, int C, void* dx, void* stream)
 {
     if (H % 2 == 0 && W % 2 == 0 && pieces(C | Ctot | cofs, dy, dx)) {
-        k_up_back8<<<grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream>>>(
+        launch_pdl(k_up_back8, grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream, 
             (const bf16*)dy, N * (H / 2), W, Ctot, cofs, C / 8, nullptr, (bf16*)dx);
         return status(cudaGetLastError());
     }
-    k_up_back<<<grid_of((long long)N * H * W * C / 4), 256, 0, (cudaStream_t)stream>>>((const bf16*)dy, N, H, W, Ctot, cofs,
+    launch_pdl(k_up_back, grid_of((long long)N * H * W * C / 4), 256, 0, (cudaStream_t)stream, (const bf16*)dy, N, H, W, Ctot, cofs,
                                                                                        C, (bf16*)dx);
     return status(cudaGetLastError());
 }
@@ -1919,7 +1981,7 @@ int tpfnet_pool_from(const void* x, int N, int H, int W, int C, int ldx, void* y
 {
     if (!x || !y || N < 1 || H < 2 || W < 2 || H % 2 || W % 2 || C < 8 || ldx < C || !pieces(C | ldx, x, y))
         return TPF_ERR_INVALID_ARG;
-    k_pool8<<<grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, N * (H / 2), W, C / 8,
+    launch_pdl(k_pool8, grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream, (const bf16*)x, N * (H / 2), W, C / 8,
                                                                                      ldx, (bf16*)y);
     return status(cudaGetLastError());
 }
@@ -1930,7 +1992,7 @@ int tpfnet_pool_back_skip(const void* dy, int N, int H, int W, int C, const void
     if (!dy || !skip || !mask || !dx || N < 1 || H < 2 || W < 2 || H % 2 || W % 2 || C < 8 || lds < C || ldm < C ||
         !pieces(C | lds | ldm, dy, skip, mask, dx))
         return TPF_ERR_INVALID_ARG;
-    k_pool_back8<<<grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream>>>(
+    launch_pdl(k_pool_back8, grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream, 
         (const bf16*)dy, N * (H / 2), W, C / 8, (const bf16*)skip, lds, (const bf16*)mask, ldm, (bf16*)dx);
     return status(cudaGetLastError());
 }
@@ -1941,7 +2003,7 @@ int tpfnet_up_back_masked(const void* dy, int N, int H, int W, int Ctot, int cof
     if (!dy || !mask || !dx || N < 1 || H < 2 || W < 2 || H % 2 || W % 2 || C < 8 || cofs < 0 || cofs + C > Ctot ||
         !pieces(C | Ctot | cofs, dy, mask, dx))
         return TPF_ERR_INVALID_ARG;
-    k_up_back8<<<grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream>>>(
+    launch_pdl(k_up_back8, grid_rows(N * (H / 2), W / 2 * (C / 8)), 256, 0, (cudaStream_t)stream, 
         (const bf16*)dy, N * (H / 2), W, Ctot, cofs, C / 8, (const bf16*)mask, (bf16*)dx);
     return status(cudaGetLastError());
 }
@@ -1950,11 +2012,11 @@ int tpfnet_channels(const void* src, int Sc, int sofs, long long pixels, int C, 
                     int accumulate, void* stream)
 {
     if (pieces(C | Sc | sofs | Dc | dofs, src, dst)) {
-        k_channels8<<<grid_of(pixels * (C / 8)), 256, 0, (cudaStream_t)stream>>>((const bf16*)src, Sc, sofs, pixels, C / 8,
+        launch_pdl(k_channels8, grid_of(pixels * (C / 8)), 256, 0, (cudaStream_t)stream, (const bf16*)src, Sc, sofs, pixels, C / 8,
                                                                                (bf16*)dst, Dc, dofs, accumulate);
         return status(cudaGetLastError());
     }
-    k_channels<<<grid_of(pixels * C), 256, 0, (cudaStream_t)stream>>>((const bf16*)src, Sc, sofs, pixels, C, (bf16*)dst, Dc,
+    launch_pdl(k_channels, grid_of(pixels * C), 256, 0, (cudaStream_t)stream, (const bf16*)src, Sc, sofs, pixels, C, (bf16*)dst, Dc,
                                                                      dofs, accumulate);
     return status(cudaGetLastError());
 }
@@ -1966,7 +2028,7 @@ int tpfnet_head(const void* x, long long pixels, int C, const float* Wt, const f
     const int smem = (C + 256) * Cout * (int)sizeof(float);
     if (pixels > 0 && Cout >= 1 && Cout <= 8 && smem <= 48 * 1024 && pieces(C, x)) {
         cudaStream_t s = (cudaStream_t)stream;
-        auto run = [&](auto kern) { kern<<<blocks, 256, smem, s>>>((const bf16*)x, pixels, C, Wt, b, out); };
+        auto run = [&](auto kern) { launch_pdl(kern, blocks, 256, smem, s, (const bf16*)x, pixels, C, Wt, b, out); };
         switch (Cout) {
         case 1: run(k_head8<1>); break;
         case 2: run(k_head8<2>); break;
@@ -1979,7 +2041,7 @@ int tpfnet_head(const void* x, long long pixels, int C, const float* Wt, const f
         }
         return status(cudaGetLastError());
     }
-    k_head<<<grid_of(pixels * Cout), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, pixels, C, Wt, b, Cout, out);
+    launch_pdl(k_head, grid_of(pixels * Cout), 256, 0, (cudaStream_t)stream, (const bf16*)x, pixels, C, Wt, b, Cout, out);
     return status(cudaGetLastError());
 }
 
@@ -1994,7 +2056,7 @@ static int head_back_any(const void* x, const float* dout, long long pixels, int
         const int blocks = (int)((pixels + per - 1) / per < 152 * 2 ? (pixels + per - 1) / per : 152 * 2);
         cudaStream_t s = (cudaStream_t)stream;
         auto run = [&](auto kern) {
-            kern<<<blocks, 256, smem, s>>>((const bf16*)x, dout, pixels, C, Wt, (bf16*)dx, dW, db, relu);
+            launch_pdl(kern, blocks, 256, smem, s, (const bf16*)x, dout, pixels, C, Wt, (bf16*)dx, dW, db, relu);
         };
         switch (Cout) {
         case 1: run(k_head_back8<1>); break;
@@ -2008,7 +2070,7 @@ static int head_back_any(const void* x, const float* dout, long long pixels, int
         }
         return status(cudaGetLastError());
     }
-    k_head_back<<<grid_of(pixels) < 304 ? grid_of(pixels) : 304, 256, smem, (cudaStream_t)stream>>>(
+    launch_pdl(k_head_back, grid_of(pixels) < 304 ? grid_of(pixels) : 304, 256, smem, (cudaStream_t)stream, 
         (const bf16*)x, dout, pixels, C, Wt, Cout, (bf16*)dx, dW, db);
     const int rc = status(cudaGetLastError());
     return rc || !relu ? rc : tpfnet_relu_mask(dx, x, pixels * C, stream);
@@ -2026,10 +2088,47 @@ int tpfnet_head_back_masked(const void* x, const float* dout, long long pixels, 
     return head_back_any(x, dout, pixels, C, Wt, Cout, dx, dW, db, 1, stream);
 }
 
+int tpfnet_unet_forward(const tpfnet_unet* u, const void* x, int N, int H, int W, float* out, void* stream)
+{
+    if (!u || !x || !out || N < 1 || H < 8 || W < 8 || H % 8 || W % 8) return TPF_ERR_INVALID_ARG;
+    const int* c = u->ch;
+    int rc = TPF_OK, k = 0;  // k: the 3x3 layer that is next
+    auto conv = [&](const void* in, int lvl, int cin, int cout, void* y, int ldy) {
+        if (rc == TPF_OK)
+            rc = tpfnet_conv3x3_into(in, N, H >> lvl, W >> lvl, cin, u->weight[k], u->bias[k], cout, 1, y, ldy, stream);
+        ++k;
+    };
+    // encoder: each level's output goes into its half of the concatenation (the bottleneck's
+    // into a tensor of its own)
+    const void* in = x;
+    int cin = u->cin;
+    for (int l = 0; l < 4; ++l) {
+        const int ld = l < 3 ? c[l + 1] + c[l] : c[3];
+        bf16* y = l < 3 ? (bf16*)u->cat[l] + c[l + 1] : (bf16*)u->deep;
+        conv(in, l, cin, c[l], u->enc[l], c[l]);
+        conv(u->enc[l], l, c[l], c[l], y, ld);
+        if (l == 3) break;
+        if (rc == TPF_OK) rc = tpfnet_pool_from(y, N, H >> l, W >> l, c[l], ld, u->pool[l], stream);
+        in = u->pool[l];
+        cin = c[l];
+    }
+    // decoder
+    const void* up = u->deep;
+    for (int l = 2; l >= 0; --l) {
+        const int ct = c[l + 1] + c[l];
+        if (rc == TPF_OK) rc = tpfnet_up_into(up, N, H >> l, W >> l, c[l + 1], u->cat[l], ct, 0, stream);
+        conv(u->cat[l], l, ct, c[l], u->dec_a[l], c[l]);
+        conv(u->dec_a[l], l, c[l], c[l], u->dec[l], c[l]);
+        up = u->dec[l];
+    }
+    if (rc == TPF_OK) rc = tpfnet_head(u->dec[0], (long long)N * H * W, c[0], u->head_w, u->head_b, u->cout, out, stream);
+    return rc;
+}
+
 int tpfnet_mse(const float* pred, const float* target, const float* wch, long long count, int C, float* grad,
                double* loss, void* stream)
 {
-    k_mse<<<grid_of(count) < 304 ? grid_of(count) : 304, 256, 0, (cudaStream_t)stream>>>(pred, target, wch, count, C, grad,
+    launch_pdl(k_mse, grid_of(count) < 304 ? grid_of(count) : 304, 256, 0, (cudaStream_t)stream, pred, target, wch, count, C, grad,
                                                                                           loss);
     return status(cudaGetLastError());
 }
@@ -2038,7 +2137,7 @@ int tpfnet_adam(float* p, const float* g, float* m, float* v, long long count, f
                 int step, void* pb, void* stream)
 {
     const float c1 = 1.f / (1.f - powf(b1, (float)step)), c2 = 1.f / (1.f - powf(b2, (float)step));
-    k_adam<<<grid_of(count), 256, 0, (cudaStream_t)stream>>>(p, g, m, v, count, lr, b1, b2, eps, c1, c2, (bf16*)pb);
+    launch_pdl(k_adam, grid_of(count), 256, 0, (cudaStream_t)stream, p, g, m, v, count, lr, b1, b2, eps, c1, c2, (bf16*)pb);
     return status(cudaGetLastError());
 }
 
@@ -2057,7 +2156,7 @@ int tpfnet_pack(const float* src, const float* base, long long plane, int C, lon
 {
     Affine a;
     if (!src || !dst || Cd < C || plane < pixels || affine_of(C, scale, shift, &a)) return TPF_ERR_INVALID_ARG;
-    k_pack<<<grid_of(pixels * C), 256, 0, (cudaStream_t)stream>>>(src, base, plane, C, pixels, a, dst, Cd,
+    launch_pdl(k_pack, grid_of(pixels * C), 256, 0, (cudaStream_t)stream, src, base, plane, C, pixels, a, dst, Cd,
                                                                  dst_bf16 ? 1 : 0);
     return status(cudaGetLastError());
 }
@@ -2067,13 +2166,13 @@ int tpfnet_unpack(const float* src, long long pixels, int C, const float* scale,
 {
     Affine a;
     if (!src || !dst || plane < pixels || affine_of(C, scale, shift, &a)) return TPF_ERR_INVALID_ARG;
-    k_unpack<<<grid_of(pixels * C), 256, 0, (cudaStream_t)stream>>>(src, pixels, C, a, base, dst, plane);
+    launch_pdl(k_unpack, grid_of(pixels * C), 256, 0, (cudaStream_t)stream, src, pixels, C, a, base, dst, plane);
     return status(cudaGetLastError());
 }
 
 int tpfnet_to_bf16(const float* x, long long count, void* y, void* stream)
 {
-    k_to_bf16<<<grid_of(count), 256, 0, (cudaStream_t)stream>>>(x, count, (bf16*)y);
+    launch_pdl(k_to_bf16, grid_of(count), 256, 0, (cudaStream_t)stream, x, count, (bf16*)y);
     return status(cudaGetLastError());
 }
 

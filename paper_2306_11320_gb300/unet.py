@@ -29,6 +29,7 @@ SIGNATURES = {
     "tpfnet_pool_back_skip": [_vp, _ip, _ip, _ip, _ip, _vp, _ip, _vp, _ip, _vp, _vp],
     "tpfnet_up_back_masked": [_vp, _ip, _ip, _ip, _ip, _ip, _ip, _vp, _vp, _vp],
     "tpfnet_head_back_masked": [_vp, _vp, _ll, _ip, _vp, _ip, _vp, _vp, _vp, _vp],
+    "tpfnet_unet_forward": [_vp, _vp, _ip, _ip, _ip, _vp, _vp],
     "tpfnet_conv3x3_tcgen05": [_ip, _ip, _ip, _ip, _ip],
     "tpfnet_conv3x3_wgrad_tcgen05": [_ip, _ip, _ip, _ip, _ip],
     "tpfnet_status": [],
@@ -48,6 +49,14 @@ SIGNATURES = {
     "tpfnet_pack": [_vp, _vp, _ll, _ip, _ll, _vp, _vp, _vp, _ip, _ip, _vp],
     "tpfnet_unpack": [_vp, _ll, _ip, _vp, _vp, _vp, _vp, _ll, _vp],
 }
+
+
+class _Net(C.Structure):
+    """tpfnet_unet"""
+    _fields_ = [("cin", _ip), ("cout", _ip), ("ch", _ip * 4), ("weight", _vp * 14), ("bias", _vp * 14),
+                ("head_w", _vp), ("head_b", _vp), ("enc", _vp * 4), ("pool", _vp * 3), ("cat", _vp * 3),
+                ("deep", _vp), ("dec_a", _vp * 3), ("dec", _vp * 3)]
+
 
 PAD = 32  # channel granularity of the convolution kernels
 
@@ -210,11 +219,6 @@ class UNet:
         if rc != 0:
             raise RuntimeError("tpfnet kernel %s failed (%d)" % (what, rc))
 
-    def _conv(self, name, x, N, H, W, cin, cout, y, relu=1):
-        """y: (N, H, W, cout), possibly a channel range of a wider tensor."""
-        self._chk(self.lib.tpfnet_conv3x3_into(_p(x), N, H, W, cin, _p(self.Pb[name + ".W"]), _p(self.P[name + ".b"]),
-                                               cout, relu, _p(y), y.stride(2), self._s()), name)
-
     def _s(self):
         return C.c_void_p(self.stream.cuda_stream)
 
@@ -224,32 +228,19 @@ class UNet:
         N, H, W, _ = x.shape
         self._buffers(N, H, W)
         self.x = x
-        B, L = self.B, self.lib
-        c0, c1, c2, c3 = self.ch
-        s = self._s()
-        dims = [(H, W), (H // 2, W // 2), (H // 4, W // 4), (H // 8, W // 8)]
-        # encoder
-        self._conv("e0a", x, N, H, W, self.cinp, c0, B["e0a"])
-        self._conv("e0b", B["e0a"], N, H, W, c0, c0, B["e0"])
-        prev, pc = B["e0"], c0
-        for lvl, (nm, c) in enumerate((("e1", c1), ("e2", c2), ("b", c3)), start=1):
-            h, w = dims[lvl]
-            self._chk(L.tpfnet_pool_from(_p(prev), N, 2 * h, 2 * w, pc, prev.stride(2), _p(B["pool%d" % lvl]), s), "pool")
-            ka, kb = ("b_a", "b_b") if nm == "b" else (nm + "a", nm + "b")
-            self._conv(ka, B["pool%d" % lvl], N, h, w, pc, c, B[nm + "a"])
-            self._conv(kb, B[nm + "a"], N, h, w, c, c, B[nm])
-            prev, pc = B[nm], c
-        # decoder: the skip part of each concatenation is there already
-        for lvl, c in ((2, c2), (1, c1), (0, c0)):
-            h, w = dims[lvl]
-            cat = B["cat%d" % lvl]
-            ctot = pc + c
-            self._chk(L.tpfnet_up_into(_p(prev), N, h, w, pc, _p(cat), ctot, 0, s), "up")
-            self._conv("d%da" % lvl, cat, N, h, w, ctot, c, B["d%da" % lvl])
-            self._conv("d%db" % lvl, B["d%da" % lvl], N, h, w, c, c, B["d%d" % lvl])
-            prev, pc = B["d%d" % lvl], c
-        self._chk(L.tpfnet_head(_p(prev), N * H * W, c0, _p(self.P["head.W"]), _p(self.P["head.b"]), self.cout,
-                                _p(self.out), s), "head")
+        B, u = self.B, _Net()
+        u.cin, u.cout, u.ch = self.cinp, self.cout, self.ch
+        names = [n for n, _, _, taps in self.specs if taps == 9]
+        u.weight = tuple(self.Pb[n + ".W"].data_ptr() for n in names)
+        u.bias = tuple(self.P[n + ".b"].data_ptr() for n in names)
+        u.head_w, u.head_b = self.P["head.W"].data_ptr(), self.P["head.b"].data_ptr()
+        u.enc = tuple(B[k].data_ptr() for k in ("e0a", "e1a", "e2a", "ba"))
+        u.pool = tuple(B["pool%d" % k].data_ptr() for k in (1, 2, 3))
+        u.cat = tuple(B["cat%d" % k].data_ptr() for k in (0, 1, 2))
+        u.deep = B["b"].data_ptr()
+        u.dec_a = tuple(B["d%da" % k].data_ptr() for k in (0, 1, 2))
+        u.dec = tuple(B["d%d" % k].data_ptr() for k in (0, 1, 2))
+        self._chk(self.lib.tpfnet_unet_forward(C.addressof(u), _p(x), N, H, W, _p(self.out), self._s()), "forward")
         return self.out
 
     # --------------------------------------------------------- backward
