@@ -40,7 +40,7 @@ constexpr int kVarBY[kNumVariants] = {4, 8, 16, 4, kStepBY};
 // resident threads per SM the batch kernel is built for: the general tile path is
 // latency-bound.  FP32 32 x 4 tiles on the 256-lattice ensemble: 0.427 ms per step at 768 (80
 // registers, with spills), 0.403 at 640 (five CTAs, 102 registers), 0.417 at 896, 0.444 at
-// 1,024; FP16 is fastest at 512 (128 registers)
+// 1,024; FP16 is fastest at 512 (128 registers).  (0.386 at 640 since, see step_tile_general)
 template <class S>
 constexpr int kBatchThreadsPerSM = kRef<S> ? 512 : 640;
 // The instance descriptor of a work item is copied word by word by warp 0 (32-bit words;
@@ -91,7 +91,7 @@ k_step_batch(const InstDesc* __restrict__ inst, const int2* __restrict__ work, i
         int x0, y0, tw, th;
         tile_whole(d.P.nx, BX, item.y & 0xffff, x0, tw);
         tile_whole(d.P.ny, BY, item.y >> 16, y0, th);
-        step_tile_general<BX, BY, S>(d.P, A, B, d.phiu, d.ref[parity], d.ref[parity ^ 1], sm, x0, y0, tw, th);
+        step_tile_general<BX, BY, S, true>(d.P, A, B, d.phiu, d.ref[parity], d.ref[parity ^ 1], sm, x0, y0, tw, th);
         // step_tile_general ends with a barrier: buffer b ^ 1 is free (its tile ended a
         // barrier ago), and after this one the next descriptor is visible
         if (wn < nwork && threadIdx.x < 32) store(b ^ 1);
@@ -189,7 +189,7 @@ k_step_batch_tma(const BatchTmaInst* __restrict__ inst, const int4* __restrict__
         fence_proxy_async();
         mbar_expect_tx_only(&bar[s], (uint32_t)sizeof(BatchTileDesc));
         bulk_load(dsm + BL::OFF_D + k % 3 * BL::DESC, &I.d, (uint32_t)sizeof(BatchTileDesc), &bar[s]);
-        tma_issue_tile<BX, BY, S>(M, dsm + s * L::STAGE, &bar[s], x0, y0);
+        tma_issue_tile<BX, BY, S>(M, dsm + s * L::STAGE, &bar[s], x0, y0, item.z, I.d.P.nx);
     };
 
     // Where the copies are issued: as in k_step_tma, the tile after next goes into the current
@@ -228,16 +228,15 @@ k_step_batch_tma(const BatchTmaInst* __restrict__ inst, const int4* __restrict__
         auto no_refill = [&]() {};
         // the buffers are read only after the block's vote; which body runs, its extent and
         // whether the seam patch runs come from the work item, the same on every thread
-        const E* A = (const E*)D.pop[parity];
         E* B = (E*)D.pop[parity ^ 1];
         RefT* refB = D.ref[parity ^ 1];
         if (cur.w & 1) {
-            if (tma_tile<BX, BY, S, true, false>(P, A, B, D.phiu, refB, st, sm, x0, y0, cur.w >> 8 & 0xff, cur.w >> 16,
+            if (tma_tile<BX, BY, S, true, true, false>(P, B, D.phiu, refB, st, sm, x0, y0, cur.w >> 8 & 0xff, cur.w >> 16,
                                                  cur.z, ok, on_abort, no_refill))
                 return;
             __syncthreads();  // every warp is done with stage s
             refill();
-        } else if (tma_tile<BX, BY, S, false, true>(P, A, B, D.phiu, refB, st, sm, x0, y0, BX, BY, 0, ok, on_abort,
+        } else if (tma_tile<BX, BY, S, false, false, true>(P, B, D.phiu, refB, st, sm, x0, y0, BX, BY, 0, ok, on_abort,
                                                     refill)) {
             return;
         }
@@ -255,7 +254,7 @@ k_step_batch_tma(const BatchTmaInst* __restrict__ inst, const int4* __restrict__
         int x0, y0, tw, th;
         tile_whole(P.nx, BX, item.y & 0xffff, x0, tw);
         tile_whole(P.ny, BY, item.y >> 16, y0, th);
-        step_tile_general<BX, BY, S>(P, (const E*)gdesc.pop[parity], (E*)gdesc.pop[parity ^ 1], gdesc.phiu,
+        step_tile_general<BX, BY, S, true>(P, (const E*)gdesc.pop[parity], (E*)gdesc.pop[parity ^ 1], gdesc.phiu,
                                      gdesc.ref[parity], gdesc.ref[parity ^ 1],
                                      *reinterpret_cast<RingSmem<BX, BY>*>(dsm), x0, y0, tw, th);
         // step_tile_general ends with a barrier: gdesc is free again

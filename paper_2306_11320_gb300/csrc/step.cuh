@@ -217,13 +217,32 @@ __device__ __forceinline__ void node_records(const Macro& m, const float* f, con
     out(kRecH, ref_pack(m.T, jhx * kInvCs2, jhy * kInvCs2, r.h));
 }
 
+// Whether every link of node (x, y) leads to a node, and the periodic x wrap of its neighbours'
+// indices.  The nodes of a boundary tile that pass push like those of any other tile; with
+// rows as warps, the rest of a tile at a wall or at a seam does (wraps in y go the long way).
+struct Wrap {
+    int l = 0, r = 0;
+};
+__device__ __forceinline__ bool plain_node(const DevParams& P, int x, int y, Wrap& wr)
+{
+    if (P.bc_x == 0) {
+        wr.l = x == 0 ? P.nx : 0;
+        wr.r = x == P.nx - 1 ? -P.nx : 0;
+    } else if (x == 0 || x == P.nx - 1) {
+        return false;
+    }
+    return y > 0 && y < P.ny - 1;
+}
+
 // Collide the node's populations and push them to their destinations, with every
 // boundary rule; for FP16 also leave the node's reference records in refB (every
 // population this node writes is encoded against them).  hold(i, k) and irc(k) give
-// the pre-collision h_i and 1/(rho c_p) of the node in ring slot k.
+// the pre-collision h_i and 1/(rho c_p) of the node in ring slot k.  plain: every link of the
+// node leads to a node (plain_node); wr: what the wrap of a periodic x adds to the index of a
+// neighbour to the left and to the right.
 template <class S, int SX, class HOLD, class IRC>
 __device__ __forceinline__ void collide_push(const DevParams& P, typename S::elem* __restrict__ B,
-                                             RefT* __restrict__ refB, int x, int y, int kown, bool interior,
+                                             RefT* __restrict__ refB, int x, int y, int kown, bool plain, Wrap wr,
                                              const Macro& m, float* f, float* g, float* h, HOLD hold, IRC irc)
 {
     const long long pl = P.plane;
@@ -234,10 +253,10 @@ __device__ __forceinline__ void collide_push(const DevParams& P, typename S::ele
     auto put_f = [&](int i, int d, float v) { S::st_dev(B + i * pl, d, v, dev_pop(i, r.f, v), P.s_f); };
     auto put_g = [&](int i, int d, float v) { S::st_dev(B + (9 + i) * pl, d, v, dev_g(i, r.g, v), P.s_g); };
     auto put_h = [&](int i, int d, float v) { S::st_dev(B + (18 + i) * pl, d, v, dev_pop(i, r.h, v), P.s_h); };
-    if (interior) {
+    if (plain) {
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-            const int d = n + cy(i) * P.nx + cx(i);
+            const int d = n + cy(i) * P.nx + cx(i) + (cx(i) < 0 ? wr.l : cx(i) > 0 ? wr.r : 0);
             const int kd = kown + cy(i) * SX + cx(i);
             put_f(i, d, f[i]);
             put_g(i, d, g[i]);
@@ -291,7 +310,12 @@ __device__ __forceinline__ void collide_push(const DevParams& P, typename S::ele
 // One thread per ring node issues that node's loads together with its own node's, so the
 // tile waits on one round trip to memory whatever its extent; ghost ring nodes take
 // their mirror's values from shared memory once those are in.
-template <int BX, int BY, class S>
+//
+// NODES: each node of a boundary tile that can pushes like an interior one (256-lattice
+// ensemble, FP32 0.403 -> 0.386 ms per step, FP16 0.82 -> 0.67); without it a tile that touches
+// the boundary pushes by the rules as a whole, which is the better code inside the TMA kernel
+// (256 x 1024 FP16, a quarter of whose tiles come here: 22.4 us per step against 25.1).
+template <int BX, int BY, class S, bool NODES>
 __device__ __forceinline__ void step_tile_general(const DevParams& P, const typename S::elem* __restrict__ A,
                                                   typename S::elem* __restrict__ B, float* __restrict__ phiu,
                                                   const RefT* __restrict__ refA, RefT* __restrict__ refB,
@@ -304,7 +328,6 @@ __device__ __forceinline__ void step_tile_general(const DevParams& P, const type
     const long long pl = P.plane;
     const int n = y * P.nx + x;
     const int kown = (ty + 1) * SX + tx + 1;
-    const bool interior = x0 >= 1 && x0 + w <= P.nx - 1 && y0 >= 1 && y0 + h_ <= P.ny - 1;
 
     constexpr int kRing = 2 * (BX + BY) + 4;
     static_assert(kRing <= BX * BY, "one thread per ring node");
@@ -387,8 +410,11 @@ __device__ __forceinline__ void step_tile_general(const DevParams& P, const type
         const Macro m = node_macro(P, f, g, h, phin, Tn, phiu[n], phiu[pl + n]);
         phiu[n] = m.phi * m.ux;
         phiu[pl + n] = m.phi * m.uy;
+        Wrap wr;
+        const bool plain = NODES ? plain_node(P, x, y, wr)
+                                 : x0 >= 1 && x0 + w <= P.nx - 1 && y0 >= 1 && y0 + h_ <= P.ny - 1;
         collide_push<S, SX>(
-            P, B, refB, x, y, kown, interior, m, f, g, h, [&](int i, int k) { return sm.h[i][k]; },
+            P, B, refB, x, y, kown, plain, wr, m, f, g, h, [&](int i, int k) { return sm.h[i][k]; },
             [&](int k) { return sm.irc[k]; });
     }
     __syncthreads();  // the caller may reuse sm for the next tile
@@ -417,7 +443,7 @@ k_step_general(const DevParams P, const typename S::elem* __restrict__ A, typena
     int x0, y0, w, h;
     tile_whole(P.nx, BX, blockIdx.x, x0, w);
     tile_whole(P.ny, BY, blockIdx.y, y0, h);
-    step_tile_general<BX, BY, S>(P, A, B, phiu, refA, refB, sm, x0, y0, w, h);
+    step_tile_general<BX, BY, S, true>(P, A, B, phiu, refA, refB, sm, x0, y0, w, h);
 }
 
 // ------------------------------------------------------- many steps per launch
@@ -449,12 +475,12 @@ k_step_general(const DevParams P, const typename S::elem* __restrict__ A, typena
 // What a step costs (512 x 128, in cycles of a CTA): the words' way through L2 and the
 // slowest neighbour 3,700, the moments 900, the macroscopic state 1,000, collisions and
 // pushes 2,200; it is bound by this chain, not by bandwidth (about 5 MB of words per step).
-// Measured against one launch per step (us/step, same process): 128 x 32 5.4 -> 2.8, 512 x
-// 128 6.7 -> 3.7, 160 x 320 6.4 -> 3.6, 331 x 117 5.5 -> 3.5; FP16 7.8 -> 3.3, 10.3 -> 4.3,
-// 10.6 -> 4.3, 12.7 -> 4.4.  Tried: step counters per tile with release/acquire and the
+// Measured against one launch per step (us/step, same process): 128 x 32 5.4 -> 2.6, 512 x
+// 128 6.7 -> 3.6, 160 x 320 6.4 -> 3.5, 331 x 117 5.5 -> 3.4; FP16 7.8 -> 3.0, 10.3 -> 4.1,
+// 10.6 -> 4.2, 12.7 -> 4.1.  Tried: step counters per tile with release/acquire and the
 // populations in L2 (4.3 and 5.3 at 128 x 32 and 512 x 128); 32 x 4 tiles (3.8, 5.6: each
-// thread then reads twice the words); testing the kind of each link in turn instead of
-// masks (3.4, 4.1).
+// thread then reads twice the words); 16 x 8 tiles (2.5, 4.1) and 16 x 16 (2.9, 4.2); testing
+// the kind of each link in turn instead of masks (3.4, 4.1).
 //
 // The waits are bounded: a CTA that gives up raises err and returns, and so do the
 // others, which look at err now and then; with err up no later launch starts.
@@ -467,12 +493,16 @@ __device__ __forceinline__ uint4 ld_word(const uint4* p)
                  : "l"(p));
     return make_uint4((uint32_t)lo, (uint32_t)(lo >> 32), (uint32_t)hi, (uint32_t)(hi >> 32));
 }
-__device__ __forceinline__ void st_word(uint4* p, float f, float g, float h, uint32_t tag)
+// (predicated in the instruction: nine of them follow one another in every node's push, and a
+// branch around each costs more than the store)
+__device__ __forceinline__ void st_word(uint4* p, float f, float g, float h, uint32_t tag, bool on = true)
 {
     const unsigned long long lo = ((unsigned long long)__float_as_uint(g) << 32) | __float_as_uint(f);
     const unsigned long long hi = ((unsigned long long)tag << 32) | __float_as_uint(h);
-    asm volatile("{\n .reg .b128 t;\n mov.b128 t, {%1, %2};\n st.relaxed.gpu.global.b128 [%0], t;\n}\n" ::"l"(p),
-                 "l"(lo), "l"(hi));
+    asm volatile(
+        "{\n .reg .b128 t;\n .reg .pred q;\n setp.ne.b32 q, %3, 0;\n mov.b128 t, {%1, %2};\n"
+        " @q st.relaxed.gpu.global.b128 [%0], t;\n}\n" ::"l"(p),
+        "l"(lo), "l"(hi), "r"((uint32_t)on));
 }
 
 constexpr uint32_t kWordWaitLimit = 1u << 22;  // polls, about half a microsecond each
@@ -571,16 +601,16 @@ __device__ __forceinline__ void tile_push(const DevParams& P, const TileMasks& M
         for (int i = 0; i < 9; ++i) slot[i] = sm.slot[i][tid];
 #pragma unroll
         for (int i = 0; i < 9; ++i)
-            if (M.rim >> i & 1) st_word(out + (uint32_t)(i * (int)P.plane) + slot[i], f[i], g[i], h[i], tag);
+            st_word(out + (uint32_t)(i * (int)P.plane) + slot[i], f[i], g[i], h[i], tag, M.rim >> i & 1);
     }
+    // (without a test: what goes to a ring slot is replaced by the words of the next step before
+    // anything reads it, what goes to a ghost slot is never read)
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         const int kd = kown + cy(i) * SM::SX + cx(i);
-        if (M.inside >> i & 1) {
-            sm.f[i][kd] = f[i];
-            sm.g[i][kd] = g[i];
-            sm.h[i][kd] = h[i];
-        }
+        sm.f[i][kd] = f[i];
+        sm.g[i][kd] = g[i];
+        sm.h[i][kd] = h[i];
     }
 }
 
@@ -612,7 +642,6 @@ k_step_many(const DevParams P, const typename S::elem* A, typename S::elem* B, f
     const bool active = tx < w && ty < h_;
     const int n = y * P.nx + x;
     const int kown = (ty + 1) * SX + tx + 1;
-    const bool interior = x0 >= 1 && x0 + w <= P.nx - 1 && y0 >= 1 && y0 + h_ <= P.ny - 1;
     const int nring = 2 * (w + h_) + 4;
     // slot (rx, ry) of ring node r; true when it lies inside the lattice, at (wx, wy)
     auto ring_node = [&](int r, int& rx, int& ry, int& wx, int& wy) {
@@ -818,8 +847,10 @@ k_step_many(const DevParams P, const typename S::elem* A, typename S::elem* B, f
                 const uint32_t tag = base + (uint32_t)s + 1;
                 tile_push<S>(P, M, sm, words + (size_t)(tag & 1) * 9 * pl, tag, kown, m, f, g, h);
             } else {
+                Wrap wr;
+                const bool plain = plain_node(P, x, y, wr);
                 collide_push<S, SX>(
-                    P, B, refB, x, y, kown, interior, m, f, g, h, [&](int i, int k) { return sm.h[i][k]; },
+                    P, B, refB, x, y, kown, plain, wr, m, f, g, h, [&](int i, int k) { return sm.h[i][k]; },
                     [&](int k) { return sm.irc[k]; });
             }
         }
@@ -901,7 +932,10 @@ struct TmaLayout {
     static constexpr int U_BYTES = 2 * BY * BX * 4;
     static constexpr int R_BYTES = kRef<S> ? 3 * RH * RW * (int)sizeof(RefT) : 0;
     static constexpr int OFF_F = 0, OFF_H = rnd(F_BYTES), OFF_G = OFF_H + rnd(F_BYTES), OFF_U = OFF_G + rnd(G_BYTES),
-                         OFF_R = OFF_U + rnd(U_BYTES), STAGE = OFF_R + rnd(R_BYTES);
+                         OFF_R = OFF_U + rnd(U_BYTES), OFF_C = OFF_R + rnd(R_BYTES);
+    // the wrapped ring column of f and of h of a seam tile (FP32): boxes of CW columns
+    static constexpr int CW = 16 / (int)sizeof(E), C_BYTES = kRef<S> ? 0 : 9 * FH * CW * (int)sizeof(E);
+    static constexpr int OFF_CH = OFF_C + rnd(C_BYTES), STAGE = OFF_CH + rnd(C_BYTES);
     static constexpr uint32_t TX_BYTES = 2 * F_BYTES + G_BYTES + U_BYTES + R_BYTES;
 };
 
@@ -923,16 +957,26 @@ struct TmaMaps {
     CUtensorMap popF;  // populations, box FW x FH x 9 (used for f at z = 0 and h at z = 18)
     CUtensorMap popG;  // populations, box BX x BY x 9 (g at z = 9)
     CUtensorMap phiu;  // (phi u) planes, box BX x BY x 2
-    CUtensorMap ref;   // FP16 reference records (8-byte elements), box RW x RH x 3
+    CUtensorMap ref;   // FP16 reference records (8-byte elements), box RW x RH x 3; FP32: the
+                       // populations, box CW x FH x 9 (wrapped columns at a periodic x seam)
 };
 
-// The copies of one TMA tile into stage st, completing on bar (one elected thread).
+// The copies of one TMA tile into stage st, completing on bar (one elected thread).  seam: see
+// seam_side; nx is needed at a left seam only.
 template <int BX, int BY, class S>
-__device__ __forceinline__ void tma_issue_tile(const TmaMaps& M, unsigned char* st, uint64_t* bar, int x0, int y0)
+__device__ __forceinline__ void tma_issue_tile(const TmaMaps& M, unsigned char* st, uint64_t* bar, int x0, int y0,
+                                               int seam, int nx)
 {
     using L = TmaLayout<BX, BY, S>;
     fence_proxy_async();
-    mbar_expect_tx(bar, L::TX_BYTES);
+    mbar_expect_tx(bar, L::TX_BYTES + (!kRef<S> && seam ? 2 * L::C_BYTES : 0));
+    if constexpr (!kRef<S>) {
+        if (seam) {
+            const int cx0 = seam < 0 ? nx - L::CW : 0;
+            tma_load_3d(st + L::OFF_C, &M.ref, bar, cx0, y0 - 1, 0);
+            tma_load_3d(st + L::OFF_CH, &M.ref, bar, cx0, y0 - 1, 18);
+        }
+    }
     tma_load_3d(st + L::OFF_F, &M.popF, bar, x0 - L::XP, y0 - 1, 0);
     tma_load_3d(st + L::OFF_H, &M.popF, bar, x0 - L::XP, y0 - 1, 18);
     tma_load_3d(st + L::OFF_G, &M.popG, bar, x0, y0, 9);
@@ -949,27 +993,26 @@ struct PhiSmem {
     float irc[SN];
 };
 
-// Periodic x seam (FP32 storage): the wrapped ring column of f and h from global memory
-// A into the box, where the copies left zeros, before anything decodes it (rows beyond
-// a wall stay zero: nothing decodes them).  Out of line: it runs for seam tiles only,
-// which wait one memory round trip here, and the stages keep their size.  Ends with a
-// block barrier.
+// Periodic x seam (FP32 storage): the wrapped ring column of f and h into the box, where the
+// copies left zeros, from the columns staged beside it, before anything decodes it (rows beyond
+// a wall are zero on both sides).  Fetching the columns here, out of global memory, cost every
+// seam tile a memory round trip: 13.6 us per step on 256 x 1024, a quarter of whose tiles are
+// seam tiles.  Ends with a block barrier.
 template <int BX, int BY, class S>
-__device__ __noinline__ void seam_patch(unsigned char* st, int seam, const typename S::elem* __restrict__ A, int nx,
-                                        int ny, long long pl, int y0, int w)
+__device__ __forceinline__ void seam_patch(unsigned char* st, int seam, int w)
 {
     static_assert(!kRef<S>, "FP16 tiles are not staged across a seam");
     using L = TmaLayout<BX, BY, S>;
     using E = typename S::elem;
-    E* bF = (E*)(st + L::OFF_F);
-    E* bH = (E*)(st + L::OFF_H);
-    const int fc = seam < 0 ? L::XP - 1 : L::XP + w, gx = seam < 0 ? nx - 1 : 0;
-    for (int k = threadIdx.x; k < 9 * L::FH; k += BX * BY) {
-        const int i = k / L::FH, y = y0 - 1 + k % L::FH;
-        if (y < 0 || y >= ny) continue;
-        const long long n = (long long)y * nx + gx;
-        bF[k * L::FW + fc] = A[i * pl + n];
-        bH[k * L::FW + fc] = A[(18 + i) * pl + n];
+    const int fc = seam < 0 ? L::XP - 1 : L::XP + w, cc = seam < 0 ? L::CW - 1 : 0;
+    const int k = threadIdx.x;
+    static_assert(2 * 9 * L::FH <= BX * BY, "one value per thread");
+    if (k < 2 * 9 * L::FH) {
+        const bool hh = k >= 9 * L::FH;
+        const int q = hh ? k - 9 * L::FH : k;
+        E* box = (E*)(st + (hh ? L::OFF_H : L::OFF_F));
+        const E* col = (const E*)(st + (hh ? L::OFF_CH : L::OFF_C));
+        box[q * L::FW + fc] = col[q * L::CW + cc];
     }
     __syncthreads();
 }
@@ -980,20 +1023,18 @@ __device__ __noinline__ void seam_patch(unsigned char* st, int seam, const typen
 // on_abort() runs on every thread and the tile returns true when any wait ran out),
 // after_ring() on every thread, then per node the macroscopic state, the collisions
 // and the push to B.  EDGE: the tile touches the lattice boundary (ghost ring nodes,
-// boundary records, boundary-aware push for every node), and may be ragged: it covers w x h_
-// nodes (w and h_ are BX and BY otherwise); seam (seam_side): the wrapped
-// column of a periodic x seam comes from A first.  EDGE, seam, w and h_ must be the
+// boundary records, boundary-aware push for every node); RAGGED: it covers w x h_ nodes (BX x BY
+// otherwise); seam (seam_side): the wrapped
+// column of a periodic x seam is put into the box first.  EDGE, seam, w and h_ must be the
 // same on every thread and must not come from a staged P (it is not to be trusted
 // before the vote).
-template <int BX, int BY, class S, bool EDGE, bool PRELOAD, class OnAbort, class AfterRing>
-__device__ __forceinline__ bool tma_tile(const DevParams& P, const typename S::elem* __restrict__ A,
-                                         typename S::elem* __restrict__ B, float* __restrict__ phiu,
-                                         RefT* __restrict__ refB,
-                                         unsigned char* st, PhiSmem<BX, BY>& sm, int x0, int y0, int w_, int h__,
+template <int BX, int BY, class S, bool EDGE, bool RAGGED, bool PRELOAD, class OnAbort, class AfterRing>
+__device__ __forceinline__ bool tma_tile(const DevParams& P, typename S::elem* __restrict__ B,
+                                         float* __restrict__ phiu, RefT* __restrict__ refB, unsigned char* st, PhiSmem<BX, BY>& sm, int x0, int y0, int w_, int h__,
                                          int seam, bool ok, OnAbort on_abort, AfterRing after_ring)
 {
     // (constants where the tile cannot be ragged)
-    const int w = EDGE ? w_ : BX, h_ = EDGE ? h__ : BY;
+    const int w = RAGGED ? w_ : BX, h_ = RAGGED ? h__ : BY;
     using L = TmaLayout<BX, BY, S>;
     using E = typename S::elem;
     constexpr int SX = BX + 2;
@@ -1020,14 +1061,7 @@ __device__ __forceinline__ bool tma_tile(const DevParams& P, const typename S::e
     };
     if constexpr (edge) {
         if constexpr (!kRef<S>) {
-            if (seam) {
-                // vote first: a batched tile's P and buffer pointers arrive with its copies
-                if (__syncthreads_or(!ok)) {
-                    on_abort();
-                    return true;
-                }
-                seam_patch<BX, BY, S>(st, seam, A, P.nx, P.ny, P.plane, y0, w);
-            }
+            if (seam) seam_patch<BX, BY, S>(st, seam, w);
         }
     }
 
@@ -1047,7 +1081,7 @@ __device__ __forceinline__ bool tma_tile(const DevParams& P, const typename S::e
     const int lx = tx + 1, ly = ty + 1, kown = ly * SX + lx;
     const int x = x0 + tx, y = y0 + ty;
     const int n = y * P.nx + x;
-    const bool active = !edge || (tx < w && ty < h_);
+    const bool active = !RAGGED || (tx < w && ty < h_);
     const bool bnode = edge && on_boundary(x, y);
     float f[9], g[9], h[9], phin[9], Tn[9];
     {
@@ -1172,7 +1206,7 @@ __device__ __forceinline__ bool tma_tile(const DevParams& P, const typename S::e
     phiu[pl + n] = m.phi * m.uy;
     if constexpr (kRef<S> && !kPre) rown_h = ref_unpack(sR[(kRecH * L::RH + ly + 1) * L::RW + lx + 3]);
     collide_push<S, SX>(
-        P, B, refB, x, y, kown, !edge, m, f, g, h,
+        P, B, refB, x, y, kown, !edge, Wrap{}, m, f, g, h,
         [&](int i, int kd) {
             if constexpr (kPre) {
                 return hold_r[i];  // interior tiles push only to kd = own + c_i
@@ -1198,7 +1232,9 @@ __device__ __forceinline__ bool tma_tile(const DevParams& P, const typename S::e
 template <class S>
 constexpr int kTmaMinBlocks = kRef<S> ? TPF_TMA_BLOCKS_F16 : TPF_TMA_BLOCKS_F32;
 
-template <int BX, int BY, class S>
+// RAGGED: the lattice has ragged TMA tiles (a body with constant extents is 1% faster on 256 x
+// 1024, a quarter of whose tiles are boundary tiles).
+template <int BX, int BY, class S, bool RAGGED>
 __global__ void __launch_bounds__(BX * BY, kTmaMinBlocks<S>)
 k_step_tma(const DevParams P, const __grid_constant__ TmaMaps maps, const typename S::elem* __restrict__ A,
            typename S::elem* __restrict__ B, float* __restrict__ phiu, const RefT* __restrict__ refA,
@@ -1240,7 +1276,7 @@ k_step_tma(const DevParams P, const __grid_constant__ TmaMaps maps, const typena
     auto issue = [&](int t, int k, int s) {
         int x0, y0;
         tile_of(t, k, x0, y0);
-        tma_issue_tile<BX, BY, S>(maps, dsm + s * L::STAGE, &bar[s], x0, y0);
+        tma_issue_tile<BX, BY, S>(maps, dsm + s * L::STAGE, &bar[s], x0, y0, seam_side<BX>(P, x0), P.nx);
     };
 
     int it = 0;
@@ -1276,13 +1312,13 @@ k_step_tma(const DevParams P, const __grid_constant__ TmaMaps maps, const typena
         const bool edge_tile = x0 <= 1 || x0 + BX >= P.nx - 1 || y0 <= 1 || y0 + BY >= P.ny - 1;
         const int seam = seam_side<BX>(P, x0);
         if (edge_tile) {
-            if (tma_tile<BX, BY, S, true, false>(P, A, B, phiu, refB, st, sm, x0, y0, min(BX, P.nx - x0),
-                                                 min(BY, P.ny - y0), seam, ok, on_abort, no_refill))
+            if (tma_tile<BX, BY, S, true, RAGGED, false>(P, B, phiu, refB, st, sm, x0, y0, min(BX, P.nx - x0),
+                                                         min(BY, P.ny - y0), seam, ok, on_abort, no_refill))
                 return;
             __syncthreads();  // every warp is done with stage s
             refill();
-        } else if (tma_tile<BX, BY, S, false, true>(P, A, B, phiu, refB, st, sm, x0, y0, BX, BY, 0, ok, on_abort,
-                                                    refill)) {
+        } else if (tma_tile<BX, BY, S, false, false, true>(P, B, phiu, refB, st, sm, x0, y0, BX, BY, 0, ok, on_abort,
+                                                           refill)) {
             return;
         }
     }
@@ -1310,8 +1346,8 @@ k_step_tma(const DevParams P, const __grid_constant__ TmaMaps maps, const typena
         int x0, y0, w, h;
         tile_whole(P.nx, BX, bx, x0, w);
         tile_whole(P.ny, BY, by, y0, h);
-        step_tile_general<BX, BY, S>(P, A, B, phiu, refA, refB, *reinterpret_cast<RingSmem<BX, BY>*>(dsm), x0, y0, w,
-                                     h);
+        step_tile_general<BX, BY, S, false>(P, A, B, phiu, refA, refB, *reinterpret_cast<RingSmem<BX, BY>*>(dsm), x0, y0,
+                                            w, h);
     }
 }
 

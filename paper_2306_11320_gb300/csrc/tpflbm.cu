@@ -791,6 +791,13 @@ bool make_map(CUtensorMap* m, CUtensorMapDataType dt, size_t esize, void* base, 
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// the TMA step kernel of a lattice: with or without ragged tiles
+template <class S>
+auto tma_kernel(tpflbm_t h)
+{
+    return h->nx % kBX || h->ny % kBY ? k_step_tma<kBX, kBY, S, true> : k_step_tma<kBX, kBY, S, false>;
+}
+
 template <class S>
 void setup_tma(tpflbm_t h)
 {
@@ -802,7 +809,7 @@ void setup_tma(tpflbm_t h)
     // TMA tiles: every tile, the ragged last one too, along a walled or inlet/outflow axis
     // (the copies fill the box beyond the lattice with zeros and the kernel applies the
     // boundary rules there) and, with FP32 storage, along a periodic x axis more than a tile
-    // long (a seam tile fetches the wrapped columns from the other edge itself); otherwise,
+    // long (a seam tile's wrapped columns are staged beside its boxes); otherwise,
     // along a periodic axis, the tiles whose (widened) halo lies inside the lattice
     int bx_lo = 0, by_lo = 0, bx_hi = (nx + kBX - 1) / kBX - 1, by_hi = (ny + kBY - 1) / kBY - 1;
     if (h->hp.bc_x == 0 && (kRef<S> || nx <= kBX)) {
@@ -827,7 +834,7 @@ void setup_tma(tpflbm_t h)
                   make_map(&M.popG, dt, e, h->pop[c], nx, ny, 27, pl, kBX, kBY, 9) &&
                   make_map(&M.phiu, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->phiu, nx, ny, 2, pl, kBX, kBY, 2);
         if (kRef<S>) ok = ok && make_map(&M.ref, CU_TENSOR_MAP_DATA_TYPE_UINT64, 8, h->ref[c], nx, ny, 3, pl, L::RW, L::RH, 3);
-        else M.ref = M.phiu;
+        else ok = ok && make_map(&M.ref, dt, e, h->pop[c], nx, ny, 27, pl, L::CW, L::FH, 9);
         if (!ok) return;
     }
     // Tile list: first the rectangle's rows and columns that touch the lattice boundary
@@ -858,13 +865,13 @@ void setup_tma(tpflbm_t h)
         }
     }
     const int smem = 2 * L::STAGE;
-    if (cudaFuncSetAttribute(k_step_tma<kBX, kBY, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+    const auto fn = tma_kernel<S>(h);
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
         cudaGetLastError();
         return;
     }
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_tma<kBX, kBY, S>, kBX * kBY, smem) != cudaSuccess ||
-        per_sm < 1) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBX * kBY, smem) != cudaSuccess || per_sm < 1) {
         cudaGetLastError();
         return;
     }
@@ -936,7 +943,7 @@ void launch_step(tpflbm_t h)
     E* B = (E*)h->pop[c ^ 1];
     if (h->tma) {
         using L = TmaLayout<kBX, kBY, S>;
-        k_step_tma<kBX, kBY, S><<<h->grid_tma, kBX * kBY, 2 * L::STAGE, h->stream>>>(
+        tma_kernel<S>(h)<<<h->grid_tma, kBX * kBY, 2 * L::STAGE, h->stream>>>(
             P, h->maps[c], A, B, h->phiu, h->ref[c], h->ref[c ^ 1], h->tiles, h->bx0, h->by0, h->ntbx, h->ntby,
             h->err);
     } else {
