@@ -28,14 +28,15 @@ int tpfnet_conv3x3(const void *x, int N, int H, int W, int Cin, const void *wt, 
 
 /* Which kernel tpfnet_conv3x3 (and tpfnet_conv3x3_dgrad, with Cin and Cout swapped)
  * runs for a shape, given 16-byte aligned tensors: the width in output channels of the
- * tcgen05 kernel's tiles (32, 64, 128 or 256), or 0 for the mma.sync kernel.  The
- * tcgen05 kernel takes pixel blocks of 128 = BW x BH with BW = min(W, 128) dividing
- * both 128 and W and BH dividing H; it stages operands with TMA and accumulates in
- * tensor memory. */
+ * tcgen05 kernels' tiles (32, 64, 128 or 256), or 0 for the mma.sync kernel.  The
+ * tcgen05 kernels take pixel blocks of 128 (8 x 16, or BW x BH with BW = min(W, 128)
+ * dividing both 128 and W and BH dividing H) and, from 1,024 pixels up, images of any
+ * other extent; they stage operands with TMA and accumulate in tensor memory.  (From
+ * 768 input channels up an image of other extents takes the mma.sync kernel.) */
 int tpfnet_conv3x3_tcgen05(int N, int H, int W, int Cin, int Cout);
 
 /* 1 when tpfnet_conv3x3_wgrad runs a tcgen05 kernel for a shape (W a multiple of 64, or W of 8
- * and H of 16; 16-byte aligned tensors), 0 for the mma.sync kernel.  The tcgen05 weight gradient
+ * and H of 16, or at least 1,024 pixels; 16-byte aligned tensors), 0 for the mma.sync kernel.  The tcgen05 weight gradient
  * reduces over pixels with both operands staged MN-major by TMA (one pixel's channels
  * per 128-byte row) and adds each CTA's FP32 partial sums into dw with atomics. */
 int tpfnet_conv3x3_wgrad_tcgen05(int N, int H, int W, int Cin, int Cout);

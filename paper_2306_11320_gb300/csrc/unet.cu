@@ -386,7 +386,8 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUt
 // then a window into that box: 16 groups (image rows) of 8 rows (pixels), the groups one row
 // of the box apart, starting (dh + 1) box rows and dw + 1 pixels in.  The box starts on a
 // swizzle boundary and the swizzle follows the address bits, so a window may start at any of
-// its rows.  The weights of each (tap, channel chunk) come through a ring of stages; taps
+// its rows.  Images of other extents have blocks that reach past their edge: the box is zero
+// there and nothing is stored.  The weights of each (tap, channel chunk) come through a ring of stages; taps
 // outermost, as in k_conv3x3_tc, so that the FP32 sums are the same bit for bit.
 //
 // What this saves is the way from L2 to the SM, which bounded the per-tap form: 184 MB of
@@ -431,7 +432,7 @@ k_conv3x3_halo(const __grid_constant__ CUtensorMap mx, const __grid_constant__ C
     unsigned char* sA = tsm + ((1024 - (sa(tsm) & 1023)) & 1023);
     const int kc = Cin / KC, kBBytes = BN * KC * 2, kStage = st.T * st.CC * kBBytes;
     unsigned char* sB = sA + kc * kABytes;
-    const int bpr = W / (8 * MT), bpi = bpr * (H / 16);
+    const int bpr = (W + 8 * MT - 1) / (8 * MT), bpi = bpr * ((H + 15) / 16);
     const int n = blockIdx.x / bpi, rem = blockIdx.x % bpi;
     const int h0 = (rem / bpr) * 16, w0 = (rem % bpr) * 8 * MT;
     const int co0 = blockIdx.y * BN;
@@ -536,7 +537,9 @@ k_conv3x3_halo(const __grid_constant__ CUtensorMap mx, const __grid_constant__ C
     // epilogue: warps 4 q .. 4 q + 3 hold block q; thread (warp w, lane l) its pixel m = 32 (w % 4)
     // + l, at row m / 8 and column m % 8 of the block
     const int q = warp >> 2, m = (warp & 3) * 32 + lane;
-    const size_t px = ((size_t)n * H + h0 + m / 8) * W + w0 + 8 * q + m % 8;
+    const int hh = h0 + m / 8, ww = w0 + 8 * q + m % 8;
+    const bool inside = hh < H && ww < W;  // (not so for the last blocks of other extents)
+    const size_t px = inside ? ((size_t)n * H + hh) * W + ww : 0;
     bf16* out = y + px * ldy + co0;
     const bf16* mrow = mask ? mask + px * Cout + co0 : nullptr;
     mb_wait(&done, 0);
@@ -578,7 +581,7 @@ k_conv3x3_halo(const __grid_constant__ CUtensorMap mx, const __grid_constant__ C
                 const __nv_bfloat162 t2 = __floats2bfloat162_rn(v0, v1);
                 o[e] = *reinterpret_cast<const uint32_t*>(&t2);
             }
-            *reinterpret_cast<uint4*>(out + c + 8 * j) = make_uint4(o[0], o[1], o[2], o[3]);
+            if (inside) *reinterpret_cast<uint4*>(out + c + 8 * j) = make_uint4(o[0], o[1], o[2], o[3]);
         }
     }
     tc_fence_before();
@@ -941,7 +944,8 @@ __device__ __forceinline__ void relu_back8(Piece& d, const Piece& y)
 // boxes that exist, lanes hold sums that are not read), N = 3 CK, K = 16 pixels = two image
 // rows.  db is summed from the dz boxes by four more warps in the CTAs of dw = -1 and the
 // first input channels, each thread eight channels of every fourth pixel.  Partial sums of a
-// CTA go to dw in vector reductions.
+// CTA go to dw in vector reductions.  Blocks that reach past an image's edge add nothing: dz is
+// zero there.
 //
 // Weight and bias gradient, batch 4 (us, against one tap or column of taps per stage with its
 // own x box): 512 x 128 32 -> 32 62 -> 24, 96 -> 32 122 -> 44; 256 x 64 64 -> 64 29 -> 19, 192 ->
@@ -989,7 +993,7 @@ k_conv3x3_wgrad_halo(const __grid_constant__ CUtensorMap mdz, const __grid_const
     const int nb = co0 + 64 < Cout ? 2 : 1;  // dz boxes
     const int boxes = Cout > 64 ? 2 : 1;     // room for them
     const int kStage = boxes * kWhDz + kX;
-    const int bpr = W / 8, bpi = bpr * (H / 16), tiles = N * bpi;
+    const int bpr = (W + 7) / 8, bpi = bpr * ((H + 15) / 16), tiles = N * bpi;
     const int begin = split * tiles_per_cta, end = min(begin + tiles_per_cta, tiles), steps = max(end - begin, 0);
     const bool bias = db && g == 0 && blockIdx.y == 0;
 
@@ -1589,17 +1593,22 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
     return fn;
 }
 
-// Shapes the tcgen05 convolution takes: pixel blocks of BW x BH = 128 (BW = W up to
-// 128, dividing W; BH dividing H).  BN: the largest of 256, 128, 64, 32 that divides
-// Cout and still gives at least one CTA per SM (else 32).  0 when the shape is not
-// taken.
+// Images of fewer pixels whose blocks do not divide evenly stay on the mma.sync kernels.
+constexpr long long kRaggedPixels = 1024;
+
+// Shapes the tcgen05 convolutions take: images that divide into pixel blocks of BW x BH = 128
+// (BW = W up to 128, dividing W; BH dividing H; BW 0 where they do not), and any other of at
+// least kRaggedPixels pixels (halo form).  BN: the largest of 256, 128, 64, 32 that divides
+// Cout and still gives at least one CTA per SM (else 32).  0 when the shape is not taken.
 int tc_bn(int N, int H, int W, int Cout, int& BW, int& BH)
 {
     BW = W < 128 ? W : 128;
-    if (128 % BW != 0 || W % BW != 0) return 0;
-    BH = 128 / BW;
-    if (H % BH != 0) return 0;
-    const long long mtiles = (long long)N * (H / BH) * (W / BW);
+    BH = BW > 0 && 128 % BW == 0 ? 128 / BW : 0;
+    if (BH == 0 || W % BW != 0 || H % BH != 0) {
+        BW = BH = 0;
+        if ((long long)N * H * W < kRaggedPixels) return 0;
+    }
+    const long long mtiles = BW ? (long long)N * (H / BH) * (W / BW) : (long long)N * ((H + 15) / 16) * ((W + 7) / 8);
     for (int bn = 256; bn > 32; bn /= 2)
         if (Cout % bn == 0 && mtiles * (Cout / bn) >= 152) return bn;
     return 32;
@@ -1651,8 +1660,8 @@ bool launch_tc(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, cons
     return true;
 }
 
-// The halo form, for images that divide into blocks of 8 x 16 pixels and channel counts whose
-// boxes fit in shared memory; false (nothing launched) otherwise.
+// The halo form, for channel counts whose boxes fit in shared memory; false (nothing launched)
+// otherwise.
 template <int KC, int MT>
 bool launch_halo(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, const float* bias, int Cout, int relu,
                  bf16* y, int ldy, const bf16* mask, cudaStream_t s, int BN)
@@ -1664,7 +1673,7 @@ bool launch_halo(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, co
     // time, or one; where the boxes leave no room for that, the per-tap kernel is the better
     // one ((4, 32, 128, 384, 128): 22.9 us against 31.1, (4, 16, 64, 256, 256): 16.8 against
     // 17.7).  With at most one CTA per SM its whole shared memory, and parts of a tap if need be.
-    const long long ctas = (long long)N * (H / 16) * (W / (8 * MT)) * (Cout / BN);
+    const long long blocks = (long long)N * ((H + 15) / 16) * ((W + 8 * MT - 1) / (8 * MT)), ctas = blocks * (Cout / BN);
     const int limit = ctas > 152 ? 112 * 1024 : 226 * 1024;
     HaloStages st{0, 0, 0};
     auto take = [&](int T, int CC, int S) {
@@ -1690,7 +1699,7 @@ bool launch_halo(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, co
         cudaGetLastError();
         return false;
     }
-    dim3 grd(N * (H / 16) * (W / (8 * MT)), Cout / BN);
+    dim3 grd((unsigned)blocks, Cout / BN);
     launch_pdl(k_conv3x3_halo<KC, MT>, grd, 128 * MT, smem, s, mx, mw, H, W, Cin, Cout, BN, st, bias, relu, y, ldy, mask);
     return true;
 }
@@ -1701,12 +1710,14 @@ bool conv_tc(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, const 
     int BW = 0, BH = 0;
     const int bn = tc_bn(N, H, W, Cout, BW, BH);
     if (!bn || (((uintptr_t)x | (uintptr_t)wt | (uintptr_t)y | (uintptr_t)mask) & 15) || ldy % 8) return false;
-    if (H % 16 == 0 && W % 8 == 0) {
+    if ((H % 16 == 0 && W % 8 == 0) || !BW) {
         // two blocks per CTA where that still gives every SM a CTA (half the weight traffic)
-        const bool two = W % 16 == 0 && (long long)N * H * W / 256 * (Cout / bn) >= 152;
+        const long long pairs = (long long)N * ((H + 15) / 16) * ((W + 15) / 16);
+        const bool two = (W % 16 == 0 || !BW) && pairs * (Cout / bn) >= 152;
         const auto f = Cin % 64 == 0 ? (two ? launch_halo<64, 2> : launch_halo<64, 1>)
                                      : (two ? launch_halo<32, 2> : launch_halo<32, 1>);
         if (f(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, bn)) return true;
+        if (!BW) return false;
     }
     if (Cin % 64 == 0) {
         switch (bn) {
@@ -1724,8 +1735,7 @@ bool conv_tc(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, const 
     }
 }
 
-// The halo form of the weight gradient, for images that divide into blocks of 8 x 16 pixels;
-// false (nothing launched) otherwise.
+// The halo form of the weight gradient; false (nothing launched) when it cannot be.
 template <int CK>
 bool launch_wgrad_halo(const bf16* x, const bf16* dz, int N, int H, int W, int Cin, int Cout, float* dw, float* db,
                        cudaStream_t s)
@@ -1738,7 +1748,7 @@ bool launch_wgrad_halo(const bf16* x, const bf16* dz, int N, int H, int W, int C
         return false;
     }
     // split the blocks over about as many CTAs as run at once
-    const long long tiles = (long long)N * (H / 16) * (W / 8);
+    const long long tiles = (long long)N * ((H + 15) / 16) * ((W + 7) / 8);
     const int ctiles = (Cout + 127) / 128, itiles = Cin / CK;
     const long long base = 3LL * ctiles * itiles, target = smem <= 112 * 1024 ? 304 : 152;
     long long splits = target / base;
@@ -1751,13 +1761,19 @@ bool launch_wgrad_halo(const bf16* x, const bf16* dz, int N, int H, int W, int C
     return true;
 }
 
+// shapes the halo form takes: images that divide into its blocks, and any other large enough
+bool wgrad_blocks(int N, int H, int W)
+{
+    return (H % 16 == 0 && W % 8 == 0) || (W % kWgPix != 0 && (long long)N * H * W >= kRaggedPixels);
+}
+
 // The tcgen05 weight gradient for W a multiple of 64 and 16-byte aligned tensors;
 // false (nothing launched) otherwise.  Adds into dw (and db).
 bool wgrad_tc(const bf16* x, const bf16* dz, int N, int H, int W, int Cin, int Cout, float* dw, float* db,
               cudaStream_t s)
 {
     if (((uintptr_t)x | (uintptr_t)dz) & 15) return false;
-    if (H % 16 == 0 && W % 8 == 0 && (uintptr_t)dw % 16 == 0) {
+    if (wgrad_blocks(N, H, W) && (uintptr_t)dw % 16 == 0) {
         const auto f = Cin % 64 == 0 ? launch_wgrad_halo<64> : launch_wgrad_halo<32>;
         if (f(x, dz, N, H, W, Cin, Cout, dw, db, s)) return true;
     }
@@ -1872,7 +1888,7 @@ int tpfnet_conv3x3_tcgen05(int N, int H, int W, int Cin, int Cout)
 
 int tpfnet_conv3x3_wgrad_tcgen05(int N, int H, int W, int Cin, int Cout)
 {
-    const bool tiles = W % kWgPix == 0 || (H % 16 == 0 && W % 8 == 0);
+    const bool tiles = W % kWgPix == 0 || (H > 0 && W > 0 && wgrad_blocks(N, H, W));
     return N >= 1 && H >= 1 && W >= 1 && Cin % 32 == 0 && Cout % 32 == 0 && tiles && encode_fn() ? 1 : 0;
 }
 

@@ -142,7 +142,10 @@ def test_parameters_of_the_callers_own():
 # 384, 64) have too many channels for the boxes of two CTAs on an SM
 @pytest.mark.parametrize("N,H,W,Cin,Cout", [(1, 16, 8, 32, 32), (1, 16, 16, 64, 64), (2, 32, 24, 96, 96),
                                             (1, 48, 40, 64, 160), (3, 16, 32, 192, 64), (1, 16, 16, 384, 64),
-                                            (4, 16, 64, 256, 256), (2, 128, 256, 32, 128)])
+                                            (4, 16, 64, 256, 256), (2, 128, 256, 32, 128),
+                                            # blocks that reach past the image
+                                            (1, 33, 32, 32, 64), (2, 31, 17, 64, 96), (1, 107, 33, 96, 32),
+                                            (3, 18, 20, 192, 128)])
 def test_block_convolutions(N, H, W, Cin, Cout):
     """Forward, data and weight gradients against float64.  Bounds, element by element: a
     float32 sum of n terms is within n 2^-24 sum |terms|, a stored bf16 within 2^-8 of its
