@@ -42,6 +42,7 @@ struct tpflbm {
     // TMA step kernel
     bool tma = false;
     tpf::TmaMaps maps[2]{};             // maps[c]: reading pop[c]
+    tpf::SeamMaps smaps[2]{};
     int bx0 = 0, by0 = 0, ntbx = 0, ntby = 0, grid_tma = 0;
     int2* tiles = nullptr;              // (x0, y0) of the TMA tiles in the order the kernel walks them
     // many-step kernel (many_fn is null where the lattice does not take it): its tiles, the

@@ -95,18 +95,19 @@ __device__ __forceinline__ int ref_source(const DevParams& P, int x, int y, int 
 }
 
 // ref_source for a node of a TMA tile: the writer's slot in the tile's record box
-// (origin x0 - 4, y0 - 2, RW x RH).  Records exist with FP16 storage only, whose TMA
-// tiles never need a periodic wrap.  Every writer lies in the box; the clamps only keep
-// the slot inside it when P itself is not to be trusted (a batched tile whose copies,
-// parameters included, timed out).
+// (origin x0 - 4, y0 - 2, RW x RH; columns beyond a periodic x seam hold the wrapped nodes'
+// records).  Every writer lies in the box; the clamps only keep the slot inside it when P
+// itself is not to be trusted (a batched tile whose copies, parameters included, timed out).
+template <bool SEAM>
 __device__ __forceinline__ int ref_slot_box(const DevParams& P, int x, int y, int i, bool g_lbe, int x0, int y0,
                                             int RW, int RH)
 {
     int sx = x - cx(i), sy = y - cy(i);
-    if (sy < 0 || sy >= P.ny || sx < 0 || (sx >= P.nx && g_lbe)) {
+    const bool open = !SEAM || P.bc_x != 0;  // x ends at an inlet and an outflow
+    if (sy < 0 || sy >= P.ny || (open && (sx < 0 || (sx >= P.nx && g_lbe)))) {
         sx = x;
         sy = y;
-    } else if (sx >= P.nx) {
+    } else if (open && sx >= P.nx) {
         sx = P.nx - 1;
     }
     const int c = min(max(sx - x0 + 4, 0), RW - 1), r = min(max(sy - y0 + 2, 0), RH - 1);
@@ -871,8 +872,7 @@ k_step_many(const DevParams P, const typename S::elem* A, typename S::elem* B, f
 // y0 + BY + 2 <= ny), which along a walled or inlet/outflow axis are all tiles, the ragged
 // last one too: there the box reaches past the lattice, the copy fills it with zeros, and
 // the tile takes its ghost ring nodes and its boundary nodes' FP16 records by the boundary
-// rules instead (with FP32 storage, along a periodic x axis of two tiles and more, too: see
-// seam_side).  For a TMA tile one elected thread issues 3D bulk
+// rules instead (along a periodic x axis of two tiles and more, too: see seam_side).  For a TMA tile one elected thread issues 3D bulk
 // tensor copies (cp.async.bulk.tensor) of the 9 f planes and the 9 h planes over the
 // tile plus a one-node ring (widened to XP columns each side for the 16-byte rule),
 // the 9 g planes and the 2 (phi u) planes over the tile, and for FP16 the 3 planes of
@@ -933,19 +933,18 @@ struct TmaLayout {
     static constexpr int R_BYTES = kRef<S> ? 3 * RH * RW * (int)sizeof(RefT) : 0;
     static constexpr int OFF_F = 0, OFF_H = rnd(F_BYTES), OFF_G = OFF_H + rnd(F_BYTES), OFF_U = OFF_G + rnd(G_BYTES),
                          OFF_R = OFF_U + rnd(U_BYTES), OFF_C = OFF_R + rnd(R_BYTES);
-    // the wrapped ring column of f and of h of a seam tile (FP32): boxes of CW columns
-    static constexpr int CW = 16 / (int)sizeof(E), C_BYTES = kRef<S> ? 0 : 9 * FH * CW * (int)sizeof(E);
-    static constexpr int OFF_CH = OFF_C + rnd(C_BYTES), STAGE = OFF_CH + rnd(C_BYTES);
+    // the wrapped ring column of f and of h of a seam tile, boxes of CW columns, and for FP16
+    // the two wrapped columns of the records
+    static constexpr int CW = 16 / (int)sizeof(E), C_BYTES = 9 * FH * CW * (int)sizeof(E);
+    static constexpr int CR_BYTES = kRef<S> ? 3 * RH * 2 * (int)sizeof(RefT) : 0;
+    static constexpr int OFF_CH = OFF_C + rnd(C_BYTES), OFF_CR = OFF_CH + rnd(C_BYTES), STAGE = OFF_CR + rnd(CR_BYTES);
+    static constexpr int stage(bool seam) { return seam ? STAGE : OFF_C; }  // bytes in use
     static constexpr uint32_t TX_BYTES = 2 * F_BYTES + G_BYTES + U_BYTES + R_BYTES;
 };
 
 // Which side of a periodic x seam a TMA tile sits on: -1 its left ring column wraps to
-// x = nx - 1, +1 its right one to x = 0, 0 neither.  Seam tiles are staged by TMA with
-// FP32 storage only, and only in lattices more than a tile wide (so no tile has both
-// sides); otherwise they take the general path and this is 0 for every TMA tile.  With
-// FP16 storage (records to patch as well) the seam code pushed the kernel to its
-// 128-register cap and slowed every tile (the 2048 x 512 channel, which has no seam,
-// by 3.5%).
+// x = nx - 1, +1 its right one to x = 0, 0 neither.  Seam tiles are staged by TMA in lattices
+// more than a tile wide (so no tile has both sides).
 template <int BX>
 __device__ __forceinline__ int seam_side(const DevParams& P, int x0)
 {
@@ -957,25 +956,28 @@ struct TmaMaps {
     CUtensorMap popF;  // populations, box FW x FH x 9 (used for f at z = 0 and h at z = 18)
     CUtensorMap popG;  // populations, box BX x BY x 9 (g at z = 9)
     CUtensorMap phiu;  // (phi u) planes, box BX x BY x 2
-    CUtensorMap ref;   // FP16 reference records (8-byte elements), box RW x RH x 3; FP32: the
-                       // populations, box CW x FH x 9 (wrapped columns at a periodic x seam)
+    CUtensorMap ref;   // FP16 reference records (8-byte elements), box RW x RH x 3
+};
+
+struct SeamMaps {     // the wrapped columns at a periodic x seam
+    CUtensorMap pop;  // populations, box CW x FH x 9
+    CUtensorMap ref;  // FP16 reference records, box 2 x RH x 3
 };
 
 // The copies of one TMA tile into stage st, completing on bar (one elected thread).  seam: see
 // seam_side; nx is needed at a left seam only.
 template <int BX, int BY, class S>
-__device__ __forceinline__ void tma_issue_tile(const TmaMaps& M, unsigned char* st, uint64_t* bar, int x0, int y0,
+__device__ __forceinline__ void tma_issue_tile(const TmaMaps& M, const SeamMaps& C, unsigned char* st, uint64_t* bar, int x0, int y0,
                                                int seam, int nx)
 {
     using L = TmaLayout<BX, BY, S>;
     fence_proxy_async();
-    mbar_expect_tx(bar, L::TX_BYTES + (!kRef<S> && seam ? 2 * L::C_BYTES : 0));
-    if constexpr (!kRef<S>) {
-        if (seam) {
-            const int cx0 = seam < 0 ? nx - L::CW : 0;
-            tma_load_3d(st + L::OFF_C, &M.ref, bar, cx0, y0 - 1, 0);
-            tma_load_3d(st + L::OFF_CH, &M.ref, bar, cx0, y0 - 1, 18);
-        }
+    mbar_expect_tx(bar, L::TX_BYTES + (seam ? 2 * L::C_BYTES + L::CR_BYTES : 0));
+    if (seam) {
+        const int cx0 = seam < 0 ? nx - L::CW : 0;
+        tma_load_3d(st + L::OFF_C, &C.pop, bar, cx0, y0 - 1, 0);
+        tma_load_3d(st + L::OFF_CH, &C.pop, bar, cx0, y0 - 1, 18);
+        if constexpr (kRef<S>) tma_load_3d(st + L::OFF_CR, &C.ref, bar, seam < 0 ? nx - 2 : 0, y0 - 2, 0);
     }
     tma_load_3d(st + L::OFF_F, &M.popF, bar, x0 - L::XP, y0 - 1, 0);
     tma_load_3d(st + L::OFF_H, &M.popF, bar, x0 - L::XP, y0 - 1, 18);
@@ -993,26 +995,34 @@ struct PhiSmem {
     float irc[SN];
 };
 
-// Periodic x seam (FP32 storage): the wrapped ring column of f and h into the box, where the
-// copies left zeros, from the columns staged beside it, before anything decodes it (rows beyond
-// a wall are zero on both sides).  Fetching the columns here, out of global memory, cost every
-// seam tile a memory round trip: 13.6 us per step on 256 x 1024, a quarter of whose tiles are
-// seam tiles.  Ends with a block barrier.
+// Periodic x seam: the wrapped ring column of f and h, and for FP16 the wrapped columns of the
+// records, into the boxes, where the copies left zeros, from the columns staged beside them,
+// before anything decodes them (rows beyond a wall are zero on both sides).  Fetching the columns
+// here, out of global memory, cost every seam tile a memory round trip (256 x 1024 FP32, a
+// quarter of whose tiles are seam tiles: 13.6 us per step against 13.1).  Ends with a block
+// barrier.
 template <int BX, int BY, class S>
 __device__ __forceinline__ void seam_patch(unsigned char* st, int seam, int w)
 {
-    static_assert(!kRef<S>, "FP16 tiles are not staged across a seam");
     using L = TmaLayout<BX, BY, S>;
     using E = typename S::elem;
-    const int fc = seam < 0 ? L::XP - 1 : L::XP + w, cc = seam < 0 ? L::CW - 1 : 0;
     const int k = threadIdx.x;
-    static_assert(2 * 9 * L::FH <= BX * BY, "one value per thread");
-    if (k < 2 * 9 * L::FH) {
-        const bool hh = k >= 9 * L::FH;
-        const int q = hh ? k - 9 * L::FH : k;
+    constexpr int kCol = 9 * L::FH, kRec = kRef<S> ? 3 * L::RH * 2 : 0;
+    static_assert(2 * kCol + kRec <= BX * BY, "one value per thread");
+    if (k < 2 * kCol) {
+        const int fc = seam < 0 ? L::XP - 1 : L::XP + w, cc = seam < 0 ? L::CW - 1 : 0;
+        const bool hh = k >= kCol;
+        const int q = hh ? k - kCol : k;
         E* box = (E*)(st + (hh ? L::OFF_H : L::OFF_F));
         const E* col = (const E*)(st + (hh ? L::OFF_CH : L::OFF_C));
         box[q * L::FW + fc] = col[q * L::CW + cc];
+    } else if (k < 2 * kCol + kRec) {
+        // record row q / 2 (of 3 RH), column q % 2 of the two beyond the seam: x = -2, -1 or
+        // x0 + w, x0 + w + 1, in a box that starts at x0 - 4
+        const int q = k - 2 * kCol, c0 = seam < 0 ? 2 : w + 4;
+        RefT* box = (RefT*)(st + L::OFF_R);
+        const RefT* col = (const RefT*)(st + L::OFF_CR);
+        box[(q >> 1) * L::RW + c0 + (q & 1)] = col[q];
     }
     __syncthreads();
 }
@@ -1024,11 +1034,11 @@ __device__ __forceinline__ void seam_patch(unsigned char* st, int seam, int w)
 // after_ring() on every thread, then per node the macroscopic state, the collisions
 // and the push to B.  EDGE: the tile touches the lattice boundary (ghost ring nodes,
 // boundary records, boundary-aware push for every node); RAGGED: it covers w x h_ nodes (BX x BY
-// otherwise); seam (seam_side): the wrapped
+// otherwise); seam (seam_side; SEAM: it may be set): the wrapped
 // column of a periodic x seam is put into the box first.  EDGE, seam, w and h_ must be the
 // same on every thread and must not come from a staged P (it is not to be trusted
 // before the vote).
-template <int BX, int BY, class S, bool EDGE, bool RAGGED, bool PRELOAD, class OnAbort, class AfterRing>
+template <int BX, int BY, class S, bool EDGE, bool RAGGED, bool SEAM, bool PRELOAD, class OnAbort, class AfterRing>
 __device__ __forceinline__ bool tma_tile(const DevParams& P, typename S::elem* __restrict__ B,
                                          float* __restrict__ phiu, RefT* __restrict__ refB, unsigned char* st, PhiSmem<BX, BY>& sm, int x0, int y0, int w_, int h__,
                                          int seam, bool ok, OnAbort on_abort, AfterRing after_ring)
@@ -1050,17 +1060,16 @@ __device__ __forceinline__ bool tma_tile(const DevParams& P, typename S::elem* _
     (void)sR;
     constexpr bool edge = EDGE;
     // nodes on a walled, inlet or outflow boundary (a periodic one has none), and ring
-    // nodes beyond one.  Only FP32 TMA tiles reach a periodic edge (x seams): the other
-    // TMA tiles keep one node clear of every periodic edge, where the plain tests agree.
-    constexpr bool kSeams = !kRef<S>;
+    // nodes beyond one.  Without SEAM the TMA tiles keep one node clear of every periodic
+    // edge, where the plain tests agree.
     auto on_boundary = [&](int gx, int gy) {
-        return ((!kSeams || P.bc_x != 0) && (gx == 0 || gx == P.nx - 1)) || gy == 0 || gy == P.ny - 1;
+        return ((!SEAM || P.bc_x != 0) && (gx == 0 || gx == P.nx - 1)) || gy == 0 || gy == P.ny - 1;
     };
     auto is_ghost = [&](int gx, int gy) {
-        return ((!kSeams || P.bc_x != 0) && (gx < 0 || gx >= P.nx)) || gy < 0 || gy >= P.ny;
+        return ((!SEAM || P.bc_x != 0) && (gx < 0 || gx >= P.nx)) || gy < 0 || gy >= P.ny;
     };
     if constexpr (edge) {
-        if constexpr (!kRef<S>) {
+        if constexpr (SEAM) {
             if (seam) seam_patch<BX, BY, S>(st, seam, w);
         }
     }
@@ -1069,7 +1078,7 @@ __device__ __forceinline__ bool tma_tile(const DevParams& P, typename S::elem* _
     auto decF = [&](const E* box, float is, int rplane, int i, int lx, int ly, bool bnode) {
         float r = 0.f;
         if constexpr (kRef<S>) {
-            const int k = bnode ? ref_slot_box(P, x0 + lx - 1, y0 + ly - 1, i, false, x0, y0, L::RW, L::RH)
+            const int k = bnode ? ref_slot_box<SEAM>(P, x0 + lx - 1, y0 + ly - 1, i, false, x0, y0, L::RW, L::RH)
                                 : (ly + 1 - cy(i)) * L::RW + lx + 3 - cx(i);
             r = ref_pop(i, ref_unpack(sR[rplane * L::RH * L::RW + k]));
         }
@@ -1092,8 +1101,8 @@ __device__ __forceinline__ bool tma_tile(const DevParams& P, typename S::elem* _
             if constexpr (kRef<S>) {
                 int k = (ly + 1 - cy(i)) * L::RW + lx + 3 - cx(i), kg = k;
                 if (bnode) {
-                    k = ref_slot_box(P, x, y, i, false, x0, y0, L::RW, L::RH);
-                    kg = ref_slot_box(P, x, y, i, true, x0, y0, L::RW, L::RH);
+                    k = ref_slot_box<SEAM>(P, x, y, i, false, x0, y0, L::RW, L::RH);
+                    kg = ref_slot_box<SEAM>(P, x, y, i, true, x0, y0, L::RW, L::RH);
                 }
                 rf = ref_pop(i, ref_unpack(sR[kRecF * L::RH * L::RW + k]));
                 rg = ref_g(i, ref_unpack(sR[kRecG * L::RH * L::RW + kg]));
@@ -1170,7 +1179,7 @@ __device__ __forceinline__ bool tma_tile(const DevParams& P, typename S::elem* _
             int rx, ry;
             ring_slot(tid, rx, ry);
             const int gx = x0 + rx - 1, gy = y0 + ry - 1;
-            const bool ox = (!kSeams || P.bc_x != 0) && (gx < 0 || gx >= P.nx), oy = gy < 0 || gy >= P.ny;
+            const bool ox = (!SEAM || P.bc_x != 0) && (gx < 0 || gx >= P.nx), oy = gy < 0 || gy >= P.ny;
             if (ox || oy) {
                 const int mx = ox ? (gx < 0 ? 0 : P.nx - 1) : gx;
                 const int my = oy ? (gy < 0 ? 0 : P.ny - 1) : gy;
@@ -1234,15 +1243,18 @@ constexpr int kTmaMinBlocks = kRef<S> ? TPF_TMA_BLOCKS_F16 : TPF_TMA_BLOCKS_F32;
 
 // RAGGED: the lattice has ragged TMA tiles (a body with constant extents is 1% faster on 256 x
 // 1024, a quarter of whose tiles are boundary tiles).
-template <int BX, int BY, class S, bool RAGGED>
+// SEAM: x is periodic, so the lattice has seam tiles (the 2048 x 512 inlet/outflow channel, which
+// has none, takes 44.9 us per step with FP32 without their code and 45.2 with it).
+template <int BX, int BY, class S, bool RAGGED, bool SEAM>
 __global__ void __launch_bounds__(BX * BY, kTmaMinBlocks<S>)
 k_step_tma(const DevParams P, const __grid_constant__ TmaMaps maps, const typename S::elem* __restrict__ A,
            typename S::elem* __restrict__ B, float* __restrict__ phiu, const RefT* __restrict__ refA,
            RefT* __restrict__ refB, const int2* __restrict__ tiles, int bx0, int by0, int ntbx, int ntby,
-           int* __restrict__ err)
+           int* __restrict__ err, const __grid_constant__ SeamMaps smaps)
 {
     using L = TmaLayout<BX, BY, S>;
-    static_assert(sizeof(RingSmem<BX, BY>) <= 2 * L::STAGE, "general-path tiles reuse the stages");
+    constexpr int kStage = SEAM ? L::STAGE : L::OFF_C;  // = L::stage(SEAM)
+    static_assert(sizeof(RingSmem<BX, BY>) <= 2 * kStage, "general-path tiles reuse the stages");
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ __align__(8) uint64_t bar[2];
     // Where a tile's copies are issued: tile t + 2 (this CTA's after next) goes into the
@@ -1276,7 +1288,7 @@ k_step_tma(const DevParams P, const __grid_constant__ TmaMaps maps, const typena
     auto issue = [&](int t, int k, int s) {
         int x0, y0;
         tile_of(t, k, x0, y0);
-        tma_issue_tile<BX, BY, S>(maps, dsm + s * L::STAGE, &bar[s], x0, y0, seam_side<BX>(P, x0), P.nx);
+        tma_issue_tile<BX, BY, S>(maps, smaps, dsm + s * kStage, &bar[s], x0, y0, SEAM ? seam_side<BX>(P, x0) : 0, P.nx);
     };
 
     int it = 0;
@@ -1308,18 +1320,21 @@ k_step_tma(const DevParams P, const __grid_constant__ TmaMaps maps, const typena
             if (t2 < ntma && tid == 0) issue(t2, it + 2, s);
         };
         auto no_refill = [&]() {};
-        unsigned char* st = dsm + s * L::STAGE;
+        unsigned char* st = dsm + s * kStage;
         const bool edge_tile = x0 <= 1 || x0 + BX >= P.nx - 1 || y0 <= 1 || y0 + BY >= P.ny - 1;
-        const int seam = seam_side<BX>(P, x0);
-        if (edge_tile) {
-            if (tma_tile<BX, BY, S, true, RAGGED, false>(P, B, phiu, refB, st, sm, x0, y0, min(BX, P.nx - x0),
-                                                         min(BY, P.ny - y0), seam, ok, on_abort, no_refill))
+        const int seam = SEAM ? seam_side<BX>(P, x0) : 0;
+        // interior tiles first: with the two bodies the other way round 512 x 512 takes 13.3 us per
+        // step with FP32 and 18.8 with FP16, so 13.05 and 18.55
+        if (!edge_tile) {
+            if (tma_tile<BX, BY, S, false, false, false, true>(P, B, phiu, refB, st, sm, x0, y0, BX, BY, 0, ok,
+                                                               on_abort, refill))
+                return;
+        } else {
+            if (tma_tile<BX, BY, S, true, RAGGED, SEAM, false>(P, B, phiu, refB, st, sm, x0, y0, min(BX, P.nx - x0),
+                                                               min(BY, P.ny - y0), seam, ok, on_abort, no_refill))
                 return;
             __syncthreads();  // every warp is done with stage s
             refill();
-        } else if (tma_tile<BX, BY, S, false, false, true>(P, B, phiu, refB, st, sm, x0, y0, BX, BY, 0, ok, on_abort,
-                                                           refill)) {
-            return;
         }
     }
 

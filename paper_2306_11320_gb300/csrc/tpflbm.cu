@@ -791,11 +791,16 @@ bool make_map(CUtensorMap* m, CUtensorMapDataType dt, size_t esize, void* base, 
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// the TMA step kernel of a lattice: with or without ragged tiles
+// the TMA step kernel of a lattice: with or without ragged tiles, and with or without a seam (x
+// periodic), and its two stages
+template <class S>
+int tma_smem(tpflbm_t h) { return 2 * TmaLayout<kBX, kBY, S>::stage(h->hp.bc_x == 0); }
 template <class S>
 auto tma_kernel(tpflbm_t h)
 {
-    return h->nx % kBX || h->ny % kBY ? k_step_tma<kBX, kBY, S, true> : k_step_tma<kBX, kBY, S, false>;
+    const bool ragged = h->nx % kBX || h->ny % kBY;
+    if (h->hp.bc_x == 0) return ragged ? k_step_tma<kBX, kBY, S, true, true> : k_step_tma<kBX, kBY, S, false, true>;
+    return ragged ? k_step_tma<kBX, kBY, S, true, false> : k_step_tma<kBX, kBY, S, false, false>;
 }
 
 template <class S>
@@ -808,11 +813,11 @@ void setup_tma(tpflbm_t h)
     if (((size_t)nx * e) % 16 != 0 || ((size_t)nx * 4) % 16 != 0) return;
     // TMA tiles: every tile, the ragged last one too, along a walled or inlet/outflow axis
     // (the copies fill the box beyond the lattice with zeros and the kernel applies the
-    // boundary rules there) and, with FP32 storage, along a periodic x axis more than a tile
-    // long (a seam tile's wrapped columns are staged beside its boxes); otherwise,
+    // boundary rules there) and along a periodic x axis more than a tile long (a seam tile's
+    // wrapped columns are staged beside its boxes); otherwise,
     // along a periodic axis, the tiles whose (widened) halo lies inside the lattice
     int bx_lo = 0, by_lo = 0, bx_hi = (nx + kBX - 1) / kBX - 1, by_hi = (ny + kBY - 1) / kBY - 1;
-    if (h->hp.bc_x == 0 && (kRef<S> || nx <= kBX)) {
+    if (h->hp.bc_x == 0 && nx <= kBX) {
         bx_lo = (L::XP + kBX - 1) / kBX;
         bx_hi = -1;  // last tile index with x0 + BX + XP <= nx
         for (int b = 0; (b + 1) * kBX + L::XP <= nx; ++b) bx_hi = b;
@@ -830,11 +835,14 @@ void setup_tma(tpflbm_t h)
     const long long pl = h->dp.plane;
     for (int c = 0; c < 2; ++c) {
         TmaMaps& M = h->maps[c];
+        SeamMaps& C = h->smaps[c];
         bool ok = make_map(&M.popF, dt, e, h->pop[c], nx, ny, 27, pl, L::FW, L::FH, 9) &&
                   make_map(&M.popG, dt, e, h->pop[c], nx, ny, 27, pl, kBX, kBY, 9) &&
                   make_map(&M.phiu, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->phiu, nx, ny, 2, pl, kBX, kBY, 2);
         if (kRef<S>) ok = ok && make_map(&M.ref, CU_TENSOR_MAP_DATA_TYPE_UINT64, 8, h->ref[c], nx, ny, 3, pl, L::RW, L::RH, 3);
-        else ok = ok && make_map(&M.ref, dt, e, h->pop[c], nx, ny, 27, pl, L::CW, L::FH, 9);
+        ok = ok && make_map(&C.pop, dt, e, h->pop[c], nx, ny, 27, pl, L::CW, L::FH, 9);
+        if (kRef<S>) ok = ok && make_map(&C.ref, CU_TENSOR_MAP_DATA_TYPE_UINT64, 8, h->ref[c], nx, ny, 3, pl, 2, L::RH, 3);
+        else C.ref = C.pop;
         if (!ok) return;
     }
     // Tile list: first the rectangle's rows and columns that touch the lattice boundary
@@ -864,7 +872,7 @@ void setup_tma(tpflbm_t h)
             return;
         }
     }
-    const int smem = 2 * L::STAGE;
+    const int smem = tma_smem<S>(h);
     const auto fn = tma_kernel<S>(h);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
         cudaGetLastError();
@@ -942,10 +950,9 @@ void launch_step(tpflbm_t h)
     const E* A = (const E*)h->pop[c];
     E* B = (E*)h->pop[c ^ 1];
     if (h->tma) {
-        using L = TmaLayout<kBX, kBY, S>;
-        tma_kernel<S>(h)<<<h->grid_tma, kBX * kBY, 2 * L::STAGE, h->stream>>>(
+        tma_kernel<S>(h)<<<h->grid_tma, kBX * kBY, tma_smem<S>(h), h->stream>>>(
             P, h->maps[c], A, B, h->phiu, h->ref[c], h->ref[c ^ 1], h->tiles, h->bx0, h->by0, h->ntbx, h->ntby,
-            h->err);
+            h->err, h->smaps[c]);
     } else {
         dim3 grd((P.nx + kBX - 1) / kBX, (P.ny + kBY - 1) / kBY);
         k_step_general<kBX, kBY, S><<<grd, kBX * kBY, 0, h->stream>>>(P, A, B, h->phiu, h->ref[c], h->ref[c ^ 1]);
