@@ -897,8 +897,8 @@ __global__ void __launch_bounds__(256) k_flip_weights(const FlipList L)
 // where every channel count and offset is a multiple of eight and every tensor 16-byte
 // aligned (all of the network's calls), and one element per thread for the rest.  They
 // move memory and nothing else; the scalar forms spent their time on 2-byte accesses and
-// 64-bit divisions per element (batch 4 at 512 x 128: upsampling the last level 98 us, now
-// see below).
+// 64-bit divisions per element (a training step of batch 4 at 512 x 128: upsampling 144 us,
+// now 16; pooling's gradient 75, now 15).
 struct Piece {
     float v[8];
 };
