@@ -10,6 +10,8 @@
 #include <cudaTypedefs.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "../../include/tpflbm.h"
 #include "../../include/tpfnet.h"
 
@@ -679,191 +681,6 @@ k_conv3x3_wgrad(const bf16* __restrict__ x, const bf16* __restrict__ dz, int N, 
     if (do_bias && tid < WM) atomicAdd(db + co0 + tid, bacc);
 }
 
-// ------------------------------------------------ tcgen05 weight gradient
-//
-// dW[tap][co][ci] += sum_p dz[p][co] x[p + off(tap)][ci] as GEMMs with M = 128 output
-// channels (co), N = 64 input channels (ci) and K = pixels, over a range of 64-pixel
-// row segments per CTA (split over CTAs, partial sums added with FP32 atomics), for one
-// tap or for the three taps of one column offset, which share each dz box (one 64-column
-// TMEM accumulator per tap).  The reduction runs over pixels, which NHWC stores outermost, so both
-// operands are staged MN-major: a TMA box of 64 channels (128 bytes, 128-byte
-// swizzle) by 64 pixels puts one pixel's channels in each 128-byte row.  A is two such
-// boxes of dz (co0 and co0 + 64), B one box of x at the tap's shifted pixels
-// (w0 + dw, h + dh), whose out-of-range pixels and channels arrive as zeros (the
-// padding, and the channels past Cin or Cout).  The tap's shift is on the pixel
-// coordinates, never on the innermost (channel) one, so every copy starts on a
-// 16-byte boundary.  Same roles as the forward kernel: one thread copies, one thread
-// issues tcgen05.mma (FP32 accumulator in 64 TMEM columns), four warps read TMEM and
-// add into dW.  db[co] += sum_p dz[p][co] is summed by the two warps left over, from the
-// staged dz boxes, in the CTAs of the first tap group and input-channel tile (partial sums
-// per 64-pixel stage, so no longer chains of additions than 64 and the stages of a CTA).  As a
-// kernel of its own, one thread per channel and pixel range, it read dz again and took
-// 9.6 us beside the 25 us of the weight gradient at (4, 64, 256, 64, 64).
-constexpr int kWgStages = 4;
-constexpr int kWgPix = 64;   // pixels per K step (one row segment)
-// taps per CTA: one, or the three rows (dh) of one column offset (dw), which share their
-// dz boxes; three measured faster from 2^17 pixels up (the 512 x 128 level), one below
-constexpr long long kWgTaps3Pixels = 1 << 17;
-
-// shared-memory matrix descriptor of an MN-major tile: 128-byte rows of 64 bf16 along
-// M (or N), one row per K index, 128-byte swizzle; blocks of 64 along M lbo bytes
-// apart, groups of 8 rows 1024 bytes apart (descriptor version 1)
-__device__ __forceinline__ uint64_t mnmajor_desc(uint32_t addr, uint32_t lbo)
-{
-    return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
-           ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
-
-template <int TAPS>
-__global__ void __launch_bounds__(128, 1)
-k_conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap mdz, const __grid_constant__ CUtensorMap mx, int N, int H,
-                   int W, int Cin, int Cout, int chunks_per_cta, float* __restrict__ dw, float* __restrict__ db)
-{
-    static_assert(TAPS == 1 || TAPS == 3, "one tap, or the three rows of one column offset");
-    constexpr int kBlk = kWgPix * 128;      // one 64-channel x 64-pixel box
-    constexpr int kStage = (2 + TAPS) * kBlk;  // A: two boxes (128 co), B: one box (64 ci) per tap
-    constexpr uint32_t kCols = TAPS == 1 ? 64 : 256;  // TMEM columns: 64 per tap, a power of two
-    // MN-major A and B (transpose bits), FP32 accumulator, BF16 operands, M 128, N 64
-    constexpr uint32_t idesc = tc_idesc(128, 64) | (1u << 15) | (1u << 16);
-    extern __shared__ __align__(1024) unsigned char tsm[];
-    __shared__ __align__(8) uint64_t full[kWgStages], empty[kWgStages], done;
-    __shared__ uint32_t tmem_base;
-    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-    unsigned char* st0 = tsm + ((1024 - (sa(tsm) & 1023)) & 1023);
-    const int co0 = blockIdx.x * 128, ci0 = blockIdx.y * 64;
-    // TAPS 1: tap = z % 9; TAPS 3: taps dwi, dwi + 3, dwi + 6 (dh = -1, 0, 1) with dwi = z % 3
-    constexpr int kGroups = 9 / TAPS;
-    const int g = blockIdx.z % kGroups, split = blockIdx.z / kGroups;
-    const int tap0 = g;  // the CTA's first tap (dh = -1 when TAPS is 3)
-    const int dwd = tap0 % 3 - 1;
-    const int segs = W / kWgPix, nchunks = N * H * segs;
-    const int c_begin = split * chunks_per_cta;
-    const int c_end = min(c_begin + chunks_per_cta, nchunks);
-    const int ksteps = c_end > c_begin ? c_end - c_begin : 0;
-    const bool bias = db && g == 0 && blockIdx.y == 0;
-
-    if (tid == 0) {
-        for (int s = 0; s < kWgStages; ++s) {
-            mb_init(&full[s], 1);
-            mb_init(&empty[s], bias ? 3 : 1);  // the MMAs and, with the bias, its two warps
-        }
-        mb_init(&done, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sa(&tmem_base)),
-                     "r"(kCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    pdl_wait();
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    pdl_next();
-    const uint32_t tmem = tmem_base;
-
-    if (warp == 0) {
-        int issued = 0;
-        for (int k = 0; k < ksteps; ++k) {
-            const int s = k % kWgStages;
-            if (k >= kWgStages && !mb_wait(&empty[s], ((k / kWgStages) - 1) & 1)) break;
-            const int c = c_begin + k, row = c / segs;  // row = n * H + h
-            const int w0 = (c - row * segs) * kWgPix, n = row / H, h = row - n * H;
-            unsigned char* a = st0 + s * kStage;
-            // the second dz box only when it holds channels: otherwise TMEM lanes 64-127
-            // accumulate whatever that smem holds and are never read
-            const bool a2 = co0 + 64 < Cout;
-            if (elect_one()) {
-                mb_expect_tx(&full[s], a2 ? kStage : kStage - kBlk);
-                tma_4d(a, &mdz, &full[s], co0, w0, h, n);
-                if (a2) tma_4d(a + kBlk, &mdz, &full[s], co0 + 64, w0, h, n);
-#pragma unroll
-                for (int t = 0; t < TAPS; ++t) {
-                    const int dh = (tap0 + 3 * t) / 3 - 1;
-                    tma_4d(a + (2 + t) * kBlk, &mx, &full[s], ci0, w0 + dwd, h + dh, n);
-                }
-            }
-            __syncwarp();
-            issued = k + 1;
-        }
-        for (int k = issued > kWgStages ? issued - kWgStages : 0; k < issued; ++k)
-            mb_wait(&full[k % kWgStages], (k / kWgStages) & 1);
-    } else if (warp == 1) {
-        for (int k = 0; k < ksteps; ++k) {
-            const int s = k % kWgStages;
-            if (!mb_wait(&full[s], (k / kWgStages) & 1)) break;
-            tc_fence_after();
-            const uint32_t a = sa(st0 + s * kStage);
-            if (elect_one()) {
-#pragma unroll
-                for (int t = 0; t < TAPS; ++t)
-#pragma unroll
-                    for (int kk = 0; kk < kWgPix / 16; ++kk)  // 16 K rows = two 8-row groups
-                        tc_mma(tmem + 64 * t, mnmajor_desc(a + 2048 * kk, kBlk),
-                               mnmajor_desc(a + (2 + t) * kBlk + 2048 * kk, kBlk), idesc, (k | kk) != 0);
-                tc_commit(&empty[s]);
-            }
-            __syncwarp();
-        }
-        if (elect_one()) tc_commit(&done);
-    } else if (warp >= 2 && bias) {
-        // warp 2 + q sums box q, lane l its channels 2 l and 2 l + 1: 16-byte piece l / 4 of
-        // the 128-byte rows, which the swizzle puts at piece (l / 4) ^ (pixel % 8)
-        const int q = warp - 2, cb = co0 + 64 * q + 2 * lane;
-        float b0 = 0.f, b1 = 0.f;
-        for (int k = 0; k < ksteps; ++k) {
-            const int s = k % kWgStages;
-            if (!mb_wait(&full[s], (k / kWgStages) & 1)) break;
-            if (co0 + 64 * q < Cout) {
-                const unsigned char* a = st0 + s * kStage + q * kBlk + 4 * (lane & 3);
-                float p0 = 0.f, p1 = 0.f;
-#pragma unroll 16
-                for (int p = 0; p < kWgPix; ++p) {
-                    const float2 v = __bfloat1622float2(
-                        *reinterpret_cast<const __nv_bfloat162*>(a + 128 * p + 16 * ((lane >> 2) ^ (p & 7))));
-                    p0 += v.x;
-                    p1 += v.y;
-                }
-                b0 += p0;
-                b1 += p1;
-            }
-            __syncwarp();
-            if (lane == 0)
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sa(&empty[s])) : "memory");
-        }
-        if (cb < Cout) {  // (Cout is even)
-            atomicAdd(db + cb, b0);
-            atomicAdd(db + cb + 1, b1);
-        }
-    }
-    __syncwarp();
-
-    // thread (warp w, lane l) owns output channel co0 + 32 w + l (TMEM lane 32 w + l)
-    mb_wait(&done, 0);
-    tc_fence_after();
-    const int co = co0 + warp * 32 + lane;
-#pragma unroll 1
-    for (int c = 0; c < 64 * TAPS; c += 8) {
-        uint32_t r[8];
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                     : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        const int tap = tap0 + 3 * (c / 64), cc = c % 64;
-        if (ksteps > 0 && co < Cout) {
-            float* dst = dw + ((size_t)tap * Cout + co) * Cin + ci0 + cc;
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (ci0 + cc + j < Cin) atomicAdd(dst + j, __uint_as_float(r[j]));
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
-}
-
 // flipped transposes for the data gradients: wd[tap][ci][co] = w[8 - tap][co][ci], of up to
 // kMaxFlips layers in one launch (blockIdx.y; 3 us each on its own)
 constexpr int kMaxFlips = 16;
@@ -932,30 +749,37 @@ __device__ __forceinline__ void relu_back8(Piece& d, const Piece& y)
         if (!(y.v[j] > 0.f)) d.v[j] = 0.f;
 }
 
-// ------------------------------------------ tcgen05 weight gradient on halo tiles
+// ------------------------------------------------ tcgen05 weight gradient
 //
-// The weight gradient with 8 x 16 pixel blocks as K steps of 128 and one column offset dw of
-// the taps per CTA: a stage holds the block of dz (64 output channels per box, two boxes when
-// there are more) and the block of x shifted by dw with a row above and below, 18 rows of 8
-// pixels by CK input channels.  Both are MN-major, one pixel's channels per row.  The three
-// taps of the column are one MMA: its N runs over three blocks of CK channels that lie one
-// image row (eight rows of shared memory) apart, so the operand's windows are the taps' shifts
-// and dz is read from shared memory once for the three.  M = 128 output channels (past the
-// boxes that exist, lanes hold sums that are not read), N = 3 CK, K = 16 pixels = two image
-// rows.  db is summed from the dz boxes by four more warps in the CTAs of dw = -1 and the
-// first input channels, each thread eight channels of every fourth pixel.  Partial sums of a
-// CTA go to dw in vector reductions.  Blocks that reach past an image's edge add nothing: dz is
-// zero there.
+// dW[tap][co][ci] += sum_p dz[p][co] x[p + off(tap)][ci], with blocks of BW x BH pixels as K steps
+// and one column offset dw of the taps per CTA: a stage holds the block of dz (64 output channels
+// per box, two boxes when there are more) and the block of x shifted by dw with a row above and
+// below, BH + 2 rows of BW pixels by CK input channels.  Both are MN-major, one pixel's channels
+// per row.  The three taps of the column are one MMA: its N runs over three blocks of CK channels
+// that lie one image row (BW rows of shared memory) apart, so the operand's windows are the taps'
+// shifts and dz is read from shared memory once for the three.  M = 128 output channels (past the
+// boxes that exist, lanes hold sums that are not read), N = 3 CK, K = 16 pixels, 16 rows of the
+// block.  db is summed from the dz boxes by four more warps in the CTAs of dw = -1 and the first
+// input channels, each thread eight channels of every fourth pixel.  Partial sums of a CTA go to
+// dw in vector reductions (dw off the 16-byte rule: one by one).  Blocks that reach past an image's
+// edge add nothing: dz is zero there.
 //
-// Weight and bias gradient, batch 4 (us, against one tap or column of taps per stage with its
-// own x box): 512 x 128 32 -> 32 62 -> 24, 96 -> 32 122 -> 44; 256 x 64 64 -> 64 29 -> 19, 192 ->
-// 64 62 -> 22; 64 x 16 256 -> 256 31 -> 13.  Bound by the MMAs (N = 192 takes the tensor pipe as
-// long as shared memory takes to deliver its operands) and, at 64 channels and fewer, by the
-// kernel's start and the reductions at its end.  The sums are more accurate than before
-// (fewer accumulations in a row): 2.5e-6 -> 1.1e-6 of dw at 512 x 128, 7.5e-7 -> 4.9e-7 at 256 x
-// 64 (relative L2 against float64).
-constexpr int kWhDz = 128 * 128;  // a dz box: 128 pixels of 64 channels
-constexpr int kWhStages = 4;
+// Blocks: segments of 64 x 1 where the width allows, else 8 x 16.  The segments' order and their
+// split over CTAs decide which products meet in which float32 sum, and training amplifies that: a
+// first step of Adam turns a change of a gradient near zero into one of up to a whole step, and
+// sums over 8 x 16 blocks, as accurate as these, moved the second step's gradients by 1e-4.  So the
+// order is fixed (wgrad_splits): every tap's sum runs through its CTA's segments from left to right
+// and from top to bottom, 16 pixels at a time.
+//
+// Weight and bias gradient, batch 4 (us, against one tap or column of taps per MMA in the same
+// order): 512 x 128 32 -> 32 82 -> 30, 96 -> 32 188 -> 57; 256 x 64 64 -> 64 35 -> 13, 192 -> 64 78 ->
+// 28; 64 x 16 256 -> 256 37 -> 10 (8 x 16 blocks, which stage x 1.1 times instead of 3: 17, 40, 11, 19
+// and 9).  Bound by staging from L2 and by the reductions at the end.
+constexpr int kWgStages = 4;
+constexpr int kWgPix = 64;  // pixels of a row segment
+// bytes of a dz box (BW x BH pixels of 64 channels) and of the x box
+__host__ __device__ constexpr int wg_dz(int BW, int BH) { return BW * BH * 128; }
+__host__ __device__ constexpr int wg_x(int BW, int BH, int CK) { return BW * (BH + 2) * 2 * CK; }
 
 // MN-major descriptor: rows of CK channels (64 or 128 bytes, swizzled over the row), groups of
 // eight rows sbo bytes apart along K, blocks of a row's channels lbo bytes apart along M or N
@@ -973,17 +797,19 @@ __device__ __forceinline__ void red_add4(float* p, const uint32_t* r)
                  : "memory");
 }
 
-template <int CK>
+template <int CK, int BW, int BH>
 __global__ void __launch_bounds__(256)
-k_conv3x3_wgrad_halo(const __grid_constant__ CUtensorMap mdz, const __grid_constant__ CUtensorMap mx, int N, int H,
-                     int W, int Cin, int Cout, int tiles_per_cta, float* __restrict__ dw, float* __restrict__ db)
+k_conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap mdz, const __grid_constant__ CUtensorMap mx, int N, int H,
+                   int W, int Cin, int Cout, int tiles_per_cta, float* __restrict__ dw, float* __restrict__ db)
 {
-    constexpr int kX = 18 * 8 * 2 * CK, kRow = 8 * 2 * CK;  // x box, one image row of it
+    static_assert(BW % 8 == 0 && BW * BH % 64 == 0, "whole groups of eight rows, sixteen pixels per MMA and bias warp");
+    constexpr int kPix = BW * BH, kDz = wg_dz(BW, BH), kX = wg_x(BW, BH, CK);
+    constexpr int kRow = BW * 2 * CK;  // one image row of the x box
     constexpr uint32_t kCols = CK == 64 ? 256 : 128;        // TMEM columns: 3 CK in use
     // MN-major A and B (transpose bits)
     constexpr uint32_t idesc = tc_idesc(128, 3 * CK) | (1u << 15) | (1u << 16);
     extern __shared__ __align__(1024) unsigned char tsm[];
-    __shared__ __align__(8) uint64_t full[kWhStages], empty[kWhStages], done;
+    __shared__ __align__(8) uint64_t full[kWgStages], empty[kWgStages], done;
     __shared__ uint32_t tmem_base;
     __shared__ float sdb[4][128];
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -992,13 +818,13 @@ k_conv3x3_wgrad_halo(const __grid_constant__ CUtensorMap mdz, const __grid_const
     const int g = blockIdx.z % 3, split = blockIdx.z / 3;
     const int nb = co0 + 64 < Cout ? 2 : 1;  // dz boxes
     const int boxes = Cout > 64 ? 2 : 1;     // room for them
-    const int kStage = boxes * kWhDz + kX;
-    const int bpr = (W + 7) / 8, bpi = bpr * ((H + 15) / 16), tiles = N * bpi;
+    const int kStage = boxes * kDz + kX;
+    const int bpr = (W + BW - 1) / BW, bpi = bpr * ((H + BH - 1) / BH), tiles = N * bpi;
     const int begin = split * tiles_per_cta, end = min(begin + tiles_per_cta, tiles), steps = max(end - begin, 0);
     const bool bias = db && g == 0 && blockIdx.y == 0;
 
     if (tid == 0) {
-        for (int s = 0; s < kWhStages; ++s) {
+        for (int s = 0; s < kWgStages; ++s) {
             mb_init(&full[s], 1);
             mb_init(&empty[s], bias ? 5 : 1);  // the MMAs and, with the bias, its four warps
         }
@@ -1021,14 +847,14 @@ k_conv3x3_wgrad_halo(const __grid_constant__ CUtensorMap mdz, const __grid_const
     if (warp == 0) {
         int n = begin / bpi, rem = begin - n * bpi, row = rem / bpr, col = rem - row * bpr, issued = 0;
         for (; issued < steps; ++issued) {
-            const int s = issued % kWhStages;
-            if (issued >= kWhStages && !mb_wait(&empty[s], (issued / kWhStages - 1) & 1)) break;
+            const int s = issued % kWgStages;
+            if (issued >= kWgStages && !mb_wait(&empty[s], (issued / kWgStages - 1) & 1)) break;
             if (elect_one()) {
                 unsigned char* a = st0 + s * kStage;
-                mb_expect_tx(&full[s], nb * kWhDz + kX);
-                tma_4d(a, &mdz, &full[s], co0, 8 * col, 16 * row, n);
-                if (nb == 2) tma_4d(a + kWhDz, &mdz, &full[s], co0 + 64, 8 * col, 16 * row, n);
-                tma_4d(a + boxes * kWhDz, &mx, &full[s], ci0, 8 * col + g - 1, 16 * row - 1, n);
+                mb_expect_tx(&full[s], nb * kDz + kX);
+                tma_4d(a, &mdz, &full[s], co0, BW * col, BH * row, n);
+                if (nb == 2) tma_4d(a + kDz, &mdz, &full[s], co0 + 64, BW * col, BH * row, n);
+                tma_4d(a + boxes * kDz, &mx, &full[s], ci0, BW * col + g - 1, BH * row - 1, n);
             }
             __syncwarp();
             if (++col == bpr) {
@@ -1037,39 +863,39 @@ k_conv3x3_wgrad_halo(const __grid_constant__ CUtensorMap mdz, const __grid_const
             }
         }
         if (issued < steps)  // a wait ran out: the copies still in flight land before the CTA ends
-            for (int k = max(issued - kWhStages, 0); k < issued; ++k) mb_wait(&full[k % kWhStages], (k / kWhStages) & 1);
+            for (int k = max(issued - kWgStages, 0); k < issued; ++k) mb_wait(&full[k % kWgStages], (k / kWgStages) & 1);
     } else if (warp == 1) {
         for (int k = 0; k < steps; ++k) {
-            const int s = k % kWhStages;
-            if (!mb_wait(&full[s], (k / kWhStages) & 1)) break;
+            const int s = k % kWgStages;
+            if (!mb_wait(&full[s], (k / kWgStages) & 1)) break;
             tc_fence_after();
             if (elect_one()) {
-                const uint32_t a = sa(st0 + s * kStage), b = a + boxes * kWhDz;
+                const uint32_t a = sa(st0 + s * kStage), b = a + boxes * kDz;
                 // (with one dz box the second block of M is the first one's rows 8 and on)
-                const uint64_t ad = mnmajor_desc2<64>(a, nb == 2 ? kWhDz : 1024, 1024);
-                const uint64_t bd = mnmajor_desc2<CK>(b, kRow, kRow);
+                const uint64_t ad = mnmajor_desc2<64>(a, nb == 2 ? kDz : 1024, 1024);
+                const uint64_t bd = mnmajor_desc2<CK>(b, kRow, 8 * 2 * CK);
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk)  // two image rows each
-                    tc_mma(tmem, ad + 2048 / 16 * kk, bd + 2 * kRow / 16 * kk, idesc, (k | kk) != 0);
+                for (int kk = 0; kk < kPix / 16; ++kk)
+                    tc_mma(tmem, ad + 16 * 128 / 16 * kk, bd + 16 * 2 * CK / 16 * kk, idesc, (k | kk) != 0);
                 tc_commit(&empty[s]);
             }
             __syncwarp();
         }
         if (elect_one()) tc_commit(&done);
     } else if (warp >= 4 && bias) {
-        // lane: 16-byte piece lane % 8 of a row, pixels 32 (warp - 4) + 4 j + lane / 8
-        const int piece = lane & 7, p0 = 32 * (warp - 4) + (lane >> 3);
+        // lane: 16-byte piece lane % 8 of a row, pixels kPix / 4 (warp - 4) + 4 j + lane / 8
+        const int piece = lane & 7, p0 = kPix / 4 * (warp - 4) + (lane >> 3);
         float acc[2][8] = {};
         for (int k = 0; k < steps; ++k) {
-            const int s = k % kWhStages;
-            if (!mb_wait(&full[s], (k / kWhStages) & 1)) break;
+            const int s = k % kWgStages;
+            if (!mb_wait(&full[s], (k / kWgStages) & 1)) break;
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 if (q >= nb) break;
-                const unsigned char* a = st0 + s * kStage + q * kWhDz;
+                const unsigned char* a = st0 + s * kStage + q * kDz;
                 float part[8] = {};
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
+                for (int j = 0; j < kPix / 16; ++j) {
                     const int p = p0 + 4 * j;
                     const Piece v = ld8(reinterpret_cast<const bf16*>(a + 128 * p + 16 * (piece ^ (p & 7))));
 #pragma unroll
@@ -1100,7 +926,7 @@ k_conv3x3_wgrad_halo(const __grid_constant__ CUtensorMap mdz, const __grid_const
     mb_wait(&done, 0);
     tc_fence_after();
     const int co = co0 + (warp & 3) * 32 + lane;
-    const bool mine = steps > 0 && co < Cout;
+    const bool mine = steps > 0 && co < Cout, vec = ((uintptr_t)dw & 15) == 0;
     constexpr int kHalf = 3 * CK / 2;
 #pragma unroll 1
     for (int c = (warp >> 2) * kHalf; c < ((warp >> 2) + 1) * kHalf; c += 16) {
@@ -1116,7 +942,14 @@ k_conv3x3_wgrad_halo(const __grid_constant__ CUtensorMap mdz, const __grid_const
             // columns c .. c + 15: tap 3 (c / CK) + g, input channels ci0 + c % CK and on
             float* dst = dw + ((size_t)(3 * (c / CK) + g) * Cout + co) * Cin + ci0 + c % CK;
 #pragma unroll
-            for (int j = 0; j < 16; j += 4) red_add4(dst + j, r + j);
+            for (int j = 0; j < 16; j += 4) {
+                if (vec) {
+                    red_add4(dst + j, r + j);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) atomicAdd(dst + j + e, __uint_as_float(r[j + e]));
+                }
+            }
         }
     }
     tc_fence_before();
@@ -1735,86 +1568,69 @@ bool conv_tc(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, const 
     }
 }
 
-// The halo form of the weight gradient; false (nothing launched) when it cannot be.
-template <int CK>
-bool launch_wgrad_halo(const bf16* x, const bf16* dz, int N, int H, int W, int Cin, int Cout, float* dw, float* db,
-                       cudaStream_t s)
+// CTAs over which the 64 x 1 segments of an image batch are split, `per` segments each: about as
+// many as run at once when each takes 64 input channels of one tap (from kWgTaps3Pixels pixels up
+// of three).  Part of the results (see k_conv3x3_wgrad_tc), not of the launch: what a CTA takes
+// otherwise does not move it.
+constexpr long long kWgTaps3Pixels = 1 << 17;
+long long wgrad_splits(int N, int H, int W, int Cin, int Cout, long long& per)
 {
+    const long long P = (long long)N * H * W, nchunks = (long long)N * H * (W / kWgPix);
+    const int taps = P >= kWgTaps3Pixels ? 3 : 1;
+    const long long base = (9 / taps) * (long long)((Cout + 127) / 128) * ((Cin + 63) / 64);
+    const long long target = taps == 1 ? 2 * 152 : 152;
+    const long long splits = std::max(1LL, std::min(nchunks, (target + base - 1) / base));
+    per = (nchunks + splits - 1) / splits;
+    return (nchunks + per - 1) / per;
+}
+
+// The weight gradient on blocks of BW x BH; false (nothing launched) when it cannot be.
+template <int CK, int BW, int BH>
+bool launch_wgrad(const bf16* x, const bf16* dz, int N, int H, int W, int Cin, int Cout, float* dw, float* db,
+                  cudaStream_t s)
+{
+    const auto kern = k_conv3x3_wgrad_tc<CK, BW, BH>;
     CUtensorMap mdz, mx;
-    if (!pixel_map(&mdz, dz, N, H, W, Cout, 64, 8, 16) || !pixel_map(&mx, x, N, H, W, Cin, CK, 8, 18)) return false;
-    const int stage = (Cout > 64 ? 2 : 1) * kWhDz + 18 * 8 * 2 * CK, smem = kWhStages * stage + 1024;
-    if (cudaFuncSetAttribute(k_conv3x3_wgrad_halo<CK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+    if (!pixel_map(&mdz, dz, N, H, W, Cout, 64, BW, BH) || !pixel_map(&mx, x, N, H, W, Cin, CK, BW, BH + 2)) return false;
+    const int stage = (Cout > 64 ? 2 : 1) * wg_dz(BW, BH) + wg_x(BW, BH, CK), smem = kWgStages * stage + 1024;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    // split the blocks over about as many CTAs as run at once
-    const long long tiles = (long long)N * ((H + 15) / 16) * ((W + 7) / 8);
     const int ctiles = (Cout + 127) / 128, itiles = Cin / CK;
-    const long long base = 3LL * ctiles * itiles, target = smem <= 112 * 1024 ? 304 : 152;
-    long long splits = target / base;
-    if (splits > tiles) splits = tiles;
-    if (splits < 1) splits = 1;
-    const long long per = (tiles + splits - 1) / splits;
-    splits = (tiles + per - 1) / per;
-    launch_pdl(k_conv3x3_wgrad_halo<CK>, dim3(ctiles, itiles, 3 * (unsigned)splits), 256, smem, s, mdz, mx, N, H, W, Cin, Cout,
-                                                                                          (int)per, dw, db);
+    long long splits, per;
+    if (BH == 1) {
+        splits = wgrad_splits(N, H, W, Cin, Cout, per);
+    } else {
+        // split the blocks over about as many CTAs as run at once
+        const long long tiles = (long long)N * ((H + BH - 1) / BH) * ((W + BW - 1) / BW);
+        const long long base = 3LL * ctiles * itiles, target = smem <= 112 * 1024 ? 304 : 152;
+        splits = std::max(1LL, std::min(tiles, target / base));
+        per = (tiles + splits - 1) / splits;
+        splits = (tiles + per - 1) / per;
+    }
+    launch_pdl(kern, dim3(ctiles, itiles, 3 * (unsigned)splits), 256, smem, s, mdz, mx, N, H, W, Cin, Cout, (int)per, dw, db);
     return true;
 }
 
-// shapes the halo form takes: images that divide into its blocks, and any other large enough
+// shapes the tcgen05 weight gradient takes: rows of whole segments, images that divide into blocks
+// of 8 x 16, and any other large enough
 bool wgrad_blocks(int N, int H, int W)
 {
-    return (H % 16 == 0 && W % 8 == 0) || (W % kWgPix != 0 && (long long)N * H * W >= kRaggedPixels);
+    return W % kWgPix == 0 || (H % 16 == 0 && W % 8 == 0) || (long long)N * H * W >= kRaggedPixels;
 }
 
-// The tcgen05 weight gradient for W a multiple of 64 and 16-byte aligned tensors;
-// false (nothing launched) otherwise.  Adds into dw (and db).
+// The tcgen05 weight gradient for those shapes and 16-byte aligned x and dz; false (nothing
+// launched) otherwise.  Adds into dw (and db).
 bool wgrad_tc(const bf16* x, const bf16* dz, int N, int H, int W, int Cin, int Cout, float* dw, float* db,
               cudaStream_t s)
 {
-    if (((uintptr_t)x | (uintptr_t)dz) & 15) return false;
-    if (wgrad_blocks(N, H, W) && (uintptr_t)dw % 16 == 0) {
-        const auto f = Cin % 64 == 0 ? launch_wgrad_halo<64> : launch_wgrad_halo<32>;
-        if (f(x, dz, N, H, W, Cin, Cout, dw, db, s)) return true;
-    }
-    if (W % kWgPix != 0) return false;
-    auto fn = encode_fn();
-    if (!fn) return false;
-    CUtensorMap mdz, mx;
-    auto make = [&](CUtensorMap* m, const bf16* base, int C) {
-        cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
-        cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
-        cuuint32_t box[4] = {64, (cuuint32_t)kWgPix, 1, 1};
-        cuuint32_t es[4] = {1, 1, 1, 1};
-        return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void*)base, dims, strides, box, es,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-    };
-    if (!make(&mdz, dz, Cout) || !make(&mx, x, Cin)) return false;
-    const long long P = (long long)N * H * W;
-    const int taps = P >= kWgTaps3Pixels ? 3 : 1;
-    const int smem = kWgStages * (2 + taps) * kWgPix * 128 + 1024;
-    if (cudaFuncSetAttribute(taps == 3 ? (const void*)k_conv3x3_wgrad_tc<3> : (const void*)k_conv3x3_wgrad_tc<1>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    // split the pixel segments so that the grid fills the GPU about twice
-    const long long nchunks = (long long)N * H * (W / kWgPix);
-    const int ctiles = (Cout + 127) / 128, itiles = (Cin + 63) / 64;
-    const long long base = (9 / taps) * (long long)ctiles * itiles;
-    const long long target = taps == 1 ? 2 * 152 : 152;  // CTAs per SM the shared memory allows
-    long long splits = (target + base - 1) / base;
-    if (splits > nchunks) splits = nchunks;
-    if (splits < 1) splits = 1;
-    const long long per = (nchunks + splits - 1) / splits;
-    splits = (nchunks + per - 1) / per;
-    dim3 grd(ctiles, itiles, (9 / taps) * (unsigned)splits);
-    if (taps == 3)
-        launch_pdl(k_conv3x3_wgrad_tc<3>, grd, 128, smem, s, mdz, mx, N, H, W, Cin, Cout, (int)per, dw, db);
-    else
-        launch_pdl(k_conv3x3_wgrad_tc<1>, grd, 128, smem, s, mdz, mx, N, H, W, Cin, Cout, (int)per, dw, db);
-    return true;
+    if ((((uintptr_t)x | (uintptr_t)dz) & 15) || !wgrad_blocks(N, H, W)) return false;
+    if (W % kWgPix == 0)
+        return Cin % 64 == 0 ? launch_wgrad<64, kWgPix, 1>(x, dz, N, H, W, Cin, Cout, dw, db, s)
+                             : launch_wgrad<32, kWgPix, 1>(x, dz, N, H, W, Cin, Cout, dw, db, s);
+    return Cin % 64 == 0 ? launch_wgrad<64, 8, 16>(x, dz, N, H, W, Cin, Cout, dw, db, s)
+                         : launch_wgrad<32, 8, 16>(x, dz, N, H, W, Cin, Cout, dw, db, s);
 }
 
 }  // namespace
@@ -1888,8 +1704,7 @@ int tpfnet_conv3x3_tcgen05(int N, int H, int W, int Cin, int Cout)
 
 int tpfnet_conv3x3_wgrad_tcgen05(int N, int H, int W, int Cin, int Cout)
 {
-    const bool tiles = W % kWgPix == 0 || (H > 0 && W > 0 && wgrad_blocks(N, H, W));
-    return N >= 1 && H >= 1 && W >= 1 && Cin % 32 == 0 && Cout % 32 == 0 && tiles && encode_fn() ? 1 : 0;
+    return N >= 1 && H >= 1 && W >= 1 && Cin % 32 == 0 && Cout % 32 == 0 && wgrad_blocks(N, H, W) && encode_fn() ? 1 : 0;
 }
 
 int tpfnet_status(void)
