@@ -558,6 +558,8 @@ int tpflbm_batch_create(int n, const int* nx, const int* ny, const tpflbm_params
         if (e == cudaSuccess && !work.empty())
             e = cudaMemcpy(b->d_work[v], work.data(), work.size() * sizeof(int2), cudaMemcpyHostToDevice);
     }
+    // the descriptors and work lists have to be in place before anything runs on the batch's stream
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         std::string why = std::string("batch set-up: ") + cudaGetErrorString(e);

@@ -938,6 +938,10 @@ int finish_create(tpflbm_t h, int nx, int ny, const tpflbm_params* p, void* ws, 
         if (f16) setup_many<StoreF16>(h);
         else setup_many<StoreF32>(h);
     }
+    // The clears and the tile list went over the legacy default stream and may still be under way
+    // when their calls return.  The handle's stream need not be ordered after that one, and a
+    // step kernel that starts early would take step counts and words of whatever the memory held.
+    if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) return cuda_fail(h, cudaGetLastError(), "set-up");
     return TPF_OK;
 }
 

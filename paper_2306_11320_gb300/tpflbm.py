@@ -166,6 +166,8 @@ class Lattice:
             if nbytes == 0:
                 raise TpfError(-1, "invalid lattice size or parameters")
             self._ws = torch.empty(nbytes + 256, dtype=torch.uint8, device="cuda")
+            # the block may have been another tensor's, with work of this stream still to run on it
+            torch.cuda.current_stream().synchronize()
             base = self._ws.data_ptr()
             aligned = (base + 255) & ~255
             rc = self.lib.tpflbm_create_in(self.nx, self.ny, C.byref(self._p), C.c_void_p(aligned),
