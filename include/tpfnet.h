@@ -46,6 +46,11 @@ int tpfnet_conv3x3_wgrad_tcgen05(int N, int H, int W, int Cin, int Cout);
  * TPF_ERR_CUDA if the flag cannot be read.  Synchronises with the device. */
 int tpfnet_status(void);
 
+/* Checks that a warp of the tcgen05 kernels leaves a wait as one: a warp waits on a barrier that
+ * completes, first with every lane's polls, then with a lane that has none.  out: lanes that left
+ * and error flag, for each (0, 0 and 32, 1). */
+int tpfnet_check_bounded_wait(int polls, int out[4]);
+
 /* Data gradient of conv3x3: dx = conv3x3 of dz (the gradient at the convolution's
  * output, ReLU mask already applied) with the flipped, transposed weights, which are
  * written to wflip (9 * Cin * Cout bf16 of caller scratch). */

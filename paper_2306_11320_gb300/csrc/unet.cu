@@ -191,18 +191,21 @@ __device__ __forceinline__ void mb_expect_tx(uint64_t* b, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(sa(b)), "r"(bytes) : "memory");
 }
-__device__ __forceinline__ bool mb_wait(uint64_t* b, uint32_t parity)
+// Bounded wait of a whole warp: false, on every lane, when the polls of any lane ran out.  (Lanes
+// poll each for itself; one that gave up alone would leave the others in an elect.sync or a
+// __syncwarp that waits for it.)
+constexpr uint32_t kMbPolls = 1u << 22;
+__device__ __forceinline__ bool mb_wait(uint64_t* b, uint32_t parity, uint32_t polls = kMbPolls, int* err = &g_tc_err)
 {
-    for (uint32_t it = 0; it < (1u << 22); ++it) {
-        uint32_t ok;
+    uint32_t ok = 0;
+    for (uint32_t it = 0; it < polls && !ok; ++it)
         asm volatile(
             "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
             : "=r"(ok)
             : "r"(sa(b)), "r"(parity)
             : "memory");
-        if (ok) return true;
-    }
-    atomicExch(&g_tc_err, 1);
+    if (__all_sync(0xffffffffu, ok != 0)) return true;
+    atomicExch(err, 1);
     return false;
 }
 __device__ __forceinline__ void tma_3d(void* dst, const CUtensorMap* m, uint64_t* b, int c0, int c1, int c2)
@@ -1391,6 +1394,32 @@ __global__ void k_unpack(const float* __restrict__ src, long long pixels, int C,
     }
 }
 
+// One warp waits in the manner of the issuing warps' loops on a barrier that completes: in block
+// 0 with every lane's polls, in block 1 with one lane that has none.  out[2 block]: lanes that
+// left the loop, out[2 block + 1]: the error flag.
+__global__ void __launch_bounds__(64) k_wait_check(uint32_t polls, int* out)
+{
+    __shared__ __align__(8) uint64_t bar;
+    if (threadIdx.x == 0) {
+        mb_init(&bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    if (threadIdx.x == 32) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sa(&bar)) : "memory");
+    if (threadIdx.x >= 32) return;
+    bool left = false;
+    for (int k = 0; k < 2; ++k) {
+        if (!mb_wait(&bar, 0, blockIdx.x == 1 && threadIdx.x == 5 ? 0 : polls, out + 2 * blockIdx.x + 1)) {
+            left = true;
+            break;
+        }
+        elect_one();
+        __syncwarp();
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, left);
+    if (threadIdx.x == 0) out[2 * blockIdx.x] = __popc(m);
+}
+
 int grid_of(long long count)
 {
     long long b = (count + 255) / 256;
@@ -1712,6 +1741,21 @@ int tpfnet_status(void)
     int v = 0;
     if (cudaMemcpyFromSymbol(&v, g_tc_err, sizeof(int)) != cudaSuccess) return TPF_ERR_CUDA;
     return v ? TPF_ERR_TIMEOUT : TPF_OK;
+}
+
+int tpfnet_check_bounded_wait(int polls, int out[4])
+{
+    if (polls < 1 || !out) return TPF_ERR_INVALID_ARG;
+    int* d = nullptr;
+    cudaError_t e = cudaMalloc(&d, 4 * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(d, 0, 4 * sizeof(int));
+    if (e == cudaSuccess) {
+        k_wait_check<<<2, 64>>>((uint32_t)polls, d);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(out, d, 4 * sizeof(int), cudaMemcpyDeviceToHost);
+    cudaFree(d);
+    return status(e);
 }
 
 int tpfnet_conv3x3_dgrad(const void* dz, int N, int H, int W, int Cout, const void* wt, int Cin, void* wflip, void* dx,

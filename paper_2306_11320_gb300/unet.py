@@ -33,6 +33,7 @@ SIGNATURES = {
     "tpfnet_conv3x3_tcgen05": [_ip, _ip, _ip, _ip, _ip],
     "tpfnet_conv3x3_wgrad_tcgen05": [_ip, _ip, _ip, _ip, _ip],
     "tpfnet_status": [],
+    "tpfnet_check_bounded_wait": [_ip, _vp],
     "tpfnet_conv3x3_dgrad": [_vp, _ip, _ip, _ip, _ip, _vp, _ip, _vp, _vp, _vp],
     "tpfnet_conv3x3_wgrad": [_vp, _vp, _ip, _ip, _ip, _ip, _ip, _vp, _vp, _vp],
     "tpfnet_relu_mask": [_vp, _vp, _ll, _vp],
