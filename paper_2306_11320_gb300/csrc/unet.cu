@@ -401,6 +401,8 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUt
 constexpr int kHaloChunks = 12;  // channel chunks of a box (Cin <= 768)
 constexpr int kHaloStages = 8;   // weight stages at most
 constexpr int kHaloRows = 18;    // box rows: 16 image rows and the frame
+// dynamic shared memory at most: what 227 KB leave beside the kernel's own 1.3 KB, in whole KB
+constexpr int kHaloSmem = 225 * 1024;
 
 // K-major descriptor with 8-row groups sbo bytes apart (kmajor_desc: 16 KC)
 template <int KC>
@@ -1536,7 +1538,7 @@ bool launch_halo(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, co
     // one ((4, 32, 128, 384, 128): 22.9 us against 31.1, (4, 16, 64, 256, 256): 16.8 against
     // 17.7).  With at most one CTA per SM its whole shared memory, and parts of a tap if need be.
     const long long blocks = (long long)N * ((H + 15) / 16) * ((W + 8 * MT - 1) / (8 * MT)), ctas = blocks * (Cout / BN);
-    const int limit = ctas > 152 ? 112 * 1024 : 226 * 1024;
+    const int limit = ctas > 152 ? 112 * 1024 : kHaloSmem;
     HaloStages st{0, 0, 0};
     auto take = [&](int T, int CC, int S) {
         if (st.S || CC < 1 || kc % CC || (long long)a + (long long)S * T * CC * b > limit) return;
@@ -1556,8 +1558,9 @@ bool launch_halo(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, co
     CUtensorMap mx, mw;
     if (!pixel_map(&mx, x, N, H, W, Cin, KC, 8 * MT + 2, kHaloRows) || !weight_map(&mw, wt, Cin, Cout, KC, BN, st.T))
         return false;
-    // set on every call: the attribute belongs to the current device
-    if (cudaFuncSetAttribute(k_conv3x3_halo<KC, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+    // set on every call (the attribute belongs to the current device), and always to the same size:
+    // another thread may be between its setting and its launch
+    if (cudaFuncSetAttribute(k_conv3x3_halo<KC, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHaloSmem) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -1622,7 +1625,9 @@ bool launch_wgrad(const bf16* x, const bf16* dz, int N, int H, int W, int Cin, i
     CUtensorMap mdz, mx;
     if (!pixel_map(&mdz, dz, N, H, W, Cout, 64, BW, BH) || !pixel_map(&mx, x, N, H, W, Cin, CK, BW, BH + 2)) return false;
     const int stage = (Cout > 64 ? 2 : 1) * wg_dz(BW, BH) + wg_x(BW, BH, CK), smem = kWgStages * stage + 1024;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+    // (always the size of two dz boxes: another thread may be between its setting and its launch)
+    constexpr int kMost = kWgStages * (2 * wg_dz(BW, BH) + wg_x(BW, BH, CK)) + 1024;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
