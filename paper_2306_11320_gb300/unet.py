@@ -117,6 +117,13 @@ class UNet:
             self._add(name + ".b", (0.01 * rng.standard_normal(b)).astype(np.float32), bf16=False)
         self.adam_t = 0
         self._shape = None
+        # all of that was queued on the current stream
+        self.stream.wait_stream(torch.cuda.current_stream())
+
+    def _on_stream(self):
+        """torch's current stream is the network's own inside: what torch clears, copies and
+        reads between the kernels is ordered with them."""
+        return self.torch.cuda.stream(self.stream)
 
     def _add(self, key, arr, bf16):
         t = self.torch
@@ -184,6 +191,10 @@ class UNet:
         if self._shape == (N, H, W):
             return
         assert H % 8 == 0 and W % 64 == 0, "H multiple of 8, W multiple of 64"
+        with self._on_stream():
+            self._new_buffers(N, H, W)
+
+    def _new_buffers(self, N, H, W):
         t = self.torch
         c0, c1, c2, c3 = self.ch
         bf = dict(dtype=t.bfloat16, device="cuda")
@@ -308,11 +319,9 @@ class UNet:
         self._block_back("e0a", "e0b", self.x, self.cinp, B["e0a"], c0, D["e0"], None, N, H, W)
 
     def zero_grad(self):
-        if self._is_flat(("G",)):
-            self._flat["G"].zero_()
-            return
-        for g in self.G.values():
-            g.zero_()
+        with self._on_stream():
+            for g in [self._flat["G"]] if self._is_flat(("G",)) else self.G.values():
+                g.zero_()
 
     def adam(self, lr=1e-3, b1=0.9, b2=0.999, eps=1e-8):
         self.adam_t += 1
@@ -330,10 +339,12 @@ class UNet:
     def mse(self, pred, target, wch=None, want_grad=True):
         """Loss (float, synchronises) and, when want_grad, its gradient in self.D['out']."""
         self._mse(pred, target, wch, want_grad)
-        return float(self.loss.item())
+        with self._on_stream():
+            return float(self.loss.item())
 
     def _mse(self, pred, target, wch, want_grad=True):
-        self.loss.zero_()
+        with self._on_stream():
+            self.loss.zero_()
         C_ = pred.shape[-1]
         self._chk(self.lib.tpfnet_mse(_p(pred), _p(target), _p(wch), pred.numel(), C_,
                                       _p(self.D["out"]) if want_grad else None, _p(self.loss), self._s()), "mse")
@@ -347,7 +358,7 @@ class UNet:
         t = self.torch
         host = t.empty(1, dtype=t.float64, pin_memory=True)
         done = t.cuda.Event()
-        with t.cuda.stream(self.stream):
+        with self._on_stream():
             host.copy_(self.loss, non_blocking=True)
             done.record()
         self.backward(self.D["out"])
