@@ -1434,8 +1434,12 @@ bool pieces(int channels, P... p)
 {
     return channels % 8 == 0 && ((... | (uintptr_t)p) & 15) == 0;
 }
-// grid of the row kernels: `per_row` pieces in each of `rows` rows
-dim3 grid_rows(int rows, int per_row) { return dim3((per_row + 255) / 256, rows < 65535 ? rows : 65535); }
+// grid of the row kernels: `per_row` pieces in each of `rows` rows (one idle block for none: an
+// empty batch is no error)
+dim3 grid_rows(int rows, int per_row)
+{
+    return dim3(std::max(1, (per_row + 255) / 256), std::max(1, std::min(rows, 65535)));
+}
 
 int status(cudaError_t e) { return e == cudaSuccess ? TPF_OK : TPF_ERR_CUDA; }
 
