@@ -100,7 +100,8 @@ typedef struct tpflbm_params {
 
 /* Device bytes tpflbm_create_in needs for an nx x ny lattice with these
  * parameters (both population buffers, (phi u) of the previous step, field and
- * reduction scratch).  Returns 0 for invalid sizes. */
+ * reduction scratch, and for a lattice of up to 304 tiles of 32 x 8 nodes the words its tiles
+ * exchange when it advances many steps per launch).  Returns 0 for invalid sizes. */
 size_t tpflbm_workspace_bytes(int nx, int ny, const tpflbm_params *p);
 
 /* Create a lattice; the library allocates its device memory (cudaMalloc) on the
@@ -110,7 +111,9 @@ int tpflbm_create(int nx, int ny, const tpflbm_params *p, tpflbm_t *out);
 
 /* Same, in caller-owned device memory `workspace` of at least
  * tpflbm_workspace_bytes(nx, ny, p) bytes, 256-byte aligned, on the current
- * device; the caller keeps it alive until tpflbm_destroy and frees it after. */
+ * device; the caller keeps it alive until tpflbm_destroy and frees it after.  Without the
+ * last part, the words (288 bytes per node, nodes rounded up to 64, and 4 bytes per tile, each
+ * rounded up to 256 bytes), it is taken too, and the lattice steps with one launch per step. */
 int tpflbm_create_in(int nx, int ny, const tpflbm_params *p, void *workspace, size_t bytes,
                      tpflbm_t *out);
 

@@ -1093,10 +1093,12 @@ int tpflbm_create_in(int nx, int ny, const tpflbm_params* p, void* workspace, si
     int rc = validate(nx, ny, p, why);
     if (rc != TPF_OK) return fail(nullptr, rc, why);
     if (!workspace || ((uintptr_t)workspace & 255)) return fail(nullptr, TPF_ERR_INVALID_ARG, "workspace must be 256-byte aligned device memory");
-    if (bytes < layout_of(nx, ny, p->storage, true).total) return fail(nullptr, TPF_ERR_INVALID_ARG, "workspace too small");
+    if (bytes < layout_of(nx, ny, p->storage, false).total) return fail(nullptr, TPF_ERR_INVALID_ARG, "workspace too small");
+    // (without room for the words of the many-step kernel the lattice does without it)
+    const bool many = bytes >= layout_of(nx, ny, p->storage, true).total;
     tpflbm_t h = new (std::nothrow) tpflbm;
     if (!h) return fail(nullptr, TPF_ERR_OOM, "host allocation failed");
-    rc = finish_create(h, nx, ny, p, workspace, bytes, false, true);
+    rc = finish_create(h, nx, ny, p, workspace, bytes, false, many);
     if (rc != TPF_OK) {
         g_create_error = h->err_msg;
         delete h;
