@@ -617,9 +617,15 @@ constexpr int kStagePlanes = 9;
 // CTAs on each of 152 SMs (its registers allow no more: the line lies where the tiles stop
 // having a CTA each; setup_many checks it against the device).  kManySteps steps per launch,
 // so that no launch holds the GPU for more than a few milliseconds.
+//
+// kManyMin: steps of a call, or its rest, from which it takes the many-step kernel.  A launch of
+// that kernel costs its set-up (word list, masks, walls) and a cooperative start.  us per call of
+// 1, 2, 3, 4 steps, many-step kernel / one launch per step: 128 x 32 12.3/8.2, 14.4/16.4, 16.4/24.6,
+// 20.4/32.8; 512 x 128 14.4/8.2, 18.4/16.4, 20.5/24.6, 24.6/32.8, with FP16 16.9/12.2, 22.5/24.4,
+// 26.6/36.7, 30.7/48.8.  The states are the same bit for bit.
 constexpr int kManyBX = 32, kManyBY = 8;
 constexpr int kManyMaxTiles = 2 * 152;
-constexpr long long kManySteps = 1024;
+constexpr long long kManySteps = 1024, kManyMin = 3;
 bool many_tiles(int nx, int ny, int& tx, int& ty)
 {
     tx = (nx + kManyBX - 1) / kManyBX;
@@ -1160,13 +1166,12 @@ int tpflbm_step(tpflbm_t h, long long nsteps)
 {
     if (!h || nsteps < 0) return TPF_ERR_INVALID_ARG;
     if (h->many_fn) {
-        while (nsteps > 0) {
+        while (nsteps >= kManyMin) {
             const int n = (int)(nsteps < kManySteps ? nsteps : kManySteps);
             TPF_CUDA(h, launch_many(h, n));
             nsteps -= n;
             h->t += n;
         }
-        return TPF_OK;
     }
     // whole chunks from a CUDA graph when the stream can be captured (not the legacy
     // default stream); kGraphSteps is even, so a chunk leaves the parity unchanged
