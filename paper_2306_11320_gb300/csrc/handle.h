@@ -49,6 +49,10 @@ struct tpflbm {
     // steps each has done, and the words they exchange
     const void* many_fn = nullptr;
     int many_tx = 0, many_ty = 0;
+    // end of its last call and that call's stream, where its grid shares the GPU badly (null
+    // otherwise; see grid_has_room)
+    cudaEvent_t many_ev = nullptr;
+    cudaStream_t many_stream = nullptr;
     uint32_t* count = nullptr;
     uint4* words = nullptr;
     // CUDA graphs of kGraphSteps steps starting from pop[0] / pop[1] (captured on first use)
