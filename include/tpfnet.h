@@ -30,9 +30,11 @@ int tpfnet_conv3x3(const void *x, int N, int H, int W, int Cin, const void *wt, 
  * runs for a shape, given 16-byte aligned tensors: the width in output channels of the
  * tcgen05 kernels' tiles (32, 64, 128 or 256), or 0 for the mma.sync kernel.  The
  * tcgen05 kernels take pixel blocks of 128 (8 x 16, or BW x BH with BW = min(W, 128)
- * dividing both 128 and W and BH dividing H) and, from 1,024 pixels up, images of any
- * other extent; they stage operands with TMA and accumulate in tensor memory.  (From
- * 768 input channels up an image of other extents takes the mma.sync kernel.) */
+ * dividing both 128 and W and BH dividing H); they stage operands with TMA and accumulate
+ * in tensor memory.  Images of other extents take them too, from 1,024 pixels up, where the
+ * staged blocks of all input channels and the weights fit: with more than 152 tiles two CTAs
+ * have to share an SM's memory, and wide layers (from 128 or 192 input channels on, by the
+ * tile's width) take the mma.sync kernel then. */
 int tpfnet_conv3x3_tcgen05(int N, int H, int W, int Cin, int Cout);
 
 /* 1 when tpfnet_conv3x3_wgrad runs a tcgen05 kernel for a shape (W a multiple of 64, or W of 8

@@ -1461,7 +1461,10 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
     return fn;
 }
 
-// Images of fewer pixels whose blocks do not divide evenly stay on the mma.sync kernels.
+// Images of fewer pixels whose blocks do not divide evenly stay on the mma.sync kernels: no level
+// of a network has them, and they keep those kernels in use.  It is not where the two are level
+// (us forward and weight gradient, tcgen05 / mma.sync: 31 x 33, 64 -> 64 4.9/17.5 and 4.4/9.1, 9 x 11
+// 4.8/16.1 and 4.3/7.1).
 constexpr long long kRaggedPixels = 1024;
 
 // Shapes the tcgen05 convolutions take: images that divide into pixel blocks of BW x BH = 128
@@ -1528,39 +1531,63 @@ bool launch_tc(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, cons
     return true;
 }
 
-// The halo form, for channel counts whose boxes fit in shared memory; false (nothing launched)
-// otherwise.
-template <int KC, int MT>
-bool launch_halo(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, const float* bias, int Cout, int relu,
-                 bf16* y, int ldy, const bf16* mask, cudaStream_t s, int BN)
+// The kernel that a convolution of 16-byte aligned tensors takes: bn output channels per tile (0:
+// the mma.sync kernel), KC channels per chunk, and the halo form (MT blocks per CTA, its weight
+// stages, its shared memory) or the per-tap one (st.S = 0; blocks of BW x BH).  The one place
+// where this is decided, for the launches and for tpfnet_conv3x3_tcgen05.
+struct ConvPlan {
+    int bn, KC, MT, smem, BW, BH;
+    HaloStages st;
+};
+ConvPlan plan_conv(int N, int H, int W, int Cin, int Cout)
 {
-    const int kc = Cin / KC, a = kc * halo_bytes(MT, KC) + 1024, b = BN * KC * 2;
-    if (kc > kHaloChunks) return false;
-    // The fewest and largest weight stages that fit: a wait and its loop cost about as much as
-    // eight MMAs.  With more CTAs than SMs, two to an SM: all nine taps at once, three at a
-    // time, or one; where the boxes leave no room for that, the per-tap kernel is the better
-    // one ((4, 32, 128, 384, 128): 22.9 us against 31.1, (4, 16, 64, 256, 256): 16.8 against
-    // 17.7).  With at most one CTA per SM its whole shared memory, and parts of a tap if need be.
-    const long long blocks = (long long)N * ((H + 15) / 16) * ((W + 8 * MT - 1) / (8 * MT)), ctas = blocks * (Cout / BN);
-    const int limit = ctas > 152 ? 112 * 1024 : kHaloSmem;
-    HaloStages st{0, 0, 0};
-    auto take = [&](int T, int CC, int S) {
-        if (st.S || CC < 1 || kc % CC || (long long)a + (long long)S * T * CC * b > limit) return;
-        st = {T, CC, S};
-    };
-    take(9, kc, 1);
-    take(3, kc, 3);
-    take(1, kc, 4);
-    take(1, kc, 3);
-    if (ctas <= 152) {
-        take(1, kc / 2, 4);
-        take(1, kc / 3, 4);
-        take(1, 1, 4);
+    ConvPlan p{};
+    p.bn = tc_bn(N, H, W, Cout, p.BW, p.BH);
+    p.KC = Cin % 64 == 0 ? 64 : 32;
+    const int kc = Cin / p.KC;
+    if (!p.bn || kc < 1) return ConvPlan{};
+    const bool any = p.BW == 0;  // an extent that only the halo form takes
+    if ((H % 16 == 0 && W % 8 == 0) || any) {
+        // two blocks per CTA where that still gives every SM a CTA (half the weight traffic)
+        const long long pairs = (long long)N * ((H + 15) / 16) * ((W + 15) / 16);
+        p.MT = (W % 16 == 0 || any) && pairs * (Cout / p.bn) >= 152 ? 2 : 1;
+        const int a = kc * halo_bytes(p.MT, p.KC) + 1024, b = p.bn * p.KC * 2;
+        // The fewest and largest weight stages that fit: a wait and its loop cost about as much as
+        // eight MMAs.  With more CTAs than SMs, two to an SM: all nine taps at once, three at a
+        // time, or one; where the boxes leave no room for that, the per-tap kernel is the better
+        // one ((4, 32, 128, 384, 128): 22.9 us against 31.1, (4, 16, 64, 256, 256): 16.8 against
+        // 17.7).  With at most one CTA per SM its whole shared memory, and parts of a tap if need be.
+        const long long blocks = (long long)N * ((H + 15) / 16) * ((W + 8 * p.MT - 1) / (8 * p.MT));
+        const long long ctas = blocks * (Cout / p.bn);
+        const int limit = ctas > 152 ? 112 * 1024 : kHaloSmem;
+        auto take = [&](int T, int CC, int S) {
+            if (p.st.S || CC < 1 || kc % CC || (long long)a + (long long)S * T * CC * b > limit) return;
+            p.st = {T, CC, S};
+        };
+        if (kc <= kHaloChunks) {
+            take(9, kc, 1);
+            take(3, kc, 3);
+            take(1, kc, 4);
+            take(1, kc, 3);
+            if (ctas <= 152) {
+                take(1, kc / 2, 4);
+                take(1, kc / 3, 4);
+                take(1, 1, 4);
+            }
+        }
+        p.smem = a + p.st.S * p.st.T * p.st.CC * b;
+        if (!p.st.S && any) return ConvPlan{};
     }
-    if (!st.S) return false;
-    const int smem = a + st.S * st.T * st.CC * b;
+    return p;
+}
+
+// The halo form; false (nothing launched) when it cannot be.
+template <int KC, int MT>
+bool launch_halo(const ConvPlan& p, const bf16* x, int N, int H, int W, int Cin, const bf16* wt, const float* bias, int Cout,
+                 int relu, bf16* y, int ldy, const bf16* mask, cudaStream_t s)
+{
     CUtensorMap mx, mw;
-    if (!pixel_map(&mx, x, N, H, W, Cin, KC, 8 * MT + 2, kHaloRows) || !weight_map(&mw, wt, Cin, Cout, KC, BN, st.T))
+    if (!pixel_map(&mx, x, N, H, W, Cin, KC, 8 * MT + 2, kHaloRows) || !weight_map(&mw, wt, Cin, Cout, KC, p.bn, p.st.T))
         return false;
     // set on every call (the attribute belongs to the current device), and always to the same size:
     // another thread may be between its setting and its launch
@@ -1568,40 +1595,27 @@ bool launch_halo(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, co
         cudaGetLastError();
         return false;
     }
-    dim3 grd((unsigned)blocks, Cout / BN);
-    launch_pdl(k_conv3x3_halo<KC, MT>, grd, 128 * MT, smem, s, mx, mw, H, W, Cin, Cout, BN, st, bias, relu, y, ldy, mask);
+    const dim3 grd((unsigned)(N * ((H + 15) / 16) * ((W + 8 * MT - 1) / (8 * MT))), Cout / p.bn);
+    launch_pdl(k_conv3x3_halo<KC, MT>, grd, 128 * MT, p.smem, s, mx, mw, H, W, Cin, Cout, p.bn, p.st, bias, relu, y, ldy, mask);
     return true;
 }
 
 bool conv_tc(const bf16* x, int N, int H, int W, int Cin, const bf16* wt, const float* bias, int Cout, int relu,
              bf16* y, int ldy, const bf16* mask, cudaStream_t s)
 {
-    int BW = 0, BH = 0;
-    const int bn = tc_bn(N, H, W, Cout, BW, BH);
-    if (!bn || (((uintptr_t)x | (uintptr_t)wt | (uintptr_t)y | (uintptr_t)mask) & 15) || ldy % 8) return false;
-    if ((H % 16 == 0 && W % 8 == 0) || !BW) {
-        // two blocks per CTA where that still gives every SM a CTA (half the weight traffic)
-        const long long pairs = (long long)N * ((H + 15) / 16) * ((W + 15) / 16);
-        const bool two = (W % 16 == 0 || !BW) && pairs * (Cout / bn) >= 152;
-        const auto f = Cin % 64 == 0 ? (two ? launch_halo<64, 2> : launch_halo<64, 1>)
-                                     : (two ? launch_halo<32, 2> : launch_halo<32, 1>);
-        if (f(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, bn)) return true;
-        if (!BW) return false;
+    if ((((uintptr_t)x | (uintptr_t)wt | (uintptr_t)y | (uintptr_t)mask) & 15) || ldy % 8) return false;
+    const ConvPlan p = plan_conv(N, H, W, Cin, Cout);
+    if (!p.bn) return false;
+    if (p.st.S) {
+        const auto f = p.KC == 64 ? (p.MT == 2 ? launch_halo<64, 2> : launch_halo<64, 1>)
+                                  : (p.MT == 2 ? launch_halo<32, 2> : launch_halo<32, 1>);
+        return f(p, x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s);
     }
-    if (Cin % 64 == 0) {
-        switch (bn) {
-        case 256: return launch_tc<256, 64>(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, BW, BH);
-        case 128: return launch_tc<128, 64>(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, BW, BH);
-        case 64: return launch_tc<64, 64>(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, BW, BH);
-        default: return launch_tc<32, 64>(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, BW, BH);
-        }
-    }
-    switch (bn) {
-    case 256: return launch_tc<256, 32>(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, BW, BH);
-    case 128: return launch_tc<128, 32>(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, BW, BH);
-    case 64: return launch_tc<64, 32>(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, BW, BH);
-    default: return launch_tc<32, 32>(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, BW, BH);
-    }
+    const auto f = p.KC == 64 ? (p.bn == 256 ? launch_tc<256, 64> : p.bn == 128 ? launch_tc<128, 64>
+                                 : p.bn == 64 ? launch_tc<64, 64> : launch_tc<32, 64>)
+                              : (p.bn == 256 ? launch_tc<256, 32> : p.bn == 128 ? launch_tc<128, 32>
+                                 : p.bn == 64 ? launch_tc<64, 32> : launch_tc<32, 32>);
+    return f(x, N, H, W, Cin, wt, bias, Cout, relu, y, ldy, mask, s, p.BW, p.BH);
 }
 
 // CTAs over which the 64 x 1 segments of an image batch are split, `per` segments each: about as
@@ -1735,9 +1749,8 @@ int tpfnet_flip_weights(int layers, const void* const* wt, const int* cin, const
 
 int tpfnet_conv3x3_tcgen05(int N, int H, int W, int Cin, int Cout)
 {
-    int BW = 0, BH = 0;
     if (N < 1 || H < 1 || W < 1 || Cin % kKC || Cout % 32 || !encode_fn()) return 0;
-    return tc_bn(N, H, W, Cout, BW, BH);
+    return plan_conv(N, H, W, Cin, Cout).bn;
 }
 
 int tpfnet_conv3x3_wgrad_tcgen05(int N, int H, int W, int Cin, int Cout)
