@@ -43,7 +43,7 @@ struct tpflbm {
     bool tma = false;
     tpf::TmaMaps maps[2]{};             // maps[c]: reading pop[c]
     tpf::SeamMaps smaps[2]{};
-    int bx0 = 0, by0 = 0, ntbx = 0, ntby = 0, grid_tma = 0;
+    int bx0 = 0, by0 = 0, ntbx = 0, ntby = 0, grid_tma = 0, lead = 0;
     int2* tiles = nullptr;              // (x0, y0) of the TMA tiles in the order the kernel walks them
     // many-step kernel (many_fn is null where the lattice does not take it): its tiles, the
     // steps each has done, and the words they exchange

@@ -303,10 +303,9 @@ __device__ __forceinline__ void collide_push(const DevParams& P, typename S::ele
 }
 
 // One tile through the general path: thread loads, ghost values and every boundary
-// rule.  Used for lattices whose rows do not meet TMA alignment, by the batched
-// ensemble, in the TMA kernel for the tiles next to a periodic seam and the ragged
-// tiles, and by the many-step kernel.  The tile covers nodes [x0, x0 + w) x [y0, y0 + h),
-// 1 <= w <= BX, 1 <= h <= BY.
+// rule.  Used for lattices whose rows do not meet TMA alignment or that are periodic in x and at
+// most one tile wide, by the batched ensemble, and in the TMA kernel for the tiles next to a
+// periodic y seam.  The tile covers nodes [x0, x0 + w) x [y0, y0 + h), 1 <= w <= BX, 1 <= h <= BY.
 //
 // One thread per ring node issues that node's loads together with its own node's, so the
 // tile waits on one round trip to memory whatever its extent; ghost ring nodes take
@@ -315,7 +314,9 @@ __device__ __forceinline__ void collide_push(const DevParams& P, typename S::ele
 // NODES: each node of a boundary tile that can pushes like an interior one (256-lattice
 // ensemble, FP32 0.403 -> 0.386 ms per step, FP16 0.82 -> 0.67); without it a tile that touches
 // the boundary pushes by the rules as a whole, which is the better code inside the TMA kernel
-// (256 x 1024 FP16, a quarter of whose tiles come here: 22.4 us per step against 25.1).
+// (both axes periodic, us per step without / with: 1024 x 1024 FP16 70.8 / 74.0, 2048 x 64 FP16
+// 13.8 / 14.5, FP32 9.4 / 9.8, 256 x 1024 FP32 18.6 / 18.9, all before the CTAs with such tiles
+// took fewer others).
 template <int BX, int BY, class S, bool NODES>
 __device__ __forceinline__ void step_tile_general(const DevParams& P, const typename S::elem* __restrict__ A,
                                                   typename S::elem* __restrict__ B, float* __restrict__ phiu,
@@ -423,7 +424,7 @@ __device__ __forceinline__ void step_tile_general(const DevParams& P, const type
 // Tile b of an axis of n nodes: start and extent.  Whole tiles of B nodes first, the
 // ragged one last (tile_whole), or nt = ceil(n / B) tiles of nearly equal extent (tile_even:
 // the many-step kernel, whose step takes as long as its fullest tile; where tiles come in
-// waves, whole ones are 1% faster).
+// waves, whole ones are faster: 1702 x 226 51.5 us per step against 54.9).
 __device__ __forceinline__ void tile_whole(int n, int B, int b, int& x0, int& w)
 {
     x0 = b * B;
@@ -867,12 +868,12 @@ k_step_many(const DevParams P, const typename S::elem* A, typename S::elem* B, f
 // ------------------------------------------------------------ TMA kernel
 //
 // Persistent CTAs walk a tile list: first the TMA tiles, then the remaining tiles
-// through the general path.  TMA tiles are the whole tiles whose halo lies inside the
-// lattice along each periodic axis (x0 >= XP, x0 + BX + XP <= nx; y0 >= 2,
-// y0 + BY + 2 <= ny), which along a walled or inlet/outflow axis are all tiles, the ragged
-// last one too: there the box reaches past the lattice, the copy fills it with zeros, and
+// through the general path.  TMA tiles are, along a walled or inlet/outflow axis, all tiles, the
+// ragged last one too: there the box reaches past the lattice, the copy fills it with zeros, and
 // the tile takes its ghost ring nodes and its boundary nodes' FP16 records by the boundary
-// rules instead (along a periodic x axis of two tiles and more, too: see seam_side).  For a TMA tile one elected thread issues 3D bulk
+// rules instead; along a periodic x axis of two tiles and more, all tiles too (see seam_side); along
+// a periodic y axis, the tiles whose halo lies inside the lattice (y0 >= 2, y0 + BY + 2 <= ny).
+// For a TMA tile one elected thread issues 3D bulk
 // tensor copies (cp.async.bulk.tensor) of the 9 f planes and the 9 h planes over the
 // tile plus a one-node ring (widened to XP columns each side for the 16-byte rule),
 // the 9 g planes and the 2 (phi u) planes over the tile, and for FP16 the 3 planes of
@@ -1245,12 +1246,14 @@ constexpr int kTmaMinBlocks = kRef<S> ? TPF_TMA_BLOCKS_F16 : TPF_TMA_BLOCKS_F32;
 // 1024, a quarter of whose tiles are boundary tiles).
 // SEAM: x is periodic, so the lattice has seam tiles (the 2048 x 512 inlet/outflow channel, which
 // has none, takes 44.9 us per step with FP32 without their code and 45.2 with it).
-template <int BX, int BY, class S, bool RAGGED, bool SEAM>
+// REST: with the general path, for the tiles that a periodic y leaves to it (the 2048 x 512 channel,
+// which has none, takes 50.7 us per step with FP16 without that code and 51.3 with it).
+template <int BX, int BY, class S, bool RAGGED, bool SEAM, bool REST>
 __global__ void __launch_bounds__(BX * BY, kTmaMinBlocks<S>)
 k_step_tma(const DevParams P, const __grid_constant__ TmaMaps maps, const typename S::elem* __restrict__ A,
            typename S::elem* __restrict__ B, float* __restrict__ phiu, const RefT* __restrict__ refA,
            RefT* __restrict__ refB, const int2* __restrict__ tiles, int bx0, int by0, int ntbx, int ntby,
-           int* __restrict__ err, const __grid_constant__ SeamMaps smaps)
+           int* __restrict__ err, const __grid_constant__ SeamMaps smaps, int lead)
 {
     using L = TmaLayout<BX, BY, S>;
     constexpr int kStage = SEAM ? L::STAGE : L::OFF_C;  // = L::stage(SEAM)
@@ -1291,15 +1294,23 @@ k_step_tma(const DevParams P, const __grid_constant__ TmaMaps maps, const typena
         tma_issue_tile<BX, BY, S>(maps, smaps, dsm + s * kStage, &bar[s], x0, y0, SEAM ? seam_side<BX>(P, x0) : 0, P.nx);
     };
 
+    // This CTA's tiles: t, next(t), ...  With REST, the first `more` CTAs have one general tile more
+    // than the others and sit out the first `lead` rounds of the TMA tiles (tma_lead).
+    const int grid = gridDim.x, more = REST && lead > 0 ? nedge % grid : 0, early = lead * (grid - more);
+    auto next = [&](int t) {
+        if (REST && more > 0 && t < early) return t + grid - more < early ? t + grid - more : early + (int)blockIdx.x;
+        return t + grid;
+    };
     int it = 0;
     int t = blockIdx.x;
+    if (REST && more > 0) t = t < more ? early + t : t - more;
     if (tid == 0) {
         if (t < ntma) issue(t, 0, 0);
-        if (t + (int)gridDim.x < ntma) issue(t + gridDim.x, 1, 1);
+        if (next(t) < ntma) issue(next(t), 1, 1);
     }
-    for (; t < ntma; t += gridDim.x, ++it) {
+    for (; t < ntma; t = next(t), ++it) {
         const int s = it & 1;
-        const int tn = t + gridDim.x, t2 = t + 2 * gridDim.x;
+        const int tn = next(t), t2 = next(tn);
         PhiSmem<BX, BY>& sm = smb[s];
         // every thread waits for the stage itself; a thread whose wait ran out reads
         // stale (in-bounds) shared memory until the block votes at the next barrier
@@ -1337,32 +1348,32 @@ k_step_tma(const DevParams P, const __grid_constant__ TmaMaps maps, const typena
             refill();
         }
     }
-
-    // the tiles outside the TMA rectangle (periodic seams, ragged edges) through the
-    // general path, continuing this CTA's round-robin share; their ring lives in the
-    // stages, which the last TMA tile may still be reading
-    if (t - ntma < nedge) __syncthreads();
-    for (int e = t - ntma; e < nedge; e += gridDim.x) {
-        // map edge index e to the e-th tile outside the TMA rectangle
-        int idx = e, bx = 0, by = 0;
-        {
-            // tiles in row-major order, skipping the TMA rectangle
-            int row = 0;
-            for (row = 0; row < tilesy; ++row) {
-                const bool inner = row >= by0 && row < by0 + ntby;
-                const int cnt = inner ? tilesx - ntbx : tilesx;
-                if (idx < cnt) break;
-                idx -= cnt;
+    // the tiles outside the TMA rectangle (next to a periodic y seam) through the general path; their
+    // ring lives in the stages, which the last TMA tile may still be reading
+    if constexpr (REST) {
+        if ((int)blockIdx.x < nedge) __syncthreads();
+        for (int e = blockIdx.x; e < nedge; e += grid) {
+            // map edge index e to the e-th tile outside the TMA rectangle
+            int idx = e, bx = 0, by = 0;
+            {
+                // tiles in row-major order, skipping the TMA rectangle
+                int row = 0;
+                for (row = 0; row < tilesy; ++row) {
+                    const bool inner = row >= by0 && row < by0 + ntby;
+                    const int cnt = inner ? tilesx - ntbx : tilesx;
+                    if (idx < cnt) break;
+                    idx -= cnt;
+                }
+                by = row;
+                const bool inner = by >= by0 && by < by0 + ntby;
+                bx = (inner && idx >= bx0) ? idx + ntbx : idx;
             }
-            by = row;
-            const bool inner = by >= by0 && by < by0 + ntby;
-            bx = (inner && idx >= bx0) ? idx + ntbx : idx;
+            int x0, y0, w, h;
+            tile_whole(P.nx, BX, bx, x0, w);
+            tile_whole(P.ny, BY, by, y0, h);
+            step_tile_general<BX, BY, S, false>(P, A, B, phiu, refA, refB, *reinterpret_cast<RingSmem<BX, BY>*>(dsm), x0, y0,
+                                                w, h);
         }
-        int x0, y0, w, h;
-        tile_whole(P.nx, BX, bx, x0, w);
-        tile_whole(P.ny, BY, by, y0, h);
-        step_tile_general<BX, BY, S, false>(P, A, B, phiu, refA, refB, *reinterpret_cast<RingSmem<BX, BY>*>(dsm), x0, y0,
-                                            w, h);
     }
 }
 

@@ -798,16 +798,55 @@ bool make_map(CUtensorMap* m, CUtensorMapDataType dt, size_t esize, void* base, 
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// the TMA step kernel of a lattice: with or without ragged tiles, and with or without a seam (x
-// periodic), and its two stages
+// the TMA step kernel of a lattice: with or without ragged tiles, with or without a seam (x
+// periodic), with or without tiles for the general path (y periodic), and its two stages
 template <class S>
 int tma_smem(tpflbm_t h) { return 2 * TmaLayout<kBX, kBY, S>::stage(h->hp.bc_x == 0); }
 template <class S>
 auto tma_kernel(tpflbm_t h)
 {
     const bool ragged = h->nx % kBX || h->ny % kBY;
-    if (h->hp.bc_x == 0) return ragged ? k_step_tma<kBX, kBY, S, true, true> : k_step_tma<kBX, kBY, S, false, true>;
-    return ragged ? k_step_tma<kBX, kBY, S, true, false> : k_step_tma<kBX, kBY, S, false, false>;
+    // (y periodic: x is too.  With FP32 the kernel that has the general path is the faster one without
+    // tiles for it, too: 512 x 512 12.7 us per step against 13.0, 256 x 1024 12.6 against 12.8; with
+    // FP16 17.1 against 17.0.)
+    constexpr bool rest = !kRef<S>;
+    if (h->hp.bc_y == 1 && !rest) return k_step_tma<kBX, kBY, S, true, true, true>;
+    if (h->hp.bc_x == 0)
+        return ragged ? k_step_tma<kBX, kBY, S, true, true, rest> : k_step_tma<kBX, kBY, S, false, true, rest>;
+    return ragged ? k_step_tma<kBX, kBY, S, true, false, false> : k_step_tma<kBX, kBY, S, false, false, false>;
+}
+
+// Rounds of TMA tiles that the CTAs with the most general tiles sit out (k_step_tma): of 1 to 3 the
+// fewest that make the fullest CTA least full, when a general tile counts as 2.5 TMA tiles, or as
+// 1.6 where such CTAs are more than an eighth of all (by differences of step times: among
+// themselves they are quicker); one where they are more than half.  When those tiles came on top
+// of a full share, the step waited for them.  us per step with both axes periodic, on top / by this
+// rule: 256 x 1024 18.5 / 12.9, FP16 24.2 / 19.5; 2048 x 512 48.9 / 47.1, FP16 67.3 / 56.7; 4096 x 24 9.3 /
+// 8.1, FP16 15.2 / 11.2.
+int tma_lead(int ntma, int nedge, int grid)
+{
+    const int more = nedge % grid;
+    if (more == 0) return 0;
+    if (2 * more > grid) return 1;
+    const double weight = 8 * more > grid ? 1.6 : 2.5;
+    int best = 1;
+    double least = 1e30;
+    for (int lead = 1; lead <= 3; ++lead) {
+        const int n0 = grid - more, early = lead * n0;
+        double most = 0.0;
+        for (int b = 0; b < grid; ++b) {
+            double load = weight * (nedge / grid + (b < more));
+            if (b >= more)
+                for (int r = 0; r < lead; ++r) load += b - more + r * n0 < ntma;
+            if (ntma > early + b) load += (ntma - early - b + grid - 1) / grid;
+            most = std::max(most, load);
+        }
+        if (most < least) {
+            least = most;
+            best = lead;
+        }
+    }
+    return best;
 }
 
 template <class S>
@@ -892,6 +931,7 @@ void setup_tma(tpflbm_t h)
     }
     const int ntiles = ((nx + kBX - 1) / kBX) * ((ny + kBY - 1) / kBY);
     h->grid_tma = std::min(ntiles, per_sm * h->num_sms);
+    h->lead = tma_lead(h->ntbx * h->ntby, ntiles - h->ntbx * h->ntby, h->grid_tma);
     h->tma = true;
 }
 
@@ -1012,7 +1052,7 @@ void launch_step(tpflbm_t h)
     if (h->tma) {
         tma_kernel<S>(h)<<<h->grid_tma, kBX * kBY, tma_smem<S>(h), h->stream>>>(
             P, h->maps[c], A, B, h->phiu, h->ref[c], h->ref[c ^ 1], h->tiles, h->bx0, h->by0, h->ntbx, h->ntby,
-            h->err, h->smaps[c]);
+            h->err, h->smaps[c], h->lead);
     } else {
         dim3 grd((P.nx + kBX - 1) / kBX, (P.ny + kBY - 1) / kBY);
         k_step_general<kBX, kBY, S><<<grd, kBX * kBY, 0, h->stream>>>(P, A, B, h->phiu, h->ref[c], h->ref[c ^ 1]);
