@@ -33,6 +33,17 @@ __device__ __forceinline__ void pdl_enter()
     pdl_wait();
     pdl_next();
 }
+// The mma.sync kernels run for tens of microseconds and at one CTA after another on an SM: where
+// they have more CTAs than SMs, early ones pile up on the SMs that the kernel before left first, and
+// the kernel takes longer than its launch saved ((4, 15, 60, 256, 256) data gradient 148 us against
+// 88, (8, 30, 120, 128, 128) forward 83 against 68; with at most one CTA per SM (1, 31, 33, 64, 64)
+// forward 17.3 against 18.6).  So they start early, and let others, up to that many CTAs only.
+constexpr unsigned kPdlCtas = 152;
+__device__ __forceinline__ void pdl_enter_small()
+{
+    pdl_wait();
+    if (gridDim.x * gridDim.y * gridDim.z <= kPdlCtas) pdl_next();
+}
 template <class... K, class... A>
 cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
 {
@@ -47,6 +58,14 @@ cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem,
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, K(args)...);
+}
+template <class... K, class... A>
+void launch_pdl_small(void (*kernel)(K...), dim3 grid, dim3 block, cudaStream_t s, A... args)
+{
+    if ((unsigned long long)grid.x * grid.y * grid.z <= kPdlCtas)
+        launch_pdl(kernel, grid, block, 0, s, args...);
+    else
+        kernel<<<grid, block, 0, s>>>(K(args)...);
 }
 
 constexpr int kBM = 64;  // output pixels per CTA (one row segment)
@@ -72,7 +91,7 @@ k_conv3x3(const bf16* __restrict__ x, int N, int H, int W, int Cin, const bf16* 
           const float* __restrict__ bias, int Cout, int relu, bf16* __restrict__ y, int ldy,
           const bf16* __restrict__ mask)
 {
-    pdl_enter();
+    pdl_enter_small();
     __shared__ __align__(16) bf16 As[kBM][kKC + kPad];
     __shared__ __align__(16) bf16 Bs[BN][kKC + kPad];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -607,7 +626,7 @@ __global__ void __launch_bounds__(128)
 k_conv3x3_wgrad(const bf16* __restrict__ x, const bf16* __restrict__ dz, int N, int H, int W, int Cin, int Cout,
                 int pix_per_cta, float* __restrict__ dw, float* __restrict__ db)
 {
-    pdl_enter();
+    pdl_enter_small();
     constexpr int RB = WM / 16;        // row blocks
     constexpr int NG = 4 / RB;         // n-tile groups
     constexpr int NTW = 4 / NG;        // n-tiles (of 8 ci) per warp
@@ -1699,11 +1718,11 @@ static int conv_any(const void* x, int N, int H, int W, int Cin, const void* wt,
     const int wblocks = (W + kBM - 1) / kBM;
     if (Cout % 64 == 0) {
         dim3 grd(wblocks * N * H, Cout / 64);
-        launch_pdl(k_conv3x3<64>, grd, 128, 0, s, (const bf16*)x, N, H, W, Cin, (const bf16*)wt, bias, Cout, relu, (bf16*)y,
+        launch_pdl_small(k_conv3x3<64>, grd, 128, s, (const bf16*)x, N, H, W, Cin, (const bf16*)wt, bias, Cout, relu, (bf16*)y,
                                       ldy, (const bf16*)mask);
     } else {
         dim3 grd(wblocks * N * H, Cout / 32);
-        launch_pdl(k_conv3x3<32>, grd, 128, 0, s, (const bf16*)x, N, H, W, Cin, (const bf16*)wt, bias, Cout, relu, (bf16*)y,
+        launch_pdl_small(k_conv3x3<32>, grd, 128, s, (const bf16*)x, N, H, W, Cin, (const bf16*)wt, bias, Cout, relu, (bf16*)y,
                                       ldy, (const bf16*)mask);
     }
     return status(cudaGetLastError());
@@ -1808,10 +1827,10 @@ int tpfnet_conv3x3_wgrad(const void* x, const void* dz, int N, int H, int W, int
     splits = (P + per - 1) / per;
     dim3 grd(Cin / kWN, Cout / WM, 9 * (int)splits);
     if (WM == 64)
-        launch_pdl(k_conv3x3_wgrad<64>, grd, 128, 0, (cudaStream_t)stream, (const bf16*)x, (const bf16*)dz, N, H, W, Cin, Cout,
+        launch_pdl_small(k_conv3x3_wgrad<64>, grd, 128, (cudaStream_t)stream, (const bf16*)x, (const bf16*)dz, N, H, W, Cin, Cout,
                                                                    (int)per, dw, db);
     else
-        launch_pdl(k_conv3x3_wgrad<32>, grd, 128, 0, (cudaStream_t)stream, (const bf16*)x, (const bf16*)dz, N, H, W, Cin, Cout,
+        launch_pdl_small(k_conv3x3_wgrad<32>, grd, 128, (cudaStream_t)stream, (const bf16*)x, (const bf16*)dz, N, H, W, Cin, Cout,
                                                                    (int)per, dw, db);
     return status(cudaGetLastError());
 }
