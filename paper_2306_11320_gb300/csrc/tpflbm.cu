@@ -658,11 +658,12 @@ Layout layout_of(int nx, int ny, int storage, bool many)
     L.phiu = off; off = align256(off + 2 * (size_t)pl * 4);
     L.stage = off; off = align256(off + kStagePlanes * (size_t)pl * 4);
     L.red = off; off = align256(off + kRedDoubles * sizeof(double));
-    L.err = off; off = align256(off + 256);
     L.snap = off; off = align256(off + 3 * (size_t)pl * 4);
     // the TMA step kernel's tile list (x0, y0 per tile)
     L.tiles = off; off = align256(off + (size_t)((nx + kBX - 1) / kBX) * ((ny + kBY - 1) / kBY) * sizeof(int2));
-    // the many-step kernel's step counts per tile and its two word sets
+    // what create clears, in one piece: the error flag, the many-step kernel's step counts per tile
+    // and its two word sets
+    L.err = off; off = align256(off + 256);
     int mtx = 0, mty = 0;
     const bool words = many && many_tiles(nx, ny, mtx, mty);
     L.count = off; off = align256(off + (words ? (size_t)mtx * mty * sizeof(uint32_t) : 0));
@@ -1023,14 +1024,12 @@ int finish_create(tpflbm_t h, int nx, int ny, const tpflbm_params* p, void* ws, 
     h->tiles = (int2*)(b + L.tiles);
     h->count = (uint32_t*)(b + L.count);
     h->words = (uint4*)(b + L.words);
-    if (cudaMemset(h->err, 0, sizeof(int)) != cudaSuccess) return cuda_fail(h, cudaGetLastError(), "cudaMemset");
+    // (steps are numbered from 1: no word of a new lattice is valid)
+    if (cudaMemset(h->err, 0, L.total - L.err) != cudaSuccess) return cuda_fail(h, cudaGetLastError(), "cudaMemset");
     const bool f16 = p->storage == TPF_STORAGE_FP16;
     if (f16) setup_tma<StoreF16>(h);
     else setup_tma<StoreF32>(h);
-    if (many && L.total > L.count) {
-        // steps are numbered from 1: no word of a new lattice is valid
-        if (cudaMemset(h->count, 0, L.total - L.count) != cudaSuccess)
-            return cuda_fail(h, cudaGetLastError(), "cudaMemset");
+    if (L.total > L.count) {
         if (f16) setup_many<StoreF16>(h);
         else setup_many<StoreF32>(h);
     }

@@ -167,7 +167,9 @@ class Lattice:
                 raise TpfError(-1, "invalid lattice size or parameters")
             self._ws = torch.empty(nbytes + 256, dtype=torch.uint8, device="cuda")
             # the block may have been another tensor's, with work of this stream still to run on it
-            torch.cuda.current_stream().synchronize()
+            # (create itself waits for the default stream)
+            if torch.cuda.current_stream().cuda_stream:
+                torch.cuda.current_stream().synchronize()
             base = self._ws.data_ptr()
             aligned = (base + 255) & ~255
             rc = self.lib.tpflbm_create_in(self.nx, self.ny, C.byref(self._p), C.c_void_p(aligned),
