@@ -62,7 +62,7 @@ int tpfnet_conv3x3_dgrad(const void *dz, int N, int H, int W, int Cout, const vo
 /* The same pieces in the forms that a whole network's passes join, so that no concatenation,
  * split or ReLU mask is a pass of its own:
  *   conv3x3_into: the output goes to Cout channels of a tensor with ldy channels per pixel
- *     (y points at the first of them; ldy even);
+ *     (y points at the first of them, 4-byte aligned; ldy even);
  *   flip_weights: the flipped, transposed weights of up to 16 layers (host arrays of device
  *     pointers and sizes) in one launch;
  *   dgrad_masked: the data gradient from weights flipped before, zero where mask (laid out as

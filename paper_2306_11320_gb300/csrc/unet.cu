@@ -1715,6 +1715,8 @@ static int conv_any(const void* x, int N, int H, int W, int Cin, const void* wt,
     cudaStream_t s = (cudaStream_t)stream;
     if (conv_tc((const bf16*)x, N, H, W, Cin, (const bf16*)wt, bias, Cout, relu, (bf16*)y, ldy, (const bf16*)mask, s))
         return status(cudaGetLastError());
+    // the mma.sync kernel reads 16-byte pieces and writes pairs of channels
+    if ((((uintptr_t)x | (uintptr_t)wt) & 15) || ((uintptr_t)y & 3) || ldy % 2) return TPF_ERR_INVALID_ARG;
     const int wblocks = (W + kBM - 1) / kBM;
     if (Cout % 64 == 0) {
         dim3 grd(wblocks * N * H, Cout / 64);
