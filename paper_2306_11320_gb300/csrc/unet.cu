@@ -1813,7 +1813,7 @@ int tpfnet_conv3x3_dgrad(const void* dz, int N, int H, int W, int Cout, const vo
 int tpfnet_conv3x3_wgrad(const void* x, const void* dz, int N, int H, int W, int Cin, int Cout, float* dw, float* db,
                          void* stream)
 {
-    if (!x || !dz || !dw || Cin % kWN || Cout % 32) return TPF_ERR_INVALID_ARG;
+    if (!x || !dz || !dw || N < 1 || H < 1 || W < 1 || Cin % kWN || Cout % 32) return TPF_ERR_INVALID_ARG;
     if (wgrad_tc((const bf16*)x, (const bf16*)dz, N, H, W, Cin, Cout, dw, db, (cudaStream_t)stream))
         return status(cudaGetLastError());
     const int WM = Cout % 64 == 0 ? 64 : 32;
