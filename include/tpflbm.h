@@ -142,7 +142,9 @@ int tpflbm_init_forced(tpflbm_t h, const float *phi, const float *ux, const floa
 
 /* Advance nsteps >= 0 time steps, enqueued on the handle's stream; returns after
  * enqueueing.  Each step is one fused kernel launch, except that a lattice of up to 304
- * tiles of 32 x 8 nodes advances up to 1,024 steps per (cooperative) launch. */
+ * tiles of 32 x 8 nodes advances up to 1,024 steps per (cooperative) launch when the call has
+ * three steps and more and, from 153 to 228 tiles, no call of another such lattice is in
+ * flight on another stream.  The states do not depend on it. */
 int tpflbm_step(tpflbm_t h, long long nsteps);
 
 /* Wait for the steps enqueued so far and report whether they completed: TPF_OK, or
@@ -204,8 +206,8 @@ int tpflbm_diagnostics(tpflbm_t h, double out[8]);
  *   out   8 doubles, host or device memory; same meaning as tpflbm_diagnostics.
  *   stream cudaStream_t (NULL = legacy default stream); the call synchronises it.
  * tpflbm_state_buffers gives these pointers for a handle's own state.
- * The kernel's scratch (per-block partial sums) is a fixed array of 1024 x 8 + 8
- * doubles (65,600 bytes) compiled into the library; every GPU that loads the
+ * The kernel's scratch (per-block partial sums) is a fixed array of 1024 x 8 + 16
+ * doubles (65,664 bytes) compiled into the library; every GPU that loads the
  * library holds it until the process exits.  Any lattice the library accepts
  * (nx, ny >= 3, nx * ny <= 2^30) fits, because the kernel walks the lattice with
  * at most 1024 blocks; larger sizes and invalid arguments return
