@@ -93,6 +93,24 @@ int tpfnet_head_back_masked(const void *x, const float *dout, long long pixels, 
 int tpfnet_conv3x3_wgrad(const void *x, const void *dz, int N, int H, int W, int Cin, int Cout, float *dw,
                          float *db, void *stream);
 
+/* Parameter gradients whose float32 sums come out the same on every run: the kernels store what
+ * they would have added to dw and db, and one launch adds that up in one order.
+ *   wgrad_parts: the number of partial sums of conv3x3_wgrad_part for a shape (0: no such shape);
+ *   conv3x3_wgrad_part: partial sum p is stored at part + p (9 Cout Cin + Cout), laid out as dw and
+ *     then db; x, dz and part 16-byte aligned;
+ *   head_parts, head_back_part: the same for head_back_masked (p (C + 1) Cout; dW and then db; C 8,
+ *     16, ... 256, up to 8 outputs, x and dx 16-byte aligned);
+ *   sum_parts: for n <= 32 ranges, dst[i][k] += sum over p < parts[i] of part[i][p stride[i] + k],
+ *     k < count[i] (host arrays of device pointers and sizes; the ranges of dst do not overlap). */
+int tpfnet_wgrad_parts(int N, int H, int W, int Cin, int Cout);
+int tpfnet_conv3x3_wgrad_part(const void *x, const void *dz, int N, int H, int W, int Cin, int Cout, float *part,
+                              void *stream);
+int tpfnet_head_parts(long long pixels, int C, int Cout);
+int tpfnet_head_back_part(const void *x, const float *dout, long long pixels, int C, const float *Wt, int Cout,
+                          void *dx, float *part, void *stream);
+int tpfnet_sum_parts(int n, const float *const *part, const long long *stride, const int *count, const int *parts,
+                     float *const *dst, void *stream);
+
 /* d[k] = 0 where y[k] <= 0 (ReLU backward on bf16 tensors of `count` elements). */
 int tpfnet_relu_mask(void *d, const void *y, long long count, void *stream);
 

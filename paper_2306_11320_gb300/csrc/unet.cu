@@ -621,10 +621,10 @@ k_conv3x3_halo(const __grid_constant__ CUtensorMap mx, const __grid_constant__ C
 // accumulates in FP32 and adds into dW with atomics.  4 warps: WM/16 row blocks of
 // 16 output channels times 64/WM groups of n-tiles.
 constexpr int kWN = 32, kWK = 32;
-template <int WM>
+template <int WM, bool PART>
 __global__ void __launch_bounds__(128)
 k_conv3x3_wgrad(const bf16* __restrict__ x, const bf16* __restrict__ dz, int N, int H, int W, int Cin, int Cout,
-                int pix_per_cta, float* __restrict__ dw, float* __restrict__ db)
+                int pix_per_cta, float* __restrict__ dw, float* __restrict__ db, float* __restrict__ part)
 {
     pdl_enter_small();
     constexpr int RB = WM / 16;        // row blocks
@@ -645,6 +645,10 @@ k_conv3x3_wgrad(const bf16* __restrict__ x, const bf16* __restrict__ dz, int N, 
 #pragma unroll
     for (int j = 0; j < NTW; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
     float bacc = 0.f;
+    if constexpr (PART) {  // this split's own sums, stored (as in k_conv3x3_wgrad_tc)
+        dw = part + (size_t)split * ((size_t)9 * Cout * Cin + Cout);
+        db = dw + (size_t)9 * Cout * Cin;
+    }
     const bool do_bias = db && tap == 4 && blockIdx.x == 0;
 
     for (long long p0 = p_begin; p0 < p_end; p0 += kWK) {
@@ -698,11 +702,19 @@ k_conv3x3_wgrad(const bf16* __restrict__ x, const bf16* __restrict__ dz, int N, 
             const int co = co0 + rb * 16 + g + 8 * r;
             const int ci = ci0 + (ng * NTW + j) * 8 + 2 * tig;
             float* dst = dw + ((size_t)tap * Cout + co) * Cin + ci;
-            atomicAdd(dst, acc[j][2 * r]);
-            atomicAdd(dst + 1, acc[j][2 * r + 1]);
+            if constexpr (PART) {
+                dst[0] = acc[j][2 * r];
+                dst[1] = acc[j][2 * r + 1];
+            } else {
+                atomicAdd(dst, acc[j][2 * r]);
+                atomicAdd(dst + 1, acc[j][2 * r + 1]);
+            }
         }
     }
-    if (do_bias && tid < WM) atomicAdd(db + co0 + tid, bacc);
+    if (do_bias && tid < WM) {
+        if constexpr (PART) db[co0 + tid] = bacc;
+        else atomicAdd(db + co0 + tid, bacc);
+    }
 }
 
 // flipped transposes for the data gradients: wd[tap][ci][co] = w[8 - tap][co][ci], of up to
@@ -786,7 +798,8 @@ __device__ __forceinline__ void relu_back8(Piece& d, const Piece& y)
 // block.  db is summed from the dz boxes by four more warps in the CTAs of dw = -1 and the first
 // input channels, each thread eight channels of every fourth pixel.  Partial sums of a CTA go to
 // dw in vector reductions (dw off the 16-byte rule: one by one).  Blocks that reach past an image's
-// edge add nothing: dz is zero there.
+// edge add nothing: dz is zero there.  With PART the sums of each split are stored instead, for
+// k_sum_parts to add up in one order.
 //
 // Blocks: segments of 64 x 1 where the width allows, else 8 x 16.  The segments' order and their
 // split over CTAs decide which products meet in which float32 sum, and training amplifies that: a
@@ -821,10 +834,11 @@ __device__ __forceinline__ void red_add4(float* p, const uint32_t* r)
                  : "memory");
 }
 
-template <int CK, int BW, int BH>
+template <int CK, int BW, int BH, bool PART>
 __global__ void __launch_bounds__(256)
 k_conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap mdz, const __grid_constant__ CUtensorMap mx, int N, int H,
-                   int W, int Cin, int Cout, int tiles_per_cta, float* __restrict__ dw, float* __restrict__ db)
+                   int W, int Cin, int Cout, int tiles_per_cta, float* __restrict__ dw, float* __restrict__ db,
+                   float* __restrict__ part)
 {
     static_assert(BW % 8 == 0 && BW * BH % 64 == 0, "whole groups of eight rows, sixteen pixels per MMA and bias warp");
     constexpr int kPix = BW * BH, kDz = wg_dz(BW, BH), kX = wg_x(BW, BH, CK);
@@ -845,6 +859,10 @@ k_conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap mdz, const __grid_constan
     const int kStage = boxes * kDz + kX;
     const int bpr = (W + BW - 1) / BW, bpi = bpr * ((H + BH - 1) / BH), tiles = N * bpi;
     const int begin = split * tiles_per_cta, end = min(begin + tiles_per_cta, tiles), steps = max(end - begin, 0);
+    if constexpr (PART) {  // this split's own sums (of all taps, then of the bias), stored
+        dw = part + (size_t)split * ((size_t)9 * Cout * Cin + Cout);
+        db = dw + (size_t)9 * Cout * Cin;
+    }
     const bool bias = db && g == 0 && blockIdx.y == 0;
 
     if (tid == 0) {
@@ -967,7 +985,9 @@ k_conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap mdz, const __grid_constan
             float* dst = dw + ((size_t)(3 * (c / CK) + g) * Cout + co) * Cin + ci0 + c % CK;
 #pragma unroll
             for (int j = 0; j < 16; j += 4) {
-                if (vec) {
+                if constexpr (PART) {
+                    *reinterpret_cast<uint4*>(dst + j) = make_uint4(r[j], r[j + 1], r[j + 2], r[j + 3]);
+                } else if (vec) {
                     red_add4(dst + j, r + j);
                 } else {
 #pragma unroll
@@ -978,10 +998,80 @@ k_conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap mdz, const __grid_constan
     }
     tc_fence_before();
     __syncthreads();
-    if (bias && tid < 128 && co0 + tid < Cout)  // one atomic per CTA and channel
-        atomicAdd(db + co0 + tid, (sdb[0][tid] + sdb[1][tid]) + (sdb[2][tid] + sdb[3][tid]));
+    if (bias && tid < 128 && co0 + tid < Cout) {  // one atomic per CTA and channel
+        const float v = (sdb[0][tid] + sdb[1][tid]) + (sdb[2][tid] + sdb[3][tid]);
+        if constexpr (PART) db[co0 + tid] = v;
+        else atomicAdd(db + co0 + tid, v);
+    }
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
+}
+
+// dst[k] += the sum over p of part[p * stride + k], for up to kMaxSums ranges in one launch: the
+// parameter gradients of a backward pass from the partial sums that its kernels stored.  Added in
+// one order, with the rounding errors carried along, so the result is the same on every run and the
+// nearest float32 to the partial sums' sum but for one rounding.  A thread takes four words of a
+// range of up to 64 partial sums that allows it, a warp one word of any other (the head's: 304).  Bound by
+// reading the partial sums (22 M words, 88 MB, for the whole network at batch 4).
+constexpr int kMaxSums = 32;
+struct SumList {
+    const float* part[kMaxSums];
+    float* dst[kMaxSums];
+    long long stride[kMaxSums];
+    int count[kMaxSums], parts[kMaxSums];
+    int first[kMaxSums + 1];  // first block of each range
+    uint32_t four;            // bit i: range i goes by four words
+};
+struct Carried {  // a float32 sum and the rounding errors it left
+    float s, c;
+    __device__ __forceinline__ void add(float v)
+    {
+        const float t = s + v, b = t - s;
+        c += (s - (t - b)) + (v - b);
+        s = t;
+    }
+};
+__global__ void __launch_bounds__(256) k_sum_parts(const SumList L, int n)
+{
+    pdl_enter();
+    int i = 0;
+    while (i + 1 < n && (int)blockIdx.x >= L.first[i + 1]) ++i;
+    const int block = (int)blockIdx.x - L.first[i], parts = L.parts[i];
+    const long long stride = L.stride[i];
+    if (L.four >> i & 1) {
+        const int k = 4 * (block * 256 + (int)threadIdx.x);
+        if (k >= L.count[i]) return;
+        float4* dst = reinterpret_cast<float4*>(L.dst[i] + k);
+        const float* p = L.part[i] + k;
+        const float4 d = *dst;
+        Carried a[4] = {{d.x, 0.f}, {d.y, 0.f}, {d.z, 0.f}, {d.w, 0.f}};
+        for (int q = 0; q < parts; q += 8, p += 8 * stride) {
+            float4 v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                v[j] = q + j < parts ? *reinterpret_cast<const float4*>(p + j * stride) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {  // (adding zero changes nothing)
+                a[0].add(v[j].x);
+                a[1].add(v[j].y);
+                a[2].add(v[j].z);
+                a[3].add(v[j].w);
+            }
+        }
+        *dst = make_float4(a[0].s + a[0].c, a[1].s + a[1].c, a[2].s + a[2].c, a[3].s + a[3].c);
+        return;
+    }
+    const int k = block * 8 + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (k >= L.count[i]) return;
+    const float* p = L.part[i] + k;
+    Carried a{lane == 0 ? L.dst[i][k] : 0.f, 0.f};
+    for (int q = lane; q < parts; q += 32) a.add(p[q * stride]);
+    for (int o = 16; o > 0; o >>= 1) {
+        const float s = __shfl_down_sync(0xffffffffu, a.s, o), c = __shfl_down_sync(0xffffffffu, a.c, o);
+        a.add(s);
+        a.c += c;
+    }
+    if (lane == 0) L.dst[i][k] = a.s + a.c;
 }
 
 __global__ void k_relu_mask8(bf16* __restrict__ d, const bf16* __restrict__ y, long long pieces)
@@ -1229,14 +1319,14 @@ k_head8(const bf16* __restrict__ x, long long pixels, int C, const float* __rest
 // Head gradients, C = 8 G with G a power of two up to 32: lane l of a warp holds channels
 // 8 (l % G) .. + 7 of pixel l / G, their weights and the FP32 partial sums of dW and db in
 // registers over all its pixels; shuffles, shared memory and one atomic per block and
-// parameter add them up.  Bound by reading x and dout and writing dx.  (Adding every
+// parameter add them up (with `part` a block stores its sums, of dW and then of db).  Bound by reading x and dout and writing dx.  (Adding every
 // pixel's products into shared memory with atomics serialised each warp on the same C x CO
 // words: 1,147 us at 262,144 pixels, C = 32, 5 outputs.)
 template <int CO>
 __global__ void __launch_bounds__(256)
 k_head_back8(const bf16* __restrict__ x, const float* __restrict__ dout, long long pixels, int C,
              const float* __restrict__ Wt, bf16* __restrict__ dx, float* __restrict__ dW, float* __restrict__ db,
-             int relu)
+             int relu, float* __restrict__ part)
 {
     pdl_enter();
     extern __shared__ float sh[];  // C * CO + CO sums
@@ -1283,15 +1373,21 @@ k_head_back8(const bf16* __restrict__ x, const float* __restrict__ dout, long lo
             for (int j = 0; j < 8; ++j) acc[j][o] += __shfl_xor_sync(0xffffffffu, acc[j][o], m);
         }
     }
-    if (ps == 0) {
+    for (int q = 0; q < 8; ++q) {  // warp by warp, in one order
+        if (warp == q && ps == 0) {
 #pragma unroll
-        for (int o = 0; o < CO; ++o) {
+            for (int o = 0; o < CO; ++o) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) atomicAdd(&sh[(8 * cg + j) * CO + o], acc[j][o]);
-            if (cg == 0) atomicAdd(&sh[C * CO + o], accb[o]);
+                for (int j = 0; j < 8; ++j) sh[(8 * cg + j) * CO + o] += acc[j][o];
+                if (cg == 0) sh[C * CO + o] += accb[o];
+            }
         }
+        __syncthreads();
     }
-    __syncthreads();
+    if (part) {
+        for (int k = threadIdx.x; k < (C + 1) * CO; k += 256) part[(size_t)blockIdx.x * ((C + 1) * CO) + k] = sh[k];
+        return;
+    }
     for (int k = threadIdx.x; k < C * CO; k += 256) atomicAdd(&dW[k], sh[k]);
     for (int k = threadIdx.x; k < CO; k += 256) atomicAdd(&db[k], sh[C * CO + k]);
 }
@@ -1653,55 +1749,82 @@ long long wgrad_splits(int N, int H, int W, int Cin, int Cout, long long& per)
     return (nchunks + per - 1) / per;
 }
 
+// Which weight gradient a shape takes, for 16-byte aligned x and dz, and how its pixels are split
+// over CTAs: rows of whole segments, images that divide into blocks of 8 x 16, and any other large
+// enough take the tcgen05 kernel with CK input channels per CTA (CK = 0: the mma.sync kernel, WM
+// output channels per CTA), in `splits` runs of `per` blocks (pixels).
+struct WgradPlan {
+    int CK, WM, splits, per;
+    bool rows;
+};
+WgradPlan plan_wgrad(int N, int H, int W, int Cin, int Cout, bool aligned)
+{
+    WgradPlan p{};
+    const long long P = (long long)N * H * W;
+    long long splits, per;
+    p.rows = W % kWgPix == 0;
+    if (!aligned || !encode_fn() || (!p.rows && !(H % 16 == 0 && W % 8 == 0) && P < kRaggedPixels)) {
+        p.WM = Cout % 64 == 0 ? 64 : 32;
+        // split the pixels so that the grid fills the GPU a few times over
+        const long long base = 9LL * (Cin / kWN) * (Cout / p.WM);
+        splits = std::max(1LL, std::min((152LL * 8 + base - 1) / base, (P + kWK - 1) / kWK));
+        per = ((P + splits - 1) / splits + kWK - 1) / kWK * kWK;
+        splits = (P + per - 1) / per;
+    } else {
+        p.CK = Cin % 64 == 0 ? 64 : 32;
+        if (p.rows) {
+            splits = wgrad_splits(N, H, W, Cin, Cout, per);
+        } else {
+            // split the blocks over about as many CTAs as run at once
+            const int stage = (Cout > 64 ? 2 : 1) * wg_dz(8, 16) + wg_x(8, 16, p.CK);
+            const long long tiles = (long long)N * ((H + 15) / 16) * ((W + 7) / 8);
+            const long long base = 3LL * ((Cout + 127) / 128) * (Cin / p.CK);
+            const long long target = kWgStages * stage + 1024 <= 112 * 1024 ? 304 : 152;
+            splits = std::max(1LL, std::min(tiles, target / base));
+            per = (tiles + splits - 1) / splits;
+            splits = (tiles + per - 1) / per;
+        }
+    }
+    p.splits = (int)splits;
+    p.per = (int)per;
+    return p;
+}
+
 // The weight gradient on blocks of BW x BH; false (nothing launched) when it cannot be.
 template <int CK, int BW, int BH>
-bool launch_wgrad(const bf16* x, const bf16* dz, int N, int H, int W, int Cin, int Cout, float* dw, float* db,
-                  cudaStream_t s)
+bool launch_wgrad(const WgradPlan& p, const bf16* x, const bf16* dz, int N, int H, int W, int Cin, int Cout, float* dw,
+                  float* db, float* part, cudaStream_t s)
 {
-    const auto kern = k_conv3x3_wgrad_tc<CK, BW, BH>;
+    const auto kern = part ? k_conv3x3_wgrad_tc<CK, BW, BH, true> : k_conv3x3_wgrad_tc<CK, BW, BH, false>;
     CUtensorMap mdz, mx;
     if (!pixel_map(&mdz, dz, N, H, W, Cout, 64, BW, BH) || !pixel_map(&mx, x, N, H, W, Cin, CK, BW, BH + 2)) return false;
-    const int stage = (Cout > 64 ? 2 : 1) * wg_dz(BW, BH) + wg_x(BW, BH, CK), smem = kWgStages * stage + 1024;
+    const int smem = kWgStages * ((Cout > 64 ? 2 : 1) * wg_dz(BW, BH) + wg_x(BW, BH, CK)) + 1024;
     // (always the size of two dz boxes: another thread may be between its setting and its launch)
     constexpr int kMost = kWgStages * (2 * wg_dz(BW, BH) + wg_x(BW, BH, CK)) + 1024;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    const int ctiles = (Cout + 127) / 128, itiles = Cin / CK;
-    long long splits, per;
-    if (BH == 1) {
-        splits = wgrad_splits(N, H, W, Cin, Cout, per);
-    } else {
-        // split the blocks over about as many CTAs as run at once
-        const long long tiles = (long long)N * ((H + BH - 1) / BH) * ((W + BW - 1) / BW);
-        const long long base = 3LL * ctiles * itiles, target = smem <= 112 * 1024 ? 304 : 152;
-        splits = std::max(1LL, std::min(tiles, target / base));
-        per = (tiles + splits - 1) / splits;
-        splits = (tiles + per - 1) / per;
-    }
-    launch_pdl(kern, dim3(ctiles, itiles, 3 * (unsigned)splits), 256, smem, s, mdz, mx, N, H, W, Cin, Cout, (int)per, dw, db);
+    launch_pdl(kern, dim3((Cout + 127) / 128, Cin / CK, 3 * (unsigned)p.splits), 256, smem, s, mdz, mx, N, H, W, Cin, Cout,
+               p.per, dw, db, part);
     return true;
 }
 
-// shapes the tcgen05 weight gradient takes: rows of whole segments, images that divide into blocks
-// of 8 x 16, and any other large enough
-bool wgrad_blocks(int N, int H, int W)
+// The weight gradient by p; false (nothing launched) when that cannot be.  Adds into dw (and db),
+// or stores the splits' sums into part.
+bool wgrad(const WgradPlan& p, const bf16* x, const bf16* dz, int N, int H, int W, int Cin, int Cout, float* dw, float* db,
+           float* part, cudaStream_t s)
 {
-    return W % kWgPix == 0 || (H % 16 == 0 && W % 8 == 0) || (long long)N * H * W >= kRaggedPixels;
-}
-
-// The tcgen05 weight gradient for those shapes and 16-byte aligned x and dz; false (nothing
-// launched) otherwise.  Adds into dw (and db).
-bool wgrad_tc(const bf16* x, const bf16* dz, int N, int H, int W, int Cin, int Cout, float* dw, float* db,
-              cudaStream_t s)
-{
-    if ((((uintptr_t)x | (uintptr_t)dz) & 15) || !wgrad_blocks(N, H, W)) return false;
-    if (W % kWgPix == 0)
-        return Cin % 64 == 0 ? launch_wgrad<64, kWgPix, 1>(x, dz, N, H, W, Cin, Cout, dw, db, s)
-                             : launch_wgrad<32, kWgPix, 1>(x, dz, N, H, W, Cin, Cout, dw, db, s);
-    return Cin % 64 == 0 ? launch_wgrad<64, 8, 16>(x, dz, N, H, W, Cin, Cout, dw, db, s)
-                         : launch_wgrad<32, 8, 16>(x, dz, N, H, W, Cin, Cout, dw, db, s);
+    if (p.CK) {
+        const auto f = p.rows ? (p.CK == 64 ? launch_wgrad<64, kWgPix, 1> : launch_wgrad<32, kWgPix, 1>)
+                              : (p.CK == 64 ? launch_wgrad<64, 8, 16> : launch_wgrad<32, 8, 16>);
+        return f(p, x, dz, N, H, W, Cin, Cout, dw, db, part, s);
+    }
+    const dim3 grd(Cin / kWN, Cout / p.WM, 9 * p.splits);
+    const auto f = part ? (p.WM == 64 ? k_conv3x3_wgrad<64, true> : k_conv3x3_wgrad<32, true>)
+                        : (p.WM == 64 ? k_conv3x3_wgrad<64, false> : k_conv3x3_wgrad<32, false>);
+    launch_pdl_small(f, grd, 128, s, x, dz, N, H, W, Cin, Cout, p.per, dw, db, part);
+    return true;
 }
 
 }  // namespace
@@ -1774,9 +1897,16 @@ int tpfnet_conv3x3_tcgen05(int N, int H, int W, int Cin, int Cout)
     return plan_conv(N, H, W, Cin, Cout).bn;
 }
 
+int tpfnet_wgrad_parts(int N, int H, int W, int Cin, int Cout)
+{
+    if (N < 1 || H < 1 || W < 1 || Cin < 32 || Cout < 32 || Cin % 32 || Cout % 32) return 0;
+    return plan_wgrad(N, H, W, Cin, Cout, true).splits;
+}
+
 int tpfnet_conv3x3_wgrad_tcgen05(int N, int H, int W, int Cin, int Cout)
 {
-    return N >= 1 && H >= 1 && W >= 1 && Cin % 32 == 0 && Cout % 32 == 0 && wgrad_blocks(N, H, W) && encode_fn() ? 1 : 0;
+    if (N < 1 || H < 1 || W < 1 || Cin < 32 || Cout < 32 || Cin % 32 || Cout % 32) return 0;
+    return plan_wgrad(N, H, W, Cin, Cout, true).CK > 0 ? 1 : 0;
 }
 
 int tpfnet_status(void)
@@ -1813,27 +1943,46 @@ int tpfnet_conv3x3_dgrad(const void* dz, int N, int H, int W, int Cout, const vo
 int tpfnet_conv3x3_wgrad(const void* x, const void* dz, int N, int H, int W, int Cin, int Cout, float* dw, float* db,
                          void* stream)
 {
-    if (!x || !dz || !dw || N < 1 || H < 1 || W < 1 || Cin % kWN || Cout % 32) return TPF_ERR_INVALID_ARG;
-    if (wgrad_tc((const bf16*)x, (const bf16*)dz, N, H, W, Cin, Cout, dw, db, (cudaStream_t)stream))
-        return status(cudaGetLastError());
-    const int WM = Cout % 64 == 0 ? 64 : 32;
-    const long long P = (long long)N * H * W;
-    // split the pixels so that the grid fills the GPU a few times over
-    const long long ctas_per_split = 9LL * (Cin / kWN) * (Cout / WM);
-    long long splits = (152LL * 8 + ctas_per_split - 1) / ctas_per_split;
-    const long long maxsplits = (P + kWK - 1) / kWK;
-    if (splits > maxsplits) splits = maxsplits;
-    if (splits < 1) splits = 1;
-    long long per = (P + splits - 1) / splits;
-    per = (per + kWK - 1) / kWK * kWK;
-    splits = (P + per - 1) / per;
-    dim3 grd(Cin / kWN, Cout / WM, 9 * (int)splits);
-    if (WM == 64)
-        launch_pdl_small(k_conv3x3_wgrad<64>, grd, 128, (cudaStream_t)stream, (const bf16*)x, (const bf16*)dz, N, H, W, Cin, Cout,
-                                                                   (int)per, dw, db);
-    else
-        launch_pdl_small(k_conv3x3_wgrad<32>, grd, 128, (cudaStream_t)stream, (const bf16*)x, (const bf16*)dz, N, H, W, Cin, Cout,
-                                                                   (int)per, dw, db);
+    if (!x || !dz || !dw || N < 1 || H < 1 || W < 1 || Cin < kWN || Cout < 32 || Cin % kWN || Cout % 32)
+        return TPF_ERR_INVALID_ARG;
+    const bool aligned = !(((uintptr_t)x | (uintptr_t)dz) & 15);
+    for (const bool tc : {aligned, false})  // (the mma.sync kernel where the other cannot be launched)
+        if (wgrad(plan_wgrad(N, H, W, Cin, Cout, tc), (const bf16*)x, (const bf16*)dz, N, H, W, Cin, Cout, dw, db, nullptr,
+                  (cudaStream_t)stream))
+            break;
+    return status(cudaGetLastError());
+}
+
+int tpfnet_conv3x3_wgrad_part(const void* x, const void* dz, int N, int H, int W, int Cin, int Cout, float* part,
+                              void* stream)
+{
+    if (!x || !dz || !part || !tpfnet_wgrad_parts(N, H, W, Cin, Cout) ||
+        (((uintptr_t)x | (uintptr_t)dz | (uintptr_t)part) & 15))
+        return TPF_ERR_INVALID_ARG;
+    const bool ok = wgrad(plan_wgrad(N, H, W, Cin, Cout, true), (const bf16*)x, (const bf16*)dz, N, H, W, Cin, Cout, nullptr,
+                          nullptr, part, (cudaStream_t)stream);
+    return ok ? status(cudaGetLastError()) : TPF_ERR_CUDA;
+}
+
+int tpfnet_sum_parts(int n, const float* const* part, const long long* stride, const int* count, const int* parts,
+                     float* const* dst, void* stream)
+{
+    if (n < 1 || n > kMaxSums || !part || !stride || !count || !parts || !dst) return TPF_ERR_INVALID_ARG;
+    SumList L{};
+    for (int i = 0; i < n; ++i) {
+        if (!part[i] || !dst[i] || count[i] < 1 || parts[i] < 1 || stride[i] < count[i]) return TPF_ERR_INVALID_ARG;
+        L.part[i] = part[i];
+        L.dst[i] = dst[i];
+        L.stride[i] = stride[i];
+        L.count[i] = count[i];
+        L.parts[i] = parts[i];
+        // (more partial sums than that are a chain too long for one thread)
+        const bool four = parts[i] <= 64 && ((uintptr_t)part[i] & 15) == 0 && ((uintptr_t)dst[i] & 15) == 0 &&
+                          stride[i] % 4 == 0 && count[i] % 4 == 0;
+        L.four |= (uint32_t)four << i;
+        L.first[i + 1] = L.first[i] + (four ? (count[i] + 1023) / 1024 : (count[i] + 7) / 8);
+    }
+    launch_pdl(k_sum_parts, L.first[n], 256, 0, (cudaStream_t)stream, L, n);
     return status(cudaGetLastError());
 }
 
@@ -1963,18 +2112,26 @@ int tpfnet_head(const void* x, long long pixels, int C, const float* Wt, const f
     return status(cudaGetLastError());
 }
 
+// blocks of k_head_back8, 0 where it does not take the shape
+int tpfnet_head_parts(long long pixels, int C, int Cout)
+{
+    const int G = C / 8;
+    if (pixels < 1 || Cout < 1 || Cout > 8 || C % 8 || G < 1 || G > 32 || (G & (G - 1))) return 0;
+    const long long per = 8 * (32 / G);  // pixels per block and turn
+    return (int)((pixels + per - 1) / per < 152 * 2 ? (pixels + per - 1) / per : 152 * 2);
+}
+
 static int head_back_any(const void* x, const float* dout, long long pixels, int C, const float* Wt, int Cout, void* dx,
-                         float* dW, float* db, int relu, void* stream)
+                         float* dW, float* db, int relu, float* part, void* stream)
 {
     const int smem = (C * Cout + Cout) * (int)sizeof(float);
     if (smem > 48 * 1024) return TPF_ERR_INVALID_ARG;
-    const int G = C / 8;
-    if (pixels > 0 && Cout >= 1 && Cout <= 8 && G >= 1 && G <= 32 && (G & (G - 1)) == 0 && pieces(C, x, dx)) {
-        const long long per = 8 * (32 / G);  // pixels per block and turn
-        const int blocks = (int)((pixels + per - 1) / per < 152 * 2 ? (pixels + per - 1) / per : 152 * 2);
+    const int blocks = pieces(C, x, dx) ? tpfnet_head_parts(pixels, C, Cout) : 0;
+    if (part && !blocks) return TPF_ERR_INVALID_ARG;
+    if (blocks) {
         cudaStream_t s = (cudaStream_t)stream;
         auto run = [&](auto kern) {
-            launch_pdl(kern, blocks, 256, smem, s, (const bf16*)x, dout, pixels, C, Wt, (bf16*)dx, dW, db, relu);
+            launch_pdl(kern, blocks, 256, smem, s, (const bf16*)x, dout, pixels, C, Wt, (bf16*)dx, dW, db, relu, part);
         };
         switch (Cout) {
         case 1: run(k_head_back8<1>); break;
@@ -1997,13 +2154,20 @@ static int head_back_any(const void* x, const float* dout, long long pixels, int
 int tpfnet_head_back(const void* x, const float* dout, long long pixels, int C, const float* Wt, int Cout, void* dx,
                      float* dW, float* db, void* stream)
 {
-    return head_back_any(x, dout, pixels, C, Wt, Cout, dx, dW, db, 0, stream);
+    return head_back_any(x, dout, pixels, C, Wt, Cout, dx, dW, db, 0, nullptr, stream);
 }
 
 int tpfnet_head_back_masked(const void* x, const float* dout, long long pixels, int C, const float* Wt, int Cout,
                             void* dx, float* dW, float* db, void* stream)
 {
-    return head_back_any(x, dout, pixels, C, Wt, Cout, dx, dW, db, 1, stream);
+    return head_back_any(x, dout, pixels, C, Wt, Cout, dx, dW, db, 1, nullptr, stream);
+}
+
+int tpfnet_head_back_part(const void* x, const float* dout, long long pixels, int C, const float* Wt, int Cout,
+                          void* dx, float* part, void* stream)
+{
+    if (!part) return TPF_ERR_INVALID_ARG;
+    return head_back_any(x, dout, pixels, C, Wt, Cout, dx, nullptr, nullptr, 1, part, stream);
 }
 
 int tpfnet_unet_forward(const tpfnet_unet* u, const void* x, int N, int H, int W, float* out, void* stream)
