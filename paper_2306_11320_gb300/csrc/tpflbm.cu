@@ -962,8 +962,6 @@ void setup_many(tpflbm_t h)
             cudaGetLastError();
             return;
         }
-        std::lock_guard<std::mutex> lock(g_wide_lock);
-        g_wide.push_back(h);
     }
     h->many_fn = (const void*)fn;
 }
@@ -1036,7 +1034,15 @@ int finish_create(tpflbm_t h, int nx, int ny, const tpflbm_params* p, void* ws, 
     // The clears and the tile list went over the legacy default stream and may still be under way
     // when their calls return.  The handle's stream need not be ordered after that one, and a
     // step kernel that starts early would take step counts and words of whatever the memory held.
-    if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) return cuda_fail(h, cudaGetLastError(), "set-up");
+    const cudaError_t e = cudaStreamSynchronize(cudaStreamLegacy);
+    if (e != cudaSuccess) {
+        if (h->many_ev) cudaEventDestroy(h->many_ev);
+        return cuda_fail(h, e, "set-up");
+    }
+    if (h->many_ev) {
+        std::lock_guard<std::mutex> lock(g_wide_lock);
+        g_wide.push_back(h);
+    }
     return TPF_OK;
 }
 
