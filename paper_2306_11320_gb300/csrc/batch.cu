@@ -41,8 +41,10 @@ constexpr int kVarBY[kNumVariants] = {4, 8, 16, 4, kStepBY};
 // latency-bound.  FP32 32 x 4 tiles on the 256-lattice ensemble: 0.427 ms per step at 768 (80
 // registers, with spills), 0.403 at 640 (five CTAs, 102 registers), 0.417 at 896, 0.444 at
 // 1,024; FP16 is fastest at 512 (128 registers).  (0.386 at 640 since, see step_tile_general)
-template <class S>
-constexpr int kBatchThreadsPerSM = kRef<S> ? 512 : 640;
+// Tiles of 256 threads come to three CTAs at 768 and to two at 640: 32 x 8 0.432 against 0.443, 64 x
+// 4 0.433 against 0.454.
+template <class S, int TILE>
+constexpr int kBatchThreadsPerSM = kRef<S> ? 512 : (TILE == 256 ? 768 : 640);
 // The instance descriptor of a work item is copied word by word by warp 0 (32-bit words;
 // InstDesc is plain data).  The next item's copy is loaded into registers while the
 // current tile runs and stored into the other shared buffer after it, so no tile waits
@@ -52,7 +54,7 @@ constexpr int kDescPerLane = (kDescWords + 31) / 32;
 static_assert(sizeof(InstDesc) % 4 == 0, "descriptor copied in 32-bit words");
 
 template <int BX, int BY, class S>
-__global__ void __launch_bounds__(BX * BY, kBatchThreadsPerSM<S> / (BX * BY) > 0 ? kBatchThreadsPerSM<S> / (BX * BY) : 1)
+__global__ void __launch_bounds__(BX * BY, kBatchThreadsPerSM<S, BX * BY> / (BX * BY) > 0 ? kBatchThreadsPerSM<S, BX * BY> / (BX * BY) : 1)
 k_step_batch(const InstDesc* __restrict__ inst, const int2* __restrict__ work, int nwork, int parity)
 {
     __shared__ RingSmem<BX, BY> sm;
