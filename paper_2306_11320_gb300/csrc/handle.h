@@ -63,6 +63,7 @@ struct tpflbm {
     std::string err_msg;
 };
 
-// tpflbm_create for a member of an ensemble (without the many-step kernel's memory)
+// tpflbm_create for a member of an ensemble (without the many-step kernel's memory; the caller
+// waits for the default stream, which the set-up goes over, before it uses the member)
 extern "C" __attribute__((visibility("hidden"))) int tpf_create_member(int nx, int ny, const tpflbm_params* p,
                                                                        tpflbm_t* out);

@@ -1000,8 +1000,9 @@ cudaError_t mark_call(tpflbm_t h)
     return cudaEventRecord(h->many_ev, h->stream);
 }
 
+// `wait`: for the set-up (a batch waits once for all its members')
 int finish_create(tpflbm_t h, int nx, int ny, const tpflbm_params* p, void* ws, size_t bytes, bool owns,
-                  bool many)
+                  bool many, bool wait)
 {
     h->nx = nx; h->ny = ny; h->hp = *p;
     h->dp = make_dev_params(nx, ny, *p);
@@ -1034,7 +1035,7 @@ int finish_create(tpflbm_t h, int nx, int ny, const tpflbm_params* p, void* ws, 
     // The clears and the tile list went over the legacy default stream and may still be under way
     // when their calls return.  The handle's stream need not be ordered after that one, and a
     // step kernel that starts early would take step counts and words of whatever the memory held.
-    const cudaError_t e = cudaStreamSynchronize(cudaStreamLegacy);
+    const cudaError_t e = wait ? cudaStreamSynchronize(cudaStreamLegacy) : cudaSuccess;
     if (e != cudaSuccess) {
         if (h->many_ev) cudaEventDestroy(h->many_ev);
         return cuda_fail(h, e, "set-up");
@@ -1148,8 +1149,9 @@ size_t tpflbm_workspace_bytes(int nx, int ny, const tpflbm_params* p)
     return layout_of(nx, ny, p->storage, true).total;
 }
 
-static int create_impl(int nx, int ny, const tpflbm_params* p, bool many, tpflbm_t* out)
+static int create_impl(int nx, int ny, const tpflbm_params* p, bool member, tpflbm_t* out)
 {
+    const bool many = !member;  // an ensemble is stepped as a whole
     if (!out) return fail(nullptr, TPF_ERR_INVALID_ARG, "out is NULL");
     *out = nullptr;
     std::string why;
@@ -1168,7 +1170,7 @@ static int create_impl(int nx, int ny, const tpflbm_params* p, bool many, tpflbm
         cudaFree(ws);
         return fail(nullptr, TPF_ERR_OOM, "host allocation failed");
     }
-    rc = finish_create(h, nx, ny, p, ws, bytes, true, many);
+    rc = finish_create(h, nx, ny, p, ws, bytes, true, many, !member);
     if (rc != TPF_OK) {
         g_create_error = h->err_msg;
         cudaFree(ws);
@@ -1179,11 +1181,11 @@ static int create_impl(int nx, int ny, const tpflbm_params* p, bool many, tpflbm
     return TPF_OK;
 }
 
-int tpflbm_create(int nx, int ny, const tpflbm_params* p, tpflbm_t* out) { return create_impl(nx, ny, p, true, out); }
+int tpflbm_create(int nx, int ny, const tpflbm_params* p, tpflbm_t* out) { return create_impl(nx, ny, p, false, out); }
 
 int tpf_create_member(int nx, int ny, const tpflbm_params* p, tpflbm_t* out)
 {
-    return create_impl(nx, ny, p, false, out);
+    return create_impl(nx, ny, p, true, out);
 }
 
 int tpflbm_create_in(int nx, int ny, const tpflbm_params* p, void* workspace, size_t bytes, tpflbm_t* out)
@@ -1199,7 +1201,7 @@ int tpflbm_create_in(int nx, int ny, const tpflbm_params* p, void* workspace, si
     const bool many = bytes >= layout_of(nx, ny, p->storage, true).total;
     tpflbm_t h = new (std::nothrow) tpflbm;
     if (!h) return fail(nullptr, TPF_ERR_OOM, "host allocation failed");
-    rc = finish_create(h, nx, ny, p, workspace, bytes, false, many);
+    rc = finish_create(h, nx, ny, p, workspace, bytes, false, many, true);
     if (rc != TPF_OK) {
         g_create_error = h->err_msg;
         delete h;
